@@ -62,14 +62,9 @@ void free_rings(lb_handle* h)
     dfree(h->node_force);
     dfree(h->ubox);
     dfree(h->fpbox);
-    dfree(h->node_work);
-    dfree(h->ring_cta0);
-    dfree(h->ring_ctas);
-    dfree(h->ring_tickets);
     dfree(h->box_tickets);
-    dfree(h->ring_claim);
-    dfree(h->node_partials);
-    h->n_node_ctas = 1;
+    h->body_ok = false;
+    h->ckpt_blocks = 1;
     h->n_rings = h->n_total = 0;
     h->tile_rot = 0;
     h->row_len = 6;
@@ -147,12 +142,7 @@ NodeArgs node_args(lb_handle* h, int advance)
     a.walls_y = h->p.walls_y;
     a.walls_x = h->p.walls_x;
     a.advance = advance;
-    a.n_ctas = h->n_node_ctas;
-    a.work = h->node_work;
-    a.ring_cta0 = h->ring_cta0;
-    a.ring_ctas = h->ring_ctas;
-    a.ring_tickets = h->ring_tickets;
-    a.node_partials = h->node_partials;
+    a.n_ctas = std::max(h->n_rings, 1);
     return a;
 }
 
@@ -365,16 +355,7 @@ int lb_create(const lb_params* pin, void* stream, lb_handle** out)
         rc = cuda_fail(nullptr, e, "cudaMalloc(series)");
         return bail(rc);
     }
-    {
-        const int2 w0 = make_int2(-1, 0);
-        if ((e = cudaMalloc(&h->node_work, sizeof(int2))) != cudaSuccess ||
-            (e = cudaMemcpy(h->node_work, &w0, sizeof(int2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-            (e = cudaMalloc(&h->node_partials, sizeof(double) * NODE_PARTIALS)) != cudaSuccess) {
-            rc = cuda_fail(nullptr, e, "cudaMalloc(node work)");
-            return bail(rc);
-        }
-        h->n_node_ctas = 1;
-    }
+    h->body_ok = true;
     *out = h;
     return LB_OK;
 }
@@ -425,7 +406,6 @@ int lb_init_fields(lb_handle* h, const double* noise)
     if (h->n_rings > 0) {
         // restart at t = 0: the work box of the current positions into the slot of even steps
         CK(h, cudaMemsetAsync(h->box_tickets, 0, sizeof(unsigned) * h->n_rings, h->stream));
-        CK(h, cudaMemsetAsync(h->ring_claim, 0, sizeof(unsigned long long) * h->n_rings, h->stream));
         CK(h, launch_nodes(node_args(h, 0), h->stream));
     }
     h->fields_ready = true;
@@ -446,7 +426,7 @@ int lb_set_body(lb_handle* h, int32_t n_rings, const lb_ring* rings, const doubl
     int off = 0;
     for (int r = 0; r < n_rings; ++r) {
         const lb_ring& g = rings[r];
-        if (g.n_nodes < 3 || g.n_nodes > 1024) return fail(h, LB_EINVAL, "ring %d: 3 <= n_nodes <= 1024", r);
+        if (g.n_nodes < 3 || g.n_nodes > MAX_RING_NODES) return fail(h, LB_EINVAL, "ring %d: 3 <= n_nodes <= 1024", r);
         if (!(g.l_eq > 0.0) || g.k_spring < 0.0) return fail(h, LB_EINVAL, "ring %d: bad spring", r);
         if (!(g.trap_k >= 0.0) || (g.trap_k > 0.0 && !(g.trap_width > 0.0 && g.trap_pull > 0.0 &&
                                                        std::isfinite(g.trap_dx) && std::isfinite(g.trap_dy) &&
@@ -517,29 +497,12 @@ int lb_set_body(lb_handle* h, int32_t n_rings, const lb_ring* rings, const doubl
     h->n_total = off;
     h->row_len = 6 + 4 * n_rings;
     h->box_floats = box_off;
-    // node-kernel work: NB owned nodes per CTA (one CTA with no ring when there are no rings)
-    std::vector<int2> work;
-    std::vector<int> cta0(std::max(n_rings, 1)), nctas(std::max(n_rings, 1));
-    for (int r = 0; r < n_rings; ++r) {
-        cta0[r] = (int)work.size();
-        for (int k0 = 0; k0 < rd[r].n_nodes; k0 += NB) work.push_back(make_int2(r, k0));
-        nctas[r] = (int)work.size() - cta0[r];
-    }
-    if (work.empty()) work.push_back(make_int2(-1, 0));
-    h->n_node_ctas = (int)work.size();
-    CK(h, cudaMalloc(&h->node_work, sizeof(int2) * work.size()));
-    CK(h, cudaMalloc(&h->ring_cta0, sizeof(int) * cta0.size()));
-    CK(h, cudaMalloc(&h->ring_ctas, sizeof(int) * nctas.size()));
-    CK(h, cudaMalloc(&h->ring_tickets, sizeof(unsigned) * nctas.size()));
-    CK(h, cudaMalloc(&h->node_partials, sizeof(double) * NODE_PARTIALS * work.size()));
-    CK(h, cudaMemcpy(h->node_work, work.data(), sizeof(int2) * work.size(), cudaMemcpyHostToDevice));
-    CK(h, cudaMemcpy(h->ring_cta0, cta0.data(), sizeof(int) * cta0.size(), cudaMemcpyHostToDevice));
-    CK(h, cudaMemcpy(h->ring_ctas, nctas.data(), sizeof(int) * nctas.size(), cudaMemcpyHostToDevice));
-    CK(h, cudaMemset(h->ring_tickets, 0, sizeof(unsigned) * nctas.size()));
-    CK(h, cudaMalloc(&h->box_tickets, sizeof(unsigned) * nctas.size()));
-    CK(h, cudaMemset(h->box_tickets, 0, sizeof(unsigned) * nctas.size()));
-    CK(h, cudaMalloc(&h->ring_claim, sizeof(unsigned long long) * nctas.size()));
-    CK(h, cudaMemset(h->ring_claim, 0, sizeof(unsigned long long) * nctas.size()));
+    int blocks60 = 0;
+    for (const RingDev& d : rd) blocks60 += (d.n_nodes + 59) / 60;
+    h->ckpt_blocks = std::max(blocks60, 1);
+    CK(h, cudaMalloc(&h->box_tickets, sizeof(unsigned) * std::max(n_rings, 1)));
+    CK(h, cudaMemset(h->box_tickets, 0, sizeof(unsigned) * std::max(n_rings, 1)));
+    h->body_ok = true;
     if (n_rings > 0) {
         CK(h, cudaMalloc(&h->rings, sizeof(RingDev) * n_rings));
         CK(h, cudaMalloc(&h->X, sizeof(double2) * off));
@@ -569,7 +532,7 @@ int lb_step(lb_handle* h, int64_t n)
     if (!h) return fail(nullptr, LB_EINVAL, "null handle");
     if (n < 0) return fail(h, LB_EINVAL, "n < 0");
     if (!h->fields_ready) return fail(h, LB_ESTATE, "lb_init_fields not called");
-    if (!h->node_work) return fail(h, LB_ESTATE, "no valid body: call lb_set_body again");
+    if (!h->body_ok) return fail(h, LB_ESTATE, "no valid body: call lb_set_body again");
     for (int64_t k = 0; k < n; ++k) {
         FusedArgs fa = fused_args(h);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -603,7 +566,6 @@ int lb_step(lb_handle* h, int64_t n)
                 fa.t = h->t;
                 fa.tile_rot = h->tile_rot;
                 fa.box_tickets = h->box_tickets;
-                fa.ring_claim = h->ring_claim;
                 fa.na = node_args(h, 1);
             }
             // without the tail, a lattice kernel stages the state before its dependency wait,

@@ -3,7 +3,7 @@
 //
 // Default (phase launches): each step is one launch per phase and tile-shape group -- all
 // instances' lattice tiles (k_batch_tiles, the tile kernel's occupancy of three CTAs per SM),
-// their diffusion sub-steps, then their node blocks -- in stream order, so no kernel waits on
+// their diffusion sub-steps, then their rings' node steps -- in stream order, so no kernel waits on
 // another inside a launch.  Alternatively (lb_batch_set_persistent) one persistent cooperative
 // kernel per group runs the whole chunk, each step having three phases separated by a grid
 // barrier:
@@ -45,7 +45,10 @@ __host__ __device__ constexpr int shape_ty(int s) { return s == 0 ? 16 : (s == 1
 constexpr size_t cmaxz(size_t a, size_t b) { return a > b ? a : b; }
 // dynamic shared memory of the kernel of one tile shape
 template <int TX, int TY>
-constexpr size_t batch_smem() { return cmaxz(tile::TileGeo<TX, TY>::SMEM_BYTES, sizeof(float) * dif::SMEM); }
+constexpr size_t batch_smem()
+{
+    return cmaxz(cmaxz(tile::TileGeo<TX, TY>::SMEM_BYTES, sizeof(float) * dif::SMEM), sizeof(node::NodeSmem));
+}
 
 struct BatchInst {
     FusedArgs fa[2];            // lattice step from buffer p to buffer p^1, p = 0, 1
@@ -62,7 +65,7 @@ struct BatchArgs {
     const BatchInst* inst;
     int n_inst;
     const int* tile_begin;      // prefix sums of lattice tiles over instances (n_inst + 1)
-    const int* node_begin;      // prefix sums of node blocks
+    const int* node_begin;      // prefix sums of rings (one for an instance without)
     const int* dif_begin;       // prefix sums of diffusion tiles (instances with dsub > 0)
     int max_dsub;
     int* cur;                   // buffer parity of the current state (device)
@@ -182,7 +185,7 @@ __global__ void __launch_bounds__(BT, 2) k_batch(const BatchArgs B, int nsteps)
             na.X = B.inst[i].xb[par];
             na.X_out = B.inst[i].xb[par ^ 1];
             // the tiles' shared memory is free in this phase
-            node::node_block(na, item - __ldg(B.node_begin + i), *reinterpret_cast<node::NodeSmem*>(sm));
+            node::node_ring(na, na.n_rings > 0 ? item - __ldg(B.node_begin + i) : -1, *reinterpret_cast<node::NodeSmem*>(sm));
             __syncthreads();
         }
         ok = grid_sync(B);
@@ -261,7 +264,7 @@ __global__ void __launch_bounds__(NODE_THREADS) k_batch_nodes(const BatchArgs B,
     NodeArgs na = B.inst[i].na;
     na.X = B.inst[i].xb[par];
     na.X_out = B.inst[i].xb[par ^ 1];
-    node::node_block(na, item - __ldg(B.node_begin + i), S);
+    node::node_ring(na, na.n_rings > 0 ? item - __ldg(B.node_begin + i) : -1, S);
 }
 
 // the buffer parity after a chunk of n steps
@@ -372,7 +375,7 @@ int build_plan(lb_batch* b)
             I.dif_ty = diffuse_tiles_y(h->p.ny);
             b->max_dsub[sh] = std::max(b->max_dsub[sh], I.dsub);
             tb.push_back(tb.back() + I.tiles_x * I.tiles_y);
-            nb.push_back(nb.back() + h->n_node_ctas);
+            nb.push_back(nb.back() + I.na.n_ctas);
             db.push_back(db.back() + (I.dsub > 0 ? I.dif_tx * I.dif_ty : 0));
             inst.push_back(I);
         }
@@ -582,7 +585,7 @@ int lb_batch_create(lb_handle* const* handles, int32_t n, lb_batch** out)
     *out = nullptr;
     for (int i = 0; i < n; ++i) {
         const lb_handle* h = handles[i];
-        if (!h || !h->fields_ready || !h->node_work) return LB_ESTATE;
+        if (!h || !h->fields_ready || !h->body_ok) return LB_ESTATE;
         if (h->p.precision != LB_FP32 || h->p.model != handles[0]->p.model || h->cur != handles[0]->cur ||
             h->stream != handles[0]->stream)
             return LB_EINVAL;

@@ -28,7 +28,7 @@ struct Header {
     lb_params p;
     int64_t plane, box_floats;
     int32_t esz, partial_cap, series_cap, row_len;
-    int32_t n_rings, n_total, n_node_ctas, n_bufs;
+    int32_t n_rings, n_total, node_blocks, n_bufs;
     int64_t payload_bytes;
     // host state
     int64_t t;
@@ -40,14 +40,17 @@ struct Buf {
     size_t bytes;
 };
 
-// The buffers of the snapshot, in file order; a null pointer stands for a buffer the handle does
-// not have (no rings yet), and is stored as zero bytes.
+// The buffers of the snapshot, in file order; a buffer the handle does not have (no rings yet)
+// takes no bytes, a null pointer with bytes is a section of zeros that a load skips.
 std::vector<Buf> snapshot_bufs(lb_handle* h)
 {
     const size_t state_bytes = (size_t)h->esz * vlb::N_PLANES * (size_t)h->plane;
     const size_t nr = (size_t)(h->n_rings > 0 ? h->n_rings : 1);     // ticket arrays hold >= 1
     const size_t nt = (size_t)h->n_total;
     auto B = [](void* p, size_t n) { return Buf{p, p ? n : 0}; };
+    // reserved sections of the file format (zero bytes): per-ring and per-block scratch that an
+    // earlier node step kept between its launches, dead between steps
+    auto Z = [](size_t n) { return Buf{nullptr, n}; };
     return {
         B(h->state[0], state_bytes),
         B(h->state[1], state_bytes),
@@ -62,10 +65,10 @@ std::vector<Buf> snapshot_bufs(lb_handle* h)
         B(h->node_force, sizeof(float2) * nt),
         B(h->ubox, sizeof(float) * (size_t)h->box_floats),
         B(h->fpbox, sizeof(float) * (size_t)h->box_floats),
-        B(h->ring_tickets, sizeof(unsigned) * nr),
+        Z(h->box_tickets ? sizeof(unsigned) * nr : 0),
         B(h->box_tickets, sizeof(unsigned) * nr),
-        B(h->ring_claim, sizeof(unsigned long long) * nr),
-        B(h->node_partials, sizeof(double) * vlb::NODE_PARTIALS * (size_t)h->n_node_ctas),
+        Z(h->box_tickets ? sizeof(unsigned long long) * nr : 0),
+        Z(sizeof(double) * 10 * (size_t)h->ckpt_blocks),
     };
 }
 
@@ -85,7 +88,7 @@ Header make_header(lb_handle* h, const std::vector<Buf>& bufs)
     hd.row_len = h->row_len;
     hd.n_rings = h->n_rings;
     hd.n_total = h->n_total;
-    hd.n_node_ctas = h->n_node_ctas;
+    hd.node_blocks = h->ckpt_blocks;
     hd.n_bufs = (int32_t)bufs.size();
     hd.payload_bytes = 0;
     for (const Buf& b : bufs) hd.payload_bytes += (int64_t)b.bytes;
@@ -115,7 +118,7 @@ bool same_layout(const Header& a, const Header& b)
 {
     return same_params(a.p, b.p) && a.plane == b.plane && a.box_floats == b.box_floats && a.esz == b.esz &&
            a.partial_cap == b.partial_cap && a.series_cap == b.series_cap && a.row_len == b.row_len &&
-           a.n_rings == b.n_rings && a.n_total == b.n_total && a.n_node_ctas == b.n_node_ctas &&
+           a.n_rings == b.n_rings && a.n_total == b.n_total && a.node_blocks == b.node_blocks &&
            a.n_bufs == b.n_bufs && a.payload_bytes == b.payload_bytes;
 }
 
@@ -147,7 +150,7 @@ int lb_save(lb_handle* h, const char* path)
     std::vector<char> host((size_t)hd.payload_bytes);
     size_t off = 0;
     for (const Buf& b : bufs) {
-        if (b.bytes) {
+        if (b.ptr && b.bytes) {
             e = cudaMemcpyAsync(host.data() + off, b.ptr, b.bytes, cudaMemcpyDeviceToHost, h->stream);
             if (e != cudaSuccess) return cuda_err(h, e, "lb_save: copy to host");
         }
@@ -228,7 +231,7 @@ int lb_load(lb_handle* h, const char* path)
     }
     size_t off = 0;
     for (const Buf& b : bufs) {
-        if (b.bytes) {
+        if (b.ptr && b.bytes) {
             e = cudaMemcpyAsync(b.ptr, host.data() + off, b.bytes, cudaMemcpyHostToDevice, h->stream);
             if (e != cudaSuccess) return cuda_err(h, e, "lb_load: copy to device (handle state undefined)");
         }

@@ -27,159 +27,88 @@ __device__ __forceinline__ int tiles_meeting(int n_tiles, int T, int RW, int b, 
     return cnt;
 }
 
-// One open node block of a ring at step tag (t + 1): increments the claim count of
-// ring_claim (tag << 16 | count) while it is below nc and returns the claimed block, or -1.
-// Each failed exchange means another CTA claimed a block, so at most nc + 1 rounds run; the
-// bound only guards that argument.
-__device__ __forceinline__ int claim_block(unsigned long long* p, unsigned long long tag, int nc, int* err)
-{
-    unsigned long long w = __ldcg(p);
-    for (int it = 0; it < 4096; ++it) {
-        if ((w >> 16) != tag || (int)(w & 0xffffu) >= nc) return -1;
-        const unsigned long long old = atomicCAS(p, w, w + 1);
-        if (old == w) return (int)(w & 0xffffu);
-        w = old;
-    }
-    atomicExch(err, 1);
-    return -1;
-}
-
-// Node blocks of the rings in `open` (bits; ring r0 + bit), claimed one at a time, then (last)
-// the lattice readout sums: the rare parts of the node tail, kept out of line so that the tiles
-// that have none of it pay nothing for them.  The node blocks take the tile's shared memory,
-// whose staged fields are dead once every thread has passed the barrier at the start.
-__device__ __noinline__ void tail_work(const FusedArgs& a, unsigned open, int r0, bool last, float* sm)
-{
-    node::NodeSmem& S = *reinterpret_cast<node::NodeSmem*>(sm);
-    const int tid = threadIdx.x;
-    const long long t = a.t;
-    const unsigned long long tag = (unsigned long long)(t + 1);
-    __syncthreads();
-    while (open) {
-        const int r = r0 + __ffs(open) - 1;
-        open &= open - 1;
-        const int c0 = a.na.ring_cta0[r], nc = a.na.ring_ctas[r];
-        for (;;) {
-            __syncthreads();
-            if (tid == 0) S.flag[0] = claim_block(a.ring_claim + r, tag, nc, &a.ctl->err_timeout);
-            __syncthreads();
-            const int c = S.flag[0];
-            if (c < 0) break;
-            __threadfence();
-            node::node_block(a.na, c0 + c, S, false, t);
-        }
-    }
-    if (last) {
-        __syncthreads();
-        __threadfence();
-        if (tid == 0) a.ctl->tile_ticket = 0u;
-        node::lattice_readout(a.na, t, S.dred);
-    }
-}
-
-// tiles that look for open node blocks in their tail: one in 32 in launch order, and all of the
-// last thirty-second (rings whose tiles run late still find helpers)
-__device__ __forceinline__ bool helper_tile()
-{
-    const int order = blockIdx.y * gridDim.x + blockIdx.x, total = gridDim.x * gridDim.y;
-    return (order & 31) == 0 || order >= total - total / 32;
-}
-
 // The node step in the tail of the lattice kernel (FusedArgs::node_tail), after this tile's
 // step (App. A).  A ring's nodes are read (spreading) only by the tiles whose region meets its
 // box of step t, and the node update writes only the box of step t + 1 (RingDev::box), the
 // nodes and the other position buffer: so once the last of those tiles has written u(t) and
-// f^p(t) onto the box, the ring can advance while the remaining tiles run.  That tile opens the
-// ring's node blocks; it and the helper tiles that finish later (helper_tile, and any tile that
-// met a ring) run them, one claimed block at a time.  On readout steps every tile counts itself
-// and the last one sums the lattice readout.  Flags live in the scan scratch of ib_gather (free
-// by now; the ring masks after it stay intact).  Out of line: node_tail below calls it only for
-// the tiles that have something to do.
+// f^p(t) onto the box, the ring can advance while the remaining tiles run.  That tile advances
+// it (node_ring), in the tile's shared memory, whose staged fields are dead by then.  On readout
+// steps every tile counts itself and the last one sums the lattice readout.  A thread's arrival
+// stands for the whole CTA: the barrier orders the CTA's writes before its fence.  Out of line:
+// node_tail below calls it only for the tiles that have something to do.
 template <int TX, int TY>
-__device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm)
+__device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm, unsigned meet)
 {
     using G = TileGeo<TX, TY>;
-    static_assert(sizeof(node::NodeSmem) <= sizeof(float) * G::OFF_SC, "node blocks overlay the staged fields only");
-    int* sT = reinterpret_cast<int*>(sm + G::OFF_SC);
-    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    node::NodeSmem& S = *reinterpret_cast<node::NodeSmem*>(sm);
+    const int tid = threadIdx.x;
     const int nr = a.n_rings;
     const long long t = a.t;
     const int bx = blockIdx.x;
     int by = blockIdx.y + a.tile_rot;
     if (by >= (int)gridDim.y) by -= gridDim.y;
-    bool helper = helper_tile();
-    const bool readout = (t % a.every) == 0;
-    const unsigned meet = nr > 32 ? 0xffffffffu : (unsigned)sT[NT / 32 + 2];
-    const unsigned long long tag = (unsigned long long)(t + 1);
-    // the CTA's global writes of the step (state, boxes, partials) before any of its arrivals
-    __threadfence();
+    __syncthreads();            // the tile's writes are out, its shared memory is free
     for (int r = 0; r < nr && meet != 0u; ++r) {
         if (nr <= 32 && !((meet >> r) & 1u)) continue;
         const int4 B = ring_box(a.rings[r], t);
         if (nr > 32 &&
             (!meets(bx * TX - 2, G::R2W, B.x, B.z, a.nx) || !meets(by * TY - 2, G::R2H, B.y, B.w, a.ny)))
             continue;
-        helper = true;
-        if (wid == 0) {
-            const int c = tiles_meeting(gridDim.x, TX, G::R2W, B.x, B.z, a.nx);
-            if (lane == 0) sT[0] = c;
-        } else if (wid == 1) {
-            const int c = tiles_meeting(gridDim.y, TY, G::R2H, B.y, B.w, a.ny);
-            if (lane == 0) sT[1] = c;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            const unsigned prev = atomicAdd(&a.box_tickets[r], 1u);
-            if (prev == (unsigned)(sT[0] * sT[1] - 1)) {
-                // every tile meeting the box is done with it: open the ring's node blocks
-                a.box_tickets[r] = 0u;
+        if (tid < 32) {
+            const int c = tiles_meeting(gridDim.x, TX, G::R2W, B.x, B.z, a.nx) *
+                          tiles_meeting(gridDim.y, TY, G::R2H, B.y, B.w, a.ny);
+            if (tid == 0) {
                 __threadfence();
-                atomicExch(&a.ring_claim[r], tag << 16);
+                const bool last = atomicAdd(&a.box_tickets[r], 1u) == (unsigned)(c - 1);
+                if (last) {
+                    a.box_tickets[r] = 0u;
+                    __threadfence();
+                }
+                S.flag = last;
             }
         }
         __syncthreads();
+        const bool last = S.flag != 0;
+        if (last) node::node_ring(a.na, r, S, false, t);
+        __syncthreads();
     }
-    // open node blocks of any ring (helpers), 32 rings at a time
-    for (int r0 = 0; r0 < (helper ? nr : 0); r0 += 32) {
-        if (wid == 0) {
-            const int r = r0 + lane;
-            bool open = false;
-            if (r < nr) {
-                const unsigned long long w = __ldcg(a.ring_claim + r);
-                open = (w >> 16) == tag && (int)(w & 0xffffu) < a.na.ring_ctas[r];
+    if ((t % a.every) == 0) {
+        if (tid == 0) {
+            __threadfence();
+            const bool last = atomicAdd(&a.ctl->tile_ticket, 1u) == gridDim.x * gridDim.y - 1u;
+            if (last) {
+                a.ctl->tile_ticket = 0u;
+                __threadfence();
             }
-            const unsigned m = __ballot_sync(0xffffffffu, open);
-            if (lane == 0) sT[2] = (int)m;
+            S.flag = last;
         }
         __syncthreads();
-        const unsigned m = (unsigned)sT[2];
-        if (m) tail_work(a, m, r0, false, sm);
-        __syncthreads();
-    }
-    if (readout) {
-        // every tile counts itself; the last one sums the lattice readout
-        __syncthreads();
-        if (tid == 0) sT[3] = atomicAdd(&a.ctl->tile_ticket, 1u) == gridDim.x * gridDim.y - 1u;
-        __syncthreads();
-        if (sT[3]) tail_work(a, 0u, 0, true, sm);
+        if (S.flag) node::lattice_readout(a.na, t, S.dred);
     }
 }
 
 // The node tail of one tile: the step counter (one tile), then node_tail_work where this tile
-// meets a ring's box, is a helper, or the step is a readout step; nothing else for most tiles.
+// meets a ring's box or the step is a readout step; nothing else for most tiles.
 template <int TX, int TY>
 __device__ __forceinline__ void node_tail(const FusedArgs& a, float* sm)
 {
     using G = TileGeo<TX, TY>;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) a.ctl->t = a.t + 1;   // nothing here reads it
-    const int* sT = reinterpret_cast<const int*>(sm + G::OFF_SC);
     // the rings whose box meets this tile's staged region (tested in ib_gather for up to 32 rings)
-    if (a.n_rings > 32 || sT[NT / 32 + 2] != 0 || helper_tile() || (a.t % a.every) == 0)
-        node_tail_work<TX, TY>(a, sm);
+    const unsigned meet =
+        a.n_rings > 32 ? 0xffffffffu : (unsigned)reinterpret_cast<const int*>(sm + G::OFF_SC)[NT / 32 + 2];
+    if (meet != 0u || (a.t % a.every) == 0) node_tail_work<TX, TY>(a, sm, meet);
+}
+
+// dynamic shared memory of a tile kernel: the tile's, or a ring's node step after it
+template <int TX, int TY>
+constexpr size_t tile_smem()
+{
+    return TileGeo<TX, TY>::SMEM_BYTES > sizeof(node::NodeSmem) ? TileGeo<TX, TY>::SMEM_BYTES : sizeof(node::NodeSmem);
 }
 
 template <int MODE, int PREC, bool SCALAR = false>
-__global__ void __launch_bounds__(NT, 3) k_fused(const FusedArgs a)
+__global__ void __launch_bounds__(NT, 3) k_fused(const __grid_constant__ FusedArgs a)
 {
     extern __shared__ __align__(16) float sm[];
     const bool tail = MODE == MODE_STEP && a.node_tail;
@@ -195,7 +124,7 @@ __global__ void __launch_bounds__(NT, 3) k_fused(const FusedArgs a)
 }
 
 template <int MODE, int PREC>
-__global__ void __launch_bounds__(NT, 2) k_fused_pair(const FusedArgs a)
+__global__ void __launch_bounds__(NT, 2) k_fused_pair(const __grid_constant__ FusedArgs a)
 {
     extern __shared__ __align__(16) float sm[];
     const bool tail = MODE == MODE_STEP && a.node_tail;
@@ -229,7 +158,7 @@ static cudaError_t launch_one(const FusedArgs& a, dim3 grid, cudaStream_t s, boo
     auto kern = PAIR ? k_fused_pair<MODE, PREC> : k_fused<MODE, PREC, SCALAR>;
     if (!done_on_device(attr_done)) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)TileGeo<TILE_X, TILE_Y>::SMEM_BYTES);
+                                             (int)tile_smem<TILE_X, TILE_Y>());
         if (e != cudaSuccess) {
             attr_done = 0;
             return e;
@@ -238,7 +167,7 @@ static cudaError_t launch_one(const FusedArgs& a, dim3 grid, cudaStream_t s, boo
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = TileGeo<TILE_X, TILE_Y>::SMEM_BYTES;
+    cfg.dynamicSmemBytes = tile_smem<TILE_X, TILE_Y>();
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

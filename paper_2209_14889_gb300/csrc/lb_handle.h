@@ -46,17 +46,13 @@ struct lb_handle {
     float2* node_force = nullptr;
     float* ubox = nullptr;
     float* fpbox = nullptr;
-    int n_node_ctas = 1;
-    int2* node_work = nullptr;
-    int* ring_cta0 = nullptr;
-    int* ring_ctas = nullptr;
-    unsigned* ring_tickets = nullptr;
+    bool body_ok = false;                   // the ring set-up (or none) is complete
+    int ckpt_blocks = 1;                    // blocks of 60 nodes of all rings (at least 1): sizes the
+                                            // reserved sections of a checkpoint file
     unsigned* box_tickets = nullptr;        // per ring: tile arrivals of the node tail
-    unsigned long long* ring_claim = nullptr;   // per ring: open node blocks of the node tail
     bool node_tail = true;                  // node step in the lattice kernel's tail (tile kernels)
     bool after_tail = false;                // the last lattice launch ran the node tail
     int tile_rot = 0;                       // first tile row of the tail launches
-    double* node_partials = nullptr;
     long long box_floats = 0;
     bool fields_ready = false;
     long long t = 0;

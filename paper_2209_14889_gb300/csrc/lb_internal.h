@@ -68,21 +68,14 @@ struct Ctl {
     unsigned int tile_ticket;    // tile arrivals of a lattice kernel with the node tail (readout steps)
 };
 
-// Node kernel geometry: NB owned nodes per CTA, NODE_THREADS >= NB + 4 threads.
-constexpr int NB = 60;
-constexpr int NODE_PARTIALS = 10;
-constexpr int NODE_THREADS = 64;
+// Node step geometry: one CTA of NODE_THREADS threads per ring of up to MAX_RING_NODES nodes.
+constexpr int NODE_THREADS = 256;
+constexpr int MAX_RING_NODES = 1024;
 
 struct NodeArgs {
     int n_rings;
     RingDev* rings;
-    int n_ctas;                  // node-kernel CTAs (>= 1)
-    const int2* work;            // per CTA: (ring or -1, first owned node)
-    const int* ring_cta0;        // per ring: first CTA, number of CTAs
-    const int* ring_ctas;
-    unsigned* ring_tickets;      // per ring: arrival counter
-    double* node_partials;       // per CTA (NODE_PARTIALS): F_rest (2), COM (2), box min/max (4),
-                                 // COM of the advanced positions (2)
+    int n_ctas;                  // CTAs of a node launch: one per ring, at least one
     const double2* X;            // FP64 master node positions, wrapped into [0, n) (read)
     double2* X_out;              // the advanced positions (written; a different buffer than X when
                                  // advancing: other CTAs read their halo nodes from X meanwhile)
@@ -130,18 +123,16 @@ struct FusedArgs {
     float* forces_out;           // MOMENTS mode, optional: Fx, Fy planes (total lattice force)
     // STEP mode with node_tail = 1: the node step of the same time step runs in the kernel's
     // tail.  Every tile whose staged region meets a ring's work box counts itself in
-    // box_tickets[ring] once its u (and f^p) box writes are out; the last of them opens the
-    // ring's node blocks (na, as the node kernel would run them) in ring_claim, and every tile
-    // that finishes later claims and runs open blocks one at a time.  Only the tiles that meet
-    // the box of step t read a ring's nodes, and the node update writes the box of step t + 1,
-    // so the update needs no second launch.  The step index comes from the host (t), and
-    // ctl->t is advanced during the launch.
+    // box_tickets[ring] once its u (and f^p) box writes are out; the last of them runs the ring's
+    // node step (na, as the node kernel would run it).  Only the tiles that meet the box of step t
+    // read a ring's nodes, and the node update writes the box of step t + 1, so the update needs
+    // no second launch.  The step index comes from the host (t), and ctl->t is advanced during
+    // the launch.
     int node_tail;
     int tile_rot;                // node_tail: the launch order starts at this tile row, so that
                                  // the tiles over the first ring run early
     long long t;                 // node_tail: the step index
     unsigned* box_tickets;       // node_tail, per ring: arrivals of the tiles meeting its box
-    unsigned long long* ring_claim;   // node_tail, per ring: (t + 1) << 16 | blocks claimed
     NodeArgs na;                 // node step of this time step (node_tail)
 };
 

@@ -1,22 +1,26 @@
-// lb_node.cuh -- the node step (device code shared by the node kernel and the batched persistent
-// kernel; App. A).
+// lb_node.cuh -- the node step (device code shared by the node kernel, the tail of the tile
+// kernels and the batched kernels; App. A).
 //
-// Per step, after the fused lattice kernel of the same step has written u(t) (and, on readout
-// steps, f^p(t)) onto the ring's work box:
+// Per step, after the lattice kernel of the same step has written u(t) (and, on readout steps,
+// f^p(t)) onto the ring's work box:
 //   * readout (t % every == 0): restoring force sum_a sum_r f^p(r) K(R_a - r) and the centre of
-//     mass of R(t), FP64 sums in a fixed order; CTA 0 also reduces the per-CTA partial sums of
-//     the lattice kernel (mass, momentum, total force) in a fixed order;
+//     mass of R(t), FP64 sums in a fixed order; the last CTA also reduces the per-CTA partial sums
+//     of the lattice kernel (mass, momentum, total force) in a fixed order;
 //   * overdamped advection dR/dt = v(R) by Heun on the frozen u(t): R* = R + v(R),
 //     R' = R + (v(R) + v(R*))/2, v interpolated with the cosine kernel (FP32 weights);
 //   * Lagrangian forces of R' (Eq. Const: springs, angle terms, constant pull split over the
 //     nodes), gathered per node without atomics, and the work box of R' for the next step.
 // Node positions are kept in FP64 (O(N_nodes) data) and advanced in FP64; the forces are
-// evaluated in FP32 except the spring extension, whose l^2 - l_eq^2 is formed in FP64 (FP64 is
-// a narrow unit on this GPU, so it is kept to a few operations per node).  The lattice kernel
-// sees the nodes as int32 cell + FP32 fraction with FP32 forces.  One CTA owns NB nodes of one
-// ring and recomputes the advance of HALO neighbours on each side, so no CTA waits for
-// another; the last CTA of a ring writes the ring's box and readouts, the last CTA overall the
-// lattice readouts and the step counter.
+// evaluated in FP32 except the spring extension, whose l^2 - l_eq^2 is formed in FP64.  The
+// lattice kernel sees the nodes as int32 cell + FP32 fraction with FP32 forces.
+//
+// The node step of a small lattice is pure latency: it stands between the last tile of a step and
+// the first gather of the next.  So one CTA advances a whole ring (thread k the nodes k, k + 256,
+// ...), with the edges exchanged through shared memory: three barriers, no partial results in
+// global memory, no arrival counters between CTAs.  Blocks of 60 nodes on CTAs of their own, with
+// the ring's sums and box put together by the last of them, took 27 000 cycles a block (157 nodes
+// and the trap: 110 000 cycles, 53 of the 74 us of a 250^2 step).  FP64 instructions occupy the SM's FP64
+// pipe for 16 cycles each, so cells and offsets are integers and FP32 wherever they are exact.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -25,8 +29,6 @@
 
 namespace vlb {
 namespace node {
-
-constexpr int HALO = 2;                       // neighbours whose advance a CTA recomputes
 
 // Node positions are kept in [0, n); one step moves a node by less than one cell, and offsets
 // between nodes of a ring are below n/2, so single conditional corrections replace fmod.
@@ -51,42 +53,25 @@ __device__ __forceinline__ int wrapi1(int i, int n)
     return i;
 }
 
-// The four cosine-kernel weights phi(f + 1), phi(f), phi(f - 1), phi(f - 2) of a node at
-// fraction f in [0, 1) (App. A): with c = cos(pi f / 2), s = sin(pi f / 2) they are
-// (1 - s)/4, (1 + c)/4, (1 + s)/4, (1 - c)/4 (quarter-period shifts of the cosine).
-__device__ __forceinline__ void phi4(float f, float* w)
+// Interpolate a 2-component box field for a node at cell (cx, cy) in [0, n) with fractions
+// (fx, fy); returns false if a support cell lies outside the box.
+__device__ __forceinline__ bool interp_box(const float* box, int cap_w, long long cap, const int4& B, int nx, int ny,
+                                           int cx, int cy, float fx, float fy, float& vx, float& vy)
 {
-    float sn, cs;
-    sincospif(0.5f * f, &sn, &cs);
-    w[0] = 0.25f * (1.f - sn);
-    w[1] = 0.25f * (1.f + cs);
-    w[2] = 0.25f * (1.f + sn);
-    w[3] = 0.25f * (1.f - cs);
-}
-
-// Interpolate a 2-component box field at the position (X, Y) in [0, n); returns false if a
-// support cell lies outside the box.
-__device__ __forceinline__ bool interp_box(const float* box, const RingDev& R, int bx0, int by0,
-                                           int bw, int bh, int nx, int ny, double X, double Y,
-                                           float& vx, float& vy)
-{
-    const int cx = (int)X, cy = (int)Y;              // X, Y >= 0
-    const long long cap = (long long)R.cap_w * R.cap_h;
-    const int ox = wrapi1(cx - 1 - bx0, nx), oy = wrapi1(cy - 1 - by0, ny);
+    const int ox = wrapi1(wrapi1(cx - 1, nx) - B.x, nx), oy = wrapi1(wrapi1(cy - 1, ny) - B.y, ny);
     vx = 0.f;
     vy = 0.f;
-    if (ox + 3 >= bw || oy + 3 >= bh) return false;   // the box never wraps onto itself
-    float wx[4], wy[4];
-    phi4((float)(X - cx), wx);
-    phi4((float)(Y - cy), wy);
-    const float* p = box + R.box_off + (long long)oy * R.cap_w + ox;
+    if (ox < 0 || oy < 0 || ox + 3 >= B.z || oy + 3 >= B.w) return false;   // the box never wraps onto itself
+    const float4 a = cell::phi4(fx), b = cell::phi4(fy);
+    const float wx[4] = {a.x, a.y, a.z, a.w}, wy[4] = {b.x, b.y, b.z, b.w};
+    const float* p = box + (long long)oy * cap_w + ox;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float w = wx[i] * wy[j];
-            vx += w * __ldcg(p + j * R.cap_w + i);      // written by the lattice step
-            vy += w * __ldcg(p + j * R.cap_w + i + cap);
+            vx += w * __ldcg(p + j * cap_w + i);        // written by the lattice step
+            vy += w * __ldcg(p + j * cap_w + i + cap);
         }
     }
     return true;
@@ -96,12 +81,20 @@ __device__ __forceinline__ bool interp_box(const float* box, const RingDev& R, i
 // sigmoids s(t; c) = 1 / (1 + exp(-8 (t - c) / w)).
 __device__ __forceinline__ double trap_sigmoid(double t, double c, double w) { return 1.0 / (1.0 + exp(-8.0 * (t - c) / w)); }
 __device__ __forceinline__ double trap_softplus(double z) { return z > 0.0 ? z + log1p(exp(-z)) : log1p(exp(z)); }
+// k(t) and g(t) by four lanes at once (lanes 0, 1: the two sigmoids; 2, 3: the two softplus), valid
+// in lane 0; the whole warp calls it.
 __device__ __forceinline__ void trap_at(const RingDev& R, double t, double& k, double& g)
 {
+    const int lane = threadIdx.x & 31;
     const double w = R.trap_w, te = R.trap_t_eq, T = R.trap_pull;
-    k = R.trap_k * trap_sigmoid(t, 0.5 * w, w) * (1.0 - trap_sigmoid(t, te + T + 0.5 * w, w));
     const double a = 8.0 / w;
-    g = (trap_softplus(a * (t - te)) - trap_softplus(a * (t - te - T))) / (a * T);
+    double v = 0.0;
+    if (lane < 2) v = trap_sigmoid(t, lane == 0 ? 0.5 * w : te + T + 0.5 * w, w);
+    else if (lane < 4) v = trap_softplus(a * (lane == 2 ? t - te : t - te - T));
+    const double s1 = __shfl_sync(0xffffffffu, v, 1), p0 = __shfl_sync(0xffffffffu, v, 2),
+                 p1 = __shfl_sync(0xffffffffu, v, 3);
+    k = R.trap_k * v * (1.0 - s1);
+    g = (p0 - p1) / (a * T);
 }
 
 __device__ __forceinline__ int half_wrap(int d, int n)   // d in (-n, n) -> [-n/2, n/2)
@@ -111,46 +104,21 @@ __device__ __forceinline__ int half_wrap(int d, int n)   // d in (-n, n) -> [-n/
     return d;
 }
 
-// Fixed-order sums over the warps of a CTA (K values per thread); result valid in thread 0.
-template <int K, class T>
-__device__ void cta_reduce(T (&v)[K], T* red, bool is_min)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-        for (int o = 16; o > 0; o >>= 1) {
-            const T u = __shfl_down_sync(0xffffffffu, v[k], o);
-            v[k] = is_min ? (u < v[k] ? u : v[k]) : v[k] + u;
-        }
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < K; ++k) red[k * 32 + wid] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            T s = red[k * 32];
-            for (int w = 1; w < nw; ++w) s = is_min ? (red[k * 32 + w] < s ? red[k * 32 + w] : s) : s + red[k * 32 + w];
-            v[k] = s;
-        }
-    __syncthreads();
-}
-
-// Shared memory of one node block.  It is passed in rather than declared static: a kernel that
-// runs node blocks after other work hands over space it no longer needs, so the node code takes
+// Shared memory of one ring's node step.  It is passed in rather than declared static: a kernel
+// that runs it after other work hands over space it no longer needs, so the node code takes
 // nothing from the L1 share of that kernel's main work.
 struct NodeSmem {
-    double sx[NODE_THREADS], sy[NODE_THREADS];     // new positions relative to node j = 0
+    double2 pos[MAX_RING_NODES];                   // new positions; later the threads' sums
+    float2 edge[MAX_RING_NODES];                   // R_(k+1) - R_k
+    float2 tens[MAX_RING_NODES];                   // spring tension vector of that edge
+    float ilen[MAX_RING_NODES];                    // 1 / its length
     double dred[4 * 32];
-    float tex[NODE_THREADS], tey[NODE_THREADS];    // spring tension vector of edge (j, j+1)
-    float dpx[NODE_THREADS], dpy[NODE_THREADS];    // d cos(gamma_j) / d p, / d q
-    float dqx[NODE_THREADS], dqy[NODE_THREADS];
-    int ired[4 * 32];
+    double trap[2];                                // k(t), g(t) of the next step
+    int ext[4];                                    // cell extent: min x, -max x, min y, -max y
+    int flag;                                      // free for the caller
     int s_last;
-    int flag[3];                                   // free for the caller
-    unsigned mask;                                 // free for the caller
 };
+static_assert(6 * NODE_THREADS * sizeof(double) <= MAX_RING_NODES * sizeof(double2), "sums overlay the positions");
 
 // Lattice readout of step t, run by the last CTA to arrive (all its threads): the sums of the
 // per-CTA partials (double-float pairs, cell::store_partial) in a fixed order, merged in
@@ -180,213 +148,215 @@ __device__ __forceinline__ void lattice_readout(const NodeArgs& a, long long t, 
     if (tid == 0) row[0] = (double)t;
 }
 
-// One CTA per block of NB nodes of one ring, with a halo of HALO nodes on each side whose
-// advance is recomputed (identically) so that the forces of the owned nodes need no other CTA.
-// One node block (cta: index into a.work) of the node step; called by k_nodes (one block per
-// CTA), by the batched persistent kernel, and (whole_step = false: without the end of the step,
+// The node step of one ring (-1: none) by the whole CTA of NODE_THREADS threads; called by k_nodes
+// and the batched kernels (one ring per CTA) and (whole_step = false: without the end of the step,
 // which the caller then runs itself; t_in: the step index, else read from ctl->t) by the tail of
 // the lattice kernel.
-__device__ __forceinline__ void node_block(const NodeArgs& a, int cta, NodeSmem& S, bool whole_step = true,
-                                           long long t_in = -1)
+__device__ __forceinline__ void node_ring(const NodeArgs& a, int ring, NodeSmem& S, bool whole_step = true,
+                                          long long t_in = -1)
 {
-    double* sx = S.sx;
-    double* sy = S.sy;
-    float* tex = S.tex;
-    float* tey = S.tey;
-    float* dpx = S.dpx;
-    float* dpy = S.dpy;
-    float* dqx = S.dqx;
-    float* dqy = S.dqy;
-    double* dred = S.dred;
-    int* ired = S.ired;
-    int& s_last = S.s_last;
-
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nx = a.nx, ny = a.ny;
     const double Lx = nx, Ly = ny;
     const long long t = t_in >= 0 ? t_in : a.ctl->t;
     const bool readout = a.advance && (t % a.every) == 0;
-    double* row = a.series + (long long)((t / a.every) % a.series_cap) * a.row_len;
-    const int2 wk = a.work[cta];                           // (ring, first owned node)
 
-    if (wk.x >= 0) {
-        const RingDev R = a.rings[wk.x];
-        const int n = R.n_nodes, off = R.node_off;
-        const int k0 = wk.y, n_own = min(NB, n - k0);
-        const int4 B0 = ring_box(R, t);
-        const int bx0 = B0.x, by0 = B0.y, bw = B0.z, bh = B0.w;
-        const int j = tid;                                   // local slot: node k0 - HALO + j
-        const bool active = j < NODE_THREADS && j < n_own + 2 * HALO;   // larger CTAs: extra threads idle
-        const bool own = j >= HALO && j < HALO + n_own;
-        int k = k0 - HALO + j;
-        k %= n;
-        if (k < 0) k += n;
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-        int bad = 0;
-        double2 Xn = make_double2(0.0, 0.0);
-        double2 X = make_double2(0.0, 0.0);
-        if (active) X = a.X[off + k];              // written by the previous node kernel
+    if (ring >= 0) {
+        RingDev& R = a.rings[ring];
+        const int n = R.n_nodes, off = R.node_off, cap_w = R.cap_w;
+        const long long cap = (long long)cap_w * R.cap_h;
+        const float* ubox = a.ubox + R.box_off;
+        const float* fpbox = a.fpbox + R.box_off;
+        const int4 B = ring_box(R, t);
+        const bool trap = R.trap_k > 0.0;
+        double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};     // F_rest, COM of R(t), COM of R(t+1)
+        bool bad = false;
+        int m0 = 1 << 30, m1 = 1 << 30, m2 = 1 << 30, m3 = 1 << 30;   // this thread's cell extent
+        const float hx = 0.5f * (float)nx, hy = 0.5f * (float)ny;
+        if (tid < 4) S.ext[tid] = 1 << 30;
         // u(t), f^p(t) and the lattice readout sums come from the lattice kernel just before
         cell::pdl_wait();
         cell::pdl_trigger();
-        if (active) {
-            Xn = X;
+        __syncthreads();
+        if (trap && wid == NODE_THREADS / 32 - 1) {         // a warp that holds no node of most rings
+            double kt, g;
+            trap_at(R, (double)(t + a.advance), kt, g);
+            if (lane == 0) {
+                S.trap[0] = kt;
+                S.trap[1] = g;
+            }
+        }
+        // ---- advance: Heun on the frozen u(t) --------------------------------------------------
+        for (int k = tid; k < n; k += NODE_THREADS) {
+            const double2 X = a.X[off + k];
+            int cx = (int)X.x, cy = (int)X.y;               // X, Y >= 0
+            float fx = (float)(X.x - cx), fy = (float)(X.y - cy);
+            double2 Xn = X;
             if (a.advance) {
-                if (readout && own) {
-                    float fx, fy;
-                    if (!interp_box(a.fpbox, R, bx0, by0, bw, bh, nx, ny, X.x, X.y, fx, fy)) bad = 1;
-                    acc[0] = (double)fx;
-                    acc[1] = (double)fy;
-                    acc[2] = mimg1(X.x - (double)bx0, Lx);        // centre of mass relative to the box
-                    acc[3] = mimg1(X.y - (double)by0, Ly);
+                if (readout) {
+                    float px, py;
+                    bad |= !interp_box(fpbox, cap_w, cap, B, nx, ny, cx, cy, fx, fy, px, py);
+                    acc[0] += (double)px;
+                    acc[1] += (double)py;
+                    acc[2] += mimg1(X.x - (double)B.x, Lx);       // centre of mass relative to the box
+                    acc[3] += mimg1(X.y - (double)B.y, Ly);
                 }
                 float vx, vy, wx, wy;
-                if (!interp_box(a.ubox, R, bx0, by0, bw, bh, nx, ny, X.x, X.y, vx, vy)) bad = 1;
-                const double Xs = wrap1(X.x + (double)vx, Lx), Ys = wrap1(X.y + (double)vy, Ly);
-                if (!interp_box(a.ubox, R, bx0, by0, bw, bh, nx, ny, Xs, Ys, wx, wy)) bad = 1;
-                const double dX = 0.5 * ((double)vx + (double)wx), dY = 0.5 * ((double)vy + (double)wy);
-                if (!(fabs(dX) < 1.0 && fabs(dY) < 1.0)) bad = 1;
-                Xn = make_double2(wrap1(X.x + dX, Lx), wrap1(X.y + dY, Ly));
-                if (a.walls_y && (Xn.y < 4.0 || Xn.y > Ly - 5.0)) bad = 1;   // supports stay off the walls
-                if (a.walls_x && (Xn.x < 4.0 || Xn.x > Lx - 5.0)) bad = 1;
+                bad |= !interp_box(ubox, cap_w, cap, B, nx, ny, cx, cy, fx, fy, vx, vy);
+                // R* = R + v: its cell from the FP32 fraction, its fraction from the FP64 position (a
+                // cell off by one at the very edge leaves a fraction of -1e-7 or 1, where the
+                // weights run on continuously)
+                const bool slow = fabsf(vx) < hx && fabsf(vy) < hy;     // false for NaN
+                const int sx = cx + (slow ? (int)floorf(fx + vx) : 0), sy = cy + (slow ? (int)floorf(fy + vy) : 0);
+                const float gx = (float)((X.x + (double)vx) - (double)sx), gy = (float)((X.y + (double)vy) - (double)sy);
+                bad |= !slow;
+                bad |= !interp_box(ubox, cap_w, cap, B, nx, ny, wrapi1(sx, nx), wrapi1(sy, ny), slow ? gx : 0.f,
+                                   slow ? gy : 0.f, wx, wy);
+                // a node that moves by a cell or more in one step is an error
+                const bool far = !(fabsf(0.5f * (vx + wx)) < 1.f && fabsf(0.5f * (vy + wy)) < 1.f);
+                bad |= far;
+                Xn.x = fma(0.5, (double)vx + (double)wx, X.x);
+                Xn.y = fma(0.5, (double)vy + (double)wy, X.y);
+                // else only a node in the lattice's outermost cells can leave [0, n)
+                if (far || cx == 0 || cx >= nx - 1) Xn.x = wrap1(Xn.x, Lx);
+                if (far || cy == 0 || cy >= ny - 1) Xn.y = wrap1(Xn.y, Ly);
+                if (a.walls_y && (Xn.y < 4.0 || Xn.y > Ly - 5.0)) bad = true;   // supports stay off the walls
+                if (a.walls_x && (Xn.x < 4.0 || Xn.x > Lx - 5.0)) bad = true;
+                cx = (int)Xn.x;
+                cy = (int)Xn.y;
+                fx = (float)(Xn.x - cx);
+                fy = (float)(Xn.y - cy);
             }
-        }
-        if (bad && own) atomicExch(&a.ctl->err_body, 1);
-        // positions relative to local slot 0 (the ring spans less than half the lattice)
-        if (tid == 0) { dred[0] = Xn.x; dred[1] = Xn.y; }
-        __syncthreads();
-        const double X0x = dred[0], X0y = dred[1];
-        __syncthreads();
-        if (active) {
-            sx[j] = mimg1(Xn.x - X0x, Lx);
-            sy[j] = mimg1(Xn.y - X0y, Ly);
-        }
-        __syncthreads();
-        const int last = n_own + 2 * HALO - 1;
-        const float ks = (float)R.k_spring, leq = (float)R.l_eq, eps = (float)R.eps_angle;
-        if (j >= 1 && j < last) {
-            // Eq. Const.  Spring on the edge (j, j+1): the extension l - l_eq = (l^2 - l_eq^2) /
-            // (l + l_eq) with l^2 - l_eq^2 formed in FP64 from the FP64 edge vector, so it keeps
-            // its relative precision; the rest in FP32.
-            const double qxd = sx[j + 1] - sx[j], qyd = sy[j + 1] - sy[j];
-            const double ext2 = fma(qxd, qxd, fma(qyd, qyd, -R.l_eq * R.l_eq));
-            const float qx = (float)qxd, qy = (float)qyd;
-            const float px = (float)(sx[j - 1] - sx[j]), py = (float)(sy[j - 1] - sy[j]);
-            const float lq = sqrtf(qx * qx + qy * qy), lp = sqrtf(px * px + py * py);
-            const float T = ks * (float)ext2 / ((lq + leq) * lq);
-            tex[j] = T * qx;
-            tey[j] = T * qy;
-            // angle term at j: gradients of cos(gamma_j) = p.q / (|p||q|)
-            const float ip = 1.f / lp, iq = 1.f / lq;
-            const float ipq = ip * iq;
-            const float c = (px * qx + py * qy) * ipq;
-            const float cp = c * ip * ip, cq = c * iq * iq;
-            dpx[j] = qx * ipq - cp * px;
-            dpy[j] = qy * ipq - cp * py;
-            dqx[j] = px * ipq - cq * qx;
-            dqy[j] = py * ipq - cq * qy;
-        }
-        __syncthreads();
-        int mm[4] = {1 << 30, 1 << 30, 1 << 30, 1 << 30};   // min x, -max x, min y, -max y
-        const bool trap = R.trap_k > 0.0;
-        double cn[2] = {0.0, 0.0};                          // advanced positions, for the trap
-        if (own && trap) {
-            cn[0] = mimg1(Xn.x - (double)bx0, Lx);
-            cn[1] = mimg1(Xn.y - (double)by0, Ly);
-        }
-        if (own) {
-            // f_a = -dU/dR_a: springs (a, a+1) and (a-1, a); angle terms at a-1 (a is its next),
-            // a, a+1 (a is its prev); the pull
-            const float fx = tex[j] - tex[j - 1] - eps * (dpx[j + 1] + dqx[j - 1] - dpx[j] - dqx[j]) + (float)R.pull_x;
-            const float fy = tey[j] - tey[j - 1] - eps * (dpy[j + 1] + dqy[j - 1] - dpy[j] - dqy[j]) + (float)R.pull_y;
-            a.node_force[off + k] = make_float2(fx, fy);
+            S.pos[k] = Xn;
+            if (trap) {                                      // advanced positions, for the trap
+                acc[4] += mimg1(Xn.x - (double)B.x, Lx);
+                acc[5] += mimg1(Xn.y - (double)B.y, Ly);
+            }
             a.X_out[off + k] = Xn;
-            int cx = (int)Xn.x, cy = (int)Xn.y;
-            float frx = (float)(Xn.x - cx), fry = (float)(Xn.y - cy);
-            if (frx >= 1.f) { frx = 0.f; cx += 1; }
-            if (fry >= 1.f) { fry = 0.f; cy += 1; }
-            a.node_cell[off + k] = make_int2(wrapi1(cx, nx), wrapi1(cy, ny));
-            a.node_frac[off + k] = make_float2(frx, fry);
+            if (fx >= 1.f) { fx = 0.f; cx += 1; }
+            if (fy >= 1.f) { fy = 0.f; cy += 1; }
+            cx = wrapi1(cx, nx);
+            cy = wrapi1(cy, ny);
+            a.node_cell[off + k] = make_int2(cx, cy);
+            a.node_frac[off + k] = make_float2(fx, fy);
             // cell offsets from the previous box origin, for the new box
-            const int ux = half_wrap(wrapi1(cx, nx) - bx0, nx), uy = half_wrap(wrapi1(cy, ny) - by0, ny);
-            mm[0] = ux; mm[1] = -ux; mm[2] = uy; mm[3] = -uy;
+            const int ux = half_wrap(cx - B.x, nx), uy = half_wrap(cy - B.y, ny);
+            m0 = min(m0, ux);
+            m1 = min(m1, -ux);
+            m2 = min(m2, uy);
+            m3 = min(m3, -uy);
+        }
+        m0 = __reduce_min_sync(0xffffffffu, m0);
+        m1 = __reduce_min_sync(0xffffffffu, m1);
+        m2 = __reduce_min_sync(0xffffffffu, m2);
+        m3 = __reduce_min_sync(0xffffffffu, m3);
+        if (lane < 4 && wid * 32 < n) atomicMin(&S.ext[lane], lane == 0 ? m0 : (lane == 1 ? m1 : (lane == 2 ? m2 : m3)));
+        if (bad) atomicExch(&a.ctl->err_body, 1);
+        __syncthreads();
+        // ---- edges: Eq. Const.  Spring on the edge (k, k+1): the extension l - l_eq = (l^2 -
+        // l_eq^2) / (l + l_eq) with l^2 - l_eq^2 formed in FP64 from the FP64 edge vector, so it
+        // keeps its relative precision; the rest in FP32.
+        const float ks = (float)R.k_spring, leq = (float)R.l_eq, eps = (float)R.eps_angle;
+        const double leq2 = R.l_eq * R.l_eq;
+        for (int k = tid; k < n; k += NODE_THREADS) {
+            const double2 p0 = S.pos[k], p1 = S.pos[k + 1 == n ? 0 : k + 1];
+            double qxd = p1.x - p0.x, qyd = p1.y - p0.y;
+            if (fabsf((float)qxd) >= hx) qxd = mimg1(qxd, Lx);   // across the seam
+            if (fabsf((float)qyd) >= hy) qyd = mimg1(qyd, Ly);
+            const double ext2 = fma(qxd, qxd, fma(qyd, qyd, -leq2));
+            const float qx = (float)qxd, qy = (float)qyd;
+            const float l = sqrtf(qx * qx + qy * qy);
+            const float T = ks * (float)ext2 / ((l + leq) * l);
+            S.edge[k] = make_float2(qx, qy);
+            S.tens[k] = make_float2(T * qx, T * qy);
+            S.ilen[k] = 1.f / l;
+        }
+        __syncthreads();
+        // ---- forces: f_a = -dU/dR_a: springs (a, a+1) and (a-1, a); angle terms at a-1 (a is its
+        // next), a, a+1 (a is its prev); the pull
+        for (int k = tid; k < n; k += NODE_THREADS) {
+            // gradients of cos(gamma_j) = p.q / (|p||q|) at j, p = R_(j-1) - R_j, q = R_(j+1) - R_j
+            auto angle = [&](int j, float2& dp, float2& dq) {
+                const int jm = j == 0 ? n - 1 : j - 1;
+                const float2 q = S.edge[j], e = S.edge[jm];
+                const float iq = S.ilen[j], ip = S.ilen[jm];
+                const float2 p = make_float2(-e.x, -e.y);
+                const float ipq = ip * iq;
+                const float c = (p.x * q.x + p.y * q.y) * ipq;
+                const float cp = c * ip * ip, cq = c * iq * iq;
+                dp = make_float2(q.x * ipq - cp * p.x, q.y * ipq - cp * p.y);
+                dq = make_float2(p.x * ipq - cq * q.x, p.y * ipq - cq * q.y);
+            };
+            const int km = k == 0 ? n - 1 : k - 1, kp = k + 1 == n ? 0 : k + 1;
+            float2 dpm, dqm, dp0, dq0, dpp, dqp;
+            angle(km, dpm, dqm);
+            angle(k, dp0, dq0);
+            angle(kp, dpp, dqp);
+            const float2 t0 = S.tens[k], tm = S.tens[km];
+            const float fx = t0.x - tm.x - eps * (dpp.x + dqm.x - dp0.x - dq0.x) + (float)R.pull_x;
+            const float fy = t0.y - tm.y - eps * (dpp.y + dqm.y - dp0.y - dq0.y) + (float)R.pull_y;
+            a.node_force[off + k] = make_float2(fx, fy);
             if (!isfinite(fx) || !isfinite(fy)) atomicExch(&a.ctl->err_nonfinite, 1);
         }
-        cta_reduce<4, int>(mm, ired, true);
-        if (readout) cta_reduce<4, double>(acc, dred, false);
-        if (trap) cta_reduce<2, double>(cn, dred, false);
-        double* np_ = a.node_partials + (long long)cta * NODE_PARTIALS;
+        // the box of the step the nodes advance to: cells min-2 .. max+3
         if (tid == 0) {
-            for (int q = 0; q < 4; ++q) np_[q] = acc[q];
-            for (int q = 0; q < 4; ++q) np_[4 + q] = (double)mm[q];
-            np_[8] = cn[0];
-            np_[9] = cn[1];
-            __threadfence();
-            const unsigned prev = atomicAdd(&a.ring_tickets[wk.x], 1u);
-            s_last = (prev == (unsigned)(a.ring_ctas[wk.x] - 1));
-        }
-        __syncthreads();
-        if (s_last && tid == 0) {
-            // the ring's last CTA: box of the new positions and the ring's readouts
-            __threadfence();
-            const int c0 = a.ring_cta0[wk.x], nc = a.ring_ctas[wk.x];
-            double sum[4] = {0.0, 0.0, 0.0, 0.0}, scn[2] = {0.0, 0.0};
-            int m[4] = {1 << 30, 1 << 30, 1 << 30, 1 << 30};
-            for (int c = 0; c < nc; ++c) {
-                const volatile double* p = a.node_partials + (long long)(c0 + c) * NODE_PARTIALS;
-                for (int q = 0; q < 4; ++q) {
-                    sum[q] += p[q];
-                    m[q] = min(m[q], (int)p[4 + q]);
-                }
-                scn[0] += p[8];
-                scn[1] += p[9];
-            }
-            if (trap) {
-                // Eq. Utrap at the step the nodes advance to: k (R_ext - R_com) / N on each node
-                const double tn = (double)(t + a.advance);
-                double kt, g;
-                trap_at(R, tn, kt, g);
-                const double ex = mimg1(R.trap_x0 + R.trap_dx * g - ((double)bx0 + scn[0] / n), Lx);
-                const double ey = mimg1(R.trap_y0 + R.trap_dy * g - ((double)by0 + scn[1] / n), Ly);
-                a.rings[wk.x].trap_f[(t + a.advance) & 1] = make_float2((float)(kt * ex / n), (float)(kt * ey / n));
-            }
-            int w = -m[1] - m[0] + 6, h = -m[3] - m[2] + 6;      // cells min-2 .. max+3
-            if (w > R.cap_w || h > R.cap_h) {
+            int w = -S.ext[1] - S.ext[0] + 6, h = -S.ext[3] - S.ext[2] + 6;
+            if (w > cap_w || h > R.cap_h) {
                 atomicExch(&a.ctl->err_body, 1);
-                w = min(w, R.cap_w);
+                w = min(w, cap_w);
                 h = min(h, R.cap_h);
             }
-            // the box of the step the nodes advance to
-            a.rings[wk.x].box[(t + a.advance) & 1] =
-                make_int4(wrapi1(wrapi1(bx0 + m[0] - 2, nx), nx), wrapi1(wrapi1(by0 + m[2] - 2, ny), ny), w, h);
-            if (readout) {
-                double* rr = row + 6 + 4 * wk.x;
-                rr[0] = sum[0];
-                rr[1] = sum[1];
-                rr[2] = wrap1((double)bx0 + sum[2] / n, Lx);
-                rr[3] = wrap1((double)by0 + sum[3] / n, Ly);
-                for (int q = 0; q < 4; ++q)
-                    if (!isfinite(sum[q])) atomicExch(&a.ctl->err_nonfinite, 1);
+            R.box[(t + a.advance) & 1] = make_int4(wrapi1(wrapi1(B.x + S.ext[0] - 2, nx), nx),
+                                                   wrapi1(wrapi1(B.y + S.ext[2] - 2, ny), ny), w, h);
+        }
+        if (readout || trap) {
+            // fixed-order FP64 sums: each thread's nodes in order, then warp c < 6 adds value c (a
+            // strided run per lane, a shuffle tree)
+            double* sum = reinterpret_cast<double*>(S.pos);  // the positions were last read before the barrier
+#pragma unroll
+            for (int c = 0; c < 6; ++c) sum[c * NODE_THREADS + tid] = acc[c];
+            __syncthreads();
+            double v = 0.0;
+            if (wid < 6 && (readout || wid >= 4)) {
+                const int m = min(n, NODE_THREADS);
+                for (int j = lane; j < m; j += 32) v += sum[wid * NODE_THREADS + j];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
             }
-            a.ring_tickets[wk.x] = 0u;
+            if (lane == 0 && wid < 6) S.dred[wid] = v;
+            __syncthreads();
+            if (tid == 0 && trap) {
+                // Eq. Utrap at the step the nodes advance to: k (R_ext - R_com) / N on each node
+                const double kt = S.trap[0], g = S.trap[1];
+                const double ex = mimg1(R.trap_x0 + R.trap_dx * g - ((double)B.x + S.dred[4] / n), Lx);
+                const double ey = mimg1(R.trap_y0 + R.trap_dy * g - ((double)B.y + S.dred[5] / n), Ly);
+                R.trap_f[(t + a.advance) & 1] = make_float2((float)(kt * ex / n), (float)(kt * ey / n));
+            }
+            if (readout && tid >= 32 && tid < 36) {
+                const int c = tid - 32;
+                double* rr = a.series + (long long)((t / a.every) % a.series_cap) * a.row_len + 6 + 4 * ring;
+                const double s = S.dred[c];
+                rr[c] = c < 2 ? s : (c == 2 ? wrap1((double)B.x + s / n, Lx) : wrap1((double)B.y + s / n, Ly));
+                if (!isfinite(s)) atomicExch(&a.ctl->err_nonfinite, 1);
+            }
         }
     }
 
     if (!whole_step) return;
     // the last CTA overall: lattice readout sums (fixed order) and the step counter
-    if (wk.x < 0) {
+    if (ring < 0) {
         cell::pdl_wait();
         cell::pdl_trigger();
     }
+    __syncthreads();
     if (tid == 0) {
         __threadfence();
         const unsigned prev = atomicAdd(&a.ctl->ticket, 1u);
-        s_last = (prev == (unsigned)a.n_ctas - 1u);
+        S.s_last = (prev == (unsigned)a.n_ctas - 1u);
     }
     __syncthreads();
-    if (s_last) {
+    if (S.s_last) {
         __threadfence();
-        if (readout) lattice_readout(a, t, dred);
+        if (readout) lattice_readout(a, t, S.dred);
         if (tid == 0) {
             a.ctl->ticket = 0u;
             if (a.advance) a.ctl->t = t + a.advance;      // advance: steps taken (1, or a jump)

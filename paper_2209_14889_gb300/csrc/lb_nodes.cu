@@ -1,4 +1,4 @@
-// lb_nodes.cu -- the node kernel: one CTA per block of ring nodes (lb_node.cuh).
+// lb_nodes.cu -- the node kernel: one CTA per ring (lb_node.cuh).
 #include <cuda_runtime.h>
 
 #include "lb_node.cuh"
@@ -12,7 +12,7 @@ using namespace node;
 __global__ void __launch_bounds__(NODE_THREADS) k_nodes(const NodeArgs a)
 {
     __shared__ NodeSmem S;
-    node_block(a, blockIdx.x, S);
+    node_ring(a, a.n_rings > 0 ? (int)blockIdx.x : -1, S);
 }
 
 }  // namespace

@@ -51,16 +51,21 @@ struct TileGeo {
     static constexpr int OFF_M = OFF_H + 2 * R3;                  // drho, ux, uy [3][R2]
     static constexpr int OFF_R = OFF_M + 3 * R2;                  // RHS(y)   [5][R0] | f_IB [2][R2]
     static constexpr int SZ_R = cmax(5 * R0, 2 * R2);
-    static constexpr int OFF_N = al4(OFF_R + SZ_R);               // nodes    [NT] float4 (cell, frac)
-    static constexpr int OFF_NF = OFF_N + 4 * NT;                 // node forces [NT] float2
-    static constexpr int OFF_XI = OFF_NF + 2 * NT;                // wrapped x index [R4W] (int)
+    static constexpr int OFF_N = al4(OFF_R + SZ_R);               // nodes: y weights [NT] float4,
+    static constexpr int OFF_NC = OFF_N + 4 * NT;                 // cells [NT] int2
+    // the rest of the gather's node data: x weights [NT] float4, forces [NT] float2 and the row and
+    // column masks, over the moments (written in C only) where they fit
+    static constexpr int SZ_G = 6 * NT + (R2H + R2W) * (NT / 32);
+    static constexpr bool G_OVER = al4(OFF_M) - OFF_M + SZ_G <= 3 * R2;
+    static constexpr int OFF_G = G_OVER ? al4(OFF_M) : OFF_NC + 2 * NT;
+    static constexpr int OFF_XI = OFF_NC + 2 * NT + (G_OVER ? 0 : al4(SZ_G));   // wrapped x index [R4W] (int)
     static constexpr int OFF_YI = OFF_XI + R4W;                   // wrapped y index [R4H] (int)
     static constexpr int OFF_SC = OFF_YI + R4H;                   // scan scratch [NT/32 + 1] (int),
                                                                   // then the tile's ring masks [2]
     static constexpr int OFF_RED = al4(OFF_SC + NT / 32 + 3);     // readout [5][NT/32] (double)
     static constexpr int SMEM_FLOATS = OFF_RED + 2 * 5 * (NT / 32);
     static constexpr size_t SMEM_BYTES = sizeof(float) * SMEM_FLOATS;
-    static_assert(OFF_N % 4 == 0 && OFF_NF % 2 == 0 && OFF_RED % 2 == 0, "shared-memory alignment");
+    static_assert(OFF_N % 4 == 0 && OFF_G % 4 == 0 && OFF_NC % 2 == 0 && OFF_RED % 2 == 0, "shared-memory alignment");
 };
 
 // Shared-memory views of one tile (layout of TileGeo<TX, TY>).
@@ -75,8 +80,12 @@ struct TileMem {
     float* sM;          // drho (moments mode only), ux, uy  [3][R2]
     float* sR;          // RHS(y)       [5][R0]
     float* sFib;        // f_IB         [2][R2]  (over RHS(y) until D)
-    float4* sNode;
+    float4* sNodeWy;
+    int2* sNodeC;
+    float4* sNodeWx;
     float2* sNodeF;
+    unsigned* sRow;     // node masks of the halo-2 region's rows [NT / 32][R2H], columns [NT / 32][R2W]
+    unsigned* sCol;
     int* sXi;
     int* sYi;
     int* sScan;
@@ -84,7 +93,9 @@ struct TileMem {
     __device__ __forceinline__ explicit TileMem(float* sm)
         : sP(sm + G::OFF_P), sS(sm + G::OFF_S), sE(sm + G::OFF_E), sY(sm + G::OFF_E), sH(sm + G::OFF_H),
           sM(sm + G::OFF_M), sR(sm + G::OFF_R), sFib(sm + G::OFF_R),
-          sNode(reinterpret_cast<float4*>(sm + G::OFF_N)), sNodeF(reinterpret_cast<float2*>(sm + G::OFF_NF)),
+          sNodeWy(reinterpret_cast<float4*>(sm + G::OFF_N)), sNodeC(reinterpret_cast<int2*>(sm + G::OFF_NC)),
+          sNodeWx(reinterpret_cast<float4*>(sm + G::OFF_G)), sNodeF(reinterpret_cast<float2*>(sm + G::OFF_G + 4 * NT)),
+          sRow(reinterpret_cast<unsigned*>(sm + G::OFF_G + 6 * NT)), sCol(sRow + G::R2H * (NT / 32)),
           sXi(reinterpret_cast<int*>(sm + G::OFF_XI)), sYi(reinterpret_cast<int*>(sm + G::OFF_YI)),
           sScan(reinterpret_cast<int*>(sm + G::OFF_SC)), sRed(reinterpret_cast<double*>(sm + G::OFF_RED))
     {
@@ -230,9 +241,12 @@ __device__ __forceinline__ void stage(const FusedArgs& a, const TileMem<TX, TY>&
 }
 
 // ---- IB: gather f_IB on the halo-2 region from the nodes of every ring near the tile ----
-// A node at cell c with fraction f sits at (c - o) + f relative to the region origin o; the
-// integer part is kept apart from the fraction so that kernel arguments stay exact in FP32.
-// Each cell sums the nodes in ring and index order, so the result does not depend on the tile.
+// A node at cell c with fraction f reaches the cells c - 1 .. c + 2 per axis with the weights
+// phi4(f).  Each cell sums the nodes in ring and index order, so the result does not depend on the
+// tile.  A ring is taken 256 nodes at a time, one per thread; the chunk's nodes are listed per row
+// and per column of the region as bit masks, and a cell visits only the nodes in both of its lists
+// (a handful: testing every node of the ring at every cell and evaluating the kernel there made the
+// gather 16 000 of the 28 000 cycles of a tile that holds a ring of 157 nodes).
 // the step index of a lattice launch: from the host with the node tail (which advances ctl->t
 // while tiles still run), else from the device step counter
 __device__ __forceinline__ long long step_index(const FusedArgs& a) { return a.node_tail ? a.t : a.ctl->t; }
@@ -245,6 +259,10 @@ __device__ __forceinline__ void ib_gather(const FusedArgs& a, const TileMem<TX, 
     const int tid = threadIdx.x;
     const int nx = a.nx, ny = a.ny;
     const bool small = (nx < R2W + 8) || (ny < R2H + 8);   // region may wrap onto itself
+    unsigned* sRow = m.sRow;
+    unsigned* sCol = m.sCol;
+    const float* wX = reinterpret_cast<const float*>(m.sNodeWx);
+    const float* wY = reinterpret_cast<const float*>(m.sNodeWy);
     const long long t = step_index(a);
     const int nr = a.n_rings;
     // with up to 32 rings every warp tests one ring per lane: the rings whose box meets the
@@ -290,44 +308,48 @@ __device__ __forceinline__ void ib_gather(const FusedArgs& a, const TileMem<TX, 
                 if (cyr > R2H) cyr -= ny;
                 keep = small || (cxr >= -2 && cyr >= -2);
             }
-            // order-preserving compaction of the kept nodes
+            // which of the chunk's nodes reach each row and each column of the region: bit j of word
+            // w is the node of thread 32 w + j, so the words list the nodes in index order
             const unsigned bal = __ballot_sync(0xffffffffu, keep);
             const int lane = tid & 31, wid = tid >> 5;
-            if (lane == 0) m.sScan[wid] = __popc(bal);
-            __syncthreads();
-            if (tid == 0) {
-                int acc = 0;
-                for (int w = 0; w < NT / 32; ++w) {
-                    const int c = m.sScan[w];
-                    m.sScan[w] = acc;
-                    acc += c;
+            if (lane == 0) m.sScan[wid] = (int)bal;
+            if (bal) {
+                m.sNodeC[tid] = make_int2(cxr, cyr);
+                m.sNodeF[tid] = f;
+                m.sNodeWx[tid] = phi4(fr.x);
+                m.sNodeWy[tid] = phi4(fr.y);
+                for (int ly = 0; ly < R2H; ++ly) {
+                    const int d = small ? mimg(cyr - ly, ny) : cyr - ly;
+                    const unsigned b = __ballot_sync(0xffffffffu, keep && (unsigned)(d + 2) < 4u);
+                    if (lane == 0) sRow[wid * R2H + ly] = b;
                 }
-                m.sScan[NT / 32] = acc;
+                for (int lx = 0; lx < R2W; ++lx) {
+                    const int d = small ? mimg(cxr - lx, nx) : cxr - lx;
+                    const unsigned b = __ballot_sync(0xffffffffu, keep && (unsigned)(d + 2) < 4u);
+                    if (lane == 0) sCol[wid * R2W + lx] = b;
+                }
             }
             __syncthreads();
-            if (keep) {
-                const int slot = m.sScan[wid] + __popc(bal & ((1u << lane) - 1u));
-                m.sNode[slot] = make_float4(__int_as_float(cxr), __int_as_float(cyr), fr.x, fr.y);
-                m.sNodeF[slot] = f;
-            }
-            __syncthreads();
-            const int cnt = m.sScan[NT / 32];
-            for (int i = tid; i < R2; i += NT) {
+            unsigned words = 0u;                  // the words that hold a node of this region
+#pragma unroll
+            for (int w = 0; w < NT / 32; ++w) words |= (m.sScan[w] != 0 ? 1u : 0u) << w;
+            for (int i = tid; words != 0u && i < R2; i += NT) {
                 const int ly = i / R2W, lx = i - ly * R2W;
                 float fx = 0.f, fy = 0.f;
-                for (int j = 0; j < cnt; ++j) {
-                    const float4 q = m.sNode[j];
-                    int ddx = __float_as_int(q.x) - lx, ddy = __float_as_int(q.y) - ly;
-                    if (small) {
-                        ddx = mimg(ddx, nx);
-                        ddy = mimg(ddy, ny);
-                    }
-                    const float dx = (float)ddx + q.z, dy = (float)ddy + q.w;
-                    if (fabsf(dx) < 2.f && fabsf(dy) < 2.f) {
-                        const float w = phi(dx) * phi(dy);
+                for (unsigned ws = words; ws; ws &= ws - 1) {
+                    const int w = __ffs(ws) - 1;
+                    for (unsigned hit = sRow[w * R2H + ly] & sCol[w * R2W + lx]; hit; hit &= hit - 1) {
+                        const int j = 32 * w + __ffs(hit) - 1;
+                        const int2 c = m.sNodeC[j];
+                        int ddx = lx - c.x, ddy = ly - c.y;      // -1 .. 2 (modulo the lattice)
+                        if (small) {
+                            ddx = -mimg(-ddx, nx);
+                            ddy = -mimg(-ddy, ny);
+                        }
+                        const float wt = wX[4 * j + 1 + ddx] * wY[4 * j + 1 + ddy];
                         const float2 fq = m.sNodeF[j];
-                        fx += fq.x * w;
-                        fy += fq.y * w;
+                        fx += fq.x * wt;
+                        fy += fq.y * wt;
                     }
                 }
                 m.sFib[i] += fx;
