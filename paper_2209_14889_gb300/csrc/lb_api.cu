@@ -334,15 +334,17 @@ int lb_create(const lb_params* pin, void* stream, lb_handle** out)
     h->sweep_chunk = sweep_chunk(p.nx, p.ny, n_sm);
     h->n_sm = n_sm;
     h->strip_chunk = strip_chunk(p.nx, p.ny, n_sm);
-    h->n_partials = fused_ctas(p.nx, p.ny);
+    h->n_partials = fused_ctas(p.nx, p.ny, 0);
+    h->tile_shape = fused_shape(p.nx, p.ny, n_sm, p.model == LB_MODEL_SCALAR);
     const int partial_cap = std::max(std::max(h->n_partials, sweep_ctas(p.nx, p.ny, h->sweep_chunk)),
                                      strip_ctas(p.nx, p.ny, h->strip_chunk));
     h->partial_cap = partial_cap;
+    const int partial_alloc = std::max(partial_cap, fused_ctas(p.nx, p.ny, h->tile_shape));
     h->series_cap = p.max_samples;
     cudaError_t e;
     if ((e = cudaMalloc(&h->lut, sizeof(float) * lut.size())) != cudaSuccess ||
         (e = cudaMalloc(&h->ctl, sizeof(Ctl))) != cudaSuccess ||
-        (e = cudaMalloc(&h->partials, sizeof(double) * 5 * (size_t)partial_cap)) != cudaSuccess) {
+        (e = cudaMalloc(&h->partials, sizeof(double) * 5 * (size_t)partial_alloc)) != cudaSuccess) {
         rc = cuda_fail(nullptr, e, "cudaMalloc");
         return bail(rc);
     }
@@ -560,8 +562,9 @@ int lb_step(lb_handle* h, int64_t n)
             CK(h, launch_strip(fa, h->strip_chunk, h->stream, pdl));
             h->n_partials = strip_ctas(h->p.nx, h->p.ny, h->strip_chunk);
         } else {
+            const int shape = pair ? 0 : h->tile_shape;
+            h->n_partials = fused_ctas(h->p.nx, h->p.ny, shape);
             if (tail) {
-                h->n_partials = fused_ctas(h->p.nx, h->p.ny);
                 fa.node_tail = 1;
                 fa.t = h->t;
                 fa.tile_rot = h->tile_rot;
@@ -571,7 +574,7 @@ int lb_step(lb_handle* h, int64_t n)
             // without the tail, a lattice kernel stages the state before its dependency wait,
             // which is safe behind a node kernel only: after a launch with the tail it waits for
             // that launch to complete
-            CK(h, launch_fused(fa, MODE_STEP, h->stream, &h->n_partials, pdl && (tail || !h->after_tail), pair));
+            CK(h, launch_fused(fa, MODE_STEP, h->stream, shape, pdl && (tail || !h->after_tail), pair));
         }
         h->after_tail = tail;
         if (h->p.diffusion_substeps > 0) {
@@ -633,7 +636,7 @@ int lb_readout(lb_handle* h, int32_t field, void* dst, size_t bytes, int32_t dst
     if (!h->moments) CK(h, cudaMalloc(&h->moments, sizeof(float) * 3 * N));
     if (field >= LB_FIELD_DRHO && field <= LB_FIELD_UY) {
         FusedArgs fa = fused_args(h);
-        CK(h, launch_fused(fa, MODE_MOMENTS, h->stream, nullptr));
+        CK(h, launch_fused(fa, MODE_MOMENTS, h->stream));
         srcp = h->moments + (size_t)(field - LB_FIELD_DRHO) * N;
     } else if (field >= LB_FIELD_SXX && field <= LB_FIELD_PY) {
         CK(h, plane_to_f32(h, h->cur, PL_SXX + field - LB_FIELD_SXX, h->moments));
@@ -969,7 +972,7 @@ int lb_readout_noalloc(lb_handle* h, int32_t field, void* dst, size_t bytes, int
         // every in-lattice element of the three planes is written before it is read
         FusedArgs fa = fused_args(h);
         fa.moments_out = scratch;
-        CK(h, launch_fused(fa, MODE_MOMENTS, h->stream, nullptr));
+        CK(h, launch_fused(fa, MODE_MOMENTS, h->stream));
         srcp = scratch + (size_t)(field - LB_FIELD_DRHO) * N;
     } else if (field == LB_FIELD_PX || field == LB_FIELD_PY) {
         CK(h, plane_to_f32(h, h->cur, PL_SXX + field - LB_FIELD_SXX, scratch));

@@ -28,19 +28,11 @@ __device__ __forceinline__ int mimg(int d, int n)
     return d;
 }
 
-// The cosine IB kernel phi(r) = (1 + cos(pi r / 2)) / 4 for |r| < 2 (App. A) as the four weights
-// phi(f + 1), phi(f), phi(f - 1), phi(f - 2) of a node at fraction f in [0, 1): with
-// c = cos(pi f / 2), s = sin(pi f / 2) they are (1 - s)/4, (1 + c)/4, (1 + s)/4, (1 - c)/4
-// (quarter-period shifts of the cosine).  The support cell at offset k - 1 from the node's cell
-// takes the k-th.
-__device__ __forceinline__ float4 phi4(float f)
+// cosine IB kernel phi(r) = (1 + cos(pi r / 2)) / 4 for |r| < 2 (App. A)
+__device__ __forceinline__ float phi(float r)
 {
-    float sn, cs;
-    sincospif(0.5f * f, &sn, &cs);
-    return make_float4(0.25f * (1.f - sn), 0.25f * (1.f + cs), 0.25f * (1.f + sn), 0.25f * (1.f - cs));
+    return fabsf(r) < 2.f ? 0.25f * (1.f + cospif(0.5f * r)) : 0.f;
 }
-// the weight of the support cell at offset d = -1 .. 2 from the node's cell
-__device__ __forceinline__ float phi_of(float4 w, int d) { return d < 1 ? (d < 0 ? w.x : w.y) : (d < 2 ? w.z : w.w); }
 
 __device__ __forceinline__ void lut_eval(const float* __restrict__ L, const Phys& ph, float q, float& a2,
                                          float& a4)

@@ -107,7 +107,7 @@ constexpr size_t tile_smem()
     return TileGeo<TX, TY>::SMEM_BYTES > sizeof(node::NodeSmem) ? TileGeo<TX, TY>::SMEM_BYTES : sizeof(node::NodeSmem);
 }
 
-template <int MODE, int PREC, bool SCALAR = false>
+template <int MODE, int PREC, bool SCALAR, int TX, int TY>
 __global__ void __launch_bounds__(NT, 3) k_fused(const __grid_constant__ FusedArgs a)
 {
     extern __shared__ __align__(16) float sm[];
@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(NT, 3) k_fused(const __grid_constant__ FusedAr
         by += a.tile_rot;
         if (by >= (int)gridDim.y) by -= gridDim.y;
     }
-    tile_step<MODE, PREC, TILE_X, TILE_Y, false, SCALAR>(a, blockIdx.x, by, by * gridDim.x + blockIdx.x, sm);
-    if (tail) node_tail<TILE_X, TILE_Y>(a, sm);
+    tile_step<MODE, PREC, TX, TY, false, SCALAR>(a, blockIdx.x, by, by * gridDim.x + blockIdx.x, sm);
+    if (tail) node_tail<TX, TY>(a, sm);
 }
 
 template <int MODE, int PREC>
@@ -140,7 +140,31 @@ __global__ void __launch_bounds__(NT, 2) k_fused_pair(const __grid_constant__ Fu
 
 }  // namespace
 
-int fused_ctas(int nx, int ny) { return ((nx + TILE_X - 1) / TILE_X) * ((ny + TILE_Y - 1) / TILE_Y); }
+// Tile shapes of the one-cell step: 32x16, 16x16, 16x8, 8x8.
+constexpr int SHAPE_X[FUSED_SHAPES] = {TILE_X, 16, 16, 8};
+constexpr int SHAPE_Y[FUSED_SHAPES] = {TILE_Y, 16, 8, 8};
+
+int fused_ctas(int nx, int ny, int shape)
+{
+    return ((nx + SHAPE_X[shape] - 1) / SHAPE_X[shape]) * ((ny + SHAPE_Y[shape] - 1) / SHAPE_Y[shape]);
+}
+
+// A lattice of few tiles is bound by the time of one tile (its passes of 256 threads over its regions,
+// with a barrier and the loads' latency in each), so small tiles win until they fill the SMs several
+// times over and the recomputed halo counts.  Measured on GB300 (us per step with one ring, shapes
+// 0 .. 3): tensorial 32^2 without a ring 8.5, 6.5, 5.0, 4.7; 64^2 23.1, 19.8, 18.2, 17.3; 128^2 24.8,
+// 20.9, 18.7, 19.0; 256^2 24.1, 22.2, 19.6, 19.8; 320^2 25.9, 23.5, 22.2, 24.9; 384^2 28.0, 27.3, 28.5,
+// 39.6; 512^2 31.2, 31.5, 35.6, 52.8; 1024^2 61.3, 79.2, 107.9, 184.7.  The scalar model does half the
+// work per cell: 384^2 29.4, 26.4, 24.3, 25.7; 512^2 29.2, 26.7, 26.0, 39.1; 640^2 30.7, 28.6, 34.4,
+// 58.0; 768^2 31.5, 36.8, 47.3, 81.8.  Hence the limits, in tiles per SM: 8x8 up to 1, 16x8 up to 6
+// (scalar 14), 16x16 up to 4 (scalar 12).
+int fused_shape(int nx, int ny, int n_sm, bool scalar)
+{
+    if (fused_ctas(nx, ny, 3) <= n_sm) return 3;
+    if (fused_ctas(nx, ny, 2) <= (scalar ? 14 : 6) * n_sm) return 2;
+    if (fused_ctas(nx, ny, 1) <= (scalar ? 12 : 4) * n_sm) return 1;
+    return 0;
+}
 
 int fused_tile_rot(int nx, int ny, double y_top)
 {
@@ -151,23 +175,26 @@ int fused_tile_rot(int nx, int ny, double y_top)
     return row;
 }
 
-template <int MODE, int PREC, bool PAIR, bool SCALAR = false>
-static cudaError_t launch_one(const FusedArgs& a, dim3 grid, cudaStream_t s, bool pdl)
+template <int MODE, int PREC, bool PAIR, bool SCALAR = false, int TX = TILE_X, int TY = TILE_Y>
+static cudaError_t launch_one(FusedArgs a, cudaStream_t s, bool pdl)
 {
     static unsigned long long attr_done = 0;     // per device
-    auto kern = PAIR ? k_fused_pair<MODE, PREC> : k_fused<MODE, PREC, SCALAR>;
+    auto kern = [] {
+        if constexpr (PAIR) return k_fused_pair<MODE, PREC>;
+        else return k_fused<MODE, PREC, SCALAR, TX, TY>;
+    }();
     if (!done_on_device(attr_done)) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)tile_smem<TILE_X, TILE_Y>());
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem<TX, TY>());
         if (e != cudaSuccess) {
             attr_done = 0;
             return e;
         }
     }
+    a.tile_rot = a.tile_rot * TILE_Y / TY;       // given in rows of TILE_Y cells
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
+    cfg.gridDim = dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
     cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = tile_smem<TILE_X, TILE_Y>();
+    cfg.dynamicSmemBytes = tile_smem<TX, TY>();
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -177,25 +204,28 @@ static cudaError_t launch_one(const FusedArgs& a, dim3 grid, cudaStream_t s, boo
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-template <bool PAIR>
-static cudaError_t launch_form(const FusedArgs& a, int mode, dim3 grid, cudaStream_t s, bool pdl)
+// the one-cell step with tiles of one shape
+template <int PREC, bool SCALAR>
+static cudaError_t launch_step(const FusedArgs& a, int shape, cudaStream_t s, bool pdl)
 {
-    // the scalar model's step (FP32 state, one-cell tiles); its moments pass is the tensorial one,
-    // which reads the unchanged P planes and, with the Ericksen force off, does not use them
-    if (!PAIR && a.scalar && a.prec == PREC_FP32 && mode == MODE_STEP)
-        return launch_one<MODE_STEP, PREC_FP32, false, true>(a, grid, s, pdl);
-    if (a.prec == PREC_FP32)
-        return mode == MODE_STEP ? launch_one<MODE_STEP, PREC_FP32, PAIR>(a, grid, s, pdl)
-                                 : launch_one<MODE_MOMENTS, PREC_FP32, PAIR>(a, grid, s, false);
-    return mode == MODE_STEP ? launch_one<MODE_STEP, PREC_LP, PAIR>(a, grid, s, pdl)
-                             : launch_one<MODE_MOMENTS, PREC_LP, PAIR>(a, grid, s, false);
+    switch (shape) {
+    case 1: return launch_one<MODE_STEP, PREC, false, SCALAR, 16, 16>(a, s, pdl);
+    case 2: return launch_one<MODE_STEP, PREC, false, SCALAR, 16, 8>(a, s, pdl);
+    case 3: return launch_one<MODE_STEP, PREC, false, SCALAR, 8, 8>(a, s, pdl);
+    default: return launch_one<MODE_STEP, PREC, false, SCALAR>(a, s, pdl);
+    }
 }
 
-cudaError_t launch_fused(const FusedArgs& a, int mode, cudaStream_t s, int* grid_ctas, bool pdl, bool pair)
+cudaError_t launch_fused(const FusedArgs& a, int mode, cudaStream_t s, int shape, bool pdl, bool pair)
 {
-    dim3 grid((a.nx + TILE_X - 1) / TILE_X, (a.ny + TILE_Y - 1) / TILE_Y);
-    if (grid_ctas) *grid_ctas = grid.x * grid.y;
-    return pair ? launch_form<true>(a, mode, grid, s, pdl) : launch_form<false>(a, mode, grid, s, pdl);
+    const bool lp = a.prec != PREC_FP32;
+    if (mode == MODE_MOMENTS)
+        return lp ? launch_one<MODE_MOMENTS, PREC_LP, false>(a, s, false) : launch_one<MODE_MOMENTS, PREC_FP32, false>(a, s, false);
+    if (pair) return lp ? launch_one<MODE_STEP, PREC_LP, true>(a, s, pdl) : launch_one<MODE_STEP, PREC_FP32, true>(a, s, pdl);
+    if (lp) return launch_step<PREC_LP, false>(a, shape, s, pdl);
+    // the scalar model's step (FP32 state, one-cell tiles); its moments pass is the tensorial one,
+    // which reads the unchanged P planes and, with the Ericksen force off, does not use them
+    return a.scalar ? launch_step<PREC_FP32, true>(a, shape, s, pdl) : launch_step<PREC_FP32, false>(a, shape, s, pdl);
 }
 
 }  // namespace vlb

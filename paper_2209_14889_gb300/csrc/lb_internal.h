@@ -151,7 +151,8 @@ inline bool done_on_device(unsigned long long& flags)
 
 // Launchers (return cudaError_t of the launch).
 // pair: the tile kernel with two cells per thread (paired FP32 instructions)
-cudaError_t launch_fused(const FusedArgs& a, int mode, cudaStream_t s, int* grid_ctas, bool pdl = false,
+// shape: the tile shape of a step (0: 32x16 cells, the only one of the other forms)
+cudaError_t launch_fused(const FusedArgs& a, int mode, cudaStream_t s, int shape = 0, bool pdl = false,
                          bool pair = false);
 // column-strip sweep (lb_sweep.cu): eligibility, rows per CTA chunk, CTA count, launch
 bool sweep_eligible(int nx, int ny);
@@ -166,7 +167,10 @@ bool strip_preferred(int nx, int ny, int n_sm);      // faster than the tile ker
 int strip_chunk(int nx, int ny, int n_sm);
 int strip_ctas(int nx, int ny, int chunk);
 cudaError_t launch_strip(const FusedArgs& a, int chunk, cudaStream_t s, bool pdl);
-int fused_ctas(int nx, int ny);
+constexpr int FUSED_SHAPES = 4;
+int fused_ctas(int nx, int ny, int shape);
+// the tile shape of the one-cell step measured fastest for a lattice
+int fused_shape(int nx, int ny, int n_sm, bool scalar);
 // the tile row holding the cell row y_top (any real value; wrapped): where the launch order of
 // the tile kernel with the node tail starts
 int fused_tile_rot(int nx, int ny, double y_top);

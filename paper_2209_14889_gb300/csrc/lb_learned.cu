@@ -275,7 +275,7 @@ int moments(lb_handle* h, float* frc = nullptr)
     FusedArgs fa = handle_fused_args(h);
     fa.moments_out = h->moments;
     fa.forces_out = frc;
-    return launch_fused(fa, MODE_MOMENTS, h->stream, nullptr) == cudaSuccess ? LB_OK : LB_ECUDA;
+    return launch_fused(fa, MODE_MOMENTS, h->stream) == cudaSuccess ? LB_OK : LB_ECUDA;
 }
 
 int pack(lb_handle* h, const LearnNorm& nm, float* raw, bf16* x)

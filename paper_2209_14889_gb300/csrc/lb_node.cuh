@@ -53,6 +53,19 @@ __device__ __forceinline__ int wrapi1(int i, int n)
     return i;
 }
 
+// The four cosine-kernel weights phi(f + 1), phi(f), phi(f - 1), phi(f - 2) of a node at
+// fraction f in [0, 1) (App. A): with c = cos(pi f / 2), s = sin(pi f / 2) they are
+// (1 - s)/4, (1 + c)/4, (1 + s)/4, (1 - c)/4 (quarter-period shifts of the cosine).
+__device__ __forceinline__ void phi4(float f, float* w)
+{
+    float sn, cs;
+    sincospif(0.5f * f, &sn, &cs);
+    w[0] = 0.25f * (1.f - sn);
+    w[1] = 0.25f * (1.f + cs);
+    w[2] = 0.25f * (1.f + sn);
+    w[3] = 0.25f * (1.f - cs);
+}
+
 // Interpolate a 2-component box field for a node at cell (cx, cy) in [0, n) with fractions
 // (fx, fy); returns false if a support cell lies outside the box.
 __device__ __forceinline__ bool interp_box(const float* box, int cap_w, long long cap, const int4& B, int nx, int ny,
@@ -62,8 +75,9 @@ __device__ __forceinline__ bool interp_box(const float* box, int cap_w, long lon
     vx = 0.f;
     vy = 0.f;
     if (ox < 0 || oy < 0 || ox + 3 >= B.z || oy + 3 >= B.w) return false;   // the box never wraps onto itself
-    const float4 a = cell::phi4(fx), b = cell::phi4(fy);
-    const float wx[4] = {a.x, a.y, a.z, a.w}, wy[4] = {b.x, b.y, b.z, b.w};
+    float wx[4], wy[4];
+    phi4(fx, wx);
+    phi4(fy, wy);
     const float* p = box + (long long)oy * cap_w + ox;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -203,23 +217,24 @@ __device__ __forceinline__ void node_ring(const NodeArgs& a, int ring, NodeSmem&
                 }
                 float vx, vy, wx, wy;
                 bad |= !interp_box(ubox, cap_w, cap, B, nx, ny, cx, cy, fx, fy, vx, vy);
-                // R* = R + v: its cell from the FP32 fraction, its fraction from the FP64 position (a
-                // cell off by one at the very edge leaves a fraction of -1e-7 or 1, where the
-                // weights run on continuously)
-                const bool slow = fabsf(vx) < hx && fabsf(vy) < hy;     // false for NaN
-                const int sx = cx + (slow ? (int)floorf(fx + vx) : 0), sy = cy + (slow ? (int)floorf(fy + vy) : 0);
-                const float gx = (float)((X.x + (double)vx) - (double)sx), gy = (float)((X.y + (double)vy) - (double)sy);
-                bad |= !slow;
-                bad |= !interp_box(ubox, cap_w, cap, B, nx, ny, wrapi1(sx, nx), wrapi1(sy, ny), slow ? gx : 0.f,
-                                   slow ? gy : 0.f, wx, wy);
+                // R* = R + v.  Moving by less than a cell, only a node in the lattice's outermost
+                // cells can leave [0, n); beyond half the lattice (or NaN) there is no R*
+                const bool edge_x = cx == 0 || cx >= nx - 1, edge_y = cy == 0 || cy >= ny - 1;
+                const bool here = fabsf(vx) < hx && fabsf(vy) < hy;
+                const bool far0 = !(fabsf(vx) < 1.f && fabsf(vy) < 1.f);
+                double Xs = X.x + (double)(here ? vx : 0.f), Ys = X.y + (double)(here ? vy : 0.f);
+                if (edge_x || far0) Xs = wrap1(Xs, Lx);
+                if (edge_y || far0) Ys = wrap1(Ys, Ly);
+                const int sx = (int)Xs, sy = (int)Ys;
+                bad |= !here;
+                bad |= !interp_box(ubox, cap_w, cap, B, nx, ny, sx, sy, (float)(Xs - sx), (float)(Ys - sy), wx, wy);
                 // a node that moves by a cell or more in one step is an error
                 const bool far = !(fabsf(0.5f * (vx + wx)) < 1.f && fabsf(0.5f * (vy + wy)) < 1.f);
                 bad |= far;
                 Xn.x = fma(0.5, (double)vx + (double)wx, X.x);
                 Xn.y = fma(0.5, (double)vy + (double)wy, X.y);
-                // else only a node in the lattice's outermost cells can leave [0, n)
-                if (far || cx == 0 || cx >= nx - 1) Xn.x = wrap1(Xn.x, Lx);
-                if (far || cy == 0 || cy >= ny - 1) Xn.y = wrap1(Xn.y, Ly);
+                if (edge_x || far) Xn.x = wrap1(Xn.x, Lx);
+                if (edge_y || far) Xn.y = wrap1(Xn.y, Ly);
                 if (a.walls_y && (Xn.y < 4.0 || Xn.y > Ly - 5.0)) bad = true;   // supports stay off the walls
                 if (a.walls_x && (Xn.x < 4.0 || Xn.x > Lx - 5.0)) bad = true;
                 cx = (int)Xn.x;

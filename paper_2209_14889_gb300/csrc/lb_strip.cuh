@@ -174,17 +174,15 @@ __device__ __noinline__ void strip_spread(const FusedArgs& a, unsigned meet, lon
                     const int qcx = __shfl_sync(FULL, cx, j), qcy = __shfl_sync(FULL, cyr, j);
                     const float qfx = __shfl_sync(FULL, fr.x, j), qfy = __shfl_sync(FULL, fr.y, j);
                     const float qFx = __shfl_sync(FULL, f.x, j), qFy = __shfl_sync(FULL, f.y, j);
-                    const int ddx = -mimg(qcx - gx, nx);            // cell - node: the support is -1 .. 2
-                    if (ddx >= -1 && ddx <= 2) {
-                        const float4 ax = phi4(qfx), ay = phi4(qfy);   // the weights of the gather
-                        const float wx = phi_of(ax, ddx);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int kr = qcy - 1 + q;
-                            if (kr < 0 || kr >= SUB) continue;
-                            const float w = wx * phi_of(ay, q - 1);
-                            tmp[(2 * kr) * 32 + lane] += qFx * w;
-                            tmp[(2 * kr + 1) * 32 + lane] += qFy * w;
+                    const float dx = (float)mimg(qcx - gx, nx) + qfx;   // node - cell, as in the gather
+                    if (fabsf(dx) < 2.f) {
+                        for (int kr = max(qcy - 1, 0); kr <= min(qcy + 2, SUB - 1); ++kr) {
+                            const float dy = (float)(qcy - kr) + qfy;
+                            if (fabsf(dy) < 2.f) {
+                                const float w = phi(dx) * phi(dy);
+                                tmp[(2 * kr) * 32 + lane] += qFx * w;
+                                tmp[(2 * kr + 1) * 32 + lane] += qFy * w;
+                            }
                         }
                     }
                 }

@@ -317,9 +317,10 @@ __global__ void __launch_bounds__(NT, 2) k_sweep(const FusedArgs a, const int ch
                     const int cnt = sScan[NT / 32];
                     for (int j = 0; j < cnt; ++j) {
                         const float4 q = sNode[j];
-                        const int ddx = c - __float_as_int(q.x), ddy = r - __float_as_int(q.y);
-                        if (ddx >= -1 && ddx <= 2 && ddy >= -1 && ddy <= 2) {
-                            const float w = phi_of(phi4(q.z), ddx) * phi_of(phi4(q.w), ddy);
+                        const float dx = (float)(__float_as_int(q.x) - c) + q.z;
+                        const float dy = (float)(__float_as_int(q.y) - r) + q.w;
+                        if (fabsf(dx) < 2.f && fabsf(dy) < 2.f) {
+                            const float w = phi(dx) * phi(dy);
                             const float2 fq = sNodeF[j];
                             fibx += fq.x * w;
                             fiby += fq.y * w;

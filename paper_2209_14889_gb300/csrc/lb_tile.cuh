@@ -242,7 +242,7 @@ __device__ __forceinline__ void stage(const FusedArgs& a, const TileMem<TX, TY>&
 
 // ---- IB: gather f_IB on the halo-2 region from the nodes of every ring near the tile ----
 // A node at cell c with fraction f reaches the cells c - 1 .. c + 2 per axis with the weights
-// phi4(f).  Each cell sums the nodes in ring and index order, so the result does not depend on the
+// phi(f + 1), phi(f), phi(f - 1), phi(f - 2).  Each cell sums the nodes in ring and index order, so the result does not depend on the
 // tile.  A ring is taken 256 nodes at a time, one per thread; the chunk's nodes are listed per row
 // and per column of the region as bit masks, and a cell visits only the nodes in both of its lists
 // (a handful: testing every node of the ring at every cell and evaluating the kernel there made the
@@ -316,8 +316,8 @@ __device__ __forceinline__ void ib_gather(const FusedArgs& a, const TileMem<TX, 
             if (bal) {
                 m.sNodeC[tid] = make_int2(cxr, cyr);
                 m.sNodeF[tid] = f;
-                m.sNodeWx[tid] = phi4(fr.x);
-                m.sNodeWy[tid] = phi4(fr.y);
+                m.sNodeWx[tid] = make_float4(phi(1.f + fr.x), phi(fr.x), phi(fr.x - 1.f), phi(fr.x - 2.f));
+                m.sNodeWy[tid] = make_float4(phi(1.f + fr.y), phi(fr.y), phi(fr.y - 1.f), phi(fr.y - 2.f));
                 for (int ly = 0; ly < R2H; ++ly) {
                     const int d = small ? mimg(cyr - ly, ny) : cyr - ly;
                     const unsigned b = __ballot_sync(0xffffffffu, keep && (unsigned)(d + 2) < 4u);
