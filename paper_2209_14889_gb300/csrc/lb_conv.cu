@@ -1,7 +1,9 @@
 // lb_conv.cu -- 3x3 convolutions on NHWC BF16 activations with FP32 accumulation (the network of
-// the learned stepper): forward passes and data gradients, as implicit GEMMs with the pixels as M,
-// the output channels as N and K = 9 Ci.
+// the learned stepper) as implicit GEMMs: forward passes and data gradients with the pixels as M, the
+// output channels as N and K = 9 Ci, weight gradients with the input channels as M, the output channels
+// as N and the pixels as K.
 #include <algorithm>
+#include <cstdint>
 
 #include "lb_conv.h"
 #include "lb_internal.h"
@@ -20,12 +22,6 @@ __device__ __forceinline__ unsigned smem_u32(const void* p)
 __device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const void* p)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldsm_x4_t(unsigned (&r)[4], const void* p)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(smem_u32(p)));
 }
@@ -203,7 +199,7 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* mb, unsigned bytes)
 __device__ __forceinline__ bool mbar_wait(uint64_t* mb, unsigned parity)
 {
     unsigned done = 0;
-    for (long it = 0; it < (1L << 22) && !done; ++it) {
+    for (long it = 0; it < (1L << 20) && !done; ++it) {
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
             : "=r"(done)
@@ -433,7 +429,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
                     }
                     const bool whole = co0 + j + 16 <= a.Co;
                     if (a.yf) {
-                        if (whole && ((o0 + j) & 3) == 0) {
+                        if (whole && (((uintptr_t)(a.yf + o0) | (a.yf2 ? (uintptr_t)(a.yf2 + o0) : 0)) & 15) == 0) {
 #pragma unroll
                             for (int e = 0; e < 16; e += 4) {
                                 const float4 q = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
@@ -462,7 +458,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
                             r[e] = __floats2bfloat162_rn(mm.x > 0.f ? gg.x : SLOPE * gg.x, mm.y > 0.f ? gg.y : SLOPE * gg.y);
                         }
                     }
-                    if (whole && ((o0 + j) & 7) == 0) {
+                    if (whole && ((uintptr_t)(a.y + o0) & 15) == 0) {
                         const uint4 w0 = *reinterpret_cast<const uint4*>(r), w1 = *reinterpret_cast<const uint4*>(r + 4);
                         *reinterpret_cast<uint4*>(a.y + o0 + j) = w0;
                         *reinterpret_cast<uint4*>(a.y + o0 + j + 8) = w1;
@@ -494,112 +490,276 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
 }
 
 // ------------------------------------------------------------------ weight gradient
-
-constexpr int WG_CO = 64, WG_CI = 16;           // output block of gw per CTA: [9][64][16]
-constexpr int DZS = WG_CO + 8;                  // shared row of 64 channels + 8 pad (144 bytes)
+//
+// gw[t][co][ci] = sum over pixels of gz[p][co] x[p + off_t][ci] on the tensor cores: M = input channels
+// (up to 128 per CTA), N = output channels (up to 48), K = pixels, one accumulator of N columns per tap
+// (9 N <= 432 of the 512 tensor-memory columns), so one pass over the pixels serves all nine taps.  The
+// channels are the contiguous index of both operands, so they are read MN-major: [channel group of
+// 8][position][8], where a tap is again a constant offset of the position.
+// A CTA takes units of up to RB rows of a 32-column strip, every S-th unit: stage j of a unit brings
+// input row y0 - 1 + j (34 positions) and, from j = 2, the gradient row y0 + j - 2 (32 positions, zero
+// beyond the image), whose 18 MMAs (2 x 16 positions, 9 taps) then read the input rows of the stages
+// j - 2 .. j.  Up to 16 stages are in flight; a stage is released by the MMAs that read it last and by
+// the warp that adds the gradient rows for the bias.  Each CTA writes one partial sum, k_sum_parts adds
+// the S partials in a fixed order.
+// What bounds it: the M = 128 operand of every MMA is read from shared memory (4 KB, 32 cycles; 9 x 2
+// per row); at few input channels most of its rows are not used, which costs nothing more.
 
 struct WgradArgs {
     const bf16* x;          // layer input (pixel stride ldx, offset xoff)
     long long ldx;
     int xoff;
-    const bf16* gz;         // gradient at the layer's pre-activation output [P][Co] (stride ldz)
-    long long ldz;
-    float* part;            // [S][9][Co][Ci] partial sums
-    int B, H, W, Ci, Co, S;
+    const bf16* gz;         // gradient at the layer's pre-activation output, dense [P][Co]
+    float* part;            // [S][n] partial sums: [9][Co][Ci], then the bias [Co]
+    int B, H, W, Ci, Co;
 };
 
-__global__ void __launch_bounds__(128) k_conv_wgrad(const WgradArgs a)
-{
-    __shared__ __align__(16) bf16 sdz[CT_H * CT_W * DZS];
-    __shared__ __align__(16) bf16 sx[CT_IH * CT_IW * PS];
-    const int co0 = blockIdx.x * WG_CO, ci0 = blockIdx.y * WG_CI, s = blockIdx.z;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = (a.W + CT_W - 1) / CT_W, tiles_y = (a.H + CT_H - 1) / CT_H;
-    const int n_tiles = a.B * tiles_x * tiles_y;
-    float acc[9][2][4];
-#pragma unroll
-    for (int t = 0; t < 9; ++t)
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[t][j][k] = 0.f;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+struct WgradGeo {
+    int cib, cob;           // channels per CTA
+    int RB, strips, rbs;    // rows per unit, strips per row, units per strip
+    int units, slots;
+    unsigned ncol;
+    long long n;            // values of a partial sum
+};
 
-    for (int tile = s; tile < n_tiles; tile += a.S) {
-        const int b = tile / (tiles_x * tiles_y), r = tile - b * (tiles_x * tiles_y);
-        const int ty0 = (r / tiles_x) * CT_H, tx0 = (r % tiles_x) * CT_W;
-        // gz tile: 128 pixels x 64 channels (8 chunks of 8)
-        for (int q = tid; q < CT_H * CT_W * 8; q += 128) {
-            const int p = q >> 3, h = q & 7;
-            const int gy = ty0 + p / CT_W, gx = tx0 + p % CT_W;
-            uint4 v = zero;
-            if (gy < a.H && gx < a.W && co0 + h * 8 < a.Co)
-                v = *reinterpret_cast<const uint4*>(a.gz + ((long long)(b * a.H + gy) * a.W + gx) * a.ldz + co0 + h * 8);
-            *reinterpret_cast<uint4*>(sdz + p * DZS + h * 8) = v;
+constexpr int WG_PX = 34, WG_PZ = 32;            // staged positions of an input and a gradient row
+constexpr int WG_NMAX = 48;
+
+__global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__ WgradArgs a,
+                                                         const __grid_constant__ WgradGeo g, int* err)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    TcShared& S = *reinterpret_cast<TcShared*>(smem);
+    const int zg = g.cob / 8;
+    const int xbytes = g.cib / 8 * WG_PX * 16, sbytes = xbytes + zg * WG_PZ * 16;
+    const unsigned stage0 = smem_u32(smem) + TC_HEAD;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ci0 = blockIdx.y * g.cib, co0 = blockIdx.z * g.cob;
+    const int xg = min(g.cib, a.Ci - ci0) / 8;   // input channel groups of this CTA
+    const int slots = g.slots;
+
+    if (tid == 0) {
+        for (int s = 0; s < slots; ++s) {
+            mbar_init(&S.xfull[s], 128);
+            mbar_init(&S.empty[s], 2);
         }
-        for (int q = tid; q < CT_IH * CT_IW * 2; q += 128) {
-            const int p = q >> 1, h = q & 1;
-            const int py = p / CT_IW, px = p - py * CT_IW;
-            const int gy = ty0 - 1 + py, gx = tx0 - 1 + px;
-            uint4 v = zero;
-            if (gy >= 0 && gy < a.H && gx >= 0 && gx < a.W)
-                v = *reinterpret_cast<const uint4*>(a.x + ((long long)(b * a.H + gy) * a.W + gx) * a.ldx + a.xoff + ci0 +
-                                                    h * 8);
-            *reinterpret_cast<uint4*>(sx + p * PS + h * 8) = v;
-        }
-        __syncthreads();
-        const int j = lane >> 3, rr = lane & 7;
-#pragma unroll 1
-        for (int ks = 0; ks < CT_H; ++ks) {             // 16 pixels (one tile row) per k-step
-            unsigned A[4];                               // (co, p): rows p of sdz, transposed
-            ldsm_x4_t(A, sdz + (ks * CT_W + rr + (j >> 1) * 8) * DZS + warp * 16 + (j & 1) * 8);
+        mbar_init(&S.done, 1);
+        S.fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 4) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
+                     "r"(g.ncol));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned tmem = S.tmem;
+    const int per = g.strips * g.rbs;
+
+    bool ok = true;
+    if (warp < 4) {
+        // ---- rows: 16-byte units (position, channel group), the channels of a position side by side
+        int xp[5], xd[5], zp[2], zd[2];
+        long long xs[5], zs[2];
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int dy = t / 3 - 1, dx = t % 3 - 1;
-                unsigned Bf[4];                          // (p, ci): rows p of the shifted input
-                const int k = rr + (j & 1) * 8;
-                ldsm_x4_t(Bf, sx + ((ks + 1 + dy) * CT_IW + (k + 1 + dx)) * PS + (j >> 1) * 8);
-                mma_bf16(acc[t][0], A, Bf[0], Bf[1]);
-                mma_bf16(acc[t][1], A, Bf[2], Bf[3]);
+        for (int i = 0; i < 5; ++i) {
+            const int u = tid + 128 * i, p = u / xg, q = u - p * xg;
+            xp[i] = p < WG_PX ? p : -1;
+            xd[i] = (q * WG_PX + p) * 16;
+            xs[i] = (long long)(p - 1) * a.ldx + a.xoff + ci0 + 8 * q;
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int u = tid + 128 * i, p = u / zg, q = u - p * zg;
+            zp[i] = p < WG_PZ ? p : -1;
+            zd[i] = xbytes + (q * WG_PZ + p) * 16;
+            zs[i] = co0 + 8 * q < a.Co ? (long long)p * a.Co + co0 + 8 * q : -1;
+        }
+        pdl_wait();
+        unsigned J = 0;
+        for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+            const int b = u / per, r = u - b * per;
+            const int x0 = (r / g.rbs) * 32, y0 = (r % g.rbs) * g.RB;
+            const int rows = min(g.RB, a.H - y0);
+            for (int j = 0; j < rows + 2; ++j, ++J) {
+                const unsigned s = J % (unsigned)slots;
+                if (J >= (unsigned)slots) ok = mbar_wait(&S.empty[s], (J / (unsigned)slots - 1) & 1u);
+                if (!ok) break;
+                const unsigned dst = stage0 + s * (unsigned)sbytes;
+                const int yx = y0 - 1 + j;
+                const bool rowx = yx >= 0 && yx < a.H;
+                const bf16* bx = a.x + (((long long)b * a.H + yx) * a.W + x0) * a.ldx;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) {
+                    if (xp[i] < 0) continue;
+                    const int x = x0 - 1 + xp[i];
+                    const bool in = rowx && x >= 0 && x < a.W;
+                    cp_async16(dst + (unsigned)xd[i], in ? bx + xs[i] : a.x, in ? 16 : 0);
+                }
+                if (j >= 2) {
+                    const bf16* bz = a.gz + (((long long)b * a.H + y0 + j - 2) * a.W + x0) * a.Co;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        if (zp[i] < 0) continue;
+                        const bool in = zs[i] >= 0 && x0 + zp[i] < a.W;
+                        cp_async16(dst + (unsigned)zd[i], in ? bz + zs[i] : a.gz, in ? 16 : 0);
+                    }
+                }
+                cp_async_arrive(&S.xfull[s]);
             }
         }
-        __syncthreads();
-    }
-    const int g = lane >> 2, tq = lane & 3;
+        pdl_trigger();
+    } else if (warp == 5) {
+        // ---- bias: the gradient rows added up, one position per lane
+        float acc[WG_NMAX];
 #pragma unroll
-    for (int t = 0; t < 9; ++t)
+        for (int e = 0; e < WG_NMAX; ++e) acc[e] = 0.f;
+        unsigned J = 0;
+        for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+            const int r = u % per;
+            const int rows = min(g.RB, a.H - (r % g.rbs) * g.RB);
+            for (int j = 0; j < rows + 2; ++j, ++J) {
+                const unsigned s = J % (unsigned)slots;
+                // every stage is waited for, so that this warp's arrival belongs to the stage's own phase
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], (J / (unsigned)slots) & 1u));
+                if (!ok) break;
+                if (j >= 2 && blockIdx.y == 0) {
+                    const unsigned char* z = smem + TC_HEAD + s * (unsigned)sbytes + xbytes + lane * 16;
 #pragma unroll
-        for (int jn = 0; jn < 2; ++jn)
+                    for (int q = 0; q < WG_NMAX / 8; ++q) {
+                        if (q >= zg) break;
+                        const uint4 v = *reinterpret_cast<const uint4*>(z + q * WG_PZ * 16);
+                        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int co = co0 + warp * 16 + g + 8 * hh;
-                const int ci = ci0 + jn * 8 + 2 * tq;
-                if (co < a.Co) {
-                    float* o = a.part + (((long long)s * 9 + t) * a.Co + co) * a.Ci + ci;
-                    o[0] = acc[t][jn][2 * hh];
-                    o[1] = acc[t][jn][2 * hh + 1];
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 f = __bfloat1622float2(h[e]);
+                            acc[8 * q + 2 * e] += f.x;
+                            acc[8 * q + 2 * e + 1] += f.y;
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&S.empty[s])) : "memory");
+            }
+        }
+        if (ok && blockIdx.y == 0) {
+            pdl_wait();             // the partial sums' buffer is the former reduction's
+#pragma unroll
+            for (int e = 0; e < WG_NMAX; ++e) {
+                float v = acc[e];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+                if (lane == 0 && e < g.cob && co0 + e < a.Co)
+                    a.part[blockIdx.x * g.n + 9LL * a.Co * a.Ci + co0 + e] = v;
+            }
+        }
+    } else if (lane == 0) {
+        // ---- MMAs, both operands MN-major
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                               ((uint32_t)(g.cob >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        unsigned J = 0;
+        int acc = 0;
+        for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+            const int r = u % per;
+            const int rows = min(g.RB, a.H - (r % g.rbs) * g.RB);
+            for (int j = 0; j < rows + 2; ++j, ++J) {
+                const unsigned s = J % (unsigned)slots;
+                ok = mbar_wait(&S.xfull[s], (J / (unsigned)slots) & 1u);
+                if (!ok) break;
+                if (j < 2) continue;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const unsigned sz = stage0 + s * (unsigned)sbytes + (unsigned)xbytes;
+                for (int dy = 0; dy < 3; ++dy) {
+                    const unsigned sx = stage0 + ((J - 2 + (unsigned)dy) % (unsigned)slots) * (unsigned)sbytes;
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx)
+                            tc_mma(tmem + (unsigned)((3 * dy + dx) * g.cob),
+                                   tc_desc(sx + (unsigned)((16 * ks + dx) * 16), 128, WG_PX * 16),
+                                   tc_desc(sz + (unsigned)(16 * ks * 16), 128, WG_PZ * 16), idesc, ks > 0 ? 1 : acc);
+                }
+                acc = 1;
+                tc_commit(&S.empty[(J - 2) % (unsigned)slots]);
+                if (j == rows + 1) {
+                    tc_commit(&S.empty[(J - 1) % (unsigned)slots]);
+                    tc_commit(&S.empty[s]);
                 }
             }
+        }
+        if (ok) tc_commit(&S.done);
+    }
+    if (!ok) S.fail = 1;
+
+    if (warp < 4) {
+        if (ok) ok = mbar_wait(&S.done, 0);
+        if (!ok) S.fail = 1;
+        cp_async_wait_all();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (ok) {
+            // warp w holds the input channels 32 w .., the columns are the output channels co0 .. of
+            // each tap
+            const bool valid = tid < 8 * xg;
+            float* out = a.part + blockIdx.x * g.n + ci0 + tid;
+            for (int t = 0; t < 9; ++t)
+                for (int j = 0; j < g.cob; j += 16) {
+                    unsigned v[16];
+                    tc_ld16(v, tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(t * g.cob + j));
+                    if (!valid) continue;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        if (co0 + j + e < a.Co) out[((long long)t * a.Co + co0 + j + e) * a.Ci] = __uint_as_float(v[e]);
+                }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (S.fail && tid == 0) atomicExch(err, 1);
+    if (warp == 4) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.ncol));
+    }
 }
 
-// sum of S partial arrays of n floats, in order: out[i] = sum_s part[s][i]
-__global__ void k_sum_parts(const float* part, int S, long long n, float* out)
+// Sum of S partial arrays of n floats (n a multiple of 4): eight threads per float4, each every eighth
+// partial in order, then the eight in order.  The first nw values go to gw, the others to gb.
+__global__ void __launch_bounds__(256) k_sum_parts(const float4* part, int S, int n4, int nw4, float* gw, float* gb)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float v = 0.f;
-    for (int s = 0; s < S; ++s) v += part[(long long)s * n + i];
-    out[i] = v;
-}
-
-// bias gradient partials: part[s][o] = sum over pixels p = s, s + S, ... of gz[p][o]
-__global__ void k_bias_parts(const bf16* gz, long long ldz, long long P, int Co, int S, float* part)
-{
-    const int o = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
-    if (o >= Co) return;
-    float v = 0.f;
-    for (long long p = s; p < P; p += S) v += __bfloat162float(gz[p * ldz + o]);
-    part[(long long)s * Co + o] = v;
+    __shared__ float4 red[8][32];
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    pdl_wait();
+    pdl_trigger();
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < n4) {
+#pragma unroll 4
+        for (int s = k; s < S; s += 8) {
+            const float4 q = part[(long long)s * n4 + i];
+            v.x += q.x;
+            v.y += q.y;
+            v.z += q.z;
+            v.w += q.w;
+        }
+    }
+    red[k][lane] = v;
+    __syncthreads();
+    if (k != 0 || i >= n4) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) {
+        const float4 w = red[q][lane];
+        v.x += w.x;
+        v.y += w.y;
+        v.z += w.z;
+        v.w += w.w;
+    }
+    float* o = i < nw4 ? gw + 4LL * i : gb + 4LL * (i - nw4);
+    o[0] = v.x;
+    o[1] = v.y;
+    o[2] = v.z;
+    o[3] = v.w;
 }
 
 // ------------------------------------------------------------------ weights
@@ -642,6 +802,14 @@ int sm_count()
 
 int* g_conv_err = nullptr;      // device flag: a tcgen05 kernel's bounded wait gave up
 
+cudaError_t conv_err_init()
+{
+    if (g_conv_err) return cudaSuccess;
+    cudaError_t e = cudaMalloc(&g_conv_err, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(g_conv_err, 0, sizeof(int));
+    return e;
+}
+
 template <int MT>
 cudaError_t launch_tc(const ConvArgs& a, const ConvGeo& g, unsigned m_tiles, int n_cot, cudaStream_t s, bool pdl)
 {
@@ -670,11 +838,8 @@ cudaError_t conv_pack(const PackArgs& p, cudaStream_t s)
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
 {
     if (a.Ci % 16 != 0) return cudaErrorInvalidValue;
-    if (!g_conv_err) {
-        cudaError_t e = cudaMalloc(&g_conv_err, sizeof(int));
-        if (e == cudaSuccess) e = cudaMemset(g_conv_err, 0, sizeof(int));
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = conv_err_init();
+    if (e != cudaSuccess) return e;
     static const int n_sm = sm_count();
     ConvGeo g = {};
     g.cpk = (a.Co + 15) / 16 * 16;
@@ -719,32 +884,68 @@ cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-int wgrad_splits(int B, int H, int W)
+// Units and partial sums of a layer's weight gradient; room: floats of the partial sums' buffer (0: as
+// many as wanted).  Returns S.
+static int wgrad_geo(int B, int H, int W, int Ci, int Co, long long room, WgradGeo& g)
 {
-    const int tiles = B * ((W + CT_W - 1) / CT_W) * ((H + CT_H - 1) / CT_H);
-    return tiles < 64 ? tiles : 64;
+    static const int n_sm = sm_count();
+    const int nb_o = (Co + WG_NMAX - 1) / WG_NMAX, nb_i = (Ci + 127) / 128;
+    g.cob = ((Co + nb_o - 1) / nb_o + 15) / 16 * 16;
+    g.cib = ((Ci / 8 + nb_i - 1) / nb_i) * 8;
+    g.ncol = 32;
+    while ((int)g.ncol < 9 * g.cob) g.ncol *= 2;
+    g.n = 9LL * Ci * Co + Co;
+    g.strips = (W + 31) / 32;
+    // one CTA per SM (two where the accumulators leave half the tensor memory), each with several units
+    // so that the last ones do not leave SMs idle; shorter units where the image is small
+    const int occ = (int)(512 / g.ncol);
+    long long S = std::max(1, occ * n_sm / (nb_o * nb_i));
+    if (room > 0) S = std::max(1LL, std::min(S, room / g.n));
+    for (g.RB = 32;; g.RB /= 2) {
+        g.rbs = (H + g.RB - 1) / g.RB;
+        if ((long long)B * g.strips * g.rbs >= 5 * S || g.RB == 2) break;
+    }
+    const long long units = (long long)B * g.strips * g.rbs;
+    g.units = (int)std::min<long long>(units, 0x7fffffff);
+    S = std::min(S, units);
+    const int sbytes = g.cib / 8 * WG_PX * 16 + g.cob / 8 * WG_PZ * 16;
+    const int bytes = (occ > 1 ? 108 : 216) * 1024 - TC_HEAD - 17 * WG_PX * 16;
+    g.slots = std::max(4, std::min(TC_SLOTS, bytes / sbytes));
+    return (int)S;
 }
 
 long long wgrad_part_elems(int B, int H, int W, int Ci, int Co)
 {
-    return (long long)wgrad_splits(B, H, W) * std::max<long long>(9LL * Ci * Co, Co);
+    WgradGeo g;
+    return wgrad_geo(B, H, W, Ci, Co, 0, g) * g.n;
 }
 
 cudaError_t conv_wgrad(cudaStream_t s, const bf16* x, long long ldx, int xoff, const bf16* gz, int B, int H, int W,
-                       int Ci, int Co, float* part, float* gw, float* gb)
+                       int Ci, int Co, float* part, long long room, float* gw, float* gb, bool pdl)
 {
-    const int S = wgrad_splits(B, H, W);
-    WgradArgs a;
-    a.x = x; a.ldx = ldx; a.xoff = xoff; a.gz = gz; a.ldz = Co; a.part = part;
-    a.B = B; a.H = H; a.W = W; a.Ci = Ci; a.Co = Co; a.S = S;
-    dim3 grid((Co + WG_CO - 1) / WG_CO, Ci / WG_CI, S);
-    k_conv_wgrad<<<grid, 128, 0, s>>>(a);
-    const long long nw = 9LL * Co * Ci;
-    k_sum_parts<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(part, S, nw, gw);
-    const long long P = (long long)B * H * W;
-    k_bias_parts<<<dim3((Co + 127) / 128, S), 128, 0, s>>>(gz, Co, P, Co, S, part);
-    k_sum_parts<<<(unsigned)((Co + 255) / 256), 256, 0, s>>>(part, S, Co, gb);
-    return cudaGetLastError();
+    cudaError_t e = conv_err_init();
+    if (e != cudaSuccess) return e;
+    static unsigned long long attr = 0;      // per device
+    if (!done_on_device(attr)) {
+        e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) {
+            attr = 0;
+            return e;
+        }
+    }
+    WgradGeo g;
+    const int S = wgrad_geo(B, H, W, Ci, Co, room, g);
+    WgradArgs a = {};
+    a.x = x; a.ldx = ldx; a.xoff = xoff; a.gz = gz; a.part = part;
+    a.B = B; a.H = H; a.W = W; a.Ci = Ci; a.Co = Co;
+    // the last stage's operand of 128 channels may reach past its own channels: 16 groups of slack
+    const size_t smem = TC_HEAD + (size_t)g.slots * (g.cib / 8 * WG_PX * 16 + g.cob / 8 * WG_PZ * 16) + 17 * WG_PX * 16;
+    e = launch_pdl(k_wgrad_tc, dim3(S, (Ci + g.cib - 1) / g.cib, (Co + g.cob - 1) / g.cob), TC_THREADS, smem, s, pdl, a, g,
+                   g_conv_err);
+    if (e != cudaSuccess) return e;
+    const int n4 = (int)(g.n / 4), nw4 = (int)(9LL * Ci * Co / 4);
+    return launch_pdl(k_sum_parts, dim3((n4 + 31) / 32), 256, 0, s, true, reinterpret_cast<const float4*>(part), S, n4, nw4,
+                      gw, gb);
 }
 
 }  // namespace net

@@ -61,10 +61,11 @@ cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl);
 cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s);
 
 // Weight and bias gradients of one layer from its input x and pre-activation gradient gz (dense
-// [P][Co]): gw[9][Co][Ci], gb[Co]; part: wgrad_part_elems floats of scratch.
+// [P][Co]): gw[9][Co][Ci], gb[Co]; part: scratch of `room` floats (at least 9 Ci Co + Co; with
+// wgrad_part_elems floats the reduction is split as far as it pays).  pdl: as for conv_tc.
 long long wgrad_part_elems(int B, int H, int W, int Ci, int Co);
 cudaError_t conv_wgrad(cudaStream_t s, const bf16* x, long long ldx, int xoff, const bf16* gz, int B, int H, int W,
-                       int Ci, int Co, float* part, float* gw, float* gb);
+                       int Ci, int Co, float* part, long long room, float* gw, float* gb, bool pdl);
 
 // the flag that a tcgen05 kernel raises when a bounded wait gave up (nullptr before the first launch)
 int* conv_err_flag();

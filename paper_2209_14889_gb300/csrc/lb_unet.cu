@@ -6,10 +6,10 @@
 //                                                                           K = 9 Ci)
 //   data grad    gx[q, c] = sum_{t', o} gz[q + off_t', o] w'[t', c, o],  w'[t'] = w[8 - t']^T
 //                (the forward kernel on the flipped, transposed weights)
-//   weight grad  gw[t, o, c] = sum_p gz[p, o] x[p + off_t, c]                (M = Co, N = Ci,
+//   weight grad  gw[t, o, c] = sum_p gz[p, o] x[p + off_t, c]                (M = Ci, N = Co,
 //                                                                           K = pixels)
-// with off_t = (t / 3 - 1, t % 3 - 1); by default the forward and the data gradient run on tcgen05
-// (lb_conv_kernel).  Weight gradients are reduced over pixel tiles in a fixed order (per-CTA
+// with off_t = (t / 3 - 1, t % 3 - 1), on tcgen05 (the forward and the data gradient on mma.sync by
+// choice: lb_conv_kernel).  Weight gradients are reduced over pixel tiles in a fixed order (per-CTA
 // partials, then a sum over CTAs), so training is bitwise reproducible.
 // Joins: 2x2 average pooling, nearest 2x upsampling written into a channel slice of the
 // concatenation buffer (the skip is written there by its producing convolution), LeakyReLU
@@ -109,8 +109,14 @@ __global__ void k_to_bf16(const float* x, long long n, bf16* y)
     pdl_trigger();
     const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 8;
     if (i >= n) return;
-    const float4 a = *reinterpret_cast<const float4*>(x + i), b = *reinterpret_cast<const float4*>(x + i + 4);
-    st8(y + i, Oct{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}});
+    Oct o;
+    if (((uintptr_t)x & 15) == 0) {
+        const float4 a = *reinterpret_cast<const float4*>(x + i), b = *reinterpret_cast<const float4*>(x + i + 4);
+        o = Oct{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+    } else {                                     // a caller's gradient at any address
+        for (int e = 0; e < 8; ++e) o.v[e] = x[i + e];
+    }
+    st8(y + i, o);
 }
 
 // y[b, i, j, c] = mean of x[b, 2i + {0,1}, 2j + {0,1}, c]  (x: stride ldx, offset xoff; output H x W)
@@ -371,8 +377,8 @@ cudaError_t layer_bwd(lb_net* n, int l, const bf16* x, long long ldx, int xoff, 
                       long long ldm, int moff, int H, int W)
 {
     const NetLayer& Ly = n->L[l];
-    cudaError_t e = conv_wgrad(n->stream, x, ldx, xoff, gz, n->B, H, W, Ly.ci, Ly.co, n->part, n->g + Ly.w_off,
-                               n->g + Ly.b_off);
+    cudaError_t e = conv_wgrad(n->stream, x, ldx, xoff, gz, n->B, H, W, Ly.ci, Ly.co, n->part, n->part_n,
+                               n->g + Ly.w_off, n->g + Ly.b_off, true);
     if (e != cudaSuccess || !gx) return e;
     ConvArgs a = {};
     a.x = gz; a.ldx = Ly.co;
@@ -380,7 +386,7 @@ cudaError_t layer_bwd(lb_net* n, int l, const bf16* x, long long ldx, int xoff, 
     a.y = gx; a.ldy = Ly.ci;
     a.B = n->B; a.H = H; a.W = W; a.Ci = Ly.co; a.Co = Ly.ci;
     a.ym = m; a.ldm = ldm; a.moff = moff;
-    return conv_run(a, n->stream, false);
+    return conv_run(a, n->stream, true);
 }
 
 // yout: a second copy of the output (device FP32 [P0][16]) or null
@@ -426,13 +432,13 @@ int net_backward(lb_net* n, const float* gy)
     // gradient of the nearest upsampling (the first channels of a concatenation's gradient gy), at h x w
     auto up2_bwd = [&](const bf16* gy2, long long ldg, const bf16* m, int h, int w, int ch, bf16* g) {
         const unsigned u = (unsigned)((long long)B * h * w * ch / 8);
-        return launch_pdl(k_up2_bwd, units(u), 256, 0, s, false, gy2, ldg, m, u, h, w, ch / 8, g);
+        return launch_pdl(k_up2_bwd, units(u), 256, 0, s, true, gy2, ldg, m, u, h, w, ch / 8, g);
     };
     // gradient of the pooling (gp) plus that of the skip (gs), at h x w
     auto pool_bwd = [&](const bf16* gp, const bf16* gs, long long lds, int soff, const bf16* m, int h, int w, int ch,
                         bf16* g) {
         const unsigned u = (unsigned)((long long)B * h * w * ch / 8);
-        return launch_pdl(k_pool2_bwd_add, units(u), 256, 0, s, false, gp, gs, lds, soff, m, lds, soff, u, h, w, ch / 8, g);
+        return launch_pdl(k_pool2_bwd_add, units(u), 256, 0, s, true, gp, gs, lds, soff, m, lds, soff, u, h, w, ch / 8, g);
     };
     NCK(n, launch_pdl(k_to_bf16, units(P0 * 2), 256, 0, s, false, gy, P0 * 16, Z));
     NCK(n, layer_bwd(n, HEAD, n->d0, 32, 0, Z, A, n->d0, 32, 0, H, W));               // A = g d0
@@ -784,10 +790,11 @@ int lb_conv3x3_wgrad(const void* x, const void* gz, float* gw, float* gb, int32_
     if (!x || !gz || !gw || !gb || B < 1 || H < 1 || W < 1 || Ci < 16 || Co < 8 || Ci % 16 || Co % 8) return LB_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     void* part = nullptr;
-    cudaError_t e = scratch(&part, sizeof(float) * (size_t)wgrad_part_elems(B, H, W, Ci, Co), s);
+    const long long room = wgrad_part_elems(B, H, W, Ci, Co);
+    cudaError_t e = scratch(&part, sizeof(float) * (size_t)room, s);
     if (e != cudaSuccess) return conv_code(e);
     e = conv_wgrad(s, static_cast<const bf16*>(x), Ci, 0, static_cast<const bf16*>(gz), B, H, W, Ci, Co,
-                   static_cast<float*>(part), gw, gb);
+                   static_cast<float*>(part), room, gw, gb, false);
     const cudaError_t f = cudaFreeAsync(part, s);
     return conv_code(e != cudaSuccess ? e : f);
 }

@@ -1,0 +1,83 @@
+"""The tcgen05 convolutions at the sizes where their geometry changes: one and several MMA tiles per
+CTA, the flat position space (width up to 128) and the tiles beyond, split output channels, one and
+several units of rows per CTA in the weight gradient, channel counts that leave parts of a block empty.
+
+Inputs are exact in BF16, so against FP64 the only errors are the FP32 accumulations: relative to the
+largest result 1e-5 for the FP32 outputs (as in the network's tests), plus 2^-8 relative for a BF16 one.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2209_14889_gb300 import lb
+    return torch, lb
+
+
+def _conv64(torch, x, w):
+    """x [B, H, W, Ci], w [9, Co, Ci] (FP64) by shifted products."""
+    B, H, W, _ = x.shape
+    xp = torch.nn.functional.pad(x, (0, 0, 1, 1, 1, 1))
+    return sum(torch.einsum("bhwc,oc->bhwo", xp[:, t // 3:t // 3 + H, t % 3:t % 3 + W], w[t]) for t in range(9))
+
+
+SIZES = [(1, 1, 1, 16, 16), (2, 3, 128, 32, 24), (1, 2, 129, 16, 32), (3, 31, 33, 48, 40), (1, 70, 131, 144, 136),
+         (4, 64, 64, 64, 64), (2, 130, 250, 96, 16), (5, 33, 127, 16, 128), (4, 256, 256, 32, 32)]
+
+
+@pytest.mark.parametrize("B,H,W,Ci,Co", SIZES)
+def test_forward_edges_vs_fp64(B, H, W, Ci, Co):
+    torch, lb = _gpu()
+    torch.manual_seed(B * H + W)
+    x = torch.randn(B, H, W, Ci, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(9, Co, Ci, device="cuda") / (9 * Ci) ** 0.5).to(torch.bfloat16)
+    b = torch.randn(Co, device="cuda")
+    ref = _conv64(torch, x.double(), w.double()) + b.double()
+    y = lb.conv3x3(x, w, b, act=False, out_f32=True)
+    assert (y.double() - ref).abs().max() <= 1e-5 * ref.abs().max()
+    z = lb.conv3x3(x, w, b, act=True, out_f32=False).double()
+    ref = torch.where(ref > 0, ref, 0.1 * ref)
+    assert torch.all((z - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5 * ref.abs().max())
+    lb.conv_status()
+
+
+@pytest.mark.parametrize("B,H,W,Ci,Co", SIZES)
+def test_gradients_edges_vs_fp64(B, H, W, Ci, Co):
+    torch, lb = _gpu()
+    Co = (Co + 15) // 16 * 16                       # the data gradient takes multiples of 16
+    torch.manual_seed(B + H * W)
+    x = torch.randn(B, H, W, Ci, device="cuda").to(torch.bfloat16)
+    gz = torch.randn(B, H, W, Co, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(9, Co, Ci, device="cuda") / (9 * Ci) ** 0.5).to(torch.bfloat16)
+    ref = _conv64(torch, gz.double(), w.double().flip(0).transpose(1, 2))
+    gx = lb.conv3x3_dgrad(gz, w).double()
+    assert torch.all((gx - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5 * ref.abs().max())
+    gw, gb = lb.conv3x3_wgrad(x, gz)
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 1, 1, 1, 1))
+    rw = torch.stack([torch.einsum("bhwo,bhwc->oc", gz.double(), xp[:, t // 3:t // 3 + H, t % 3:t % 3 + W])
+                      for t in range(9)])
+    assert (gw.double() - rw).abs().max() <= 1e-5 * rw.abs().max()
+    rb = gz.double().sum((0, 1, 2))
+    assert (gb.double() - rb).abs().max() <= 1e-5 * max(rb.abs().max().item(), 1.0)
+    lb.conv_status()
+
+
+def test_weight_gradient_of_few_output_channels_and_any_address():
+    # Co = 8 (half an MMA column block) and results at addresses that are multiples of 4 bytes only
+    torch, lb = _gpu()
+    x = torch.randn(2, 9, 40, 32, device="cuda").to(torch.bfloat16)
+    gz = torch.randn(2, 9, 40, 8, device="cuda").to(torch.bfloat16)
+    gw, gb = lb.conv3x3_wgrad(x, gz)
+    buf = torch.full((9 * 8 * 32 + 8 + 3,), 7.0, device="cuda")
+    rc = lb.lib().lb_conv3x3_wgrad(x.data_ptr(), gz.data_ptr(), buf.data_ptr() + 4, buf.data_ptr() + 4 * (9 * 8 * 32 + 2),
+                                   2, 9, 40, 32, 8, torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    torch.cuda.synchronize()
+    n = 9 * 8 * 32
+    assert torch.equal(buf[1:1 + n].reshape(gw.shape), gw) and torch.equal(buf[n + 2:n + 10], gb)
+    assert buf[0] == 7.0 and buf[n + 1] == 7.0 and buf[n + 10] == 7.0
