@@ -150,18 +150,20 @@ __global__ void __launch_bounds__(128) k_conv3x3(const ConvArgs a)
 // Either way a tap reads the 128 consecutive staged positions that start at (1 + dy) pitch + 1 + dx.
 // One chunk of 16 input channels is 9 MT MMAs of K = 16, in the same order for every geometry (chunk,
 // then tap), so results do not depend on it.  Operands in the canonical K-major layout without
-// swizzle: input [2 k-halves][positions][8], weights [9 taps][2 k-halves][cop][8]; 8-row groups 128
-// bytes apart.
+// swizzle: input [k-halves][positions][8], weights [chunks][9 taps][2 k-halves][cop][8]; 8-row groups
+// 128 bytes apart.
 //
-// Four warps copy the input (cp.async, the position's address formed once for all chunks), one warp
-// the weights (bulk copies of the packed layout, conv_pack), one thread issues the MMAs; the chunks
-// go through up to 16 stages, each with a barrier for its input, its weights and its release by the
-// MMAs that read it (tcgen05.commit).  The four copying warps then store the result.
+// Eight warps copy the input (cp.async; the pixels of the positions in a table formed once), one warp
+// the weights (bulk copies of the packed layout, conv_pack), one warp issues the MMAs.  A stage holds
+// cw = 1, 2 or 4 chunks, so that a copy instruction covers 32 to 128 contiguous bytes of a pixel;
+// each of up to 16 stages has a barrier for its input, its weights and its release by the MMAs that
+// read it (tcgen05.commit).  The eight copying warps then store the result, two per quarter of the
+// tensor memory's lanes.
 //
-// What bounds it: at 32 channels the 128 x 16 input operand of every MMA is read from shared memory
-// (4 KB, 32 cycles) for half as many cycles of tensor work; at few CTAs (the 1/4 and 1/8 resolution
-// layers) the latency of one CTA's chain, which is why all chunks' copies are issued ahead and the
-// channels are split until every SM has a CTA.
+// What bounds it: the 128 x 16 input operand of every MMA is read from shared memory (4 KB, 32 cycles
+// against 16 of tensor work at 32 channels); the copies of the input; at few CTAs (the 1/4 and 1/8
+// resolution layers) the latency of one CTA's chain, which is why all copies are issued ahead and the
+// channels are split until most SMs have a CTA.
 
 // shared-memory matrix descriptor: start address, leading (K-direction core-matrix) and stride
 // (8-row group) byte offsets, descriptor version 1, no swizzle
@@ -212,12 +214,21 @@ __device__ __forceinline__ void tc_commit(uint64_t* mb)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mb)) : "memory");
 }
-__device__ __forceinline__ void tc_mma(unsigned d, uint64_t ad, uint64_t bd, uint32_t idesc, int acc)
+// One lane issues the MMAs, but the whole warp runs the loop around them with warp-uniform operands: in
+// a branch of one thread the descriptors go through that thread's registers and each MMA took 130 to 160
+// cycles to issue, against 32 + N / 4 this way (measured, N = 16 .. 128: the operands' shared memory).
+__device__ __forceinline__ unsigned elect_one()
+{
+    unsigned l;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(l));
+    return l;
+}
+__device__ __forceinline__ void tc_mma(unsigned d, uint64_t ad, uint64_t bd, uint32_t idesc, int acc, unsigned lead)
 {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(lead));
 }
 __device__ __forceinline__ void tc_ld16(unsigned (&v)[16], unsigned taddr)
 {
@@ -227,18 +238,42 @@ __device__ __forceinline__ void tc_ld16(unsigned (&v)[16], unsigned taddr)
         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
           "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tc_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// 32 bytes to global memory (32-byte aligned): a whole sector per lane
+__device__ __forceinline__ void st32(void* p, const unsigned (&v)[8])
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
 }
 
-constexpr int TC_THREADS = 192;                  // 4 copying and storing warps, MMA warp, weights warp
+constexpr int TC_COPY = 256;                     // threads of the 8 copying and storing warps
+constexpr int TC_THREADS = TC_COPY + 64;         // and the MMA warp and the weights (bias) warp
 constexpr int TC_SLOTS = 16;                     // most stages
-constexpr int TC_HEAD = 512;                     // shared bytes of the barriers
+constexpr int TC_HEAD = 1024;                    // shared bytes of the barriers and the bias
+
+// division of 0 <= n < 2^31 by a constant d >= 1: n / d = (n m) >> (32 + s) with 2^s >= d
+struct FastDiv {
+    unsigned m, s, d;
+    FastDiv() = default;
+    explicit FastDiv(unsigned d_) : d(d_)
+    {
+        for (s = 0; (1u << s) < d && s < 31; ++s) {
+        }
+        m = (unsigned)((((1ull << s) - d) << 32) / d + 1);       // 2^32 (2^s - d) / d, rounded up
+    }
+    __device__ __forceinline__ unsigned div(unsigned n) const { return (unsigned)(((unsigned long long)__umulhi(n, m) + n) >> s); }
+};
 
 struct ConvGeo {
     int flat, pitch, npix;                       // npix: staged positions
     int cop, slots, tx, ty;                      // channels per CTA, stages, tile grid (tiles form)
+    int cw, lgh;                                 // chunks per stage, log2 of its k-halves
     int cpk;                                     // channels of the packed weights
     unsigned ncol;                               // tensor-memory columns (a power of two >= 32)
+    FastDiv d0, d1;                              // flat: by pitch, by H + 1; tiles: by tx, by tx ty
 };
 
 // shared state of a tcgen05 kernel ahead of its stages
@@ -246,6 +281,7 @@ struct TcShared {
     uint64_t xfull[TC_SLOTS], wfull[TC_SLOTS], empty[TC_SLOTS], done;
     unsigned tmem;
     int fail;
+    float4 bias[32];
 };
 static_assert(sizeof(TcShared) <= TC_HEAD, "barriers fit ahead of the stages");
 
@@ -255,63 +291,62 @@ __device__ __forceinline__ bool out_pixel(const ConvArgs& a, const ConvGeo& g, i
 {
     if (g.flat) {
         const int Q = (int)blockIdx.x * (128 * MT) + 128 * mt + m;
-        const int row = Q / g.pitch;
+        const int row = (int)g.d0.div((unsigned)Q);
         x = Q - row * g.pitch;
-        b = row / (a.H + 1);
+        b = (int)g.d1.div((unsigned)row);
         y = row - b * (a.H + 1);
         return x < a.W && y < a.H && b < a.B;
     }
-    const int per = g.tx * g.ty;
-    b = (int)blockIdx.x / per;
-    const int r = (int)blockIdx.x - b * per;
+    b = (int)g.d1.div(blockIdx.x);
+    const int r = (int)blockIdx.x - b * g.tx * g.ty;
+    const int ty = (int)g.d0.div((unsigned)r);
     const int c = m & 31;
-    y = (r / g.tx) * (4 * MT) + 4 * mt + (m >> 5);
-    x = (r % g.tx) * 30 + c;
+    y = ty * (4 * MT) + 4 * mt + (m >> 5);
+    x = (r - ty * g.tx) * 30 + c;
     return c < 30 && x < a.W && y < a.H;
 }
 
-// element offset of the pixel at staged position p (without the channel), or -1 where it is padding
+// pixel at staged position p, or -1 where it is padding (there are fewer than 2^31 pixels)
 template <int MT>
-__device__ __forceinline__ long long in_pixel(const ConvArgs& a, const ConvGeo& g, int p)
+__device__ __forceinline__ int in_pixel(const ConvArgs& a, const ConvGeo& g, int p)
 {
     int b, y, x;
     if (g.flat) {
         const int Q = (int)blockIdx.x * (128 * MT) - g.pitch - 1 + p;
-        if (Q < 0) return -1;
-        const int row = Q / g.pitch;
+        if (Q < 0 || p >= 128 * MT + 2 * g.pitch + 2) return -1;
+        const int row = (int)g.d0.div((unsigned)Q);
         x = Q - row * g.pitch;
-        b = row / (a.H + 1);
+        b = (int)g.d1.div((unsigned)row);
         y = row - b * (a.H + 1);
         if (b >= a.B) return -1;
     } else {
-        const int per = g.tx * g.ty;
-        b = (int)blockIdx.x / per;
-        const int r = (int)blockIdx.x - b * per;
-        y = (r / g.tx) * (4 * MT) - 1 + (p >> 5);
-        x = (r % g.tx) * 30 - 1 + (p & 31);
+        b = (int)g.d1.div(blockIdx.x);
+        const int r = (int)blockIdx.x - b * g.tx * g.ty;
+        const int ty = (int)g.d0.div((unsigned)r);
+        y = ty * (4 * MT) - 1 + (p >> 5);
+        x = (r - ty * g.tx) * 30 - 1 + (p & 31);
         if (p >= (4 * MT + 2) * 32 || y < 0 || x < 0) return -1;
     }
     if (x >= a.W || y >= a.H) return -1;
-    return (((long long)b * a.H + y) * a.W + x) * a.ldx + a.xoff;
+    return (b * a.H + y) * a.W + x;
 }
 
 template <int MT>
 __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ ConvArgs a, const __grid_constant__ ConvGeo g,
                                                         int* err)
 {
-    // copies per thread and chunk: 2 npix / 128, npix <= max(128 MT + 72, 128 MT + 260)
-    constexpr int NU = (2 * (128 * MT + 260) + 127) / 128;
     extern __shared__ __align__(128) unsigned char smem[];
     TcShared& S = *reinterpret_cast<TcShared*>(smem);
-    const int xbytes = g.npix * 32, wbytes = 288 * g.cop, sbytes = xbytes + wbytes;
-    const unsigned stage0 = smem_u32(smem) + TC_HEAD;
+    int* const spix = reinterpret_cast<int*>(smem + TC_HEAD);        // pixels of the staged positions
+    const int xbytes = g.npix * 32 * g.cw, sbytes = xbytes + 288 * g.cop * g.cw;
+    const unsigned stage0 = smem_u32(smem) + TC_HEAD + (unsigned)(g.npix * 4);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int co0 = blockIdx.y * g.cop;
-    const int nchunk = a.Ci / 16, slots = g.slots;
+    const int nstage = a.Ci / (16 * g.cw), slots = g.slots;
 
     if (tid == 0) {
         for (int s = 0; s < slots; ++s) {
-            mbar_init(&S.xfull[s], 128);
+            mbar_init(&S.xfull[s], TC_COPY);
             mbar_init(&S.wfull[s], 1);
             mbar_init(&S.empty[s], 1);
         }
@@ -319,128 +354,145 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
         S.fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4) {
+    if (warp == TC_COPY / 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
                      "r"(g.ncol));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    for (int p = tid; p < g.npix; p += TC_THREADS) spix[p] = in_pixel<MT>(a, g, p);
+    if (tid < 128) reinterpret_cast<float*>(S.bias)[tid] = a.bias && tid < g.cop && co0 + tid < a.Co ? a.bias[co0 + tid] : 0.f;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = S.tmem;
 
     bool ok = true;
-    if (warp < 4) {
-        // ---- input: 16-byte units (position, k-half); a thread's units and their addresses are the
-        // same in every chunk, 32 bytes further on
-        long long src[NU];
-#pragma unroll
-        for (int i = 0; i < NU; ++i) {
-            const int u = tid + 128 * i;
-            src[i] = u < 2 * g.npix ? in_pixel<MT>(a, g, u >> 1) : -1;
-        }
+    if (warp < TC_COPY / 32) {
+        // ---- input: 16-byte units (position, k-half), the k-halves of a position side by side
+        const int h = tid & ((1 << g.lgh) - 1), p0 = tid >> g.lgh, step = TC_COPY >> g.lgh;
         pdl_wait();                       // the input is the result of the kernel before this one
-        for (int k = 0; k < nchunk && ok; ++k) {
+        for (int k = 0; k < nstage && ok; ++k) {
             const int s = k % slots;
             if (k >= slots) ok = mbar_wait(&S.empty[s], (unsigned)((k / slots - 1) & 1));
             if (!ok) break;
-            const unsigned dst = stage0 + (unsigned)(s * sbytes);
-            const bf16* base = a.x + 16 * k + 8 * (tid & 1);
-            const int h = tid & 1;
-#pragma unroll
-            for (int i = 0; i < NU; ++i) {
-                const int u = tid + 128 * i;
-                if (u < 2 * g.npix)
-                    cp_async16(dst + (unsigned)((h * g.npix + (u >> 1)) * 16), src[i] >= 0 ? base + src[i] : a.x,
-                               src[i] >= 0 ? 16 : 0);
+            const unsigned dst = stage0 + (unsigned)(s * sbytes + h * g.npix * 16);
+            const bf16* base = a.x + a.xoff + 16 * g.cw * k + 8 * h;
+#pragma unroll 4
+            for (int p = p0; p < g.npix; p += step) {
+                const int pix = spix[p];
+                cp_async16(dst + (unsigned)(p * 16), pix >= 0 ? base + (long long)pix * a.ldx : a.x, pix >= 0 ? 16 : 0);
             }
             cp_async_arrive(&S.xfull[s]);
         }
         pdl_trigger();
-    } else if (warp == 5) {
-        // ---- weights: 18 bulk copies (tap, k-half) of the CTA's channels per chunk, one per lane
+    } else if (warp == TC_COPY / 32 + 1) {
+        // ---- weights: 18 bulk copies (tap, k-half) of the CTA's channels per chunk
         const unsigned nb = (unsigned)min(g.cop, g.cpk - co0) * 16u;
         int issued = 0;
-        for (int k = 0; k < nchunk && ok; ++k) {
+        for (int k = 0; k < nstage && ok; ++k) {
             const int s = k % slots;
             if (k >= slots) ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], (unsigned)((k / slots - 1) & 1)));
             if (!ok) break;
-            if (lane == 0) mbar_expect_tx(&S.wfull[s], 18u * nb);
+            if (lane == 0) mbar_expect_tx(&S.wfull[s], 18u * (unsigned)g.cw * nb);
             __syncwarp();
-            if (lane < 18)
-                bulk_copy(stage0 + (unsigned)(s * sbytes + xbytes + lane * g.cop * 16),
-                          a.wp + (((long long)k * 18 + lane) * g.cpk + co0) * 8, nb, &S.wfull[s]);
+            for (int q = lane; q < 18 * g.cw; q += 32)
+                bulk_copy(stage0 + (unsigned)(s * sbytes + xbytes + q * g.cop * 16),
+                          a.wp + (((long long)k * g.cw * 18 + q) * g.cpk + co0) * 8, nb, &S.wfull[s]);
             issued = k + 1;
         }
         // the CTA does not end with a weights copy in flight, whatever happened above
         for (int k = max(0, issued - slots); k < issued; ++k)
             mbar_wait(&S.wfull[k % slots], (unsigned)((k / slots) & 1));
-    } else if (lane == 0) {
+    } else {
         // ---- MMAs
+        const unsigned lead = elect_one();
         const uint32_t idesc =
             (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.cop >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-        for (int k = 0; k < nchunk && ok; ++k) {
+        for (int k = 0; k < nstage && ok; ++k) {
             const int s = k % slots;
             const unsigned par = (unsigned)((k / slots) & 1);
-            ok = mbar_wait(&S.xfull[s], par) && mbar_wait(&S.wfull[s], par);
+            ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], par) && mbar_wait(&S.wfull[s], par));
             if (!ok) break;
             // the input was written through the generic proxy, the tensor core reads through the
             // asynchronous one
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const unsigned sx = stage0 + (unsigned)(s * sbytes), sw = sx + (unsigned)xbytes;
-            for (int t = 0; t < 9; ++t) {
-                const uint64_t bd = tc_desc(sw + (unsigned)(t * 2 * g.cop * 16), (unsigned)(g.cop * 16), 128);
-                const int p0 = (t / 3) * g.pitch + t % 3;
+            // descriptors of the tap (-1, -1); their addresses count 16 bytes: positions and weights
+            const unsigned sx = stage0 + (unsigned)(s * sbytes);
+            uint64_t ad = tc_desc(sx, (unsigned)(g.npix * 16), 128);
+            uint64_t bd = tc_desc(sx + (unsigned)xbytes, (unsigned)(g.cop * 16), 128);
+            for (int kk = 0; kk < g.cw; ++kk) {
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    tc_mma(tmem + (unsigned)(mt * g.cop), tc_desc(sx + (unsigned)((p0 + 128 * mt) * 16), (unsigned)(g.npix * 16), 128),
-                           bd, idesc, (k > 0 || t > 0) ? 1 : 0);
+                for (int t = 0; t < 9; ++t) {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+                        tc_mma(tmem + (unsigned)(mt * g.cop), ad + (unsigned)((t / 3) * g.pitch + t % 3 + 128 * mt),
+                               bd + (unsigned)(t * 2 * g.cop), idesc, (k > 0 || kk > 0 || t > 0) ? 1 : 0, lead);
+                }
+                ad += (unsigned)(2 * g.npix);
+                bd += (unsigned)(18 * g.cop);
             }
-            tc_commit(&S.empty[s]);
+            if (lead) tc_commit(&S.empty[s]);
         }
-        if (ok) tc_commit(&S.done);
+        if (ok && lead) tc_commit(&S.done);
     }
     if (!ok) S.fail = 1;
 
-    if (warp < 4) {
+    if (warp < TC_COPY / 32) {
         if (ok) ok = mbar_wait(&S.done, 0);
         if (!ok) S.fail = 1;
         cp_async_wait_all();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (ok) {
-            // warp w holds the positions 32 w .. of each tile, the columns are the channels co0 ..
-            for (int mt = 0; mt < MT; ++mt) {
-                int b, y, x;
-                const bool valid = out_pixel<MT>(a, g, mt, tid, b, y, x);
-                const long long pix = ((long long)b * a.H + y) * a.W + x;
-                const long long o0 = pix * a.ldy + a.yoff + co0;
-                for (int j = 0; j < g.cop; j += 16) {
-                    unsigned v[16];
-                    tc_ld16(v, tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(mt * g.cop + j));
-                    if (!valid) continue;
+            // warp w holds the positions 32 (w % 4) .. of each tile, the columns are the channels co0 ..;
+            // blocks of 16 channels of a tile, every second one, two at a time
+            const int m = tid & 127, nj = g.cop / 16, nblk = MT * nj;
+            const unsigned lane0 = tmem + ((unsigned)(warp & 3) << 21);
+            for (int q0 = warp >> 2; q0 < nblk; q0 += 4) {
+                __syncwarp();               // the lanes that stored nothing and the others
+                unsigned v[2][16];
+                const int q1 = q0 + 2;
+                tc_ld16(v[0], lane0 + (unsigned)((q0 / nj) * g.cop + (q0 % nj) * 16));
+                if (q1 < nblk) tc_ld16(v[1], lane0 + (unsigned)((q1 / nj) * g.cop + (q1 % nj) * 16));
+                tc_ld_wait();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int q = h ? q1 : q0;
+                    if (q >= nblk) break;
+                    const int mt = q / nj, j = (q - mt * nj) * 16;
+                    int b, y, x;
+                    if (!out_pixel<MT>(a, g, mt, m, b, y, x)) continue;
+                    const long long pix = ((long long)b * a.H + y) * a.W + x;
+                    const long long o = pix * a.ldy + a.yoff + co0 + j;
                     float f[16];
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int co = co0 + j + e;
-                        float val = __uint_as_float(v[e]) + ((a.bias && co < a.Co) ? __ldg(a.bias + co) : 0.f);
-                        if (a.act) val = val > 0.f ? val : SLOPE * val;
-                        f[e] = val;
+                    for (int e = 0; e < 4; ++e) {
+                        const float4 bi = S.bias[j / 4 + e];
+                        f[4 * e] = __uint_as_float(v[h][4 * e]) + bi.x;
+                        f[4 * e + 1] = __uint_as_float(v[h][4 * e + 1]) + bi.y;
+                        f[4 * e + 2] = __uint_as_float(v[h][4 * e + 2]) + bi.z;
+                        f[4 * e + 3] = __uint_as_float(v[h][4 * e + 3]) + bi.w;
+                    }
+                    if (a.act) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) f[e] = fmaxf(f[e], SLOPE * f[e]);      // LeakyReLU, 0 < SLOPE < 1
                     }
                     const bool whole = co0 + j + 16 <= a.Co;
                     if (a.yf) {
-                        if (whole && (((uintptr_t)(a.yf + o0) | (a.yf2 ? (uintptr_t)(a.yf2 + o0) : 0)) & 15) == 0) {
-#pragma unroll
-                            for (int e = 0; e < 16; e += 4) {
-                                const float4 q = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
-                                *reinterpret_cast<float4*>(a.yf + o0 + j + e) = q;
-                                if (a.yf2) *reinterpret_cast<float4*>(a.yf2 + o0 + j + e) = q;
+                        if (whole && (((uintptr_t)(a.yf + o) | (a.yf2 ? (uintptr_t)(a.yf2 + o) : 0)) & 31) == 0) {
+                            const unsigned(*w)[8] = reinterpret_cast<const unsigned(*)[8]>(f);
+                            st32(a.yf + o, w[0]);
+                            st32(a.yf + o + 8, w[1]);
+                            if (a.yf2) {
+                                st32(a.yf2 + o, w[0]);
+                                st32(a.yf2 + o + 8, w[1]);
                             }
                         } else {
+#pragma unroll
                             for (int e = 0; e < 16; ++e)
                                 if (co0 + j + e < a.Co) {
-                                    a.yf[o0 + j + e] = f[e];
-                                    if (a.yf2) a.yf2[o0 + j + e] = f[e];
+                                    a.yf[o + e] = f[e];
+                                    if (a.yf2) a.yf2[o + e] = f[e];
                                 }
                         }
                         continue;
@@ -458,23 +510,19 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
                             r[e] = __floats2bfloat162_rn(mm.x > 0.f ? gg.x : SLOPE * gg.x, mm.y > 0.f ? gg.y : SLOPE * gg.y);
                         }
                     }
-                    if (whole && ((uintptr_t)(a.y + o0) & 15) == 0) {
-                        const uint4 w0 = *reinterpret_cast<const uint4*>(r), w1 = *reinterpret_cast<const uint4*>(r + 4);
-                        *reinterpret_cast<uint4*>(a.y + o0 + j) = w0;
-                        *reinterpret_cast<uint4*>(a.y + o0 + j + 8) = w1;
-                        if (a.up) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                bf16* d = a.up + (((long long)b * 2 * a.H + 2 * y + (q >> 1)) * 2 * a.W + 2 * x + (q & 1)) * a.ldu +
-                                          co0 + j;
-                                *reinterpret_cast<uint4*>(d) = w0;
-                                *reinterpret_cast<uint4*>(d + 8) = w1;
-                            }
-                        }
+                    const unsigned(&w)[8] = *reinterpret_cast<const unsigned(*)[8]>(r);
+                    if (whole && ((uintptr_t)(a.y + o) & 31) == 0) {
+                        st32(a.y + o, w);
                     } else {
 #pragma unroll
                         for (int e = 0; e < 16; ++e)
-                            if (co0 + j + e < a.Co) a.y[o0 + j + e] = e & 1 ? r[e >> 1].y : r[e >> 1].x;
+                            if (co0 + j + e < a.Co) a.y[o + e] = e & 1 ? r[e >> 1].y : r[e >> 1].x;
+                    }
+                    if (a.up) {                     // the network's own buffers: whole blocks, aligned
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            st32(a.up + (((long long)b * 2 * a.H + 2 * y + (u >> 1)) * 2 * a.W + 2 * x + (u & 1)) * a.ldu + co0 + j,
+                                 w);
                     }
                 }
             }
@@ -483,7 +531,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (S.fail && tid == 0) atomicExch(err, 1);
-    if (warp == 4) {
+    if (warp == TC_COPY / 32) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.ncol));
     }
@@ -492,18 +540,19 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
 // ------------------------------------------------------------------ weight gradient
 //
 // gw[t][co][ci] = sum over pixels of gz[p][co] x[p + off_t][ci] on the tensor cores: M = input channels
-// (up to 128 per CTA), N = output channels (up to 48), K = pixels, one accumulator of N columns per tap
-// (9 N <= 432 of the 512 tensor-memory columns), so one pass over the pixels serves all nine taps.  The
-// channels are the contiguous index of both operands, so they are read MN-major: [channel group of
-// 8][position][8], where a tap is again a constant offset of the position.
+// (up to 128 per CTA), N = (dx, output channel), up to 3 x 48, K = pixels q = p + dx of an input row; one
+// accumulator of N columns per dy (3 N <= 432 of the 512 tensor-memory columns), so one pass over the
+// pixels serves all nine taps.  The channels are the contiguous index of both operands, so they are read
+// MN-major: [channel group of 8][position][8].  The gradient row is staged three times, shifted by dx,
+// as three runs of channel groups.
 // A CTA takes units of up to RB rows of a 32-column strip, every S-th unit: stage j of a unit brings
-// input row y0 - 1 + j (34 positions) and, from j = 2, the gradient row y0 + j - 2 (32 positions, zero
-// beyond the image), whose 18 MMAs (2 x 16 positions, 9 taps) then read the input rows of the stages
-// j - 2 .. j.  Up to 16 stages are in flight; a stage is released by the MMAs that read it last and by
-// the warp that adds the gradient rows for the bias.  Each CTA writes one partial sum, k_sum_parts adds
-// the S partials in a fixed order.
-// What bounds it: the M = 128 operand of every MMA is read from shared memory (4 KB, 32 cycles; 9 x 2
-// per row); at few input channels most of its rows are not used, which costs nothing more.
+// gradient row y0 - 1 + j and, from j = 2, input row r = y0 + j - 2, whose 6 MMAs (2 x 16 positions,
+// 3 dy) then read the gradient rows r - dy of the stages j - 2 .. j.  Up to 16 stages are in flight; a
+// stage is released by the MMAs that read it last and by the warp that adds the gradient rows for the
+// bias.  Each CTA writes one partial sum, k_sum_parts adds the S partials in a fixed order.
+// What bounds it: the M = 128 operand of an MMA takes 32 cycles to read from shared memory, whatever its
+// N (at few input channels most of its rows are not used, which costs nothing more), so the taps of a
+// row share it: N = 96 takes 56 cycles where three of N = 32 take 3 x 40.
 
 struct WgradArgs {
     const bf16* x;          // layer input (pixel stride ldx, offset xoff)
@@ -522,7 +571,7 @@ struct WgradGeo {
     long long n;            // values of a partial sum
 };
 
-constexpr int WG_PX = 34, WG_PZ = 32;            // staged positions of an input and a gradient row
+constexpr int WG_P = 32;                         // positions of a staged row
 constexpr int WG_NMAX = 48;
 
 __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__ WgradArgs a,
@@ -531,7 +580,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
     extern __shared__ __align__(128) unsigned char smem[];
     TcShared& S = *reinterpret_cast<TcShared*>(smem);
     const int zg = g.cob / 8;
-    const int xbytes = g.cib / 8 * WG_PX * 16, sbytes = xbytes + zg * WG_PZ * 16;
+    const int xbytes = g.cib / 8 * WG_P * 16, sbytes = xbytes + 3 * zg * WG_P * 16;
     const unsigned stage0 = smem_u32(smem) + TC_HEAD;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ci0 = blockIdx.y * g.cib, co0 = blockIdx.z * g.cob;
@@ -540,14 +589,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
 
     if (tid == 0) {
         for (int s = 0; s < slots; ++s) {
-            mbar_init(&S.xfull[s], 128);
+            mbar_init(&S.xfull[s], TC_COPY);
             mbar_init(&S.empty[s], 2);
         }
         mbar_init(&S.done, 1);
         S.fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4) {
+    if (warp == TC_COPY / 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem)),
                      "r"(g.ncol));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -559,78 +608,89 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
     const int per = g.strips * g.rbs;
 
     bool ok = true;
-    if (warp < 4) {
+    if (warp < TC_COPY / 32) {
         // ---- rows: 16-byte units (position, channel group), the channels of a position side by side
-        int xp[5], xd[5], zp[2], zd[2];
-        long long xs[5], zs[2];
+        constexpr int NX = 2, NZ = 3;       // units per thread: 16 x 32 / 256, 18 x 32 / 256
+        int xp[NX], xd[NX], zp[NZ], zd[NZ];
+        long long xs[NX], zs[NZ];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            const int u = tid + 128 * i, p = u / xg, q = u - p * xg;
-            xp[i] = p < WG_PX ? p : -1;
-            xd[i] = (q * WG_PX + p) * 16;
-            xs[i] = (long long)(p - 1) * a.ldx + a.xoff + ci0 + 8 * q;
+        for (int i = 0; i < NX; ++i) {
+            const int u = tid + TC_COPY * i, p = u / xg, q = u - p * xg;
+            xp[i] = p < WG_P ? p : -1;
+            xd[i] = (q * WG_P + p) * 16;
+            xs[i] = (long long)p * a.ldx + a.xoff + ci0 + 8 * q;
         }
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int u = tid + 128 * i, p = u / zg, q = u - p * zg;
-            zp[i] = p < WG_PZ ? p : -1;
-            zd[i] = xbytes + (q * WG_PZ + p) * 16;
-            zs[i] = co0 + 8 * q < a.Co ? (long long)p * a.Co + co0 + 8 * q : -1;
+        for (int i = 0; i < NZ; ++i) {
+            // (dx, position, group): position q of copy dx holds the gradient at column q - dx
+            const int u = tid + TC_COPY * i, r = u / zg, q = u - r * zg, dx = r / WG_P - 1, p = r % WG_P;
+            const bool in = dx <= 1 && co0 + 8 * q < a.Co;
+            zp[i] = dx <= 1 ? (in ? p - dx : -2) : -3;
+            zd[i] = xbytes + (((dx + 1) * zg + q) * WG_P + p) * 16;
+            zs[i] = (long long)(p - dx) * a.Co + co0 + 8 * q;
         }
         pdl_wait();
-        unsigned J = 0;
+        int s = 0;
+        unsigned par = 1;                   // the first round finds the stages free
+        const long long zrow = (long long)a.W * a.Co, xrow = (long long)a.W * a.ldx;
         for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
             const int b = u / per, r = u - b * per;
-            const int x0 = (r / g.rbs) * 32, y0 = (r % g.rbs) * g.RB;
+            const int x0 = (r / g.rbs) * WG_P, y0 = (r % g.rbs) * g.RB;
             const int rows = min(g.RB, a.H - y0);
-            for (int j = 0; j < rows + 2; ++j, ++J) {
-                const unsigned s = J % (unsigned)slots;
-                if (J >= (unsigned)slots) ok = mbar_wait(&S.empty[s], (J / (unsigned)slots - 1) & 1u);
-                if (!ok) break;
-                const unsigned dst = stage0 + s * (unsigned)sbytes;
-                const int yx = y0 - 1 + j;
-                const bool rowx = yx >= 0 && yx < a.H;
-                const bf16* bx = a.x + (((long long)b * a.H + yx) * a.W + x0) * a.ldx;
+            // this thread's columns of the strip: inside the image or not
+            bool xin[NX], zin[NZ];
 #pragma unroll
-                for (int i = 0; i < 5; ++i) {
-                    if (xp[i] < 0) continue;
-                    const int x = x0 - 1 + xp[i];
-                    const bool in = rowx && x >= 0 && x < a.W;
-                    cp_async16(dst + (unsigned)xd[i], in ? bx + xs[i] : a.x, in ? 16 : 0);
+            for (int i = 0; i < NX; ++i) xin[i] = x0 + xp[i] < a.W;
+#pragma unroll
+            for (int i = 0; i < NZ; ++i) zin[i] = zp[i] > -2 && x0 + zp[i] >= 0 && x0 + zp[i] < a.W;
+            const bf16* bz = a.gz + (((long long)b * a.H + y0 - 1) * a.W + x0) * a.Co;
+            const bf16* bx = a.x + (((long long)b * a.H + y0 - 2) * a.W + x0) * a.ldx;
+            for (int j = 0; j < rows + 2; ++j, bz += zrow, bx += xrow) {
+                ok = mbar_wait(&S.empty[s], par);
+                if (!ok) break;
+                const unsigned dst = stage0 + (unsigned)(s * sbytes);
+                const bool rowz = y0 - 1 + j >= 0 && y0 - 1 + j < a.H;
+#pragma unroll
+                for (int i = 0; i < NZ; ++i) {
+                    if (zp[i] == -3) continue;
+                    const bool in = rowz && zin[i];
+                    cp_async16(dst + (unsigned)zd[i], in ? bz + zs[i] : a.gz, in ? 16 : 0);
                 }
                 if (j >= 2) {
-                    const bf16* bz = a.gz + (((long long)b * a.H + y0 + j - 2) * a.W + x0) * a.Co;
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        if (zp[i] < 0) continue;
-                        const bool in = zs[i] >= 0 && x0 + zp[i] < a.W;
-                        cp_async16(dst + (unsigned)zd[i], in ? bz + zs[i] : a.gz, in ? 16 : 0);
+                    for (int i = 0; i < NX; ++i) {
+                        if (xp[i] < 0) continue;
+                        cp_async16(dst + (unsigned)xd[i], xin[i] ? bx + xs[i] : a.x, xin[i] ? 16 : 0);
                     }
                 }
                 cp_async_arrive(&S.xfull[s]);
+                if (++s == slots) {
+                    s = 0;
+                    par ^= 1u;
+                }
             }
         }
         pdl_trigger();
-    } else if (warp == 5) {
+    } else if (warp == TC_COPY / 32 + 1) {
         // ---- bias: the gradient rows added up, one position per lane
         float acc[WG_NMAX];
 #pragma unroll
         for (int e = 0; e < WG_NMAX; ++e) acc[e] = 0.f;
-        unsigned J = 0;
+        int s = 0;
+        unsigned par = 0;
         for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
             const int r = u % per;
             const int rows = min(g.RB, a.H - (r % g.rbs) * g.RB);
-            for (int j = 0; j < rows + 2; ++j, ++J) {
-                const unsigned s = J % (unsigned)slots;
+            for (int j = 0; j < rows + 2; ++j) {
                 // every stage is waited for, so that this warp's arrival belongs to the stage's own phase
-                ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], (J / (unsigned)slots) & 1u));
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], par));
                 if (!ok) break;
-                if (j >= 2 && blockIdx.y == 0) {
-                    const unsigned char* z = smem + TC_HEAD + s * (unsigned)sbytes + xbytes + lane * 16;
+                if (j >= 1 && j <= rows && blockIdx.y == 0) {       // the unit's own rows, unshifted
+                    const unsigned char* z = smem + TC_HEAD + s * sbytes + xbytes + (zg * WG_P + lane) * 16;
 #pragma unroll
                     for (int q = 0; q < WG_NMAX / 8; ++q) {
                         if (q >= zg) break;
-                        const uint4 v = *reinterpret_cast<const uint4*>(z + q * WG_PZ * 16);
+                        const uint4 v = *reinterpret_cast<const uint4*>(z + q * WG_P * 16);
                         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
@@ -643,6 +703,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
                 __syncwarp();
                 if (lane == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&S.empty[s])) : "memory");
+                if (++s == slots) {
+                    s = 0;
+                    par ^= 1u;
+                }
             }
         }
         if (ok && blockIdx.y == 0) {
@@ -655,70 +719,92 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
                     a.part[blockIdx.x * g.n + 9LL * a.Co * a.Ci + co0 + e] = v;
             }
         }
-    } else if (lane == 0) {
+    } else {
         // ---- MMAs, both operands MN-major
+        const unsigned lead = elect_one();
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                               ((uint32_t)(g.cob >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-        unsigned J = 0;
-        int acc = 0;
+                               ((uint32_t)(3 * g.cob >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        int s = 0, s1 = 0, s2 = 0, acc = 0;         // this stage and the two before it
+        unsigned par = 0;
         for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
             const int r = u % per;
             const int rows = min(g.RB, a.H - (r % g.rbs) * g.RB);
-            for (int j = 0; j < rows + 2; ++j, ++J) {
-                const unsigned s = J % (unsigned)slots;
-                ok = mbar_wait(&S.xfull[s], (J / (unsigned)slots) & 1u);
+            for (int j = 0; j < rows + 2; ++j) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], par));
                 if (!ok) break;
-                if (j < 2) continue;
+                const int sn = s + 1 == slots ? 0 : s + 1;
+                if (j < 2) {
+                    s2 = s1;
+                    s1 = s;
+                    if (sn == 0) par ^= 1u;
+                    s = sn;
+                    continue;
+                }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const unsigned sz = stage0 + s * (unsigned)sbytes + (unsigned)xbytes;
-                for (int dy = 0; dy < 3; ++dy) {
-                    const unsigned sx = stage0 + ((J - 2 + (unsigned)dy) % (unsigned)slots) * (unsigned)sbytes;
+                const uint64_t ad = tc_desc(stage0 + (unsigned)(s * sbytes), 128, WG_P * 16);
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {          // gradient row r - dy: 1 + dy stages back
+                    const int sz = dy < 0 ? s : (dy == 0 ? s1 : s2);
+                    const uint64_t bd = tc_desc(stage0 + (unsigned)(sz * sbytes + xbytes), 128, WG_P * 16);
 #pragma unroll
                     for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-                        for (int dx = 0; dx < 3; ++dx)
-                            tc_mma(tmem + (unsigned)((3 * dy + dx) * g.cob),
-                                   tc_desc(sx + (unsigned)((16 * ks + dx) * 16), 128, WG_PX * 16),
-                                   tc_desc(sz + (unsigned)(16 * ks * 16), 128, WG_PZ * 16), idesc, ks > 0 ? 1 : acc);
+                        tc_mma(tmem + (unsigned)((dy + 1) * 3 * g.cob), ad + (unsigned)(16 * ks), bd + (unsigned)(16 * ks), idesc,
+                               ks > 0 ? 1 : acc, lead);
                 }
                 acc = 1;
-                tc_commit(&S.empty[(J - 2) % (unsigned)slots]);
-                if (j == rows + 1) {
-                    tc_commit(&S.empty[(J - 1) % (unsigned)slots]);
-                    tc_commit(&S.empty[s]);
+                if (lead) {
+                    tc_commit(&S.empty[s2]);
+                    if (j == rows + 1) {
+                        tc_commit(&S.empty[s1]);
+                        tc_commit(&S.empty[s]);
+                    }
                 }
+                s2 = s1;
+                s1 = s;
+                if (sn == 0) par ^= 1u;
+                s = sn;
             }
         }
-        if (ok) tc_commit(&S.done);
+        if (ok && lead) tc_commit(&S.done);
     }
     if (!ok) S.fail = 1;
 
-    if (warp < 4) {
+    if (warp < TC_COPY / 32) {
         if (ok) ok = mbar_wait(&S.done, 0);
         if (!ok) S.fail = 1;
         cp_async_wait_all();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (ok) {
-            // warp w holds the input channels 32 w .., the columns are the output channels co0 .. of
-            // each tap
-            const bool valid = tid < 8 * xg;
-            float* out = a.part + blockIdx.x * g.n + ci0 + tid;
-            for (int t = 0; t < 9; ++t)
-                for (int j = 0; j < g.cob; j += 16) {
-                    unsigned v[16];
-                    tc_ld16(v, tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(t * g.cob + j));
-                    if (!valid) continue;
+            // warp w holds the input channels 32 (w % 4) .., the columns are the output channels co0 .. of
+            // each tap; blocks of 16 of them, every second one, two at a time
+            const int m = tid & 127, nj = g.cob / 16, nblk = 9 * nj;
+            const bool valid = m < 8 * xg;
+            const unsigned lane0 = tmem + ((unsigned)(warp & 3) << 21);
+            float* out = a.part + blockIdx.x * g.n + ci0 + m;
+            for (int q0 = warp >> 2; q0 < nblk; q0 += 4) {
+                __syncwarp();               // the lanes that stored nothing and the others
+                unsigned v[2][16];
+                tc_ld16(v[0], lane0 + (unsigned)(q0 * 16));
+                if (q0 + 2 < nblk) tc_ld16(v[1], lane0 + (unsigned)((q0 + 2) * 16));
+                tc_ld_wait();
+                if (!valid) continue;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int q = q0 + 2 * h;
+                    if (q >= nblk) break;
+                    const int t = q / nj, co = co0 + (q - t * nj) * 16;
 #pragma unroll
                     for (int e = 0; e < 16; ++e)
-                        if (co0 + j + e < a.Co) out[((long long)t * a.Co + co0 + j + e) * a.Ci] = __uint_as_float(v[e]);
+                        if (co + e < a.Co) out[((long long)t * a.Co + co + e) * a.Ci] = __uint_as_float(v[h][e]);
                 }
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (S.fail && tid == 0) atomicExch(err, 1);
-    if (warp == 4) {
+    if (warp == TC_COPY / 32) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.ncol));
     }
@@ -821,7 +907,7 @@ cudaError_t launch_tc(const ConvArgs& a, const ConvGeo& g, unsigned m_tiles, int
             return e;
         }
     }
-    const size_t smem = TC_HEAD + (size_t)g.slots * (g.npix * 32 + 288 * g.cop);
+    const size_t smem = TC_HEAD + (size_t)g.npix * 4 + (size_t)g.slots * g.cw * (g.npix * 32 + 288 * g.cop);
     return launch_pdl(k_conv_tc<MT>, dim3(m_tiles, n_cot), TC_THREADS, smem, s, pdl, a, g, g_conv_err);
 }
 
@@ -838,6 +924,7 @@ cudaError_t conv_pack(const PackArgs& p, cudaStream_t s)
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
 {
     if (a.Ci % 16 != 0) return cudaErrorInvalidValue;
+    if ((long long)a.B * a.H * a.W >= (1LL << 31)) return conv_mma(a, s);      // 32-bit pixel indices
     const cudaError_t e = conv_err_init();
     if (e != cudaSuccess) return e;
     static const int n_sm = sm_count();
@@ -851,23 +938,30 @@ cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
         if (g.flat) return (flat_n + 128 * mt - 1) / (128 * mt);
         return (long long)g.tx * ((a.H + 4 * mt - 1) / (4 * mt)) * a.B;
     };
-    // channels per CTA: all up to 128, in equal parts beyond; MMA tiles per CTA: as many as leave two
-    // CTAs per SM and fit half the tensor memory; then, where the CTAs would leave SMs empty, the
+    // channels per CTA: all up to 128, in equal parts beyond; MMA tiles per CTA: as many as leave one and
+    // a half CTAs per SM and fit half the tensor memory; then, where the CTAs would leave SMs empty, the
     // channels are split further (each part stages the input again)
     int n_cot = (g.cpk + 127) / 128;
     g.cop = ((g.cpk + n_cot - 1) / n_cot + 15) / 16 * 16;
     int mt = 4;
-    while (mt > 1 && (mt * g.cop > 256 || tiles(mt) * n_cot < 2 * n_sm)) mt /= 2;
-    while (g.cop > 16 && tiles(mt) * ((g.cpk + g.cop - 1) / g.cop) < n_sm) g.cop = (g.cop / 2 + 15) / 16 * 16;
+    while (mt > 1 && (mt * g.cop > 256 || 2 * tiles(mt) * n_cot < 3 * n_sm)) mt /= 2;
+    while (g.cop > 16 && 4 * tiles(mt) * ((g.cpk + g.cop - 1) / g.cop) < 3 * n_sm) g.cop = (g.cop / 2 + 15) / 16 * 16;
     n_cot = (g.cpk + g.cop - 1) / g.cop;
     g.ty = (a.H + 4 * mt - 1) / (4 * mt);
+    // positions: a multiple of 4 that is not one of 8, which spreads the k-halves over the banks
     g.npix = g.flat ? 128 * mt + 2 * g.pitch + 2 : (4 * mt + 2) * 32 + 8;
+    g.npix = (g.npix + 3) / 8 * 8 + 4;
+    g.d0 = FastDiv((unsigned)(g.flat ? g.pitch : g.tx));
+    g.d1 = FastDiv((unsigned)(g.flat ? a.H + 1 : g.tx * g.ty));
     g.ncol = 32;
     while ((int)g.ncol < mt * g.cop) g.ncol *= 2;
-    // stages: all chunks where one CTA has an SM to itself, else what lets two share it
-    const int sbytes = g.npix * 32 + 288 * g.cop;
-    const int room = tiles(mt) * n_cot <= n_sm ? 220 * 1024 : 110 * 1024;
-    g.slots = std::max(1, std::min(std::min(a.Ci / 16, TC_SLOTS), (room - TC_HEAD) / sbytes));
+    // stages: all chunks where one CTA has an SM to itself, else what lets two share it; the widest
+    // stage of which two fit
+    const int cbytes = g.npix * 32 + 288 * g.cop, nchunk = a.Ci / 16;
+    const int room = (tiles(mt) * n_cot <= n_sm ? 220 : 110) * 1024 - TC_HEAD - g.npix * 4;
+    for (g.cw = 4, g.lgh = 3; g.cw > 1; g.cw /= 2, --g.lgh)
+        if (nchunk % g.cw == 0 && std::min(2, nchunk / g.cw) * g.cw * cbytes <= room) break;
+    g.slots = std::max(1, std::min(std::min(nchunk / g.cw, TC_SLOTS), room / (g.cw * cbytes)));
     const long long m_tiles = tiles(mt);
     if (m_tiles > 0x7fffffffLL || n_cot > 65535) return cudaErrorInvalidConfiguration;
     switch (mt) {
@@ -908,8 +1002,8 @@ static int wgrad_geo(int B, int H, int W, int Ci, int Co, long long room, WgradG
     const long long units = (long long)B * g.strips * g.rbs;
     g.units = (int)std::min<long long>(units, 0x7fffffff);
     S = std::min(S, units);
-    const int sbytes = g.cib / 8 * WG_PX * 16 + g.cob / 8 * WG_PZ * 16;
-    const int bytes = (occ > 1 ? 108 : 216) * 1024 - TC_HEAD - 17 * WG_PX * 16;
+    const int sbytes = (g.cib / 8 + 3 * (g.cob / 8)) * WG_P * 16;
+    const int bytes = (occ > 1 ? 108 : 216) * 1024 - TC_HEAD - 17 * WG_P * 16;
     g.slots = std::max(4, std::min(TC_SLOTS, bytes / sbytes));
     return (int)S;
 }
@@ -939,7 +1033,7 @@ cudaError_t conv_wgrad(cudaStream_t s, const bf16* x, long long ldx, int xoff, c
     a.x = x; a.ldx = ldx; a.xoff = xoff; a.gz = gz; a.part = part;
     a.B = B; a.H = H; a.W = W; a.Ci = Ci; a.Co = Co;
     // the last stage's operand of 128 channels may reach past its own channels: 16 groups of slack
-    const size_t smem = TC_HEAD + (size_t)g.slots * (g.cib / 8 * WG_PX * 16 + g.cob / 8 * WG_PZ * 16) + 17 * WG_PX * 16;
+    const size_t smem = TC_HEAD + (size_t)g.slots * (g.cib / 8 + 3 * (g.cob / 8)) * WG_P * 16 + 17 * WG_P * 16;
     e = launch_pdl(k_wgrad_tc, dim3(S, (Ci + g.cib - 1) / g.cib, (Co + g.cob - 1) / g.cob), TC_THREADS, smem, s, pdl, a, g,
                    g_conv_err);
     if (e != cudaSuccess) return e;
