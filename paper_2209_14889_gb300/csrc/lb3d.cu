@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "../../include/lb3d.h"
+#include "lb_vec.cuh"
 
 namespace v3 {
 
@@ -56,7 +57,6 @@ struct Args3 {
     float* u;                    // u(t) [3]
     float* ys;                   // predictor y* [9]
     float* r0;                   // RHS(y) [9]
-    float* mom;                  // moments pass: drho, ux, uy, uz [4]
     const float4* lut;           // coefficients of C:X against |P| (two float4 per entry)
     long long NP;
     int nx, ny, nz;
@@ -67,7 +67,9 @@ struct Args3 {
     int ericksen;
     int readout;                 // k3_collide: sum the readouts of this step
     long long t;
-    double* partials;            // [CTAs][7]
+    unsigned n_ctas;             // CTAs of k3_collide
+    long long ahead;             // cells ahead whose planes the stencil kernels prefetch into L2 (0: none)
+    double* partials;            // [n_ctas][7]
     double* gpartials;           // [groups of NT CTAs][7]
     double* row;                 // readout row of this step (8 values)
     int* err_nonfinite;
@@ -109,11 +111,14 @@ __device__ __forceinline__ float lap7(const float* v) { return v[1] + v[2] + v[3
 __device__ __forceinline__ float dif(const float* v, int a) { return 0.5f * (v[1 + 2 * a] - v[2 + 2 * a]); }
 
 // alpha + beta |P|^2 at P = P_ref + dP without the cancellation near the equilibrium modulus
-__device__ __forceinline__ float bulk(const Args3& a, float dx, float dy, float dz)
+template <class T>
+__device__ __forceinline__ T bulk(const Args3& a, T dx, T dy, T dz)
 {
-    const float pd = a.prx * dx + a.pry * dy + a.prz * dz;
-    const float dd = dx * dx + dy * dy + dz * dz;
-    return a.A0 + a.beta * (2.f * pd + dd);
+    using vlb::vec::vfma;
+    using vlb::vec::operator*;
+    const T pd = vfma(a.prx, dx, vfma(a.pry, dy, a.prz * dz));
+    const T dd = vfma(dx, dx, vfma(dy, dy, dz * dz));
+    return vfma(a.beta, vfma(2.f, pd, dd), vlb::vec::bc<T>(a.A0));
 }
 
 // symmetric-tensor component (xx, yy, zz, yz, xz, xy) of (i, j)
@@ -122,25 +127,90 @@ __device__ __forceinline__ int sym6(int i, int j)
     return i == j ? i : (i + j == 3 ? 3 : (i + j == 2 ? 4 : 5));
 }
 
+// One cell per thread (T = float) or the two cells x, x + 1 (T = float2, x even: nx even), whose
+// arithmetic then runs on paired FP32 instructions and whose stencil points other than +-x are 8-byte
+// loads.
+using vlb::vec::operator+;
+using vlb::vec::operator-;
+using vlb::vec::operator*;
+using vlb::vec::bc;
+using vlb::vec::vfma;
+
+// Consecutive kernels of a step overlap by programmatic dependent launch: each waits for the one before
+// it to complete before it touches memory, then lets the next one start its CTAs.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class T>
+struct Nb {                      // flat indices: the cell (pair), +x of its last cell, -x of its first, +-y, +-z
+    int c, xp, xm, yp, ym, zp, zm;
+};
+
+template <class T>
+__device__ __forceinline__ bool nb_of(const Args3& a, Nb<T>& q)
+{
+    constexpr int W = vlb::vec::Lanes<T>::N;
+    const int x = W * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z * blockDim.z + threadIdx.z;
+    if (x >= a.nx || y >= a.ny || z >= a.nz) return false;
+    const int nx = a.nx, nxy = a.nx * a.ny;
+    q.c = z * nxy + y * nx + x;
+    q.xp = q.c + (x + W == nx ? W - nx : W);
+    q.xm = q.c + (x == 0 ? nx - 1 : -1);
+    q.yp = q.c + (y + 1 == a.ny ? nx - nxy : nx);
+    q.ym = q.c + (y == 0 ? nxy - nx : -nx);
+    q.zp = q.c + (z + 1 == a.nz ? nxy - nxy * a.nz : nxy);
+    q.zm = q.c + (z == 0 ? nxy * a.nz - nxy : -nxy);
+    return true;
+}
+
+template <class T>
+__device__ __forceinline__ T ldv(const float* p) { return __ldg(reinterpret_cast<const T*>(p)); }
+template <class T>
+__device__ __forceinline__ void stv(float* p, T v) { *reinterpret_cast<T*>(p) = v; }
+
+// value, differences f(+) - f(-) along x, y, z and the sum of the six neighbours of plane f
+__device__ __forceinline__ void fold(const float* f, const Nb<float>& q, float& c, float& dx, float& dy, float& dz, float& sum)
+{
+    c = __ldg(f + q.c);
+    const float xp = __ldg(f + q.xp), xm = __ldg(f + q.xm), yp = __ldg(f + q.yp), ym = __ldg(f + q.ym),
+                zp = __ldg(f + q.zp), zm = __ldg(f + q.zm);
+    dx = xp - xm;
+    dy = yp - ym;
+    dz = zp - zm;
+    sum = ((xp + xm) + (yp + ym)) + (zp + zm);
+}
+__device__ __forceinline__ void fold(const float* f, const Nb<float2>& q, float2& c, float2& dx, float2& dy, float2& dz,
+                                     float2& sum)
+{
+    c = ldv<float2>(f + q.c);
+    const float r = __ldg(f + q.xp), l = __ldg(f + q.xm);
+    const float2 yp = ldv<float2>(f + q.yp), ym = ldv<float2>(f + q.ym), zp = ldv<float2>(f + q.zp), zm = ldv<float2>(f + q.zm);
+    const float2 xp = make_float2(c.y, r), xm = make_float2(l, c.x);
+    dx = xp - xm;
+    dy = yp - ym;
+    dz = zp - zm;
+    sum = ((xp + xm) + (yp + ym)) + (zp + zm);
+}
+
 // ---- stiffness: the transversely isotropic contraction C(P):X --------------------------------
+template <class T>
 struct Stiff {
-    float n[3];
-    float cpp_n, g;              // c_pp = cpp_n pXp + g trX
-    float cd_t;                  // c_d  = g pXp + cd_t trX
-    float cs, cX;
+    T n[3];
+    T cpp_n, g;                  // c_pp = cpp_n pXp + g trX
+    T cd_t;                      // c_d  = g pXp + cd_t trX
+    T cs, cX;
 };
 
 // The table holds, per |P|, the five scalar coefficients of C:X (formed on the host in FP64 from
 // the orientation moments and K^x, so the cancellations in e1, e2, e3 never happen in FP32):
 // (cpp_n, g, cd_t, cs) and (cX, -, -, -).
-__device__ __forceinline__ Stiff stiffness(const Args3& a, float px, float py, float pz)
+__device__ __forceinline__ void stiffness(const Args3& a, const float (&p)[3], Stiff<float>& S)
 {
-    Stiff S;
-    const float P2 = px * px + py * py + pz * pz;
-    const float Pm = sqrtf(P2);
+    const float Pm = sqrtf(p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
     if (Pm > 0.f) {
         const float r = 1.f / Pm;
-        S.n[0] = px * r; S.n[1] = py * r; S.n[2] = pz * r;
+        S.n[0] = p[0] * r; S.n[1] = p[1] * r; S.n[2] = p[2] * r;
     } else {
         S.n[0] = 1.f; S.n[1] = 0.f; S.n[2] = 0.f;
     }
@@ -155,106 +225,143 @@ __device__ __forceinline__ Stiff stiffness(const Args3& a, float px, float py, f
     S.cd_t = u0.z + f * (u1.z - u0.z);
     S.cs = u0.w + f * (u1.w - u0.w);
     S.cX = v0 + f * (v1 - v0);
-    return S;
+}
+__device__ __forceinline__ void stiffness(const Args3& a, const float2 (&p)[3], Stiff<float2>& S)
+{
+    Stiff<float> A, B;
+    const float pa[3] = {p[0].x, p[1].x, p[2].x}, pb[3] = {p[0].y, p[1].y, p[2].y};
+    stiffness(a, pa, A);
+    stiffness(a, pb, B);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) S.n[i] = make_float2(A.n[i], B.n[i]);
+    S.cpp_n = make_float2(A.cpp_n, B.cpp_n);
+    S.g = make_float2(A.g, B.g);
+    S.cd_t = make_float2(A.cd_t, B.cd_t);
+    S.cs = make_float2(A.cs, B.cs);
+    S.cX = make_float2(A.cX, B.cX);
 }
 
 // out = C:X for the symmetric X (6 components)
-__device__ __forceinline__ void apply_c(const Stiff& S, const float* X, float* out)
+template <class T>
+__device__ __forceinline__ void apply_c(const Stiff<T>& S, const T* X, T* out)
 {
-    const float* n = S.n;
-    const float Xn0 = X[0] * n[0] + X[5] * n[1] + X[4] * n[2];
-    const float Xn1 = X[5] * n[0] + X[1] * n[1] + X[3] * n[2];
-    const float Xn2 = X[4] * n[0] + X[3] * n[1] + X[2] * n[2];
-    const float nXn = n[0] * Xn0 + n[1] * Xn1 + n[2] * Xn2;
-    const float tr = X[0] + X[1] + X[2];
-    const float cpp = S.cpp_n * nXn + S.g * tr;
-    const float cd = S.g * nXn + S.cd_t * tr;
-    const float Xn[3] = {Xn0, Xn1, Xn2};
+    const T* n = S.n;
+    const T Xn[3] = {vfma(X[0], n[0], vfma(X[5], n[1], X[4] * n[2])), vfma(X[5], n[0], vfma(X[1], n[1], X[3] * n[2])),
+                     vfma(X[4], n[0], vfma(X[3], n[1], X[2] * n[2]))};
+    const T nXn = vfma(n[0], Xn[0], vfma(n[1], Xn[1], n[2] * Xn[2]));
+    const T tr = (X[0] + X[1]) + X[2];
+    const T cpp = vfma(S.cpp_n, nXn, S.g * tr);
+    const T cd = vfma(S.g, nXn, S.cd_t * tr);
+    // cpp n_i n_j + cs (n_i Xn_j + Xn_i n_j) = n_i V_j + V_i n_j with V = cpp n / 2 + cs Xn
+    const T hc = 0.5f * cpp;
+    T V[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) V[i] = vfma(hc, n[i], S.cs * Xn[i]);
     const int I[6] = {0, 1, 2, 1, 0, 0}, J[6] = {0, 1, 2, 2, 2, 1};
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
         const int i = I[c], j = J[c];
-        out[c] = cpp * n[i] * n[j] + (i == j ? cd : 0.f) + S.cs * (n[i] * Xn[j] + Xn[i] * n[j]) + S.cX * X[c];
+        if (i == j) out[c] = vfma(2.f * n[i], V[i], vfma(S.cX, X[c], cd));
+        else out[c] = vfma(n[i], V[j], vfma(V[i], n[j], S.cX * X[c]));
     }
 }
 
 // ---- right-hand sides of Eq. StiffCons (Jaumann derivative) and Eq. BE -----------------------
 // y = (sigma (6), dP = P - P_ref (3)) at the cell, reduced from each component's stencil as it is
 // loaded: the value, the advection u.grad (central differences) and the 7-point Laplacian
+template <class T>
 struct Y9 {
-    float c[9], adv[9], lap[9];
+    T c[9], adv[9], lap[9];
 };
 
-__device__ __forceinline__ void load_y9(const float* base, long long NP, const Cell& q, const float* uc, Y9& y)
+template <class T>
+__device__ __forceinline__ void load_y9(const float* base, long long NP, const Nb<T>& q, const T* uc, Y9<T>& y)
 {
+    const T hu[3] = {0.5f * uc[0], 0.5f * uc[1], 0.5f * uc[2]};
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        float v[7];
-        stencil(base + k * NP, q, v);
-        y.c[k] = v[0];
-        y.adv[k] = uc[0] * dif(v, 0) + uc[1] * dif(v, 1) + uc[2] * dif(v, 2);
-        y.lap[k] = lap7(v);
+        T dx, dy, dz, sum;
+        fold(base + k * NP, q, y.c[k], dx, dy, dz, sum);
+        y.adv[k] = vfma(hu[0], dx, vfma(hu[1], dy, hu[2] * dz));
+        y.lap[k] = vfma(-6.f, y.c[k], sum);
     }
 }
 
-// uc: u at the cell; G[i][j] = d_i u_j; h: molecular field at the cell
-__device__ __forceinline__ void rhs9(const Args3& a, const Y9& y, const float (*G)[3], const float* h, float* r)
+// u at the cell, Psi (xx, yy, zz, yz, xz, xy) and Om (01, 02, 12) of its gradient G_ij = d_i u_j
+// (central differences)
+template <class T>
+struct Flow {
+    T u[3], psi[6], om[3];
+};
+
+template <class T>
+__device__ __forceinline__ void flow(const Args3& a, const Nb<T>& q, Flow<T>& f)
 {
-    float Psi[3][3], Om[3][3], s[3][3];
+    T G[3][3], sum;              // 2 G
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) fold(a.u + j * a.NP, q, f.u[j], G[0][j], G[1][j], G[2][j], sum);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            Psi[i][j] = 0.5f * (G[i][j] + G[j][i]);
-            Om[i][j] = 0.5f * (G[i][j] - G[j][i]);
-            s[i][j] = y.c[sym6(i, j)];
-        }
-    const float P[3] = {a.prx + y.c[6], a.pry + y.c[7], a.prz + y.c[8]};
-    const Stiff S = stiffness(a, P[0], P[1], P[2]);
+    for (int i = 0; i < 3; ++i) f.psi[i] = 0.5f * G[i][i];
+    f.psi[3] = 0.25f * (G[1][2] + G[2][1]);
+    f.psi[4] = 0.25f * (G[0][2] + G[2][0]);
+    f.psi[5] = 0.25f * (G[0][1] + G[1][0]);
+    f.om[0] = 0.25f * (G[0][1] - G[1][0]);
+    f.om[1] = 0.25f * (G[0][2] - G[2][0]);
+    f.om[2] = 0.25f * (G[1][2] - G[2][1]);
+}
+
+// the right-hand side at y, h the molecular field of its P (Eq. Ffunctional)
+template <class T>
+__device__ __forceinline__ void rhs9(const Args3& a, const Y9<T>& y, const Flow<T>& f, T* r)
+{
+    const T *s = y.c, *psi = f.psi;
+    const T oa = f.om[0], ob = f.om[1], oc = f.om[2];
+    const T P[3] = {y.c[6] + a.prx, y.c[7] + a.pry, y.c[8] + a.prz};
+    Stiff<T> S;
+    stiffness(a, P, S);
     // C Psi - C sigma / eta_p = C (Psi - sigma / eta_p): one contraction (C is linear in X)
-    const float psi6[6] = {Psi[0][0], Psi[1][1], Psi[2][2], Psi[1][2], Psi[0][2], Psi[0][1]};
-    float X6[6], CX6[6];
+    T X6[6], CX[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) X6[c] = psi6[c] - a.inv_eta * y.c[c];
-    apply_c(S, X6, CX6);
-    const int I[6] = {0, 1, 2, 1, 0, 0}, J[6] = {0, 1, 2, 2, 2, 1};
+    for (int c = 0; c < 6; ++c) X6[c] = vfma(-a.inv_eta, s[c], psi[c]);
+    apply_c(S, X6, CX);
+    // -(Omega s - s Omega) with Omega = (0 a b; -a 0 c; -b -c 0)
+    T nJ[6];
+    nJ[0] = -2.f * vfma(oa, s[5], ob * s[4]);
+    nJ[1] = 2.f * vfma(oa, s[5], -1.f * (oc * s[3]));
+    nJ[2] = 2.f * vfma(ob, s[4], oc * s[3]);
+    nJ[3] = vfma(oa, s[4], vfma(ob, s[5], oc * (s[1] - s[2])));
+    nJ[4] = vfma(ob, s[0] - s[2], vfma(oc, s[5], -1.f * (oa * s[3])));
+    nJ[5] = vfma(oa, s[0] - s[1], -1.f * vfma(ob, s[3], oc * s[4]));
 #pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        const int i = I[c], j = J[c];
-        float Jc = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Jc += Om[i][k] * s[k][j] - s[i][k] * Om[k][j];
-        r[c] = -y.adv[c] - Jc + CX6[c] + a.Dp * y.lap[c];
-    }
+    for (int c = 0; c < 6; ++c) r[c] = vfma(a.Dp, y.lap[c], (CX[c] + nJ[c]) - y.adv[c]);
+    // Eq. BE with h = (alpha + beta |P|^2) P - kappa lap P
+    const T A = bulk(a, y.c[6], y.c[7], y.c[8]);
+    const T rot[3] = {vfma(oa, P[1], ob * P[2]), vfma(oc, P[2], -1.f * (oa * P[0])), -1.f * vfma(ob, P[0], oc * P[1])};
+    const T str[3] = {vfma(psi[0], P[0], vfma(psi[5], P[1], psi[4] * P[2])),
+                      vfma(psi[5], P[0], vfma(psi[1], P[1], psi[3] * P[2])),
+                      vfma(psi[4], P[0], vfma(psi[3], P[1], psi[2] * P[2]))};
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        float rot = 0.f, str = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            rot += Om[i][k] * P[k];
-            str += Psi[i][k] * P[k];
-        }
-        r[6 + i] = -y.adv[6 + i] - rot + a.xi * str - a.Gamma * h[i];
+        const T h = vfma(A, P[i], (-a.kappa) * y.lap[6 + i]);
+        r[6 + i] = vfma(-a.Gamma, h, vfma(a.xi, str[i], -1.f * (rot[i] + y.adv[6 + i])));
     }
 }
 
-// u at the cell and its gradient G[i][j] = d_i u_j (central differences)
-__device__ __forceinline__ void flow(const Args3& a, const Cell& q, float* uc, float (*G)[3])
+// n planes of a row of 32 cells, a.ahead cells further on, into L2 (one lane per row)
+__device__ __forceinline__ void prefetch_rows(const Args3& a, const float* base, int n, int c)
 {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        float v[7];
-        stencil(a.u + j * a.NP, q, v);
-        uc[j] = v[0];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) G[i][j] = dif(v, i);
-    }
+    if (c + a.ahead >= a.NP) return;
+    const float* p = base + c + a.ahead;
+    for (int k = 0; k < n; ++k, p += a.NP) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // ---- kernels ---------------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(NT) k3_molecular(const Args3 a, const float* dP)
+// row: the row i of sigma^E_ij wanted (-1: all)
+__global__ void __launch_bounds__(NT) k3_molecular(const __grid_constant__ Args3 a, const float* dP, int row)
 {
+    pdl_wait();
+    pdl_trigger();
     Cell q;
     if (!cell_of(a, q)) return;
     float v[3][7];                  // stencils of dP = P - P_ref
@@ -271,7 +378,8 @@ __global__ void __launch_bounds__(NT) k3_molecular(const Args3 a, const float* d
 #pragma unroll
         for (int k = 0; k < 3; ++k) gP[i][k] = dif(v[k], i);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 3; ++i) {
+        if (row >= 0 && i != row) continue;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             const float Pi = P[i], Pj = P[j];
@@ -279,6 +387,7 @@ __global__ void __launch_bounds__(NT) k3_molecular(const Args3 a, const float* d
             a.sE[(i * 3 + j) * a.NP + q.c] = -0.5f * (Pi * h[j] - h[i] * Pj) + 0.5f * a.xi * (Pi * h[j] + h[i] * Pj)
                                              - a.kappa * gg;
         }
+    }
 }
 
 // Fixed-order sums of the readout values v[7] of a CTA into out[7]: FP32 within each warp (a
@@ -286,7 +395,7 @@ __global__ void __launch_bounds__(NT) k3_molecular(const Args3 a, const float* d
 // is a narrow unit on this GPU: seven short chains, not one long one).
 __device__ __forceinline__ void cta_sum7(const float* v, double* out, float* sm)
 {
-    const int tid = threadIdx.x + BX * (threadIdx.y + BY * threadIdx.z);
+    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
     for (int k = 0; k < 7; ++k) {
@@ -307,7 +416,7 @@ __device__ __forceinline__ void cta_sum7(const float* v, double* out, float* sm)
 // fixed-order FP64 block sum of v[7] (thread 0 returns the totals)
 __device__ __forceinline__ void block_sum7(double* v, double* sm)
 {
-    const int tid = threadIdx.x + BX * (threadIdx.y + BY * threadIdx.z);
+    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
     for (int k = 0; k < 7; ++k) {
@@ -326,9 +435,11 @@ __device__ __forceinline__ void block_sum7(double* v, double* sm)
     }
 }
 
-// mode 0: the step's collision and streaming; mode 1: moments of the current state only
-__global__ void __launch_bounds__(NT, 4) k3_collide(const Args3 a, int mode)
+// the step's collision and streaming
+__global__ void __launch_bounds__(NT, 4) k3_collide(const __grid_constant__ Args3 a)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float sRedF[(NT / 32) * 7];
     Cell q;
     const bool in = cell_of(a, q);
@@ -361,13 +472,6 @@ __global__ void __launch_bounds__(NT, 4) k3_collide(const Args3 a, int mode)
         const float rho = a.rho0 + drho;
         const float ir = 1.f / rho;
         const float ux = (jx + 0.5f * F[0]) * ir, uy = (jy + 0.5f * F[1]) * ir, uz = (jz + 0.5f * F[2]) * ir;
-        if (mode == 1) {
-            a.mom[q.c] = drho;
-            a.mom[a.NP + q.c] = ux;
-            a.mom[2 * a.NP + q.c] = uy;
-            a.mom[3 * a.NP + q.c] = uz;
-            return;
-        }
         a.u[q.c] = ux;
         a.u[a.NP + q.c] = uy;
         a.u[2 * a.NP + q.c] = uz;
@@ -408,22 +512,55 @@ __global__ void __launch_bounds__(NT, 4) k3_collide(const Args3 a, int mode)
             acc[4] = F[0]; acc[5] = F[1]; acc[6] = F[2];
         }
     }
-    if (mode == 1 || !a.readout) return;
+    if (!a.readout) return;
     // readout: the CTA's sums; the groups of NT CTAs are added by the next kernel and the groups by
     // the one after (kernel boundaries order the writes: no fence or atomic in this kernel)
     const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     cta_sum7(acc, a.partials + (long long)cta * 7, sRedF);
 }
 
+// One moment of the current state into out: rho - rho0 (axis -1: the populations alone), or a component of
+// u (its component of the force, from sigma^p and the row of sigma^E that k3_molecular has written).
+// A readout asks for one field: forming all four moments each time read 34 planes of stress for one.
+__global__ void __launch_bounds__(NT) k3_moment(const __grid_constant__ Args3 a, int axis, float* out)
+{
+    Cell q;
+    if (!cell_of(a, q)) return;
+    float drho = 0.f, jn = 0.f;
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) {
+        const float d = __ldg(a.src + (long long)n * a.NP + q.c);
+        drho += d;
+        const int c = axis == 0 ? CX[n] : (axis == 1 ? CY[n] : CZ[n]);
+        jn += (float)c * d;
+    }
+    if (axis < 0) {
+        out[q.c] = drho;
+        return;
+    }
+    float F = axis == 0 ? a.fx : (axis == 1 ? a.fy : a.fz);
+    const int nb[3][2] = {{q.xp, q.xm}, {q.yp, q.ym}, {q.zp, q.zm}};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float* sp = a.src + (long long)(PL_S + sym6(axis, j)) * a.NP;
+        F += 0.5f * (__ldg(sp + nb[j][0]) - __ldg(sp + nb[j][1]));
+        if (a.ericksen) {
+            const float* se = a.sE + (long long)(axis * 3 + j) * a.NP;
+            F += 0.5f * (__ldg(se + nb[j][0]) - __ldg(se + nb[j][1]));
+        }
+    }
+    out[q.c] = (jn + 0.5f * F) * (1.f / (a.rho0 + drho));
+}
+
 // Readout, second level (in k3_predict): CTA g < groups adds the sums of CTAs g NT .. g NT + NT - 1
 // of k3_collide in a fixed tree.
 __device__ __forceinline__ void readout_groups(const Args3& a, double* sm)
 {
-    const unsigned n_ctas = gridDim.x * gridDim.y * gridDim.z;
+    const unsigned n_ctas = a.n_ctas;
     const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const unsigned n_grp = (n_ctas + NT - 1) / NT;
     if (!a.readout || cta >= n_grp) return;
-    const int tid = threadIdx.x + BX * (threadIdx.y + BY * threadIdx.z);
+    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const unsigned g0 = cta * NT;
     double s[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     if (g0 + tid < n_ctas) {
@@ -440,9 +577,9 @@ __device__ __forceinline__ void readout_groups(const Args3& a, double* sm)
 __device__ __forceinline__ void readout_total(const Args3& a, double* sm)
 {
     if (!a.readout || blockIdx.x + blockIdx.y + blockIdx.z != 0) return;
-    const unsigned n_ctas = gridDim.x * gridDim.y * gridDim.z;
+    const unsigned n_ctas = a.n_ctas;
     const unsigned n_grp = (n_ctas + NT - 1) / NT;
-    const int tid = threadIdx.x + BX * (threadIdx.y + BY * threadIdx.z);
+    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const unsigned per = (n_grp + NT - 1) / NT;
     const unsigned b0 = min(n_grp, tid * per), b1 = min(n_grp, b0 + per);
     double s[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -460,54 +597,61 @@ __device__ __forceinline__ void readout_total(const Args3& a, double* sm)
     }
 }
 
-__global__ void __launch_bounds__(NT) k3_predict(const Args3 a)
+// Predictor and corrector: streaming stencil kernels bound by instruction issue and load latency (63
+// stencil points of y, 21 of u), so they take two cells per thread where nx is even: half the loads and
+// arithmetic per cell, 16 warps of two cells per SM against 24 of one.
+template <class T>
+__global__ void __launch_bounds__(NT, vlb::vec::Lanes<T>::N == 2 ? 2 : 3) k3_predict(const __grid_constant__ Args3 a)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ double sRed[(NT / 32) * 7];
     readout_groups(a, sRed);
-    Cell q;
-    if (!cell_of(a, q)) return;
-    float uc[3], G[3][3];
-    flow(a, q, uc, G);
-    Y9 y;
-    load_y9(a.src + (long long)PL_S * a.NP, a.NP, q, uc, y);
-    // h(P): Eq. Ffunctional from the folded dP stencils
-    const float A = bulk(a, y.c[6], y.c[7], y.c[8]);
-    const float Pr[3] = {a.prx, a.pry, a.prz};
-    float h[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) h[i] = A * (Pr[i] + y.c[6 + i]) - a.kappa * y.lap[6 + i];
-    float r[9];
-    rhs9(a, y, G, h, r);
+    Nb<T> q;
+    if (!nb_of(a, q)) return;
+    if (a.ahead && threadIdx.x == 0) {
+        prefetch_rows(a, a.u, 3, q.c);
+        prefetch_rows(a, a.src + (long long)PL_S * a.NP, 9, q.c);
+    }
+    Flow<T> f;
+    flow(a, q, f);
+    Y9<T> y;
+    load_y9(a.src + (long long)PL_S * a.NP, a.NP, q, f.u, y);
+    T r[9];
+    rhs9(a, y, f, r);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        a.r0[k * a.NP + q.c] = r[k];
-        a.ys[k * a.NP + q.c] = y.c[k] + r[k];
+        stv(a.r0 + k * a.NP + q.c, r[k]);
+        stv(a.ys + k * a.NP + q.c, y.c[k] + r[k]);
     }
 }
 
-__global__ void __launch_bounds__(NT) k3_correct(const Args3 a)
+template <class T>
+__global__ void __launch_bounds__(NT, vlb::vec::Lanes<T>::N == 2 ? 2 : 3) k3_correct(const __grid_constant__ Args3 a)
 {
+    pdl_wait();
+    pdl_trigger();
     __shared__ double sRed[(NT / 32) * 7];
     readout_total(a, sRed);
-    Cell q;
-    if (!cell_of(a, q)) return;
-    float uc[3], G[3][3];
-    flow(a, q, uc, G);
-    Y9 y;
-    load_y9(a.ys, a.NP, q, uc, y);
-    // h(P*): Eq. Ffunctional at the predictor
-    const float A = bulk(a, y.c[6], y.c[7], y.c[8]);
-    const float Pr[3] = {a.prx, a.pry, a.prz};
-    float h[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) h[i] = A * (Pr[i] + y.c[6 + i]) - a.kappa * y.lap[6 + i];
-    float r[9];
-    rhs9(a, y, G, h, r);
+    Nb<T> q;
+    if (!nb_of(a, q)) return;
+    if (a.ahead && threadIdx.x == 0) {
+        prefetch_rows(a, a.u, 3, q.c);
+        prefetch_rows(a, a.ys, 9, q.c);
+        prefetch_rows(a, a.src + (long long)PL_S * a.NP, 9, q.c);
+        prefetch_rows(a, a.r0, 9, q.c);
+    }
+    Flow<T> f;
+    flow(a, q, f);
+    Y9<T> y;
+    load_y9(a.ys, a.NP, q, f.u, y);
+    T r[9];
+    rhs9(a, y, f, r);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const float y0 = __ldg(a.src + (long long)(PL_S + k) * a.NP + q.c);
-        const float r0 = __ldg(a.r0 + k * a.NP + q.c);
-        a.dst[(long long)(PL_S + k) * a.NP + q.c] = y0 + 0.5f * (r0 + r[k]);
+        const T y0 = ldv<T>(a.src + (long long)(PL_S + k) * a.NP + q.c);
+        const T r0 = ldv<T>(a.r0 + k * a.NP + q.c);
+        stv(a.dst + (long long)(PL_S + k) * a.NP + q.c, vfma(0.5f, r0 + r[k], y0));
     }
 }
 
@@ -615,7 +759,7 @@ struct lb3d_handle {
     float* u = nullptr;
     float* ys = nullptr;
     float* r0 = nullptr;
-    float* mom = nullptr;
+    float* scratch = nullptr;     // one plane: a formed field on its way to the host
     float4* lut = nullptr;
     double* partials = nullptr;
     double* gpartials = nullptr;
@@ -672,7 +816,7 @@ v3::Args3 args_of(lb3d_handle* h)
     v3::Args3 a = {};
     a.src = h->state[h->cur];
     a.dst = h->state[h->cur ^ 1];
-    a.sE = h->sE; a.u = h->u; a.ys = h->ys; a.r0 = h->r0; a.mom = h->mom;
+    a.sE = h->sE; a.u = h->u; a.ys = h->ys; a.r0 = h->r0;
     a.lut = h->lut;
     a.NP = h->NP;
     a.nx = p.nx; a.ny = p.ny; a.nz = p.nz;
@@ -691,29 +835,32 @@ v3::Args3 args_of(lb3d_handle* h)
     a.ericksen = p.ericksen;
     a.partials = h->partials;
     a.gpartials = h->gpartials;
+    const dim3 g = grid_of(h);
+    a.n_ctas = g.x * g.y * g.z;
+    // one plane ahead where the state does not stay in L2 (measured at 256^3: 1.825 ms per step without,
+    // 1.739, 1.763, 1.826 and 2.012 ms with 1, 2, 3 and 4 planes)
+    a.ahead = h->NP * v3::NPL * 4 > (64LL << 20) ? (long long)p.nx * p.ny : 0;
     a.err_nonfinite = h->err;
     a.t = h->t;
     return a;
 }
 
-int launch_check(lb3d_handle* h, const char* what)
+// launch with or without programmatic stream serialization
+template <class K, class... A>
+int launch3(lb3d_handle* h, const char* what, K kern, dim3 g, dim3 b, bool pdl, const A&... args)
 {
-    cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = b;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
     if (e != cudaSuccess) return fail(h, LB_ECUDA, "%s: %s", what, cudaGetErrorString(e));
     return LB_OK;
-}
-
-// h and sigma^E of the current state, then the moments pass or the step's collision
-int launch_front(lb3d_handle* h, v3::Args3& a, int mode)
-{
-    const dim3 g = grid_of(h), b(v3::BX, v3::BY, v3::BZ);
-    if (h->p.ericksen) {
-        v3::k3_molecular<<<g, b, 0, h->stream>>>(a, a.src + (long long)v3::PL_P * h->NP);
-        int rc = launch_check(h, "k3_molecular");
-        if (rc) return rc;
-    }
-    v3::k3_collide<<<g, b, 0, h->stream>>>(a, mode);
-    return launch_check(h, "k3_collide");
 }
 
 }  // namespace
@@ -749,7 +896,7 @@ int lb3d_create(const lb3d_params* p, lb3d_handle** out)
     if (e == cudaSuccess) e = cudaMalloc(&h->u, 3 * pb);
     if (e == cudaSuccess) e = cudaMalloc(&h->ys, 9 * pb);
     if (e == cudaSuccess) e = cudaMalloc(&h->r0, 9 * pb);
-    if (e == cudaSuccess) e = cudaMalloc(&h->mom, 4 * pb);
+    if (e == cudaSuccess) e = cudaMalloc(&h->scratch, pb);
     if (e == cudaSuccess) e = cudaMalloc(&h->lut, sizeof(float4) * 2 * (v3::LUT_N + 1));
     const size_t n_grp = (n_ctas + v3::NT - 1) / v3::NT;
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, sizeof(double) * 7 * n_ctas);
@@ -771,7 +918,7 @@ void lb3d_destroy(lb3d_handle* h)
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
     dfree(h->state[0]); dfree(h->state[1]);
-    dfree(h->sE); dfree(h->u); dfree(h->ys); dfree(h->r0); dfree(h->mom);
+    dfree(h->sE); dfree(h->u); dfree(h->ys); dfree(h->r0); dfree(h->scratch);
     dfree(h->lut); dfree(h->partials); dfree(h->gpartials); dfree(h->series); dfree(h->err);
     for (auto e : h->ev) cudaEventDestroy(e);
     if (h->stream) cudaStreamDestroy(h->stream);
@@ -814,6 +961,9 @@ int lb3d_step(lb3d_handle* h, int64_t n)
     if (n < 0) return fail(h, LB_EINVAL, "n < 0");
     if (!h->ready) return fail(h, LB_ESTATE, "lb3d_init_fields not called");
     const dim3 g = grid_of(h), b(v3::BX, v3::BY, v3::BZ);
+    // two cells per thread: rows of pairs that start at even indices; CTAs of 32 x 8 x 2 cells
+    const bool pairs = h->p.nx % 2 == 0;
+    const dim3 b2(16, 8, 2), g2((unsigned)((h->p.nx / 2 + 15) / 16), (unsigned)((h->p.ny + 7) / 8), (unsigned)((h->p.nz + 1) / 2));
     for (int64_t k = 0; k < n; ++k) {
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (h->timing) {
@@ -833,13 +983,17 @@ int lb3d_step(lb3d_handle* h, int64_t n)
             a.row = h->series + (size_t)(h->rows % h->p.max_samples) * 8;
             h->rows += 1;
         }
-        int rc = launch_front(h, a, 0);
-        if (rc) return rc;
-        v3::k3_predict<<<g, b, 0, h->stream>>>(a);
-        rc = launch_check(h, "k3_predict");
-        if (rc) return rc;
-        v3::k3_correct<<<g, b, 0, h->stream>>>(a);
-        rc = launch_check(h, "k3_correct");
+        const bool pdl = !h->timing;
+        int rc = LB_OK;
+        if (h->p.ericksen)
+            rc = launch3(h, "k3_molecular", v3::k3_molecular, g, b, pdl, a, a.src + (long long)v3::PL_P * h->NP, -1);
+        if (!rc) rc = launch3(h, "k3_collide", v3::k3_collide, g, b, pdl, a);
+        if (!rc)
+            rc = pairs ? launch3(h, "k3_predict", v3::k3_predict<float2>, g2, b2, pdl, a)
+                       : launch3(h, "k3_predict", v3::k3_predict<float>, g, b, pdl, a);
+        if (!rc)
+            rc = pairs ? launch3(h, "k3_correct", v3::k3_correct<float2>, g2, b2, pdl, a)
+                       : launch3(h, "k3_correct", v3::k3_correct<float>, g, b, pdl, a);
         if (rc) return rc;
         if (h->timing) CK3(h, cudaEventRecord(e1, h->stream));
         h->cur ^= 1;
@@ -869,27 +1023,30 @@ int lb3d_readout(lb3d_handle* h, int32_t field, float* dst, size_t count, int32_
     if (field < 0 || field >= LB3D_N_FIELDS) return fail(h, LB_EINVAL, "unknown field %d", field);
     if (count < (size_t)h->NP) return fail(h, LB_EINVAL, "need %lld values", h->NP);
     if (!h->ready) return fail(h, LB_ESTATE, "lb3d_init_fields not called");
-    const float* srcp;
+    // a formed field goes straight to device memory, or through the handle's scratch plane to the host
+    const float* srcp = nullptr;
+    float* out = dst_is_device ? dst : h->scratch;
+    int rc = LB_OK;
     if (field <= 3) {
         v3::Args3 a = args_of(h);
-        a.readout = 0;
-        int rc = launch_front(h, a, 1);
-        if (rc) return rc;
-        srcp = h->mom + (size_t)field * h->NP;
+        const dim3 g = grid_of(h), b(v3::BX, v3::BY, v3::BZ);
+        if (h->p.ericksen && field > 0)
+            rc = launch3(h, "k3_molecular", v3::k3_molecular, g, b, false, a, a.src + (long long)v3::PL_P * h->NP, field - 1);
+        if (!rc) rc = launch3(h, "k3_moment", v3::k3_moment, g, b, false, a, field - 1, out);
     } else if (field < LB3D_FIELD_P) {
         srcp = h->state[h->cur] + (size_t)(v3::PL_S + field - LB3D_FIELD_SIGMA) * h->NP;
     } else if (field < LB3D_FIELD_POP0) {
         const int c = field - LB3D_FIELD_P;
-        v3::k3_add<<<1024, 256, 0, h->stream>>>(h->state[h->cur] + (size_t)(v3::PL_P + c) * h->NP,
-                                                (float)h->p.P_ref[c], h->mom, h->NP);
-        int rc = launch_check(h, "k3_add");
-        if (rc) return rc;
-        srcp = h->mom;
+        const float* plane = h->state[h->cur] + (size_t)(v3::PL_P + c) * h->NP;
+        rc = launch3(h, "k3_add", v3::k3_add, dim3(1024), dim3(256), false, plane, (float)h->p.P_ref[c], out, h->NP);
     } else {
         srcp = h->state[h->cur] + (size_t)(field - LB3D_FIELD_POP0) * h->NP;
     }
-    CK3(h, cudaMemcpyAsync(dst, srcp, sizeof(float) * (size_t)h->NP,
-                           dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+    if (rc) return rc;
+    if (!srcp && !dst_is_device) srcp = h->scratch;
+    if (srcp)
+        CK3(h, cudaMemcpyAsync(dst, srcp, sizeof(float) * (size_t)h->NP,
+                               dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
     CK3(h, cudaStreamSynchronize(h->stream));
     return LB_OK;
 }
