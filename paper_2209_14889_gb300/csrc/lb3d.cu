@@ -435,8 +435,9 @@ __device__ __forceinline__ void block_sum7(double* v, double* sm)
     }
 }
 
-// the step's collision and streaming
-__global__ void __launch_bounds__(NT, 4) k3_collide(const __grid_constant__ Args3 a)
+// the step's collision and streaming; MINB: CTAs per SM that the registers leave room for
+template <int MINB>
+__global__ void __launch_bounds__(NT, MINB) k3_collide(const __grid_constant__ Args3 a)
 {
     pdl_wait();
     pdl_trigger();
@@ -600,8 +601,8 @@ __device__ __forceinline__ void readout_total(const Args3& a, double* sm)
 // Predictor and corrector: streaming stencil kernels bound by instruction issue and load latency (63
 // stencil points of y, 21 of u), so they take two cells per thread where nx is even: half the loads and
 // arithmetic per cell, 16 warps of two cells per SM against 24 of one.
-template <class T>
-__global__ void __launch_bounds__(NT, vlb::vec::Lanes<T>::N == 2 ? 2 : 3) k3_predict(const __grid_constant__ Args3 a)
+template <class T, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k3_predict(const __grid_constant__ Args3 a)
 {
     pdl_wait();
     pdl_trigger();
@@ -626,8 +627,8 @@ __global__ void __launch_bounds__(NT, vlb::vec::Lanes<T>::N == 2 ? 2 : 3) k3_pre
     }
 }
 
-template <class T>
-__global__ void __launch_bounds__(NT, vlb::vec::Lanes<T>::N == 2 ? 2 : 3) k3_correct(const __grid_constant__ Args3 a)
+template <class T, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k3_correct(const __grid_constant__ Args3 a)
 {
     pdl_wait();
     pdl_trigger();
@@ -752,6 +753,7 @@ void coefficient_table(const lb3d_params& p, std::vector<float>& out)
 struct lb3d_handle {
     lb3d_params p;
     cudaStream_t stream = nullptr;
+    int n_sm = 152;
     long long NP = 0;
     float* state[2] = {nullptr, nullptr};
     int cur = 0;
@@ -887,6 +889,8 @@ int lb3d_create(const lb3d_params* p, lb3d_handle** out)
         lb3d_destroy(h);
         return code;
     };
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking);
     const size_t pb = sizeof(float) * (size_t)h->NP;
     const dim3 g = grid_of(h);
@@ -961,8 +965,13 @@ int lb3d_step(lb3d_handle* h, int64_t n)
     if (n < 0) return fail(h, LB_EINVAL, "n < 0");
     if (!h->ready) return fail(h, LB_ESTATE, "lb3d_init_fields not called");
     const dim3 g = grid_of(h), b(v3::BX, v3::BY, v3::BZ);
-    // two cells per thread: rows of pairs that start at even indices; CTAs of 32 x 8 x 2 cells
-    const bool pairs = h->p.nx % 2 == 0;
+    // Few CTAs (at most two per SM): the kernels are bound by the latency of their loads, and registers for
+    // more of them in flight pay (us per step, 16x12x8: 11.0 -> 10.3; 32^3: 13.3 -> 11.5; 44x38x30: 17.9 ->
+    // 15.2, where two cells per thread take 18.8; beyond, 64^3 32.0 -> 34.0, 128^3 236 -> 262).  Else two
+    // cells per thread where rows of pairs start at even indices (128^3 236 -> 228, 256^3 1.92 -> 1.74 ms),
+    // CTAs of 32 x 8 x 2 cells.
+    const bool few = (long long)g.x * g.y * g.z <= 2LL * h->n_sm;
+    const bool pairs = !few && h->p.nx % 2 == 0;
     const dim3 b2(16, 8, 2), g2((unsigned)((h->p.nx / 2 + 15) / 16), (unsigned)((h->p.ny + 7) / 8), (unsigned)((h->p.nz + 1) / 2));
     for (int64_t k = 0; k < n; ++k) {
         cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -987,13 +996,15 @@ int lb3d_step(lb3d_handle* h, int64_t n)
         int rc = LB_OK;
         if (h->p.ericksen)
             rc = launch3(h, "k3_molecular", v3::k3_molecular, g, b, pdl, a, a.src + (long long)v3::PL_P * h->NP, -1);
-        if (!rc) rc = launch3(h, "k3_collide", v3::k3_collide, g, b, pdl, a);
+        if (!rc) rc = (few ? launch3(h, "k3_collide", v3::k3_collide<2>, g, b, pdl, a) : launch3(h, "k3_collide", v3::k3_collide<4>, g, b, pdl, a));
         if (!rc)
-            rc = pairs ? launch3(h, "k3_predict", v3::k3_predict<float2>, g2, b2, pdl, a)
-                       : launch3(h, "k3_predict", v3::k3_predict<float>, g, b, pdl, a);
+            rc = pairs ? launch3(h, "k3_predict", v3::k3_predict<float2, 2>, g2, b2, pdl, a)
+                 : few ? launch3(h, "k3_predict", v3::k3_predict<float, 2>, g, b, pdl, a)
+                       : launch3(h, "k3_predict", v3::k3_predict<float, 3>, g, b, pdl, a);
         if (!rc)
-            rc = pairs ? launch3(h, "k3_correct", v3::k3_correct<float2>, g2, b2, pdl, a)
-                       : launch3(h, "k3_correct", v3::k3_correct<float>, g, b, pdl, a);
+            rc = pairs ? launch3(h, "k3_correct", v3::k3_correct<float2, 2>, g2, b2, pdl, a)
+                 : few ? launch3(h, "k3_correct", v3::k3_correct<float, 2>, g, b, pdl, a)
+                       : launch3(h, "k3_correct", v3::k3_correct<float, 3>, g, b, pdl, a);
         if (rc) return rc;
         if (h->timing) CK3(h, cudaEventRecord(e1, h->stream));
         h->cur ^= 1;

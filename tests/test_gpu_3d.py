@@ -191,3 +191,26 @@ def test_3d_nonfinite_state_is_reported_and_cleared():
     assert e.value.code == lb.LB_ENONFINITE
     s.sync()                     # cleared
     s.close()
+
+
+@pytest.mark.parametrize("nx", [66, 67], ids=["two_cells_per_thread", "one_cell_per_thread"])
+def test_3d_larger_ragged_boxes_vs_oracle(nx):
+    # beyond two CTAs per SM: even rows take two cells per thread, odd ones one; ragged in every axis
+    lb3d = _gpu()
+    w = W.make3d(nx, 34, 35, seed=12, director=(0.48, 0.6, 0.64), every=2)
+    s = lb3d.Solver3D.from_workload(w)
+    s.step(4)
+    s.sync()
+    got, pops, ser = s.fields(), s.populations(), s.series()
+    s.close()
+    sim = O3.Sim3.from_workload(w)
+    sim.step(4, every=2)
+    ref = sim.fields()
+    for k in FIELDS:
+        e = _rel(got[k], ref[k])
+        assert e <= 1e-5, (k, e)
+    _, wq = O3.lattice()
+    hp = pops.astype(np.float64) + wq[:, None, None, None] * w["rho0"]
+    assert np.abs(hp - sim.h).max() <= 1e-6 * (1 + np.abs(sim.h).max())
+    rs = np.array(sim.series)
+    assert np.array_equal(ser[:, 0], rs[:, 0]) and np.abs(ser[:, 1:] - rs[:, 1:]).max() <= 1e-6 * nx * 34 * 35
