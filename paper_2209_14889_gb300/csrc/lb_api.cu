@@ -139,6 +139,8 @@ NodeArgs node_args(lb_handle* h, int advance)
     a.every = h->p.readout_every;
     a.nx = h->p.nx;
     a.ny = h->p.ny;
+    a.len_x = h->p.nx;
+    a.len_y = h->p.ny;
     a.walls_y = h->p.walls_y;
     a.walls_x = h->p.walls_x;
     a.advance = advance;

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(BT, 2) k_batch(const BatchArgs B, int nsteps)
             na.X = B.inst[i].xb[par];
             na.X_out = B.inst[i].xb[par ^ 1];
             // the tiles' shared memory is free in this phase
-            node::node_ring(na, na.n_rings > 0 ? item - __ldg(B.node_begin + i) : -1, *reinterpret_cast<node::NodeSmem*>(sm));
+            node::node_step(na, na.n_rings > 0 ? item - __ldg(B.node_begin + i) : -1, *reinterpret_cast<node::NodeSmem*>(sm));
             __syncthreads();
         }
         ok = grid_sync(B);
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(NODE_THREADS) k_batch_nodes(const BatchArgs B,
     NodeArgs na = B.inst[i].na;
     na.X = B.inst[i].xb[par];
     na.X_out = B.inst[i].xb[par ^ 1];
-    node::node_ring(na, na.n_rings > 0 ? item - __ldg(B.node_begin + i) : -1, S);
+    node::node_step(na, na.n_rings > 0 ? item - __ldg(B.node_begin + i) : -1, S);
 }
 
 // the buffer parity after a chunk of n steps

@@ -13,8 +13,12 @@
 namespace vlb {
 namespace cell {
 
+// i modulo n in [0, n).  Nearly every argument is within one period of the range; the division by a
+// variable takes some 150 cycles, and the test whether a ring meets a tile makes eight of them.
 __device__ __forceinline__ int wrapn(int i, int n)
 {
+    i += i < 0 ? n : (i >= n ? -n : 0);
+    if ((unsigned)i < (unsigned)n) return i;
     i %= n;
     return i < 0 ? i + n : i;
 }
@@ -22,7 +26,7 @@ __device__ __forceinline__ int wrapn(int i, int n)
 // minimum image of an integer offset on a periodic axis of length n, in [-n/2, n/2)
 __device__ __forceinline__ int mimg(int d, int n)
 {
-    d %= n;
+    if (d <= -n || d >= n) d %= n;
     if (d < -(n / 2)) d += n;
     else if (d >= n - n / 2) d -= n;
     return d;

@@ -27,6 +27,16 @@ __device__ __forceinline__ int tiles_meeting(int n_tiles, int T, int RW, int b, 
     return cnt;
 }
 
+// One of n arrivals; true for the last, which leaves the counter at zero.  Release and acquire in
+// the one atomic: a fence, an atomic, a store of the zero and a second fence took 3 200 cycles of
+// the chain between the last tile and the ring's nodes.
+__device__ __forceinline__ bool arrive(unsigned* counter, unsigned n)
+{
+    unsigned prev;
+    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(prev) : "l"(counter), "r"(n - 1u) : "memory");
+    return prev == n - 1u;
+}
+
 // The node step in the tail of the lattice kernel (FusedArgs::node_tail), after this tile's
 // step (App. A).  A ring's nodes are read (spreading) only by the tiles whose region meets its
 // box of step t, and the node update writes only the box of step t + 1 (RingDev::box), the
@@ -47,41 +57,27 @@ __device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm, unsig
     const int bx = blockIdx.x;
     int by = blockIdx.y + a.tile_rot;
     if (by >= (int)gridDim.y) by -= gridDim.y;
-    __syncthreads();            // the tile's writes are out, its shared memory is free
     for (int r = 0; r < nr && meet != 0u; ++r) {
         if (nr <= 32 && !((meet >> r) & 1u)) continue;
-        const int4 B = ring_box(a.rings[r], t);
+        node::RingRegs rg;      // every tile that meets the ring loads what the last one needs
+        node::load_ring(a.na, r, t, rg);
+        node::load_first_node(a.na, rg);
+        const int4 B = rg.B;
         if (nr > 32 &&
             (!meets(bx * TX - 2, G::R2W, B.x, B.z, a.nx) || !meets(by * TY - 2, G::R2H, B.y, B.w, a.ny)))
             continue;
-        if (tid < 32) {
-            const int c = tiles_meeting(gridDim.x, TX, G::R2W, B.x, B.z, a.nx) *
-                          tiles_meeting(gridDim.y, TY, G::R2H, B.y, B.w, a.ny);
-            if (tid == 0) {
-                __threadfence();
-                const bool last = atomicAdd(&a.box_tickets[r], 1u) == (unsigned)(c - 1);
-                if (last) {
-                    a.box_tickets[r] = 0u;
-                    __threadfence();
-                }
-                S.flag = last;
-            }
-        }
+        unsigned c = 0u;
+        if (tid < 32)
+            c = tiles_meeting(gridDim.x, TX, G::R2W, B.x, B.z, a.nx) *
+                tiles_meeting(gridDim.y, TY, G::R2H, B.y, B.w, a.ny);
+        __syncthreads();        // the tile's writes are out, its shared memory is free
+        if (tid == 0) S.flag = arrive(&a.box_tickets[r], c);
         __syncthreads();
-        const bool last = S.flag != 0;
-        if (last) node::node_ring(a.na, r, S, false, t);
-        __syncthreads();
+        if (S.flag) node::node_ring(a.na, r, rg, S, t, (t % a.every) == 0);
     }
     if ((t % a.every) == 0) {
-        if (tid == 0) {
-            __threadfence();
-            const bool last = atomicAdd(&a.ctl->tile_ticket, 1u) == gridDim.x * gridDim.y - 1u;
-            if (last) {
-                a.ctl->tile_ticket = 0u;
-                __threadfence();
-            }
-            S.flag = last;
-        }
+        __syncthreads();
+        if (tid == 0) S.flag = arrive(&a.ctl->tile_ticket, gridDim.x * gridDim.y);
         __syncthreads();
         if (S.flag) node::lattice_readout(a.na, t, S.dred);
     }

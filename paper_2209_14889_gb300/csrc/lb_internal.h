@@ -91,6 +91,7 @@ struct NodeArgs {
     Ctl* ctl;
     int every;
     int nx, ny;
+    double len_x, len_y;         // nx, ny
     int walls_y;                 // 1: walls in y; a node closer than 4 cells to one is an error
     int walls_x;                 // 1: walls in x; the same
     int advance;                 // 0: forces + box only (initial configuration); else the steps

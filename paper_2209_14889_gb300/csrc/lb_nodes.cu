@@ -12,7 +12,7 @@ using namespace node;
 __global__ void __launch_bounds__(NODE_THREADS) k_nodes(const NodeArgs a)
 {
     __shared__ NodeSmem S;
-    node_ring(a, a.n_rings > 0 ? (int)blockIdx.x : -1, S);
+    node_step(a, a.n_rings > 0 ? (int)blockIdx.x : -1, S);
 }
 
 }  // namespace

@@ -295,7 +295,7 @@ __device__ __forceinline__ void ib_gather(const FusedArgs& a, const TileMem<TX, 
                 const int2 c = a.node_cell[R.node_off + k];
                 fr = a.node_frac[R.node_off + k];
                 f = a.node_force[R.node_off + k];
-                if (R.trap_k > 0.0) {             // the trap's force, the same on every node
+                if (__double_as_longlong(R.trap_k) > 0) {   // the trap's force, the same on every node
                     const float2 tf = R.trap_f[t & 1];
                     f.x += tf.x;
                     f.y += tf.y;
@@ -547,7 +547,7 @@ __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, in
 
     // The state at t was written two kernels back; the node forces, ring boxes, step counter and
     // readout buffers come from the node kernel just before this one.
-    pdl_wait();
+    if (!a.node_tail) pdl_wait();       // with the tail the kernel waited before staging
     pdl_trigger();
     ib_gather(a, m, x0, y0);
 
@@ -797,7 +797,7 @@ __device__ __forceinline__ void tile_step2(const FusedArgs& a, int bx, int by, i
         }
     }
 
-    pdl_wait();
+    if (!a.node_tail) pdl_wait();       // with the tail the kernel waited before staging
     pdl_trigger();
     ib_gather(a, m, x0, y0);
 

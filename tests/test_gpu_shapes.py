@@ -106,3 +106,25 @@ def test_ring_sizes_vs_oracle(n_nodes):
         c = 6 + 4 * k
         assert np.linalg.norm(ser[:, c:c + 2] - ref[:, c:c + 2]) <= 1e-4 * np.linalg.norm(ref[:, c:c + 2])
         assert np.abs(ser[:, c + 2:c + 4] - ref[:, c + 2:c + 4]).max() <= 1e-6
+
+
+@pytest.mark.parametrize("n_nodes,radius,trap", [(129, 40.0, False), (192, 12.0, True), (193, 12.0, True), (500, 40.0, True)])
+def test_ring_boxes_and_trap_warps_vs_oracle(n_nodes, radius, trap):
+    # u(t) on a box too large for shared memory (radius 40) is read from global memory; with the trap
+    # the last two of eight warps hold no edge of a ring of up to 192 nodes and advance none of up to 256
+    lb = _gpu()
+    g = dict(pull_force=0.0, trap=TRAP) if trap else dict(pull_force=1e-3, pull_angle=0.4)
+    w = W.make(288, 256, rings=[W.ring(n_nodes, radius, (280.3, 60.2), **g)], seed=20 + n_nodes)
+    s = lb.Solver.from_workload(w)
+    s.step(40)
+    _, X, ser = _state(s)
+    s.close()
+    sim = O.Sim.from_workload(w)
+    sim.step(40, every=10)
+    ref = np.array(sim.series)
+    d = X - sim.X
+    d -= np.array([288.0, 256.0]) * np.round(d / np.array([288.0, 256.0]))
+    # as in test_ring_sizes_vs_oracle
+    assert np.abs(d).max() <= 1e-6
+    assert np.linalg.norm(ser[:, 6:8] - ref[:, 6:8]) <= 1e-4 * np.linalg.norm(ref[:, 6:8])
+    assert np.abs(ser[:, 8:10] - ref[:, 8:10]).max() <= 1e-6
