@@ -14,19 +14,6 @@ namespace {
 
 using namespace tile;
 
-// Tiles c = 0 .. n_tiles - 1 of one lattice axis whose staged region [c T - 2, c T - 2 + RW)
-// meets the box span [b, b + bw) (the test of ib_gather); one warp, result in every lane.
-__device__ __forceinline__ int tiles_meeting(int n_tiles, int T, int RW, int b, int bw, int n)
-{
-    const int lane = threadIdx.x & 31;
-    int cnt = 0;
-    for (int c0 = 0; c0 < n_tiles; c0 += 32) {
-        const int c = c0 + lane;
-        cnt += __popc(__ballot_sync(0xffffffffu, c < n_tiles && meets(c * T - 2, RW, b, bw, n)));
-    }
-    return cnt;
-}
-
 // One of n arrivals; true for the last, which leaves the counter at zero.  Release and acquire in
 // the one atomic: a fence, an atomic, a store of the zero and a second fence took 3 200 cycles of
 // the chain between the last tile and the ring's nodes.
@@ -46,7 +33,7 @@ __device__ __forceinline__ bool arrive(unsigned* counter, unsigned n)
 // steps every tile counts itself and the last one sums the lattice readout.  A thread's arrival
 // stands for the whole CTA: the barrier orders the CTA's writes before its fence.  Out of line:
 // node_tail below calls it only for the tiles that have something to do.
-template <int TX, int TY>
+template <int TX, int TY, bool EARLY>
 __device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm, unsigned meet)
 {
     using G = TileGeo<TX, TY>;
@@ -57,6 +44,27 @@ __device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm, unsig
     const int bx = blockIdx.x;
     int by = blockIdx.y + a.tile_rot;
     if (by >= (int)gridDim.y) by -= gridDim.y;
+    if constexpr (EARLY) {
+        const int* ar = reinterpret_cast<const int*>(sm + G::OFF_AR);
+        __syncthreads();        // the tile's shared memory is free, AR_LAST is known
+        if (ar[AR_COUNT] != 0) {
+            meet = 0u;
+            if (ar[AR_LAST]) {
+                node::RingRegs rg;
+                const int r = ar[AR_RING];
+                rg.n = ar[AR_NODES];
+                rg.off = ar[AR_OFF];
+                rg.cap_w = ar[AR_CAP_W];
+                rg.cap_h = ar[AR_CAP_H];
+                rg.trap = ar[AR_TRAP] != 0;
+                rg.box_off = *reinterpret_cast<const long long*>(ar + AR_BOX_OFF);
+                rg.B = *reinterpret_cast<const int4*>(ar + AR_BOX);
+                node::load_first_node(a.na, rg);
+                __syncthreads();        // the node step's shared memory lies over these values
+                node::node_ring(a.na, r, rg, S, t, (t % a.every) == 0);
+            }
+        }
+    }
     for (int r = 0; r < nr && meet != 0u; ++r) {
         if (nr <= 32 && !((meet >> r) & 1u)) continue;
         node::RingRegs rg;      // every tile that meets the ring loads what the last one needs
@@ -85,7 +93,7 @@ __device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm, unsig
 
 // The node tail of one tile: the step counter (one tile), then node_tail_work where this tile
 // meets a ring's box or the step is a readout step; nothing else for most tiles.
-template <int TX, int TY>
+template <int TX, int TY, bool EARLY = false>
 __device__ __forceinline__ void node_tail(const FusedArgs& a, float* sm)
 {
     using G = TileGeo<TX, TY>;
@@ -93,7 +101,7 @@ __device__ __forceinline__ void node_tail(const FusedArgs& a, float* sm)
     // the rings whose box meets this tile's staged region (tested in ib_gather for up to 32 rings)
     const unsigned meet =
         a.n_rings > 32 ? 0xffffffffu : (unsigned)reinterpret_cast<const int*>(sm + G::OFF_SC)[NT / 32 + 2];
-    if (meet != 0u || (a.t % a.every) == 0) node_tail_work<TX, TY>(a, sm, meet);
+    if (meet != 0u || (a.t % a.every) == 0) node_tail_work<TX, TY, EARLY>(a, sm, meet);
 }
 
 // dynamic shared memory of a tile kernel: the tile's, or a ring's node step after it
@@ -115,8 +123,9 @@ __global__ void __launch_bounds__(NT, 3) k_fused(const __grid_constant__ FusedAr
         by += a.tile_rot;
         if (by >= (int)gridDim.y) by -= gridDim.y;
     }
-    tile_step<MODE, PREC, TX, TY, false, SCALAR>(a, blockIdx.x, by, by * gridDim.x + blockIdx.x, sm);
-    if (tail) node_tail<TX, TY>(a, sm);
+    constexpr bool EARLY = MODE == MODE_STEP && TX * TY <= 128;
+    tile_step<MODE, PREC, TX, TY, false, SCALAR, EARLY>(a, blockIdx.x, by, by * gridDim.x + blockIdx.x, sm);
+    if (tail) node_tail<TX, TY, EARLY>(a, sm);
 }
 
 template <int MODE, int PREC>

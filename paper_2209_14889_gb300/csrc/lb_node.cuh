@@ -189,7 +189,6 @@ struct RingRegs {
     long long box_off;
     int4 B;
     bool trap;
-    double par;                  // lane l < 5: k_spring, eps_angle, l_eq, pull_x, pull_y
     double X0;                   // thread 2 k + (0: x, 1: y): node k
 };
 
@@ -209,8 +208,6 @@ __device__ __forceinline__ void load_ring(const NodeArgs& a, int ring, long long
     q.box_off = R.box_off;
     q.B = ring_box(R, t);
     q.trap = __double_as_longlong(R.trap_k) > 0;
-    const int lane = threadIdx.x & 31;
-    q.par = lane == 0 ? R.k_spring : (lane == 1 ? R.eps_angle : (lane == 2 ? R.l_eq : (lane == 3 ? R.pull_x : R.pull_y)));
 }
 
 // Lattice readout of step t, run by the last CTA to arrive (all its threads): the sums of the
@@ -283,9 +280,10 @@ __device__ __forceinline__ void node_ring(const NodeArgs& a, int ring, const Rin
     float* tens = reinterpret_cast<float*>(edge + n);
     float* ilen = tens + n;
     const float hx = 0.5f * (float)nx, hy = 0.5f * (float)ny;
-    if (wid == NW - 3) {
-        if (lane < 5) S.par[lane] = (float)rg.par;
-        if (lane == 2) S.leq2 = rg.par * rg.par;
+    if (wid == NW - 3 && lane < 5) {
+        const double p = lane == 0 ? R.k_spring : (lane == 1 ? R.eps_angle : (lane == 2 ? R.l_eq : (lane == 3 ? R.pull_x : R.pull_y)));
+        S.par[lane] = (float)p;
+        if (lane == 2) S.leq2 = p * p;
     }
     if (tid < 4) S.ext[tid] = 1 << 30;
     if (trap && wid >= NW - 2) trap_at(R, (double)(t + a.advance), wid - (NW - 2), S.trap);

@@ -36,6 +36,10 @@ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 constexpr int al4(int x) { return (x + 3) & ~3; }   // 16-byte alignment in floats
 
 // Geometry and shared-memory layout (in floats) of a TX x TY output tile.
+// The early arrival of a small tile at its ring (tile_step, node_tail): what the node step needs of
+// the ring, the tiles that meet it, and whether this one was the last of them.
+enum { AR_BOX = 0, AR_BOX_OFF = 4, AR_COUNT = 6, AR_RING, AR_NODES, AR_OFF, AR_CAP_W, AR_CAP_H, AR_TRAP, AR_LAST, AR_N = 16 };
+
 template <int TX, int TY>
 struct TileGeo {
     static constexpr int R4W = TX + 8, R4H = TY + 8, R4 = R4W * R4H;
@@ -62,7 +66,8 @@ struct TileGeo {
     static constexpr int OFF_YI = OFF_XI + R4W;                   // wrapped y index [R4H] (int)
     static constexpr int OFF_SC = OFF_YI + R4H;                   // scan scratch [NT/32 + 1] (int),
                                                                   // then the tile's ring masks [2]
-    static constexpr int OFF_RED = al4(OFF_SC + NT / 32 + 3);     // readout [5][NT/32] (double)
+    static constexpr int OFF_AR = al4(OFF_SC + NT / 32 + 3);      // the early arrival [AR_N] (int)
+    static constexpr int OFF_RED = OFF_AR + AR_N;     // readout [5][NT/32] (double)
     static constexpr int SMEM_FLOATS = OFF_RED + 2 * 5 * (NT / 32);
     static constexpr size_t SMEM_BYTES = sizeof(float) * SMEM_FLOATS;
     static_assert(OFF_N % 4 == 0 && OFF_G % 4 == 0 && OFF_NC % 2 == 0 && OFF_RED % 2 == 0, "shared-memory alignment");
@@ -89,6 +94,7 @@ struct TileMem {
     int* sXi;
     int* sYi;
     int* sScan;
+    int* sArr;
     double* sRed;
     __device__ __forceinline__ explicit TileMem(float* sm)
         : sP(sm + G::OFF_P), sS(sm + G::OFF_S), sE(sm + G::OFF_E), sY(sm + G::OFF_E), sH(sm + G::OFF_H),
@@ -97,7 +103,7 @@ struct TileMem {
           sNodeWx(reinterpret_cast<float4*>(sm + G::OFF_G)), sNodeF(reinterpret_cast<float2*>(sm + G::OFF_G + 4 * NT)),
           sRow(reinterpret_cast<unsigned*>(sm + G::OFF_G + 6 * NT)), sCol(sRow + G::R2H * (NT / 32)),
           sXi(reinterpret_cast<int*>(sm + G::OFF_XI)), sYi(reinterpret_cast<int*>(sm + G::OFF_YI)),
-          sScan(reinterpret_cast<int*>(sm + G::OFF_SC)), sRed(reinterpret_cast<double*>(sm + G::OFF_RED))
+          sScan(reinterpret_cast<int*>(sm + G::OFF_SC)), sArr(reinterpret_cast<int*>(sm + G::OFF_AR)), sRed(reinterpret_cast<double*>(sm + G::OFF_RED))
     {
     }
 };
@@ -251,7 +257,21 @@ __device__ __forceinline__ void stage(const FusedArgs& a, const TileMem<TX, TY>&
 // while tiles still run), else from the device step counter
 __device__ __forceinline__ long long step_index(const FusedArgs& a) { return a.node_tail ? a.t : a.ctl->t; }
 
-template <int TX, int TY>
+// Tiles c = 0 .. n_tiles - 1 of one lattice axis whose staged region [c T - 2, c T - 2 + RW)
+// meets the box span [b, b + bw) (the test of ib_gather); one warp, result in every lane.
+__device__ __forceinline__ int tiles_meeting(int n_tiles, int T, int RW, int b, int bw, int n)
+{
+    const int lane = threadIdx.x & 31;
+    int cnt = 0;
+    for (int c0 = 0; c0 < n_tiles; c0 += 32) {
+        const int c = c0 + lane;
+        cnt += __popc(__ballot_sync(0xffffffffu, c < n_tiles && meets(c * T - 2, RW, b, bw, n)));
+    }
+    return cnt;
+}
+
+// EARLY: the tile will arrive at its ring early (tile_step); its last warp notes what that takes.
+template <int TX, int TY, bool EARLY = false>
 __device__ __forceinline__ void ib_gather(const FusedArgs& a, const TileMem<TX, TY>& m, int x0, int y0)
 {
     using G = TileGeo<TX, TY>;
@@ -278,6 +298,26 @@ __device__ __forceinline__ void ib_gather(const FusedArgs& a, const TileMem<TX, 
         }
         meet = __ballot_sync(0xffffffffu, m2);
         own = __ballot_sync(0xffffffffu, mo);
+    }
+    if (EARLY && tid >= NT - 32) {
+        int c = 0;                            // tiles that meet the ring; 0: no early arrival
+        if (a.node_tail && nr <= 32 && __popc(meet) == 1) {
+            const int r = __ffs(meet) - 1;
+            const RingDev& R = a.rings[r];
+            const int4 B = ring_box(R, t);
+            if (tid == NT - 32) {
+                m.sArr[AR_RING] = r;
+                m.sArr[AR_NODES] = R.n_nodes;
+                m.sArr[AR_OFF] = R.node_off;
+                m.sArr[AR_CAP_W] = R.cap_w;
+                m.sArr[AR_CAP_H] = R.cap_h;
+                m.sArr[AR_TRAP] = __double_as_longlong(R.trap_k) > 0;
+                *reinterpret_cast<long long*>(m.sArr + AR_BOX_OFF) = R.box_off;
+                *reinterpret_cast<int4*>(m.sArr + AR_BOX) = B;
+            }
+            c = tiles_meeting(gridDim.x, TX, R2W, B.x, B.z, nx) * tiles_meeting(gridDim.y, TY, R2H, B.y, B.w, ny);
+        }
+        if (tid == NT - 32) m.sArr[AR_COUNT] = c;
     }
     for (int r = 0; r < nr; ++r) {
         if (nr <= 32 && !((meet >> r) & 1u)) continue;
@@ -489,7 +529,11 @@ __device__ __forceinline__ void st_pair(const float2* base, int W, int lx, int l
 // predictor of sigma_xx, sigma_yy and of P, and of the right-hand sides live as interleaved
 // pairs in the regions TileGeo gives their planes (same sizes), so that a stencil point is one
 // 8-byte load that feeds the paired arithmetic of lb_cell.cuh directly.
-template <int MODE, int PREC, int TX, int TY, bool COH = false, bool SCALAR = false>
+// EARLY (small tiles with the node tail, at most 8 x 16 cells): u(t) goes to the ring's box right after
+// phase C, and the tile counts itself there and then (the last warp, which holds no cell of the
+// phases that follow), so that the count's trip to L2 and back runs beside phases D and E instead of after
+// them; node_tail finds the outcome in sArr[AR_LAST].
+template <int MODE, int PREC, int TX, int TY, bool COH = false, bool SCALAR = false, bool EARLY = false>
 __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, int tile_index, float* sm)
 {
     using G = TileGeo<TX, TY>;
@@ -549,7 +593,7 @@ __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, in
     // readout buffers come from the node kernel just before this one.
     if (!a.node_tail) pdl_wait();       // with the tail the kernel waited before staging
     pdl_trigger();
-    ib_gather(a, m, x0, y0);
+    ib_gather<TX, TY, EARLY>(a, m, x0, y0);
 
     // ---- C: total force and moments on the halo-2 region; collision of the owned cells ------
     // Owned cells collide here, with their populations still in registers, and push to
@@ -628,6 +672,26 @@ __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, in
     if (MODE == MODE_MOMENTS) {
         moments_out<TX, TY, true>(a, m, x0, y0);
         return;
+    }
+    unsigned arrived = 0u, n_meet = 0u;
+    if constexpr (EARLY) {
+        static_assert(G::R1 <= NT - 32, "the last warp holds no cell of phases D and E");
+        const unsigned mask = (unsigned)m.sScan[NT / 32 + 1];
+        if (mask) {
+            for (int i = tid; i < R0; i += NT) {
+                const int ly = i / TX, lx = i - ly * TX;
+                if (x0 + lx >= nx || y0 + ly >= ny) continue;
+                const float2 u = sU2[(ly + 2) * R2W + lx + 2];
+                box_write<R3, R3W>(a, mask, t, x0 + lx, y0 + ly, u.x, u.y, readout, m.sS, (ly + 3) * R3W + lx + 3);
+            }
+            __syncthreads();
+        }
+        n_meet = (unsigned)m.sArr[AR_COUNT];
+        if (tid == NT - 32 && n_meet)
+            asm volatile("atom.release.gpu.global.inc.u32 %0, [%1], %2;"
+                         : "=r"(arrived)
+                         : "l"(a.box_tickets + m.sArr[AR_RING]), "r"(n_meet - 1u)
+                         : "memory");
     }
     if (wall) {
         // u beyond a wall: the negated image (zero velocity at the wall)
@@ -723,9 +787,14 @@ __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, in
                 st_flds<PREC>(dst, NP, g, ynew, (unsigned long long)t);
             }
         }
-        box_write<R3, R3W>(a, bmask, t, gx, gy, ux, uy, readout, m.sS, (ly + 3) * R3W + lx + 3);
+        if (!EARLY) box_write<R3, R3W>(a, bmask, t, gx, gy, ux, uy, readout, m.sS, (ly + 3) * R3W + lx + 3);
     }
     if (readout) readout_reduce(a, acc, m.sRed, tile_index);
+    if (EARLY && tid == NT - 32) {
+        const bool last = n_meet && arrived == n_meet - 1u;
+        if (last) __threadfence();              // acquires what the other tiles released
+        m.sArr[AR_LAST] = last;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
