@@ -584,7 +584,8 @@ int lb_step(lb_handle* h, int64_t n)
             float* sig_new = static_cast<float*>(h->state[h->cur ^ 1]) + (size_t)PL_SXX * h->plane;
             float* sig_old = static_cast<float*>(h->state[h->cur]) + (size_t)PL_SXX * h->plane;
             CK(h, launch_diffusion(sig_new, sig_old, h->plane, h->p.nx, h->p.ny,
-                                   (float)(h->p.Dp / h->p.diffusion_substeps), h->p.diffusion_substeps, h->stream));
+                                   (float)(h->p.Dp / h->p.diffusion_substeps), h->p.diffusion_substeps, h->stream,
+                                   pdl && !sweep, pdl && tail));
         }
         if (h->timing && e1) cudaEventRecord(e1, h->stream);
         if (!tail) {

@@ -9,7 +9,7 @@
 // barrier:
 //   lattice  the fused step of every tile of every instance (tile shape per instance, chosen by
 //            the autotuner among 32x16, 32x8, 64x8, 16x16), the tile code of lb_tile.cuh;
-//   sigma    diffusion sub-steps of the instances whose D_p exceeds the Heun bound;
+//   sigma    diffusion passes of the instances whose D_p exceeds the Heun bound;
 //   nodes    the node blocks of every ring of every instance (lb_node.cuh).
 // Work items are assigned to CTAs round-robin, so the schedule and every result are the same
 // from run to run.  The barrier spins with an iteration limit and reports LB_ETIMEOUT.
@@ -33,6 +33,7 @@ namespace vlb {
 namespace {
 
 constexpr int BT = 256;     // threads per CTA
+static_assert(BT == dif::DNT, "a diffusion tile is a CTA of a batch kernel");
 // tile shapes 0..3 (32x16, 32x8, 64x8, 16x16 cells per CTA), and shape 4: the warp-strip kernel
 // (phase launches only; a CTA = SWARPS strips of SOWN columns x STRIP_H rows)
 constexpr int N_SHAPES = 5;
@@ -151,30 +152,16 @@ __global__ void __launch_bounds__(BT, 2) k_batch(const BatchArgs B, int nsteps)
             __syncthreads();     // shared memory is reused by the next item
         }
         ok = grid_sync(B);
-        // diffusion sub-steps: sigma of the new buffer (par^1) and the old one as the other buffer
-        for (int k = 0; k <= B.max_dsub && ok && n_dif > 0; ++k) {
+        // diffusion passes: sigma of the new buffer (par^1) and the old one as the other buffer
+        for (int k = 0; k < dif::passes(B.max_dsub) && ok && n_dif > 0; ++k) {
             for (int item = blockIdx.x; item < n_dif; item += gridDim.x) {
                 const int i = find_inst(B.dif_begin, B.n_inst, item);
                 const BatchInst& I = B.inst[i];
                 const int local = item - __ldg(B.dif_begin + i);
                 const int by = local / I.dif_tx, bx = local - by * I.dif_tx;
-                float* sn = I.sig[par ^ 1];
-                float* so = I.sig[par];
-                const long long NP = I.fa[0].plane;
-                if (k < I.dsub) {
-                    const bool even = (k & 1) == 0;
-                    dif::diffuse_tile(even ? sn : so, even ? so : sn, NP, I.fa[0].nx, I.fa[0].ny, I.dsub_D, bx, by, sm);
-                } else if (k == I.dsub && (I.dsub & 1)) {
-                    // odd number of sub-steps: the result is in the other buffer; copy it back
-                    for (int q = threadIdx.x; q < dif::DX * dif::DY; q += blockDim.x) {
-                        const int ly = q / dif::DX, lx = q - ly * dif::DX;
-                        const int gx = bx * dif::DX + lx, gy = by * dif::DY + ly;
-                        if (gx < I.fa[0].nx && gy < I.fa[0].ny) {
-                            const long long g = (long long)gy * I.fa[0].nx + gx;
-                            for (int c = 0; c < 3; ++c) sn[c * NP + g] = __ldcg(so + c * NP + g);
-                        }
-                    }
-                }
+                if (k < dif::passes(I.dsub))
+                    dif::diffuse_pass(I.sig[par ^ 1], I.sig[par], I.fa[0].plane, I.fa[0].nx, I.fa[0].ny, I.dsub_D, I.dsub,
+                                      k, bx, by, sm);
             }
             ok = grid_sync(B);
         }
@@ -226,8 +213,7 @@ __global__ void __launch_bounds__(SNT, 3) k_batch_strips(const BatchArgs B, int 
     strip_body<cell::PREC_FP32, SCALAR>(I.fa[par], I.fa[par].ctl->t, STRIP_H, cx, cy, local, smem);
 }
 
-// sub-step k of the diffusion of the instances with dsub > k (or, with dsub odd and k == dsub,
-// the copy of the result back into the new state's sigma planes)
+// pass k of the diffusion of the instances with sub-steps (those of more passes than k)
 __global__ void __launch_bounds__(BT) k_batch_diffuse(const BatchArgs B, int s, int k)
 {
     extern __shared__ __align__(16) float sm[];
@@ -235,24 +221,10 @@ __global__ void __launch_bounds__(BT) k_batch_diffuse(const BatchArgs B, int s, 
     const int item = blockIdx.x;
     const int i = find_inst(B.dif_begin, B.n_inst, item);
     const BatchInst& I = B.inst[i];
+    if (k >= dif::passes(I.dsub)) return;
     const int local = item - __ldg(B.dif_begin + i);
     const int by = local / I.dif_tx, bx = local - by * I.dif_tx;
-    float* sn = I.sig[par ^ 1];
-    float* so = I.sig[par];
-    const long long NP = I.fa[0].plane;
-    if (k < I.dsub) {
-        const bool even = (k & 1) == 0;
-        dif::diffuse_tile(even ? sn : so, even ? so : sn, NP, I.fa[0].nx, I.fa[0].ny, I.dsub_D, bx, by, sm);
-    } else if (k == I.dsub && (I.dsub & 1)) {
-        for (int q = threadIdx.x; q < dif::DX * dif::DY; q += blockDim.x) {
-            const int ly = q / dif::DX, lx = q - ly * dif::DX;
-            const int gx = bx * dif::DX + lx, gy = by * dif::DY + ly;
-            if (gx < I.fa[0].nx && gy < I.fa[0].ny) {
-                const long long g = (long long)gy * I.fa[0].nx + gx;
-                for (int c = 0; c < 3; ++c) sn[c * NP + g] = so[c * NP + g];
-            }
-        }
-    }
+    dif::diffuse_pass(I.sig[par ^ 1], I.sig[par], I.fa[0].plane, I.fa[0].nx, I.fa[0].ny, I.dsub_D, I.dsub, k, bx, by, sm);
 }
 
 __global__ void __launch_bounds__(NODE_THREADS) k_batch_nodes(const BatchArgs B, int s)
@@ -481,7 +453,7 @@ cudaError_t launch_phases(const lb_batch* b, int nsteps)
         if (b->n_group[SHAPE_STRIP] && e == cudaSuccess) e = launch_strips(b, s);
         for (int sh = 0; sh < N_SHAPES && e == cudaSuccess; ++sh) {
             if (!b->n_group[sh] || !b->n_dif[sh]) continue;
-            for (int k = 0; k <= b->max_dsub[sh] && e == cudaSuccess; ++k) {
+            for (int k = 0; k < dif::passes(b->max_dsub[sh]) && e == cudaSuccess; ++k) {
                 k_batch_diffuse<<<b->n_dif[sh], BT, dsm, b->stream>>>(batch_args(b, sh), s, k);
                 e = cudaGetLastError();
             }

@@ -326,3 +326,26 @@ def test_scalar_model_batch_matches_single_handles_bitwise():
     b.close()
     for s in ss:
         s.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(41, 30), (97, 61)])
+@pytest.mark.parametrize("dsub", [1, 2, 3, 5, 6, 7, 13])
+def test_fused_diffusion_passes_match_single_substeps_bitwise(nx, ny, dsub):
+    # a batch takes up to three sub-steps per pass (one and a copy, 1 + 1, 2 + 1, 3 + 2, 3 + 3, 2 + 2 + 2 + 1,
+    # six passes of 3 or 2), a lattice alone one per launch; lattices smaller than
+    # the widest staged region, odd sides
+    lb = _gpu()
+    w = W.small(nx, ny, seed=30 + dsub, n_nodes=16, radius=2.6, Dp=0.2 * dsub, diffusion_substeps=dsub)
+    a, b = lb.Solver.from_workload(w), lb.Solver.from_workload(w)
+    a.step(12)
+    batch = lb.Batch([b])
+    batch.step(12)
+    batch.sync()
+    a.sync()
+    fa, fb = a.fields(), b.fields()
+    for k in fa:
+        assert np.array_equal(fa[k], fb[k]), k
+    assert np.array_equal(a.nodes(), b.nodes())
+    batch.close()
+    a.close()
+    b.close()
