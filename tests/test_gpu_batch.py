@@ -349,3 +349,39 @@ def test_fused_diffusion_passes_match_single_substeps_bitwise(nx, ny, dsub):
     batch.close()
     a.close()
     b.close()
+
+
+def test_groups_keep_the_parity_of_instances_that_change_shape():
+    # instances with and without sub-steps, moved to other shapes (and launch forms) after odd numbers
+    # of steps and from an odd start: the state buffer each step reads stays the right one
+    lb = _gpu()
+    ws = [W.small(96, 80, seed=50, n_nodes=24, radius=5.0, Dp=0.6, diffusion_substeps=3),
+          W.small(72, 64, seed=51, n_nodes=24, radius=5.0), W.small(64, 64, seed=52, n_nodes=0)]
+    ref = [lb.Solver.from_workload(w) for w in ws]
+    got = [lb.Solver.from_workload(w) for w in ws]
+    for s in ref:
+        s.step(3 + 5 + 7 + 11 + 3)
+    for s in got:
+        s.step(3)
+    batch = lb.Batch(got)
+    batch.set_shape(4)
+    batch.step(5)
+    batch.set_shape(1, 0)
+    batch.set_shape(3, 2)
+    batch.step(7)
+    batch.set_shape(2)
+    batch.set_persistent(True)
+    batch.step(11)
+    batch.set_persistent(False)
+    batch.set_shape(0, 1)
+    batch.step(3)
+    batch.sync()
+    for a, b in zip(ref, got):
+        a.sync()
+        fa, fb = a.fields(), b.fields()
+        for k in fa:
+            assert np.array_equal(fa[k], fb[k]), k
+        assert np.array_equal(a.nodes(), b.nodes())
+    batch.close()
+    for s in ref + got:
+        s.close()
