@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "../../include/lb3d.h"
+#include "lb_device_ptr.h"
 #include "lb_vec.cuh"
 
 namespace v3 {
@@ -1034,9 +1035,10 @@ int lb3d_readout(lb3d_handle* h, int32_t field, float* dst, size_t count, int32_
     if (field < 0 || field >= LB3D_N_FIELDS) return fail(h, LB_EINVAL, "unknown field %d", field);
     if (count < (size_t)h->NP) return fail(h, LB_EINVAL, "need %lld values", h->NP);
     if (!h->ready) return fail(h, LB_ESTATE, "lb3d_init_fields not called");
-    // a formed field goes straight to device memory, or through the handle's scratch plane to the host
+    // a formed field goes straight to memory of this device, or through the handle's scratch plane
     const float* srcp = nullptr;
-    float* out = dst_is_device ? dst : h->scratch;
+    const bool direct = dst_is_device && vlb::device_floats(dst, sizeof(float) * (size_t)h->NP);
+    float* out = direct ? dst : h->scratch;
     int rc = LB_OK;
     if (field <= 3) {
         v3::Args3 a = args_of(h);
@@ -1054,7 +1056,7 @@ int lb3d_readout(lb3d_handle* h, int32_t field, float* dst, size_t count, int32_
         srcp = h->state[h->cur] + (size_t)(field - LB3D_FIELD_POP0) * h->NP;
     }
     if (rc) return rc;
-    if (!srcp && !dst_is_device) srcp = h->scratch;
+    if (!srcp && !direct) srcp = h->scratch;
     if (srcp)
         CK3(h, cudaMemcpyAsync(dst, srcp, sizeof(float) * (size_t)h->NP,
                                dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));

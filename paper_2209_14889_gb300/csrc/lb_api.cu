@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "lb_device_ptr.h"
 #include "lb_handle.h"
 
 using namespace vlb;
@@ -105,6 +106,7 @@ FusedArgs fused_args(lb_handle* h)
     a.ctl = h->ctl;
     a.every = h->p.readout_every;
     a.moments_out = h->moments;
+    a.moments_only = 0;
     a.forces_out = nullptr;
     return a;
 }
@@ -635,22 +637,24 @@ int lb_readout(lb_handle* h, int32_t field, void* dst, size_t bytes, int32_t dst
         return LB_OK;
     }
     if (bytes != sizeof(float) * N) return fail(h, LB_EINVAL, "bytes mismatch");
-    const float* srcp = nullptr;
-    if (!h->moments) CK(h, cudaMalloc(&h->moments, sizeof(float) * 3 * N));
-    if (field >= LB_FIELD_DRHO && field <= LB_FIELD_UY) {
-        FusedArgs fa = fused_args(h);
-        CK(h, launch_fused(fa, MODE_MOMENTS, h->stream));
-        srcp = h->moments + (size_t)(field - LB_FIELD_DRHO) * N;
-    } else if (field >= LB_FIELD_SXX && field <= LB_FIELD_PY) {
-        CK(h, plane_to_f32(h, h->cur, PL_SXX + field - LB_FIELD_SXX, h->moments));
-        srcp = h->moments;
-    } else if (field >= LB_FIELD_POP0 && field < LB_FIELD_POP0 + 9) {
-        CK(h, plane_to_f32(h, h->cur, field - LB_FIELD_POP0, h->moments));
-        srcp = h->moments;
-    } else {
+    if (!(field >= LB_FIELD_DRHO && field <= LB_FIELD_PY) && !(field >= LB_FIELD_POP0 && field < LB_FIELD_POP0 + 9))
         return fail(h, LB_EINVAL, "unknown field %d", field);
+    // the field is formed where it is wanted (2048^2: a plane's copy takes 7 us), or, where that is not
+    // memory of this device that a kernel may write, in the handle's scratch and copied
+    const bool direct = dst_is_device && vlb::device_floats(dst, bytes);
+    if (!direct && !h->moments) CK(h, cudaMalloc(&h->moments, sizeof(float) * 3 * N));
+    float* out = direct ? static_cast<float*>(dst) : h->moments;
+    if (field == LB_FIELD_DRHO) {
+        CK(h, launch_drho(fused_args(h), out, h->stream));
+    } else if (field <= LB_FIELD_UY) {
+        FusedArgs fa = fused_args(h);
+        fa.moments_out = out;
+        fa.moments_only = 1 + field - LB_FIELD_DRHO;
+        CK(h, launch_fused(fa, MODE_MOMENTS, h->stream));
+    } else {
+        CK(h, plane_to_f32(h, h->cur, field <= LB_FIELD_PY ? PL_SXX + field - LB_FIELD_SXX : field - LB_FIELD_POP0, out));
     }
-    CK(h, cudaMemcpyAsync(dst, srcp, bytes, kind, h->stream));
+    if (!direct) CK(h, cudaMemcpyAsync(dst, out, bytes, kind, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     return LB_OK;
 }

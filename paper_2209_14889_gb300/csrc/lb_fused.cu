@@ -143,7 +143,30 @@ __global__ void __launch_bounds__(NT, 2) k_fused_pair(const __grid_constant__ Fu
     if (tail) node_tail<TILE_X, TILE_Y>(a, sm);
 }
 
+// rho - rho0 needs the populations alone: streaming them takes the time of one pass over nine planes,
+// the moments pass of the tile kernel (forces and all) six times as long.
+template <int PREC>
+__global__ void __launch_bounds__(256) k_drho(const void* src, float* out, long long NP, Phys ph)
+{
+    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= NP) return;
+    float d[9];
+#pragma unroll
+    for (int n = 0; n < 9; ++n) d[n] = cell::ld_pop<PREC, false>(src, NP, n, g);
+    float drho, ux, uy;
+    cell::moments(ph, d, 0.f, 0.f, drho, ux, uy);
+    out[g] = drho;
+}
+
 }  // namespace
+
+cudaError_t launch_drho(const FusedArgs& a, float* out, cudaStream_t s)
+{
+    const unsigned n = (unsigned)((a.plane + 255) / 256);
+    if (a.prec != PREC_FP32) k_drho<PREC_LP><<<n, 256, 0, s>>>(a.src, out, a.plane, a.ph);
+    else k_drho<PREC_FP32><<<n, 256, 0, s>>>(a.src, out, a.plane, a.ph);
+    return cudaGetLastError();
+}
 
 // Tile shapes of the one-cell step: 32x16, 16x16, 16x8, 8x8.
 constexpr int SHAPE_X[FUSED_SHAPES] = {TILE_X, 16, 16, 8};

@@ -120,7 +120,8 @@ struct FusedArgs {
     double* partials;            // per-CTA readout sums (5 per CTA)
     Ctl* ctl;
     int every;                   // readout period
-    float* moments_out;          // MOMENTS mode: drho, ux, uy planes
+    float* moments_out;          // MOMENTS mode: drho, ux, uy planes, or
+    int moments_only;            // ... with 1 + k the k-th of them alone (0: all three)
     float* forces_out;           // MOMENTS mode, optional: Fx, Fy planes (total lattice force)
     // STEP mode with node_tail = 1: the node step of the same time step runs in the kernel's
     // tail.  Every tile whose staged region meets a ring's work box counts itself in
@@ -177,6 +178,9 @@ int fused_shape(int nx, int ny, int n_sm, bool scalar);
 int fused_tile_rot(int nx, int ny, double y_top);
 
 enum { MODE_STEP = 0, MODE_MOMENTS = 1 };
+
+// rho - rho0 of the state a.src into out [ny][nx]
+cudaError_t launch_drho(const FusedArgs& a, float* out, cudaStream_t s);
 
 // Stress-diffusion sub-steps (lb_diffuse.cu): s Heun sub-steps of D_p/s on the sigma planes of
 // sig_new (3 planes of NP), using sig_tmp (3 planes) as the other buffer.  pdl: started by programmatic

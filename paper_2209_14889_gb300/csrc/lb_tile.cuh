@@ -452,7 +452,7 @@ __device__ __forceinline__ void readout_reduce(const FusedArgs& a, const DF* acc
     store_partial(a.partials, tile_index, acc, reinterpret_cast<float*>(sRed));
 }
 
-// the moments of the owned cells to the moments_out planes (MODE_MOMENTS)
+// the moments of the owned cells to the moments_out planes, all or the one asked for (MODE_MOMENTS)
 // IL: u staged as interleaved (u_x, u_y) pairs and drho after them (the one-cell step)
 template <int TX, int TY, bool IL = false>
 __device__ __forceinline__ void moments_out(const FusedArgs& a, const TileMem<TX, TY>& m, int x0, int y0)
@@ -465,7 +465,9 @@ __device__ __forceinline__ void moments_out(const FusedArgs& a, const TileMem<TX
         if (gx >= a.nx || gy >= a.ny) continue;
         const int j = (ly + 2) * G::R2W + lx + 2;
         const long long g = (long long)gy * a.nx + gx;
-        if (IL) {
+        if (IL && a.moments_only) {
+            a.moments_out[g] = a.moments_only == 1 ? m.sM[2 * G::R2 + j] : m.sM[2 * j + a.moments_only - 2];
+        } else if (IL) {
             const float2 u = reinterpret_cast<const float2*>(m.sM)[j];
             a.moments_out[g] = m.sM[2 * G::R2 + j];
             a.moments_out[NP + g] = u.x;
@@ -573,6 +575,8 @@ __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, in
         int lx, ly;
         region_cell<TX, TY, 3>(k, lx, ly);
         const int i = ly * R3W + lx;
+        // the moments of the owned cells need the stress one cell around them
+        if (MODE == MODE_MOMENTS && (lx < 2 || lx >= TX + 4 || ly < 2 || ly >= TY + 4)) continue;
         St px, py;
         st_pair(sP2, R4W, lx + 1, ly + 1, px, py);               // dP stencils
         float hx, hy, E[4];
@@ -602,7 +606,7 @@ __device__ __forceinline__ void tile_step(const FusedArgs& a, int bx, int by, in
     const bool readout = (t % a.every) == 0;
     DF acc[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
     void* dst = a.dst;
-    for (int k = tid; k < R2; k += NT) {
+    for (int k = tid; k < (MODE == MODE_MOMENTS ? R0 : R2); k += NT) {
         int lx, ly;
         region_cell<TX, TY, 2>(k, lx, ly);
         const int i = ly * R2W + lx;

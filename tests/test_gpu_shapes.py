@@ -128,3 +128,33 @@ def test_ring_boxes_and_trap_warps_vs_oracle(n_nodes, radius, trap):
     assert np.abs(d).max() <= 1e-6
     assert np.linalg.norm(ser[:, 6:8] - ref[:, 6:8]) <= 1e-4 * np.linalg.norm(ref[:, 6:8])
     assert np.abs(ser[:, 8:10] - ref[:, 8:10]).max() <= 1e-6
+
+
+@pytest.mark.parametrize("half", [False, True])
+@pytest.mark.parametrize("case", ["odd_71x53", "walls_131x150", "scalar_box_250"])
+def test_readout_of_one_field_matches_the_moments_of_all(case, half):
+    # a field formed alone, straight into device memory or by way of scratch (host memory, an odd address),
+    # is the plane of the pass that forms all three moments (lb_readout_noalloc)
+    import ctypes
+    lb = _gpu()
+    import torch
+    w = CASES[case]()
+    if half and (w.get("walls_x") or w.get("model")):
+        pytest.skip("the 2-byte state takes neither walls nor the scalar model")
+    s = lb.Solver.from_workload(w, precision=lb.LB_FP16_BF16 if half else lb.LB_FP32)
+    s.step(7)
+    noalloc = lb.lib().lb_readout_noalloc
+    noalloc.restype = ctypes.c_int
+    noalloc.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int32]
+    for k, fid in lb.FIELDS.items():
+        a = s.readout(k).cpu().numpy()
+        assert np.array_equal(a, s.readout(k, device=False)), k
+        n = a.size * 4
+        odd = torch.zeros(n + 8, dtype=torch.uint8, device="cuda")
+        assert lb.lib().lb_readout(s.h, fid, ctypes.c_void_p(odd.data_ptr() + 1), n, 1) == 0
+        assert np.array_equal(odd[1:1 + n].cpu().numpy().view(np.float32).reshape(a.shape), a), k
+        if k in ("drho", "ux", "uy", "Px", "Py"):
+            b = torch.zeros(a.shape, dtype=torch.float32, device="cuda")
+            assert noalloc(s.h, fid, b.data_ptr(), n, 1) == 0
+            assert np.array_equal(b.cpu().numpy(), a), k
+    s.close()
