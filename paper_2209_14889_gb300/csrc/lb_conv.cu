@@ -559,7 +559,7 @@ struct WgradArgs {
     long long ldx;
     int xoff;
     const bf16* gz;         // gradient at the layer's pre-activation output, dense [P][Co]
-    float* part;            // [S][n] partial sums: [9][Co][Ci], then the bias [Co]
+    float* part;            // [S][n] partial sums: [9][Ci][Co], then the bias [Co] (32-byte aligned)
     int B, H, W, Ci, Co;
 };
 
@@ -781,7 +781,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
             const int m = tid & 127, nj = g.cob / 16, nblk = 9 * nj;
             const bool valid = m < 8 * xg;
             const unsigned lane0 = tmem + ((unsigned)(warp & 3) << 21);
-            float* out = a.part + blockIdx.x * g.n + ci0 + m;
+            // a lane holds 16 output channels of its input channel: two whole sectors of [9][Ci][Co] (one
+            // store per value, along the input channels, took 6 to 10 us of 18 to 38)
+            float* out = a.part + blockIdx.x * g.n + (long long)(ci0 + m) * a.Co;
             for (int q0 = warp >> 2; q0 < nblk; q0 += 4) {
                 __syncwarp();               // the lanes that stored nothing and the others
                 unsigned v[2][16];
@@ -794,9 +796,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
                     const int q = q0 + 2 * h;
                     if (q >= nblk) break;
                     const int t = q / nj, co = co0 + (q - t * nj) * 16;
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (co + e < a.Co) out[((long long)t * a.Co + co + e) * a.Ci] = __uint_as_float(v[h][e]);
+                    float* o = out + (long long)t * a.Ci * a.Co + co;
+                    const unsigned(&w)[2][8] = *reinterpret_cast<const unsigned(*)[2][8]>(v[h]);
+                    if (co < a.Co) st32(o, w[0]);
+                    if (co + 8 < a.Co) st32(o + 8, w[1]);
                 }
             }
         }
@@ -811,8 +814,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const __grid_constant__
 }
 
 // Sum of S partial arrays of n floats (n a multiple of 4): eight threads per float4, each every eighth
-// partial in order, then the eight in order.  The first nw values go to gw, the others to gb.
-__global__ void __launch_bounds__(256) k_sum_parts(const float4* part, int S, int n4, int nw4, float* gw, float* gb)
+// partial in order, then the eight in order.  The first nw values ([9][Ci][Co]) go to gw ([9][Co][Ci]), the
+// others to gb.
+__global__ void __launch_bounds__(256) k_sum_parts(const float4* part, int S, int n4, int nw4, int Ci, int Co, float* gw,
+                                                   float* gb)
 {
     __shared__ float4 red[8][32];
     const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
@@ -841,11 +846,17 @@ __global__ void __launch_bounds__(256) k_sum_parts(const float4* part, int S, in
         v.z += w.z;
         v.w += w.w;
     }
-    float* o = i < nw4 ? gw + 4LL * i : gb + 4LL * (i - nw4);
+    float* o = gb + 4LL * (i - nw4);
+    long long step = 1;
+    if (i < nw4) {
+        const int r = 4 * i / Co, co = 4 * i - r * Co, t = r / Ci, ci = r - t * Ci;
+        o = gw + ((long long)t * Co + co) * Ci + ci;
+        step = Ci;
+    }
     o[0] = v.x;
-    o[1] = v.y;
-    o[2] = v.z;
-    o[3] = v.w;
+    o[step] = v.y;
+    o[2 * step] = v.z;
+    o[3 * step] = v.w;
 }
 
 // ------------------------------------------------------------------ weights
@@ -1039,7 +1050,7 @@ cudaError_t conv_wgrad(cudaStream_t s, const bf16* x, long long ldx, int xoff, c
     if (e != cudaSuccess) return e;
     const int n4 = (int)(g.n / 4), nw4 = (int)(9LL * Ci * Co / 4);
     return launch_pdl(k_sum_parts, dim3((n4 + 31) / 32), 256, 0, s, true, reinterpret_cast<const float4*>(part), S, n4, nw4,
-                      gw, gb);
+                      Ci, Co, gw, gb);
 }
 
 }  // namespace net
