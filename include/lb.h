@@ -255,8 +255,8 @@ int lb_commit_state(lb_handle* h);
  * a step carries over to the next: both state buffers and which one is current, the step
  * counter, the control block, the readout partials and series ring buffer and, with rings, the
  * ring records (parameters, trap protocol and its origin, work-box extents), both node position
- * buffers, the per-node cell, fraction and force, the work boxes, the tail's tickets and claims
- * and the node partial sums.  Native byte order; a file is read only by this library version.
+ * buffers, the per-node cell, fraction and force, the work boxes, the tail's tickets,
+ * and reserved sections of zeros.  Native byte order; a file is read only by this library version.
  * lb_load reads such a file into a handle that was created with equal lb_params (every field)
  * and given the same rings by lb_set_body (the same number of rings and nodes per ring, and
  * equal spring constant, angle constant, rest length, pull and trap protocol per ring; the node
@@ -344,8 +344,9 @@ void lb_destroy(lb_handle* h);
  * Batched form.  Many independent lattices (each with its own size, parameters, rings and
  * diffusion sub-steps; Sec. II with the parameters of Tables I-IV varied per instance) advanced
  * together, a chunk of readout_every steps at a time, the chunk captured once as a CUDA graph and
- * replayed.  By default every step is three launches per tile-shape group: all instances'
- * lattice tiles, then their diffusion sub-steps, then their node blocks.  With
+ * replayed.  By default every step is one launch per phase and group of instances (of one tile
+ * shape, with or without diffusion sub-steps), every group on a stream of its own: the lattice
+ * tiles, then the diffusion sub-steps (up to three per launch) beside the node steps.  With
  * lb_batch_set_persistent(b, 1) one persistent cooperative kernel per group runs the whole chunk
  * instead, with a grid barrier between the phases.
  * Each instance computes exactly what lb_step computes for its handle (fields and nodes bitwise

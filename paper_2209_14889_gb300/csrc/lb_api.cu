@@ -463,7 +463,7 @@ int lb_set_body(lb_handle* h, int32_t n_rings, const lb_ring* rings, const doubl
         const int lim = std::min(nx, ny) - 8;
         int cw = (int)std::ceil(mxx - mnx) + 8, chh = (int)std::ceil(mxy - mny) + 8;
         // the tail launches start at the tile row over the first ring's top (minus the box
-        // margin and the staged halo), so its node blocks run while most tiles are still to come
+        // margin and the staged halo), so its node step runs while most tiles are still to come
         if (r == 0) h->tile_rot = fused_tile_rot(nx, ny, P[1] + mny - 4.0);
         if (2 * cw > nx || 2 * chh > ny) return fail(h, LB_EINVAL, "ring %d does not fit the lattice", r);
         cw = std::min(cw + 2 * std::max(16, cw / 2), lim);

@@ -13,7 +13,7 @@
 //   lattice  the fused step of every tile of every instance (tile shape per instance, chosen by
 //            the autotuner among 32x16, 32x8, 64x8, 16x16), the tile code of lb_tile.cuh;
 //   sigma    diffusion passes of the instances whose D_p exceeds the Heun bound;
-//   nodes    the node blocks of every ring of every instance (lb_node.cuh).
+//   nodes    the node step of every ring of every instance (lb_node.cuh).
 // Work items are assigned to CTAs round-robin, so the schedule and every result are the same
 // from run to run.  The barrier spins with an iteration limit and reports LB_ETIMEOUT.
 #include <cuda_runtime.h>
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(BT, 3) k_batch_tiles(const BatchArgs B, int s)
 
 // the warp-strip step of every instance of the strip group: CTA `local` of an instance covers
 // strip columns (local % tiles_x) * SWARPS .. and rows chunk local / tiles_x; the step index comes
-// from the instance's control block (advanced by its node blocks of the step before)
+// from the instance's control block (advanced by its node step of the step before)
 template <bool SCALAR>
 __global__ void __launch_bounds__(SNT, 3) k_batch_strips(const BatchArgs B, int s)
 {
