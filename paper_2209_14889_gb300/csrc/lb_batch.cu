@@ -73,6 +73,7 @@ struct BatchArgs {
     const BatchInst* inst;
     int n_inst;
     const int* tile_begin;      // prefix sums of lattice tiles over instances (n_inst + 1)
+    const int* tile_inst;       // instance of each lattice tile (phase launches)
     const int* node_begin;      // prefix sums of rings (one for an instance without)
     const int* dif_begin;       // prefix sums of diffusion tiles (instances with dsub > 0)
     int max_dsub;
@@ -196,7 +197,8 @@ __global__ void __launch_bounds__(BT, 3) k_batch_tiles(const BatchArgs B, int s)
     extern __shared__ __align__(16) float sm[];
     const int par = (*B.cur + s) & 1;
     const int item = blockIdx.x;
-    const int i = find_inst(B.tile_begin, B.n_inst, item);
+    // one load where a search among the prefix sums is log2 n dependent ones at the start of every CTA (a sweep of 20 lattices, 30 steps: 5482 -> 5344 us)
+    const int i = __ldg(B.tile_inst + item);
     const BatchInst& I = B.inst[i];
     const int local = item - __ldg(B.tile_begin + i);
     const int by = local / I.tiles_x, bx = local - by * I.tiles_x;
@@ -213,7 +215,7 @@ __global__ void __launch_bounds__(SNT, 3) k_batch_strips(const BatchArgs B, int 
     extern __shared__ __align__(16) float smem[];
     const int par = (*B.cur + s) & 1;
     const int item = blockIdx.x;
-    const int i = find_inst(B.tile_begin, B.n_inst, item);
+    const int i = __ldg(B.tile_inst + item);
     const BatchInst& I = B.inst[i];
     const int local = item - __ldg(B.tile_begin + i);
     const int cy = local / I.tiles_x, cx = local - cy * I.tiles_x;
@@ -271,6 +273,7 @@ struct lb_batch {
     cudaEvent_t ev_main[N_GROUPS] = {}, ev_side[N_GROUPS] = {};
     BatchInst* d_inst[N_GROUPS] = {};
     int* d_tile_begin[N_GROUPS] = {};
+    int* d_tile_inst[N_GROUPS] = {};
     int* d_node_begin[N_GROUPS] = {};
     int* d_dif_begin[N_GROUPS] = {};
     int n_group[N_GROUPS] = {};
@@ -326,7 +329,7 @@ int build_plan(lb_batch* b)
     for (int g = 0; g < N_GROUPS; ++g) {
         const int sh = group_shape(g);
         std::vector<BatchInst> inst;
-        std::vector<int> tb(1, 0), nb(1, 0), db(1, 0);
+        std::vector<int> tb(1, 0), nb(1, 0), db(1, 0), ti;
         b->max_dsub[g] = 0;
         for (int i = 0; i < n; ++i) {
             lb_handle* h = b->h[i];
@@ -359,6 +362,7 @@ int build_plan(lb_batch* b)
             I.dif_ty = diffuse_tiles_y(h->p.ny);
             b->max_dsub[g] = std::max(b->max_dsub[g], I.dsub);
             tb.push_back(tb.back() + I.tiles_x * I.tiles_y);
+            ti.resize(tb.back(), (int)inst.size());
             nb.push_back(nb.back() + I.na.n_ctas);
             db.push_back(db.back() + (I.dsub > 0 ? I.dif_tx * I.dif_ty : 0));
             inst.push_back(I);
@@ -379,6 +383,11 @@ int build_plan(lb_batch* b)
             BCK(b, cudaEventCreateWithFlags(&b->ev_side[g], cudaEventDisableTiming));
         }
         BCK(b, cudaMemcpy(b->d_inst[g], inst.data(), sizeof(BatchInst) * n_in, cudaMemcpyHostToDevice));
+        // the tiles of an instance depend on its shape; nothing of the batch is in flight here
+        cudaFree(b->d_tile_inst[g]);
+        b->d_tile_inst[g] = nullptr;
+        BCK(b, cudaMalloc(&b->d_tile_inst[g], sizeof(int) * ti.size()));
+        BCK(b, cudaMemcpy(b->d_tile_inst[g], ti.data(), sizeof(int) * ti.size(), cudaMemcpyHostToDevice));
         BCK(b, cudaMemcpy(b->d_tile_begin[g], tb.data(), sizeof(int) * (n_in + 1), cudaMemcpyHostToDevice));
         BCK(b, cudaMemcpy(b->d_node_begin[g], nb.data(), sizeof(int) * (n_in + 1), cudaMemcpyHostToDevice));
         BCK(b, cudaMemcpy(b->d_dif_begin[g], db.data(), sizeof(int) * (n_in + 1), cudaMemcpyHostToDevice));
@@ -393,6 +402,7 @@ BatchArgs batch_args(const lb_batch* b, int g)
     a.inst = b->d_inst[g];
     a.n_inst = b->n_group[g];
     a.tile_begin = b->d_tile_begin[g];
+    a.tile_inst = b->d_tile_inst[g];
     a.node_begin = b->d_node_begin[g];
     a.dif_begin = b->d_dif_begin[g];
     a.max_dsub = b->max_dsub[g];
@@ -935,6 +945,7 @@ void lb_batch_destroy(lb_batch* b)
     for (int g = 0; g < N_GROUPS; ++g) {
         cudaFree(b->d_inst[g]);
         cudaFree(b->d_tile_begin[g]);
+        cudaFree(b->d_tile_inst[g]);
         cudaFree(b->d_node_begin[g]);
         cudaFree(b->d_dif_begin[g]);
         if (b->ev_main[g]) cudaEventDestroy(b->ev_main[g]);
