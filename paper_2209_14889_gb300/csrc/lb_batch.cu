@@ -4,8 +4,8 @@
 // Default (phase launches): each step is one launch per phase and group of instances -- all
 // instances' lattice tiles (k_batch_tiles, the tile kernel's occupancy of three CTAs per SM),
 // then their diffusion passes beside their rings' node steps -- in stream order, so no kernel waits
-// on another inside a launch.  A group holds the instances of one tile shape, those with diffusion
-// sub-steps apart from those without: instances are independent, so every group has a stream of its
+// on another inside a launch.  A group holds instances of one tile shape, those with diffusion
+// sub-steps apart from those without, which make two groups: instances are independent, so every group has a stream of its
 // own and its short launches run beside the lattice launches of the others (20 lattices of 128^2 to
 // 512^2, 30 steps: 6109 -> 5500 us).  Alternatively (lb_batch_set_persistent) one persistent cooperative
 // kernel per group runs the whole chunk, each step having three phases separated by a grid
@@ -43,10 +43,13 @@ constexpr int N_SHAPES = 5;
 constexpr int N_TILE_SHAPES = 4;
 constexpr int SHAPE_STRIP = 4;
 constexpr int STRIP_H = 64;
-// groups: per shape the instances without and with diffusion sub-steps (persistent launches: all in
-// the first of the two)
-constexpr int N_GROUPS = 2 * N_SHAPES;
-constexpr int group_shape(int g) { return g / 2; }
+// groups: per shape two of instances without diffusion sub-steps, of about as many tiles (the node steps
+// of the one run beside the tiles of the other), and one of those with (persistent launches: all in
+// the first of the three)
+constexpr int LANES = 3, LANE_SUB = 2;
+constexpr int N_GROUPS = LANES * N_SHAPES;
+static_assert(N_GROUPS < 32, "k_batch_parity takes a mask of groups");
+constexpr int group_shape(int g) { return g / LANES; }
 __host__ __device__ constexpr int shape_tx(int s) { return s == 0 ? 32 : (s == 1 ? 32 : (s == 2 ? 64 : 16)); }
 __host__ __device__ constexpr int shape_ty(int s) { return s == 0 ? 16 : (s == 1 ? 8 : (s == 2 ? 8 : 16)); }
 
@@ -268,7 +271,7 @@ struct lb_batch {
     std::vector<int> shape;                 // per instance
     bool scalar = false;                    // every instance runs the scalar model (else none does)
     // per group: device descriptors, prefix sums, work items, and (phase launches) its streams: the
-    // lattice and diffusion launches on one, the node steps of a sub-stepped group on the other
+    // lattice and diffusion launches on one, the node steps on the other
     cudaStream_t main[N_GROUPS] = {}, side[N_GROUPS] = {};
     cudaEvent_t ev_main[N_GROUPS] = {}, ev_side[N_GROUPS] = {};
     BatchInst* d_inst[N_GROUPS] = {};
@@ -326,6 +329,18 @@ void drop_graph(lb_batch* b)
 int build_plan(lb_batch* b)
 {
     const int n = (int)b->h.size();
+    std::vector<int> lane(n, 0);
+    if (!b->persistent) {
+        long long cells[N_SHAPES][2] = {};
+        for (int i = 0; i < n; ++i) {
+            long long* c = cells[b->shape[i]];
+            if (b->h[i]->p.diffusion_substeps > 0) lane[i] = LANE_SUB;
+            else {
+                lane[i] = c[1] < c[0] ? 1 : 0;
+                c[lane[i]] += b->h[i]->plane;
+            }
+        }
+    }
     for (int g = 0; g < N_GROUPS; ++g) {
         const int sh = group_shape(g);
         std::vector<BatchInst> inst;
@@ -333,7 +348,7 @@ int build_plan(lb_batch* b)
         b->max_dsub[g] = 0;
         for (int i = 0; i < n; ++i) {
             lb_handle* h = b->h[i];
-            if (b->shape[i] != sh || (!b->persistent && h->p.diffusion_substeps > 0) != (g % 2 == 1)) continue;
+            if (b->shape[i] != sh || lane[i] != g % LANES) continue;
             BatchInst I;
             const int save = h->cur;
             for (int p = 0; p < 2; ++p) {
@@ -374,11 +389,12 @@ int build_plan(lb_batch* b)
         if (inst.empty()) continue;
         const int n_in = (int)inst.size();
         if (!b->persistent && !b->main[g]) {
-            // sub-stepped instances have the longest chain of launches: theirs go first
+            // sub-stepped instances have the longest chain of launches, node steps are short and hold up
+            // the next tiles: theirs go first
             int least = 0, greatest = 0;
             BCK(b, cudaDeviceGetStreamPriorityRange(&least, &greatest));
-            BCK(b, cudaStreamCreateWithPriority(&b->main[g], cudaStreamNonBlocking, g % 2 ? greatest : least));
-            BCK(b, cudaStreamCreateWithPriority(&b->side[g], cudaStreamNonBlocking, g % 2 ? greatest : least));
+            BCK(b, cudaStreamCreateWithPriority(&b->main[g], cudaStreamNonBlocking, g % LANES == LANE_SUB ? greatest : least));
+            BCK(b, cudaStreamCreateWithPriority(&b->side[g], cudaStreamNonBlocking, greatest));
             BCK(b, cudaEventCreateWithFlags(&b->ev_main[g], cudaEventDisableTiming));
             BCK(b, cudaEventCreateWithFlags(&b->ev_side[g], cudaEventDisableTiming));
         }
@@ -417,7 +433,7 @@ BatchArgs batch_args(const lb_batch* b, int g)
 template <int TX, int TY>
 cudaError_t launch_shape(const lb_batch* b, int sh, int nsteps)
 {
-    BatchArgs a = batch_args(b, 2 * sh);
+    BatchArgs a = batch_args(b, LANES * sh);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(b->grid[sh]);
     cfg.blockDim = dim3(BT);
@@ -507,7 +523,7 @@ cudaError_t launch_phases(const lb_batch* b, int nsteps)
         for (int g = N_GROUPS - 1; g >= 0; --g) {
             if (!b->n_group[g]) continue;
             if (!ok(launch_lattice(b, g, s, st[g]))) return e;
-            const bool fork = b->n_dif[g] > 0 && b->n_nodes[g] > 0;
+            const bool fork = (b->n_dif[g] > 0 || used > 1) && b->n_nodes[g] > 0;
             if (b->n_nodes[g]) {
                 if (fork && !after(b->side[g], b->ev_side[g], st[g])) return e;
                 k_batch_nodes<<<b->n_nodes[g], NODE_THREADS, 0, fork ? b->side[g] : st[g]>>>(batch_args(b, g), s);
@@ -533,9 +549,9 @@ cudaError_t launch_batch(const lb_batch* b, int nsteps)
     if (!b->persistent) return launch_phases(b, nsteps);
     cudaError_t e = cudaSuccess;
     if (b->n_group[0] && e == cudaSuccess) e = launch_shape<32, 16>(b, 0, nsteps);
-    if (b->n_group[2] && e == cudaSuccess) e = launch_shape<32, 8>(b, 1, nsteps);
-    if (b->n_group[4] && e == cudaSuccess) e = launch_shape<64, 8>(b, 2, nsteps);
-    if (b->n_group[6] && e == cudaSuccess) e = launch_shape<16, 16>(b, 3, nsteps);
+    if (b->n_group[LANES] && e == cudaSuccess) e = launch_shape<32, 8>(b, 1, nsteps);
+    if (b->n_group[2 * LANES] && e == cudaSuccess) e = launch_shape<64, 8>(b, 2, nsteps);
+    if (b->n_group[3 * LANES] && e == cudaSuccess) e = launch_shape<16, 16>(b, 3, nsteps);
     unsigned others = 0;             // a persistent launch advances its own word
     for (int g = 0; g < N_GROUPS; ++g)
         if (!b->n_group[g]) others |= 1u << g;
@@ -574,7 +590,7 @@ void capture(lb_batch* b)
     }
     const cudaError_t e = launch_batch(b, b->chunk);
     const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
-    if (e == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&b->graph, g, 0) != cudaSuccess)
+    if (e == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&b->graph, g, cudaGraphInstantiateFlagUseNodePriority) != cudaSuccess)
         b->graph = nullptr;
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
