@@ -934,8 +934,7 @@ cudaError_t conv_pack(const PackArgs& p, cudaStream_t s)
 
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
 {
-    if (a.Ci % 16 != 0) return cudaErrorInvalidValue;
-    if ((long long)a.B * a.H * a.W >= (1LL << 31)) return conv_mma(a, s);      // 32-bit pixel indices
+    if (a.Ci % 16 != 0 || !a.wp || !conv_tc_fits(a.B, a.H, a.W)) return cudaErrorInvalidValue;
     const cudaError_t e = conv_err_init();
     if (e != cudaSuccess) return e;
     static const int n_sm = sm_count();

@@ -54,8 +54,12 @@ struct PackArgs {
 };
 cudaError_t conv_pack(const PackArgs& p, cudaStream_t s);
 
-// The tcgen05 convolution of a (Ci % 16 == 0).  pdl: the launch may start while the kernel before it
-// in the stream finishes (that kernel must not be the one that wrote the weights).
+// The tcgen05 kernels index pixels in 32 bits; a larger call takes the mma.sync kernel, which reads the
+// weights as they are (a.w) and not packed.
+inline bool conv_tc_fits(int B, int H, int W) { return (long long)B * H * W < (1LL << 31); }
+
+// The tcgen05 convolution of a (Ci % 16 == 0, conv_tc_fits).  pdl: the launch may start while the kernel
+// before it in the stream finishes (that kernel must not be the one that wrote the weights).
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl);
 // The mma.sync convolution (ym, up and yf2 are not supported).
 cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s);

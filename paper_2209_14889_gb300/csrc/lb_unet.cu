@@ -747,7 +747,7 @@ int lb_conv3x3(const void* x, int64_t ldx, int32_t xoff, const void* w, const fl
     a.x = static_cast<const bf16*>(x); a.ldx = ldx; a.xoff = xoff; a.w = static_cast<const bf16*>(w); a.bias = bias;
     a.y = static_cast<bf16*>(y); a.yf = yf; a.ldy = ldy; a.yoff = yoff;
     a.B = B; a.H = H; a.W = W; a.Ci = Ci; a.Co = Co; a.act = act ? 1 : 0;
-    if (g_conv_kernel == 0) return conv_code(conv_mma(a, s));
+    if (g_conv_kernel == 0 || !conv_tc_fits(B, H, W)) return conv_code(conv_mma(a, s));
     void* wp = nullptr;
     cudaError_t e = scratch(&wp, sizeof(bf16) * (size_t)conv_pack_elems(Ci, Co), s);
     if (e != cudaSuccess) return conv_code(e);
@@ -766,7 +766,7 @@ int lb_conv3x3_dgrad(const void* gz, const void* w, void* gx, int32_t B, int32_t
 {
     if (!gz || !w || !gx || B < 1 || H < 1 || W < 1 || Ci < 16 || Co < 16 || Ci % 16 || Co % 16) return LB_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    const bool tc = g_conv_kernel == 1;
+    const bool tc = g_conv_kernel == 1 && conv_tc_fits(B, H, W);
     void* wt = nullptr;
     cudaError_t e = scratch(&wt, sizeof(bf16) * 9 * (size_t)Ci * Co, s);
     if (e != cudaSuccess) return conv_code(e);
@@ -775,7 +775,8 @@ int lb_conv3x3_dgrad(const void* gz, const void* w, void* gx, int32_t B, int32_t
     p.L[0] = PackLayer{static_cast<const bf16*>(w), Ci, Co, nullptr, tc ? static_cast<bf16*>(wt) : nullptr,
                        tc ? nullptr : static_cast<bf16*>(wt)};
     ConvArgs a = {};
-    a.x = static_cast<const bf16*>(gz); a.ldx = Co; a.w = static_cast<bf16*>(wt); a.wp = static_cast<bf16*>(wt);
+    a.x = static_cast<const bf16*>(gz); a.ldx = Co;
+    (tc ? a.wp : a.w) = static_cast<bf16*>(wt);
     a.y = static_cast<bf16*>(gx); a.ldy = Ci;
     a.B = B; a.H = H; a.W = W; a.Ci = Co; a.Co = Ci;
     e = conv_pack(p, s);

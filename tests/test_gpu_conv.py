@@ -81,3 +81,29 @@ def test_weight_gradient_of_few_output_channels_and_any_address():
     n = 9 * 8 * 32
     assert torch.equal(buf[1:1 + n].reshape(gw.shape), gw) and torch.equal(buf[n + 2:n + 10], gb)
     assert buf[0] == 7.0 and buf[n + 1] == 7.0 and buf[n + 10] == 7.0
+
+
+def test_data_gradient_of_two_to_the_31_pixels():
+    # the size from which the mma.sync kernel takes the call: 64 GiB in, 64 GiB out; the gradient is
+    # non-zero around the first and the last pixels and checked there
+    torch, lb = _gpu()
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < 160 << 30:
+        pytest.skip("needs 160 GiB")
+    torch.manual_seed(31)
+    H, W, n = 32768, 65536, 20
+    gz = torch.zeros(1, H, W, 16, dtype=torch.bfloat16, device="cuda")
+    w = (torch.randn(9, 16, 16, device="cuda") / 12).to(torch.bfloat16)
+    first, last = (torch.randn(1, n, n, 16, device="cuda").to(torch.bfloat16) for _ in range(2))
+    gz[:, :n, :n] = first
+    gz[:, -n:, -n:] = last
+    gx = lb.conv3x3_dgrad(gz, w)
+    wd = w.double().flip(0).transpose(1, 2)
+    for part, got in ((first, gx[:, :n - 1, :n - 1]), (last, gx[:, 1 - n:, 1 - n:])):
+        ref = _conv64(torch, part.double(), wd)
+        ref = ref[:, :n - 1, :n - 1] if part is first else ref[:, 1:, 1:]
+        assert ref.abs().max() > 1
+        # as in test_gradients_edges_vs_fp64
+        assert torch.all((got.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5 * ref.abs().max())
+    del gz, gx
+    torch.cuda.empty_cache()
