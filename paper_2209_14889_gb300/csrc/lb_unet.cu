@@ -29,6 +29,7 @@
 
 #include "../../include/lb.h"
 #include "lb_conv.h"
+#include "lb_device_ptr.h"
 #include "lb_internal.h"
 
 namespace vlb {
@@ -587,7 +588,13 @@ int lb_net_forward(lb_net* n, const void* x, float* y)
     if (!n || !x) return LB_EINVAL;
     const long long P0 = (long long)n->B * n->H * n->W;
     NCK(n, cudaMemcpyAsync(n->x_in, x, sizeof(bf16) * P0 * 16, cudaMemcpyDeviceToDevice, n->stream));
-    return net_forward(n, y);
+    // the last convolution stores the output in y too, where a kernel may write; elsewhere a copy, which
+    // handles or refuses the address
+    const bool direct = y && vlb::device_floats(y, sizeof(float) * P0 * 16);
+    const int rc = net_forward(n, direct ? y : nullptr);
+    if (rc == LB_OK && y && !direct)
+        NCK(n, cudaMemcpyAsync(y, n->y, sizeof(float) * P0 * 16, cudaMemcpyDeviceToDevice, n->stream));
+    return rc;
 }
 
 const float* lb_net_output(const lb_net* n) { return n ? n->y : nullptr; }

@@ -107,3 +107,19 @@ def test_data_gradient_of_two_to_the_31_pixels():
         assert torch.all((got.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5 * ref.abs().max())
     del gz, gx
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 4])
+def test_network_output_at_any_address(shift):
+    torch, lb = _gpu()
+    n = lb.Net(1, 16, 24, seed=3)
+    x = torch.randn(1, 16, 24, 16, device="cuda").to(torch.bfloat16)
+    ref = n.forward(x)
+    size = ref.numel() * 4
+    buf = torch.full((size + 8,), 9, dtype=torch.uint8, device="cuda")
+    assert lb.lib().lb_net_forward(n.n, x.data_ptr(), buf.data_ptr() + shift) == 0
+    torch.cuda.synchronize()
+    got = buf[shift:shift + size].clone().view(torch.float32).reshape(ref.shape)
+    assert torch.equal(got, ref)
+    assert (buf[:shift] == 9).all() and (buf[shift + size:] == 9).all()
+    n.close()

@@ -7,7 +7,7 @@ import pytest
 
 import _fake_cuda as F
 
-LB_OK, LB_ENOMEM, LB_ECUDA = 0, -3, -4
+LB_OK, LB_ENOMEM, LB_ECUDA, LB_ESTATE = 0, -2, -3, -7
 P = ctypes.c_void_p
 I32, I64 = ctypes.c_int32, ctypes.c_int64
 
@@ -88,3 +88,39 @@ def test_data_gradient_reads_the_weights_in_the_form_that_its_kernel_takes(conv,
     else:
         assert args[0].w and args[0].w == packs[0].wt
     assert (args[0].x, args[0].y, args[0].Ci, args[0].Co) == (GZ, GX, 32, 16)
+
+
+# ---- the network's output
+
+@pytest.mark.parametrize("kind,device,shift,room,direct", [
+    (F.DEVICE, 0, 0, 0, True), (F.DEVICE, 0, 4, 0, True), (F.DEVICE, 0, 1, 0, False), (F.DEVICE, 0, 2, 0, False),
+    (F.DEVICE, 1, 0, 0, False), (F.HOST, 0, 0, 0, False), (F.MANAGED, 0, 0, 0, False), (0, -2, 0, 0, False),
+    (F.DEVICE, 0, 0, -4, False)])
+def test_network_output_goes_by_copy_where_a_kernel_must_not_write(fake, kind, device, shift, room, direct):
+    # memory of this device at a multiple of four bytes: the head convolution stores there; host, managed
+    # or another device's memory, an odd address, an end outside: the runtime's copy, which handles or refuses it
+    L = fake.L
+    L.lb_net_create.argtypes = [I32, I32, I32, ctypes.c_uint64, P, P]
+    L.lb_net_forward.argtypes = [P, P, P]
+    L.lb_net_output.argtypes, L.lb_net_output.restype = [P], P
+    L.lb_net_destroy.argtypes = [P]
+    n = P()
+    assert L.lb_net_create(1, 8, 16, 1, None, ctypes.byref(n)) == LB_OK
+    nbytes = 4 * 8 * 16 * 16
+    base = 7 << 40
+    if kind:
+        fake.memory(base, nbytes + shift + room, kind, device)
+    y = base + shift
+    x = ctypes.create_string_buffer(2 * 8 * 16 * 16)
+    if not kind:                                 # a plain host buffer
+        buf = ctypes.create_string_buffer(nbytes)
+        y = ctypes.addressof(buf)
+    fake.clear()
+    seen = arguments(fake, "k_conv_tc", ConvArgs)
+    assert L.lb_net_forward(n, x, y) == LB_OK
+    assert [a.yf2 for a in seen if a.yf2] == ([y] if direct else [])
+    copies = [c for c in fake.calls("cudaMemcpyAsync") if int(c[1], 16) == y]
+    assert [(int(c[2], 16), int(c[3])) for c in copies] == ([] if direct else [(L.lb_net_output(n), nbytes)])
+    fake.hook(None)
+    L.lb_net_destroy(n)
+    fake.memory(base, 0)
