@@ -102,10 +102,10 @@ __device__ __forceinline__ bool cell_of(const Args3& a, Cell& q)
 // value of plane f at the cell and its six neighbours: v[0] centre, then +x -x +y -y +z -z
 __device__ __forceinline__ void stencil(const float* f, const Cell& q, float* v)
 {
-    v[0] = __ldg(f + q.c);
-    v[1] = __ldg(f + q.xp); v[2] = __ldg(f + q.xm);
-    v[3] = __ldg(f + q.yp); v[4] = __ldg(f + q.ym);
-    v[5] = __ldg(f + q.zp); v[6] = __ldg(f + q.zm);
+    v[0] = f[q.c];
+    v[1] = f[q.xp]; v[2] = f[q.xm];
+    v[3] = f[q.yp]; v[4] = f[q.ym];
+    v[5] = f[q.zp]; v[6] = f[q.zm];
 }
 
 __device__ __forceinline__ float lap7(const float* v) { return v[1] + v[2] + v[3] + v[4] + v[5] + v[6] - 6.f * v[0]; }
@@ -138,7 +138,10 @@ using vlb::vec::bc;
 using vlb::vec::vfma;
 
 // Consecutive kernels of a step overlap by programmatic dependent launch: each waits for the one before
-// it to complete before it touches memory, then lets the next one start its CTAs.
+// it to complete before it touches memory, then lets the next one start its CTAs.  What the kernels before
+// have written is read by plain loads: the read-only path (__ldg) is for data that nothing writes while the
+// kernel lives, and this kernel lives before the former one has ended; a compiler may also move such a load
+// above the wait.  Only the coefficient table is read through it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -165,17 +168,34 @@ __device__ __forceinline__ bool nb_of(const Args3& a, Nb<T>& q)
     return true;
 }
 
+// The stencil kernels' loads, in program order behind the wait (256^3: 1758 us per step as with __ldg, where
+// loads that the compiler may move spill registers and take 1777).
+__device__ __forceinline__ float ldo(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 template <class T>
-__device__ __forceinline__ T ldv(const float* p) { return __ldg(reinterpret_cast<const T*>(p)); }
+__device__ __forceinline__ T ldv(const float* p);
+template <>
+__device__ __forceinline__ float ldv<float>(const float* p) { return ldo(p); }
+template <>
+__device__ __forceinline__ float2 ldv<float2>(const float* p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
 template <class T>
 __device__ __forceinline__ void stv(float* p, T v) { *reinterpret_cast<T*>(p) = v; }
 
 // value, differences f(+) - f(-) along x, y, z and the sum of the six neighbours of plane f
 __device__ __forceinline__ void fold(const float* f, const Nb<float>& q, float& c, float& dx, float& dy, float& dz, float& sum)
 {
-    c = __ldg(f + q.c);
-    const float xp = __ldg(f + q.xp), xm = __ldg(f + q.xm), yp = __ldg(f + q.yp), ym = __ldg(f + q.ym),
-                zp = __ldg(f + q.zp), zm = __ldg(f + q.zm);
+    c = ldo(f + q.c);
+    const float xp = ldo(f + q.xp), xm = ldo(f + q.xm), yp = ldo(f + q.yp), ym = ldo(f + q.ym),
+                zp = ldo(f + q.zp), zm = ldo(f + q.zm);
     dx = xp - xm;
     dy = yp - ym;
     dz = zp - zm;
@@ -185,7 +205,7 @@ __device__ __forceinline__ void fold(const float* f, const Nb<float2>& q, float2
                                      float2& sum)
 {
     c = ldv<float2>(f + q.c);
-    const float r = __ldg(f + q.xp), l = __ldg(f + q.xm);
+    const float r = ldo(f + q.xp), l = ldo(f + q.xm);
     const float2 yp = ldv<float2>(f + q.yp), ym = ldv<float2>(f + q.ym), zp = ldv<float2>(f + q.zp), zm = ldv<float2>(f + q.zm);
     const float2 xp = make_float2(c.y, r), xm = make_float2(l, c.x);
     dx = xp - xm;
@@ -447,25 +467,32 @@ __global__ void __launch_bounds__(NT, MINB) k3_collide(const __grid_constant__ A
     const bool in = cell_of(a, q);
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (in) {
-        // F_i = d_j sigma^p_ij + d_j sigma^E_ij + f_ext,i
+        // F_i = d_j sigma^p_ij + d_j sigma^E_ij + f_ext,i; every load ahead of the sums
         float F[3] = {a.fx, a.fy, a.fz};
         const int nb[3][2] = {{q.xp, q.xm}, {q.yp, q.ym}, {q.zp, q.zm}};
+        float dp[9], de[9], d[NQ];
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+        for (int n = 0; n < NQ; ++n) d[n] = a.src[(long long)n * a.NP + q.c];
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const float* sp = a.src + (long long)(PL_S + sym6(i, j)) * a.NP;
-                F[i] += 0.5f * (__ldg(sp + nb[j][0]) - __ldg(sp + nb[j][1]));
-                if (a.ericksen) {
-                    const float* se = a.sE + (long long)(i * 3 + j) * a.NP;
-                    F[i] += 0.5f * (__ldg(se + nb[j][0]) - __ldg(se + nb[j][1]));
-                }
+        for (int k = 0; k < 9; ++k) {
+            const float* sp = a.src + (long long)(PL_S + sym6(k / 3, k % 3)) * a.NP;
+            dp[k] = sp[nb[k % 3][0]] - sp[nb[k % 3][1]];
+        }
+        if (a.ericksen) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const float* se = a.sE + (long long)k * a.NP;
+                de[k] = se[nb[k % 3][0]] - se[nb[k % 3][1]];
             }
-        float d[NQ];
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            F[k / 3] += 0.5f * dp[k];
+            if (a.ericksen) F[k / 3] += 0.5f * de[k];
+        }
         float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
 #pragma unroll
         for (int n = 0; n < NQ; ++n) {
-            d[n] = __ldg(a.src + (long long)n * a.NP + q.c);
             drho += d[n];
             jx += (float)CX[n] * d[n];
             jy += (float)CY[n] * d[n];
@@ -531,7 +558,7 @@ __global__ void __launch_bounds__(NT) k3_moment(const __grid_constant__ Args3 a,
     float drho = 0.f, jn = 0.f;
 #pragma unroll
     for (int n = 0; n < NQ; ++n) {
-        const float d = __ldg(a.src + (long long)n * a.NP + q.c);
+        const float d = a.src[(long long)n * a.NP + q.c];
         drho += d;
         const int c = axis == 0 ? CX[n] : (axis == 1 ? CY[n] : CZ[n]);
         jn += (float)c * d;
@@ -545,10 +572,10 @@ __global__ void __launch_bounds__(NT) k3_moment(const __grid_constant__ Args3 a,
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         const float* sp = a.src + (long long)(PL_S + sym6(axis, j)) * a.NP;
-        F += 0.5f * (__ldg(sp + nb[j][0]) - __ldg(sp + nb[j][1]));
+        F += 0.5f * (sp[nb[j][0]] - sp[nb[j][1]]);
         if (a.ericksen) {
             const float* se = a.sE + (long long)(axis * 3 + j) * a.NP;
-            F += 0.5f * (__ldg(se + nb[j][0]) - __ldg(se + nb[j][1]));
+            F += 0.5f * (se[nb[j][0]] - se[nb[j][1]]);
         }
     }
     out[q.c] = (jn + 0.5f * F) * (1.f / (a.rho0 + drho));
@@ -649,12 +676,15 @@ __global__ void __launch_bounds__(NT, MINB) k3_correct(const __grid_constant__ A
     load_y9(a.ys, a.NP, q, f.u, y);
     T r[9];
     rhs9(a, y, f, r);
+    // all loads ahead of the stores, which they may not be moved across
+    T y0[9], r0[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const T y0 = ldv<T>(a.src + (long long)(PL_S + k) * a.NP + q.c);
-        const T r0 = ldv<T>(a.r0 + k * a.NP + q.c);
-        stv(a.dst + (long long)(PL_S + k) * a.NP + q.c, vfma(0.5f, r0 + r[k], y0));
+        y0[k] = ldv<T>(a.src + (long long)(PL_S + k) * a.NP + q.c);
+        r0[k] = ldv<T>(a.r0 + k * a.NP + q.c);
     }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) stv(a.dst + (long long)(PL_S + k) * a.NP + q.c, vfma(0.5f, r0[k] + r[k], y0[k]));
 }
 
 // out = plane + c (the readout of P = P_ref + dP)

@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
                     for (int e = 0; e < 8; ++e) r[e] = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
                     if (a.ym) {                     // the gradient through the layer below's LeakyReLU
                         const uint4* mp = reinterpret_cast<const uint4*>(a.ym + pix * a.ldm + a.moff + co0 + j);
-                        const uint4 m4[2] = {__ldg(mp), __ldg(mp + 1)};
+                        const uint4 m4[2] = {mp[0], mp[1]};     // not __ldg: a launch before wrote them
                         const __nv_bfloat162* mv = reinterpret_cast<const __nv_bfloat162*>(m4);
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
