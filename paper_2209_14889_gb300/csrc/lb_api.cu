@@ -563,7 +563,9 @@ int lb_step(lb_handle* h, int64_t n)
             h->n_partials = sweep_ctas(h->p.nx, h->p.ny, h->sweep_chunk);
         } else if (strip) {
             fa.t = h->t;
-            CK(h, launch_strip(fa, h->strip_chunk, h->stream, pdl));
+            // its read-only loads of the state are safe behind a node kernel; behind a launch with the tail it
+            // starts when that launch has completed
+            CK(h, launch_strip(fa, h->strip_chunk, h->stream, pdl && !h->after_tail));
             h->n_partials = strip_ctas(h->p.nx, h->p.ny, h->strip_chunk);
         } else {
             const int shape = pair ? 0 : h->tile_shape;

@@ -124,3 +124,43 @@ def test_network_output_goes_by_copy_where_a_kernel_must_not_write(fake, kind, d
     fake.hook(None)
     L.lb_net_destroy(n)
     fake.memory(base, 0)
+
+
+# ---- lattices
+
+def solver(fake, nx, ny, rings=0, every=4, stream=None, **kw):
+    """A handle on the stand-in, with `rings` small rings, ready to step."""
+    from paper_2209_14889_gb300 import lb
+    L = fake.L
+    base = dict(nx=nx, ny=ny, tau=0.8, rho0=1.0, K1111=2e-3, K1122=1e-3, K2222=1e-3, K1212=1e-3, eta_p=0.1,
+                lambda_steps=0.0, Dp=0.05, alpha=-0.9, beta=1.0, xi=1.1, Gamma=1.0, kappa=1e-3, P_cap=0.99,
+                director_angle=0.0, ericksen=1, precision=0, readout_every=every, max_samples=16)
+    base.update(kw)
+    h = P()
+    assert L.lb_create(ctypes.byref(lb.lb_params(**base)), P(stream), ctypes.byref(h)) == LB_OK
+    if rings:
+        import math
+        rd = (lb.lb_ring * rings)(*[lb.lb_ring(n_nodes=12, k_spring=0.1, eps_angle=0.01, l_eq=1.0) for _ in range(rings)])
+        X = [c for r in range(rings) for k in range(12)
+             for c in (nx / 2 + 0.1 * r + 2 * math.cos(k * math.pi / 6), ny / 2 + 2 * math.sin(k * math.pi / 6))]
+        X = (ctypes.c_double * len(X))(*X)
+        L.lb_set_body.argtypes = [P, I32, P, P]
+        assert L.lb_set_body(h, rings, rd, X) == LB_OK
+    L.lb_init_fields.argtypes = [P, P]
+    assert L.lb_init_fields(h, None) == LB_OK
+    L.lb_step.argtypes = [P, I64]
+    L.lb_set_kernel.argtypes = [P, I32]
+    L.lb_destroy.argtypes = [P]
+    return h
+
+
+def test_strip_step_behind_a_launch_with_the_node_tail_starts_when_that_has_ended(fake):
+    # it reads the state by the read-only path, which the launch before must no longer write
+    from paper_2209_14889_gb300 import lb
+    h = solver(fake, 128, 64, rings=1)
+    assert fake.L.lb_step(h, 2) == LB_OK
+    assert fake.L.lb_set_kernel(h, lb.LB_KERNEL_STRIP) == LB_OK
+    fake.clear()
+    assert fake.L.lb_step(h, 3) == LB_OK
+    assert [c[-1] for c in fake.launches("k_strip")] == ["0", "1", "1"]
+    fake.L.lb_destroy(h)
