@@ -421,6 +421,7 @@ void lb_batch_destroy(lb_batch* b);
  *   BF16 activations and weights w[9][Co][Ci]), exposed to test them alone: forward with optional
  *   bias and LeakyReLU into BF16 y or FP32 yf; the data gradient gx[B][H][W][Ci] from
  *   gz[B][H][W][Co]; the weight and bias gradients gw[9][Co][Ci], gb[Co] (FP32) from x and gz.
+ *   lb_conv3x3 is ordered on `stream`; the two gradients return when their results are there.
  */
 typedef struct lb_net lb_net;
 int lb_net_create(int32_t batch, int32_t height, int32_t width, uint64_t seed, void* stream, lb_net** out);
@@ -445,7 +446,8 @@ const char* lb_net_last_error(const lb_net* n);
 void lb_net_destroy(lb_net* n);
 /* Convolution kernel of the forward passes and data gradients (process-wide): 0 mma.sync
  * m16n8k16 tiles, 1 tcgen05.mma with tensor-memory accumulators (default).  lb_conv_status returns
- * LB_ETIMEOUT (once) if a tcgen05 convolution's bounded wait for its MMAs gave up. */
+ * LB_ETIMEOUT (once) if a tcgen05 convolution's bounded wait for its MMAs gave up; it waits for no
+ * stream: synchronise the one that lb_conv3x3 or a network ran on before asking. */
 int lb_conv_kernel(int32_t kernel);
 int lb_conv_status(void);
 int lb_conv3x3(const void* x, int64_t ldx, int32_t xoff, const void* w, const float* bias, void* y, float* yf,

@@ -736,6 +736,15 @@ cudaError_t scratch(void** p, size_t bytes, cudaStream_t s)
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
+// The end of a gradient call: its scratch given back and its work done, so that the results may be used from
+// anywhere and a fault of its kernels is its own return code.
+cudaError_t finish(void* p, cudaError_t e, cudaStream_t s)
+{
+    const cudaError_t f = cudaFreeAsync(p, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e != cudaSuccess ? e : f;
+}
+
 int conv_code(cudaError_t e) { return e == cudaSuccess ? LB_OK : (e == cudaErrorMemoryAllocation ? LB_ENOMEM : LB_ECUDA); }
 
 }  // namespace
@@ -788,8 +797,7 @@ int lb_conv3x3_dgrad(const void* gz, const void* w, void* gx, int32_t B, int32_t
     a.B = B; a.H = H; a.W = W; a.Ci = Co; a.Co = Ci;
     e = conv_pack(p, s);
     if (e == cudaSuccess) e = tc ? conv_tc(a, s, false) : conv_mma(a, s);
-    const cudaError_t f = cudaFreeAsync(wt, s);
-    return conv_code(e != cudaSuccess ? e : f);
+    return conv_code(finish(wt, e, s));
 }
 
 int lb_conv3x3_wgrad(const void* x, const void* gz, float* gw, float* gb, int32_t B, int32_t H, int32_t W, int32_t Ci,
@@ -803,8 +811,7 @@ int lb_conv3x3_wgrad(const void* x, const void* gz, float* gw, float* gb, int32_
     if (e != cudaSuccess) return conv_code(e);
     e = conv_wgrad(s, static_cast<const bf16*>(x), Ci, 0, static_cast<const bf16*>(gz), B, H, W, Ci, Co,
                    static_cast<float*>(part), room, gw, gb, false);
-    const cudaError_t f = cudaFreeAsync(part, s);
-    return conv_code(e != cudaSuccess ? e : f);
+    return conv_code(finish(part, e, s));
 }
 
 }  // extern "C"

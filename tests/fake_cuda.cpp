@@ -122,7 +122,13 @@ extern "C" {
 // ---- the tests' side
 const char* fake_log() { return logbuf.c_str(); }
 void fake_clear() { logbuf.clear(); }
-void fake_fail(const char* name, int nth, int e) { fail_name = name; fail_at = nth; fail_err = e; }
+void fake_fail(const char* name, int nth, int e)
+{
+    fail_name = name;
+    fail_at = nth;
+    fail_err = e;
+    last = cudaSuccess;
+}
 void fake_memory(void* p, size_t bytes, int type, int dev)
 {
     if (bytes) mems[static_cast<char*>(p)] = Mem{bytes, type, dev, false};

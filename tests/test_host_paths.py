@@ -164,3 +164,26 @@ def test_strip_step_behind_a_launch_with_the_node_tail_starts_when_that_has_ende
     assert fake.L.lb_step(h, 3) == LB_OK
     assert [c[-1] for c in fake.launches("k_strip")] == ["0", "1", "1"]
     fake.L.lb_destroy(h)
+
+
+def gradient_calls(L):
+    return {"dgrad": lambda s: L.lb_conv3x3_dgrad(GZ, WT, GX, 1, 9, 40, 32, 16, s),
+            "wgrad": lambda s: L.lb_conv3x3_wgrad(X, GZ, GW, GB, 1, 9, 40, 32, 16, s)}
+
+
+@pytest.mark.parametrize("which", ["dgrad", "wgrad"])
+@pytest.mark.parametrize("kernel", [0, 1])
+def test_single_layer_gradients_return_when_they_are_done(conv, which, kernel):
+    # the results may be read from any stream or freed; a fault of their kernels is their own return code
+    s = 0x77770
+    conv.L.lb_conv_kernel(kernel)
+    call = gradient_calls(conv.L)[which]
+    assert call(s) == LB_OK
+    kinds = [c[0] for c in conv.calls()]
+    last = len(kinds) - 1 - kinds[::-1].index("launch")
+    assert ["cudaStreamSynchronize", hex(s)] in conv.calls()[last:]
+    live = conv.L.fake_live()
+    conv.fail("cudaStreamSynchronize", 1, 700)
+    assert call(s) == LB_ECUDA
+    assert conv.L.fake_live() == live
+    conv.L.lb_conv_kernel(1)
