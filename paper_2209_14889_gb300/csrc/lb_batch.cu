@@ -270,8 +270,12 @@ struct lb_batch {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     std::vector<int> shape;                 // per instance
     bool scalar = false;                    // every instance runs the scalar model (else none does)
-    // per group: device descriptors, prefix sums, work items, and (phase launches) its streams: the
-    // lattice and diffusion launches on one, the node steps on the other
+    // per group: device descriptors, prefix sums and work items, in one buffer sized for any shapes
+    // (plan_cap), and (phase launches) its streams: the lattice and diffusion launches on one, the
+    // node steps on the other
+    char* d_plan = nullptr;
+    size_t plan_cap = 0;
+    bool planned = false;                   // the plan is complete (else no step runs)
     cudaStream_t main[N_GROUPS] = {}, side[N_GROUPS] = {};
     cudaEvent_t ev_main[N_GROUPS] = {}, ev_side[N_GROUPS] = {};
     BatchInst* d_inst[N_GROUPS] = {};
@@ -325,9 +329,42 @@ void drop_graph(lb_batch* b)
     b->graph_tried = false;
 }
 
-// (re)build the per-instance descriptors of every shape group for the current tile shapes
+// work items of a lattice step of one instance, in x and y
+void lattice_items(const lb_handle* h, int sh, int& tx, int& ty)
+{
+    if (sh == SHAPE_STRIP) {
+        tx = ((h->p.nx + SOWN - 1) / SOWN + SWARPS - 1) / SWARPS;
+        ty = (h->p.ny + STRIP_H - 1) / STRIP_H;
+    } else {
+        tx = (h->p.nx + shape_tx(sh) - 1) / shape_tx(sh);
+        ty = (h->p.ny + shape_ty(sh) - 1) / shape_ty(sh);
+    }
+}
+
+// bytes of the plan of these instances, whatever their shapes: descriptors, three prefix sums per group,
+// the instance of every tile
+size_t plan_bytes(const std::vector<lb_handle*>& hs)
+{
+    size_t ints = 3 * (hs.size() + N_GROUPS);
+    for (const lb_handle* h : hs) {
+        int most = 0;
+        for (int sh = 0; sh < N_SHAPES; ++sh) {
+            int tx, ty;
+            lattice_items(h, sh, tx, ty);
+            most = std::max(most, tx * ty);
+        }
+        ints += most;
+    }
+    return sizeof(BatchInst) * hs.size() + sizeof(int) * ints;
+}
+
+// (re)build the per-instance descriptors of every shape group for the current tile shapes; nothing of the
+// batch is in flight.  The former plan and its graph are gone first: when a call fails half way no step
+// runs until a plan is complete.
 int build_plan(lb_batch* b)
 {
+    drop_graph(b);
+    b->planned = false;
     const int n = (int)b->h.size();
     std::vector<int> lane(n, 0);
     if (!b->persistent) {
@@ -341,6 +378,15 @@ int build_plan(lb_batch* b)
             }
         }
     }
+    // the buffer: the descriptors of the groups one after the other, then each group's tables
+    std::vector<char> plan(b->plan_cap);
+    size_t inst_at = 0, int_at = sizeof(BatchInst) * (size_t)n;
+    auto table = [&](const std::vector<int>& v) {
+        memcpy(plan.data() + int_at, v.data(), sizeof(int) * v.size());
+        int* d = reinterpret_cast<int*>(b->d_plan + int_at);
+        int_at += sizeof(int) * v.size();
+        return d;
+    };
     for (int g = 0; g < N_GROUPS; ++g) {
         const int sh = group_shape(g);
         std::vector<BatchInst> inst;
@@ -362,13 +408,7 @@ int build_plan(lb_batch* b)
             I.xb[h->cur] = h->X;
             I.xb[h->cur ^ 1] = h->X_alt;
             I.shape = sh;
-            if (sh == SHAPE_STRIP) {
-                I.tiles_x = ((h->p.nx + SOWN - 1) / SOWN + SWARPS - 1) / SWARPS;
-                I.tiles_y = (h->p.ny + STRIP_H - 1) / STRIP_H;
-            } else {
-                I.tiles_x = (h->p.nx + shape_tx(sh) - 1) / shape_tx(sh);
-                I.tiles_y = (h->p.ny + shape_ty(sh) - 1) / shape_ty(sh);
-            }
+            lattice_items(h, sh, I.tiles_x, I.tiles_y);
             I.na.n_partials = I.tiles_x * I.tiles_y;
             for (int p = 0; p < 2; ++p) I.sig[p] = static_cast<float*>(h->state[p]) + (size_t)PL_SXX * h->plane;
             I.dsub = h->p.diffusion_substeps;
@@ -387,28 +427,27 @@ int build_plan(lb_batch* b)
         b->n_nodes[g] = nb.back();
         b->n_dif[g] = db.back();
         if (inst.empty()) continue;
-        const int n_in = (int)inst.size();
-        if (!b->persistent && !b->main[g]) {
+        b->d_inst[g] = reinterpret_cast<BatchInst*>(b->d_plan + inst_at);
+        memcpy(plan.data() + inst_at, inst.data(), sizeof(BatchInst) * inst.size());
+        inst_at += sizeof(BatchInst) * inst.size();
+        b->d_tile_begin[g] = table(tb);
+        b->d_node_begin[g] = table(nb);
+        b->d_dif_begin[g] = table(db);
+        b->d_tile_inst[g] = table(ti);
+        if (!b->persistent) {
             // sub-stepped instances have the longest chain of launches, node steps are short and hold up
             // the next tiles: theirs go first
             int least = 0, greatest = 0;
             BCK(b, cudaDeviceGetStreamPriorityRange(&least, &greatest));
-            BCK(b, cudaStreamCreateWithPriority(&b->main[g], cudaStreamNonBlocking, g % LANES == LANE_SUB ? greatest : least));
-            BCK(b, cudaStreamCreateWithPriority(&b->side[g], cudaStreamNonBlocking, greatest));
-            BCK(b, cudaEventCreateWithFlags(&b->ev_main[g], cudaEventDisableTiming));
-            BCK(b, cudaEventCreateWithFlags(&b->ev_side[g], cudaEventDisableTiming));
+            if (!b->main[g])
+                BCK(b, cudaStreamCreateWithPriority(&b->main[g], cudaStreamNonBlocking, g % LANES == LANE_SUB ? greatest : least));
+            if (!b->side[g]) BCK(b, cudaStreamCreateWithPriority(&b->side[g], cudaStreamNonBlocking, greatest));
+            if (!b->ev_main[g]) BCK(b, cudaEventCreateWithFlags(&b->ev_main[g], cudaEventDisableTiming));
+            if (!b->ev_side[g]) BCK(b, cudaEventCreateWithFlags(&b->ev_side[g], cudaEventDisableTiming));
         }
-        BCK(b, cudaMemcpy(b->d_inst[g], inst.data(), sizeof(BatchInst) * n_in, cudaMemcpyHostToDevice));
-        // the tiles of an instance depend on its shape; nothing of the batch is in flight here
-        cudaFree(b->d_tile_inst[g]);
-        b->d_tile_inst[g] = nullptr;
-        BCK(b, cudaMalloc(&b->d_tile_inst[g], sizeof(int) * ti.size()));
-        BCK(b, cudaMemcpy(b->d_tile_inst[g], ti.data(), sizeof(int) * ti.size(), cudaMemcpyHostToDevice));
-        BCK(b, cudaMemcpy(b->d_tile_begin[g], tb.data(), sizeof(int) * (n_in + 1), cudaMemcpyHostToDevice));
-        BCK(b, cudaMemcpy(b->d_node_begin[g], nb.data(), sizeof(int) * (n_in + 1), cudaMemcpyHostToDevice));
-        BCK(b, cudaMemcpy(b->d_dif_begin[g], db.data(), sizeof(int) * (n_in + 1), cudaMemcpyHostToDevice));
     }
-    drop_graph(b);
+    BCK(b, cudaMemcpy(b->d_plan, plan.data(), int_at, cudaMemcpyHostToDevice));
+    b->planned = true;
     return LB_OK;
 }
 
@@ -601,6 +640,7 @@ void capture(lb_batch* b)
 int run_steps(lb_batch* b, long long n)
 {
     if (n == 0) return LB_OK;
+    if (!b->planned) return bfail(b, LB_ESTATE, "no complete plan: set the shapes again");
     if (!b->graph_tried) capture(b);
     BCK(b, cudaEventRecord(b->ev_in, b->user));
     BCK(b, cudaStreamWaitEvent(b->stream, b->ev_in, 0));
@@ -653,12 +693,8 @@ int lb_batch_create(lb_handle* const* handles, int32_t n, lb_batch** out)
         cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming) != cudaSuccess)
         return cleanup(LB_ECUDA);
-    for (int g = 0; g < N_GROUPS; ++g)
-        if (cudaMalloc(&b->d_inst[g], sizeof(BatchInst) * n) != cudaSuccess ||
-            cudaMalloc(&b->d_tile_begin[g], sizeof(int) * (n + 1)) != cudaSuccess ||
-            cudaMalloc(&b->d_node_begin[g], sizeof(int) * (n + 1)) != cudaSuccess ||
-            cudaMalloc(&b->d_dif_begin[g], sizeof(int) * (n + 1)) != cudaSuccess)
-            return cleanup(LB_ENOMEM);
+    b->plan_cap = plan_bytes(b->h);
+    if (cudaMalloc(&b->d_plan, b->plan_cap) != cudaSuccess) return cleanup(LB_ENOMEM);
     if (cudaMalloc(&b->d_cur, sizeof(int) * N_GROUPS) != cudaSuccess ||
         cudaMalloc(&b->d_bar, 2 * sizeof(unsigned) * N_SHAPES) != cudaSuccess ||
         cudaMalloc(&b->d_err, sizeof(int)) != cudaSuccess)
@@ -959,16 +995,12 @@ void lb_batch_destroy(lb_batch* b)
     if (b->ev_out) cudaEventDestroy(b->ev_out);
     if (b->stream) cudaStreamDestroy(b->stream);
     for (int g = 0; g < N_GROUPS; ++g) {
-        cudaFree(b->d_inst[g]);
-        cudaFree(b->d_tile_begin[g]);
-        cudaFree(b->d_tile_inst[g]);
-        cudaFree(b->d_node_begin[g]);
-        cudaFree(b->d_dif_begin[g]);
         if (b->ev_main[g]) cudaEventDestroy(b->ev_main[g]);
         if (b->ev_side[g]) cudaEventDestroy(b->ev_side[g]);
         if (b->main[g]) cudaStreamDestroy(b->main[g]);
         if (b->side[g]) cudaStreamDestroy(b->side[g]);
     }
+    cudaFree(b->d_plan);
     cudaFree(b->d_cur);
     cudaFree(b->d_bar);
     cudaFree(b->d_err);

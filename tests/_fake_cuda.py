@@ -36,7 +36,7 @@ class Fake:
 
     def fail(self, name, nth=1, err=2):
         """The nth call of `name` from here on returns err (2: out of memory)."""
-        self.L.fake_fail(name.encode(), nth, err)
+        self.L.fake_fail(name.encode(), nth if name else 0, err)
 
     def memory(self, address, nbytes, kind=DEVICE, device=0):
         """An address that the runtime knows and nothing touches; nbytes 0 forgets it."""

@@ -187,3 +187,49 @@ def test_single_layer_gradients_return_when_they_are_done(conv, which, kernel):
     assert call(s) == LB_ECUDA
     assert conv.L.fake_live() == live
     conv.L.lb_conv_kernel(1)
+
+
+# ---- batches
+
+def batch(fake, handles):
+    L = fake.L
+    for f, a in (("lb_batch_create", [P, I32, P]), ("lb_batch_step", [P, I64]), ("lb_batch_set_shape", [P, I32, I32]),
+                 ("lb_batch_set_persistent", [P, I32]), ("lb_batch_destroy", [P]), ("lb_batch_uses_graph", [P])):
+        getattr(L, f).argtypes = a
+    arr = (P * len(handles))(*[h.value for h in handles])
+    b = P()
+    assert L.lb_batch_create(arr, len(handles), ctypes.byref(b)) == LB_OK
+    return b
+
+
+SIZES = [dict(nx=128, ny=96, rings=1), dict(nx=64, ny=64), dict(nx=160, ny=80, rings=1, Dp=0.3, diffusion_substeps=3),
+         dict(nx=71, ny=53)]
+
+
+@pytest.mark.parametrize("call", ["cudaMalloc", "cudaMemcpy", "cudaStreamCreateWithPriority", "cudaEventCreateWithFlags"])
+@pytest.mark.parametrize("nth", [1, 2, 3])
+@pytest.mark.parametrize("change", ["shape", "persistent"])
+def test_batch_with_a_plan_that_failed_launches_nothing(fake, call, nth, change):
+    # a change of plan that the runtime refuses half way: the launches and the graph of the former plan
+    # read tables that are gone or half replaced
+    L = fake.L
+    hs = [solver(fake, **kw) for kw in SIZES]
+    b = batch(fake, hs)
+    if change == "persistent":
+        assert L.lb_batch_set_persistent(b, 1) == LB_OK
+    assert L.lb_batch_step(b, 8) == LB_OK
+    change = (lambda: L.lb_batch_set_shape(b, -1, 1)) if change == "shape" else (lambda: L.lb_batch_set_persistent(b, 0))
+    fake.fail(call, nth)
+    rc = change()
+    fake.fail("")
+    fake.clear()
+    again = L.lb_batch_step(b, 4)
+    if rc != LB_OK:
+        assert again == LB_ESTATE
+        assert not fake.calls("launch") and not fake.calls("cudaGraphLaunch")
+        assert change() == LB_OK and L.lb_batch_step(b, 4) == LB_OK
+    else:
+        assert again == LB_OK
+    L.lb_batch_destroy(b)
+    for h in hs:
+        L.lb_destroy(h)
