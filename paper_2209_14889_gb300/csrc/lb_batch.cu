@@ -358,6 +358,16 @@ size_t plan_bytes(const std::vector<lb_handle*>& hs)
     return sizeof(BatchInst) * hs.size() + sizeof(int) * ints;
 }
 
+int groups_used(const lb_batch* b)
+{
+    int used = 0;
+    for (int g = 0; g < N_GROUPS; ++g) used += b->n_group[g] > 0;
+    return used;
+}
+
+// the node steps of a group run on a stream of their own: beside the group's diffusion or other groups
+bool nodes_fork(const lb_batch* b, int g, int used) { return (b->n_dif[g] > 0 || used > 1) && b->n_nodes[g] > 0; }
+
 // (re)build the per-instance descriptors of every shape group for the current tile shapes; nothing of the
 // batch is in flight.  The former plan and its graph are gone first: when a call fails half way no step
 // runs until a plan is complete.
@@ -434,15 +444,23 @@ int build_plan(lb_batch* b)
         b->d_node_begin[g] = table(nb);
         b->d_dif_begin[g] = table(db);
         b->d_tile_inst[g] = table(ti);
-        if (!b->persistent) {
-            // sub-stepped instances have the longest chain of launches, node steps are short and hold up
-            // the next tiles: theirs go first
-            int least = 0, greatest = 0;
+    }
+    // the streams and events that launch_phases will use and that are not there yet
+    const int used = groups_used(b);
+    for (int g = 0; g < N_GROUPS && !b->persistent; ++g) {
+        if (!b->n_group[g]) continue;
+        // sub-stepped instances have the longest chain of launches, node steps are short and hold up
+        // the next tiles: theirs go first
+        int least = 0, greatest = 0;
+        if (used > 1) {
             BCK(b, cudaDeviceGetStreamPriorityRange(&least, &greatest));
             if (!b->main[g])
                 BCK(b, cudaStreamCreateWithPriority(&b->main[g], cudaStreamNonBlocking, g % LANES == LANE_SUB ? greatest : least));
-            if (!b->side[g]) BCK(b, cudaStreamCreateWithPriority(&b->side[g], cudaStreamNonBlocking, greatest));
             if (!b->ev_main[g]) BCK(b, cudaEventCreateWithFlags(&b->ev_main[g], cudaEventDisableTiming));
+        }
+        if (nodes_fork(b, g, used)) {
+            BCK(b, cudaDeviceGetStreamPriorityRange(&least, &greatest));
+            if (!b->side[g]) BCK(b, cudaStreamCreateWithPriority(&b->side[g], cudaStreamNonBlocking, greatest));
             if (!b->ev_side[g]) BCK(b, cudaEventCreateWithFlags(&b->ev_side[g], cudaEventDisableTiming));
         }
     }
@@ -551,8 +569,7 @@ cudaError_t launch_phases(const lb_batch* b, int nsteps)
     auto after = [&](cudaStream_t st, cudaEvent_t ev, cudaStream_t src) {     // st goes on when src is here
         return ok(cudaEventRecord(ev, src)) && ok(cudaStreamWaitEvent(st, ev, 0));
     };
-    int used = 0;
-    for (int g = 0; g < N_GROUPS; ++g) used += b->n_group[g] > 0;
+    const int used = groups_used(b);
     cudaStream_t st[N_GROUPS];
     for (int g = 0; g < N_GROUPS; ++g) {
         st[g] = used > 1 ? b->main[g] : b->stream;
@@ -562,7 +579,7 @@ cudaError_t launch_phases(const lb_batch* b, int nsteps)
         for (int g = N_GROUPS - 1; g >= 0; --g) {
             if (!b->n_group[g]) continue;
             if (!ok(launch_lattice(b, g, s, st[g]))) return e;
-            const bool fork = (b->n_dif[g] > 0 || used > 1) && b->n_nodes[g] > 0;
+            const bool fork = nodes_fork(b, g, used);
             if (b->n_nodes[g]) {
                 if (fork && !after(b->side[g], b->ev_side[g], st[g])) return e;
                 k_batch_nodes<<<b->n_nodes[g], NODE_THREADS, 0, fork ? b->side[g] : st[g]>>>(batch_args(b, g), s);

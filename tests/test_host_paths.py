@@ -233,3 +233,42 @@ def test_batch_with_a_plan_that_failed_launches_nothing(fake, call, nth, change)
     L.lb_batch_destroy(b)
     for h in hs:
         L.lb_destroy(h)
+
+
+def test_batch_of_one_group_makes_no_streams_it_does_not_use(fake):
+    # creating a batch: one buffer for the plan, streams and events of the groups that fork only
+    hs = [solver(fake, 128, 96, rings=1)]
+    fake.clear()
+    b = batch(fake, hs)
+    assert len(fake.calls("cudaMalloc")) <= 5 and not fake.calls("cudaStreamCreateWithPriority")
+    assert fake.L.lb_batch_step(b, 9) == LB_OK
+    fake.L.lb_batch_destroy(b)
+    fake.L.lb_destroy(hs[0])
+
+
+@pytest.mark.parametrize("shapes", [(0, 0, 0, 0), (4, 1, 0, 3), (2, 2, 2, 2)])
+@pytest.mark.parametrize("members", [(0,), (2,), (0, 1), (0, 1, 2, 3)])
+def test_batch_launches_wait_for_each_other_through_streams_and_events_that_exist(fake, shapes, members):
+    # every launch of the steps is on a stream that was created, every event waited for was recorded before
+    L = fake.L
+    hs = [solver(fake, **SIZES[i]) for i in members]
+    fake.clear()
+    b = batch(fake, hs)
+    for k, i in enumerate(members):
+        if shapes[i] != 4 or i == 0:
+            assert L.lb_batch_set_shape(b, k, shapes[i]) == LB_OK
+    made = {c[1] for c in fake.calls() if c[0].startswith(("cudaStreamCreate", "cudaEventCreate"))}
+    fake.clear()
+    assert L.lb_batch_step(b, 9) == LB_OK
+    recorded = set()
+    for c in fake.calls():
+        if c[0] == "cudaEventRecord":
+            recorded.add(c[1])
+            assert c[1] in made
+        elif c[0] == "cudaStreamWaitEvent":
+            assert c[2] in recorded
+        elif c[0] == "launch":
+            assert c[7] in made
+    L.lb_batch_destroy(b)
+    for h in hs:
+        L.lb_destroy(h)
