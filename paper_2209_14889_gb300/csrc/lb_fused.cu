@@ -67,13 +67,13 @@ __device__ __noinline__ void node_tail_work(const FusedArgs& a, float* sm, unsig
     }
     for (int r = 0; r < nr && meet != 0u; ++r) {
         if (nr <= 32 && !((meet >> r) & 1u)) continue;
-        node::RingRegs rg;      // every tile that meets the ring loads what the last one needs
-        node::load_ring(a.na, r, t, rg);
-        node::load_first_node(a.na, rg);
-        const int4 B = rg.B;
+        const int4 B = ring_box(a.rings[r], t);
         if (nr > 32 &&
             (!meets(bx * TX - 2, G::R2W, B.x, B.z, a.nx) || !meets(by * TY - 2, G::R2H, B.y, B.w, a.ny)))
             continue;
+        node::RingRegs rg;      // every tile that meets the ring loads what the last one needs
+        node::load_ring(a.na, r, t, rg);
+        node::load_first_node(a.na, rg);
         unsigned c = 0u;
         if (tid < 32)
             c = tiles_meeting(gridDim.x, TX, G::R2W, B.x, B.z, a.nx) *

@@ -158,3 +158,24 @@ def test_readout_of_one_field_matches_the_moments_of_all(case, half):
             assert noalloc(s.h, fid, b.data_ptr(), n, 1) == 0
             assert np.array_equal(b.cpu().numpy(), a), k
     s.close()
+
+
+@pytest.mark.parametrize("count", [33, 70])
+def test_more_rings_than_a_warp_has_lanes_match_the_node_kernel_bitwise(count):
+    # beyond 32 rings a tile tests each ring's box by itself, in the gather and in the tail; the same steps with
+    # the node step in a launch of its own
+    lb = _gpu()
+    side = int(np.ceil(np.sqrt(count)))
+    rings = [W.ring(12, 2.0, (20.0 * (k % side) + 9.3, 20.0 * (k // side) + 8.6), pull_force=1e-3, pull_angle=0.1 * k)
+             for k in range(count)]
+    w = W.make(20 * side, 20 * side + 3, rings=rings, seed=12)
+    a, b = lb.Solver.from_workload(w), lb.Solver.from_workload(w)
+    b.set_node_tail(False)
+    a.step(33)
+    b.step(33)
+    ra, rb = _state(a), _state(b)
+    for k in ra[0]:
+        assert np.array_equal(ra[0][k], rb[0][k]), k
+    assert np.array_equal(ra[1], rb[1]) and np.array_equal(ra[2], rb[2])
+    a.close()
+    b.close()
