@@ -339,11 +339,12 @@ int lb_create(const lb_params* pin, void* stream, lb_handle** out)
     h->n_sm = n_sm;
     h->strip_chunk = strip_chunk(p.nx, p.ny, n_sm);
     h->n_partials = fused_ctas(p.nx, p.ny, 0);
-    h->tile_shape = fused_shape(p.nx, p.ny, n_sm, p.model == LB_MODEL_SCALAR);
+    for (int r = 0; r < 2; ++r) h->tile_shape[r] = fused_shape(p.nx, p.ny, n_sm, p.model == LB_MODEL_SCALAR, r == 1);
     const int partial_cap = std::max(std::max(h->n_partials, sweep_ctas(p.nx, p.ny, h->sweep_chunk)),
                                      strip_ctas(p.nx, p.ny, h->strip_chunk));
     h->partial_cap = partial_cap;
-    const int partial_alloc = std::max(partial_cap, fused_ctas(p.nx, p.ny, h->tile_shape));
+    const int partial_alloc = std::max(partial_cap, std::max(fused_ctas(p.nx, p.ny, h->tile_shape[0]),
+                                                             fused_ctas(p.nx, p.ny, h->tile_shape[1])));
     h->series_cap = p.max_samples;
     cudaError_t e;
     if ((e = cudaMalloc(&h->lut, sizeof(float) * lut.size())) != cudaSuccess ||
@@ -568,7 +569,7 @@ int lb_step(lb_handle* h, int64_t n)
             CK(h, launch_strip(fa, h->strip_chunk, h->stream, pdl && !h->after_tail));
             h->n_partials = strip_ctas(h->p.nx, h->p.ny, h->strip_chunk);
         } else {
-            const int shape = pair ? 0 : h->tile_shape;
+            const int shape = pair ? 0 : h->tile_shape[h->n_rings > 0 ? 1 : 0];
             h->n_partials = fused_ctas(h->p.nx, h->p.ny, shape);
             if (tail) {
                 fa.node_tail = 1;

@@ -186,9 +186,18 @@ int fused_ctas(int nx, int ny, int shape)
 // work per cell: 384^2 29.4, 26.4, 24.3, 25.7; 512^2 29.2, 26.7, 26.0, 39.1; 640^2 30.7, 28.6, 34.4,
 // 58.0; 768^2 31.5, 36.8, 47.3, 81.8.  Hence the limits, in tiles per SM: 8x8 up to 1, 16x8 up to 6
 // (scalar 14), 16x16 up to 4 (scalar 12).
-int fused_shape(int nx, int ny, int n_sm, bool scalar)
+// Without a ring a tile is shorter by the gather and the node step, and the halo counts sooner: tensorial
+// 96^2 9.0, 6.9, 5.3, 5.1; 224^2 9.1, 7.8, 7.0, 10.3; 250^2 9.1, 9.7, 10.4, 13.8; 320^2 10.8, 9.5, 12.1,
+// 18.7; 384^2 13.5, 14.3, 16.3, 26.2; scalar 224^2 7.3, 6.3, 5.7, 8.7; 250^2 7.3, 7.8, 8.2, 11.8; 320^2 8.1,
+// 7.5, 9.4, 15.6; 512^2 14.8, 16.9, 20.5, 34.3.  8x8 up to one tile per SM, 16x8 up to 3; beyond, 16x16 up
+// to 3 where 32x16 tiles would take a second wave.
+int fused_shape(int nx, int ny, int n_sm, bool scalar, bool rings)
 {
     if (fused_ctas(nx, ny, 3) <= n_sm) return 3;
+    if (!rings) {
+        if (fused_ctas(nx, ny, 2) <= 3 * n_sm) return 2;
+        return fused_ctas(nx, ny, 0) > n_sm && fused_ctas(nx, ny, 1) <= 3 * n_sm ? 1 : 0;
+    }
     if (fused_ctas(nx, ny, 2) <= (scalar ? 14 : 6) * n_sm) return 2;
     if (fused_ctas(nx, ny, 1) <= (scalar ? 12 : 4) * n_sm) return 1;
     return 0;

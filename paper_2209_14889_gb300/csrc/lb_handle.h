@@ -27,7 +27,7 @@ struct lb_handle {
     double* partials = nullptr;
     int partial_cap = 0;                    // partial sums of the largest launch with 32x16 tiles
     int n_partials = 0;                     // partial sums written by the last lattice launch
-    int tile_shape = 0;                     // tile shape of the one-cell step (fused_shape)
+    int tile_shape[2] = {0, 0};             // tile shapes of the one-cell step without and with rings (fused_shape)
     int kernel = 0;                         // LB_KERNEL_AUTO / TILE / SWEEP / PAIR / STRIP
     int sweep_chunk = 0;
     int strip_chunk = 0;                    // rows per warp of the strip kernel

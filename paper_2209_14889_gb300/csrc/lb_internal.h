@@ -171,8 +171,8 @@ int strip_ctas(int nx, int ny, int chunk);
 cudaError_t launch_strip(const FusedArgs& a, int chunk, cudaStream_t s, bool pdl);
 constexpr int FUSED_SHAPES = 4;
 int fused_ctas(int nx, int ny, int shape);
-// the tile shape of the one-cell step measured fastest for a lattice
-int fused_shape(int nx, int ny, int n_sm, bool scalar);
+// the tile shape of the one-cell step measured fastest for a lattice with or without rings
+int fused_shape(int nx, int ny, int n_sm, bool scalar, bool rings);
 // the tile row holding the cell row y_top (any real value; wrapped): where the launch order of
 // the tile kernel with the node tail starts
 int fused_tile_rot(int nx, int ny, double y_top);

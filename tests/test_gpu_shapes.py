@@ -179,3 +179,21 @@ def test_more_rings_than_a_warp_has_lanes_match_the_node_kernel_bitwise(count):
     assert np.array_equal(ra[1], rb[1]) and np.array_equal(ra[2], rb[2])
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("scalar", [False, True])
+@pytest.mark.parametrize("nx,ny", [(97, 96), (101, 98), (224, 226), (250, 251), (273, 272), (320, 320), (385, 384)])
+def test_tile_shapes_without_rings_match_32x16_tiles_bitwise(nx, ny, scalar):
+    # around the limits of the rule without rings: 8x8, 16x8, 32x16 in one wave, 16x16, 32x16
+    lb = _gpu()
+    w = W.make(nx, ny, seed=11, **(W.scalar_physics() if scalar else {}))
+    a, b = lb.Solver.from_workload(w), lb.Solver.from_workload(w)
+    a.step(33)
+    batch = lb.Batch([b])
+    batch.set_shape(0)
+    batch.step(33)
+    batch.sync()
+    _same(_state(a), _state(b))
+    batch.close()
+    a.close()
+    b.close()

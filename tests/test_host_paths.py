@@ -272,3 +272,19 @@ def test_batch_launches_wait_for_each_other_through_streams_and_events_that_exis
     L.lb_batch_destroy(b)
     for h in hs:
         L.lb_destroy(h)
+
+
+@pytest.mark.parametrize("nx,ny,scalar,rings,grid", [
+    (96, 96, 0, 0, (12, 12)), (224, 224, 0, 0, (14, 28)), (250, 250, 0, 0, (8, 16)), (320, 320, 0, 0, (20, 20)),
+    (384, 384, 0, 0, (12, 24)), (384, 384, 1, 0, (12, 24)), (512, 512, 1, 0, (16, 32)), (64, 1024, 0, 0, (2, 64)),
+    (250, 250, 0, 1, (16, 32)), (384, 384, 0, 1, (24, 24)), (512, 512, 1, 1, (32, 64))])
+def test_tile_shape_by_size_and_rings(fake, nx, ny, scalar, rings, grid):
+    # the grid of the step's launch: 8x8, 16x8, 16x16 or 32x16 cells per CTA; a lattice without rings leaves the
+    # small tiles sooner
+    from paper_2209_14889_gb300 import workloads as W
+    kw = dict(model=1, ericksen=0, K1111=1.875e-3, K1122=0.0, K2222=1.875e-3, K1212=0.9375e-3) if scalar else {}
+    h = solver(fake, nx, ny, rings=rings, **kw)
+    fake.clear()
+    assert fake.L.lb_step(h, 1) == LB_OK
+    assert [(int(c[2]), int(c[3])) for c in fake.launches("k_fused")] == [grid]
+    fake.L.lb_destroy(h)
