@@ -42,7 +42,10 @@ constexpr int CT_IH = CT_H + 2, CT_IW = CT_W + 2;
 constexpr int CT_CO = 64;                       // output channels per CTA
 constexpr int PS = 24;                          // shared row of 16 channels + 8 pad (48 bytes)
 
-__global__ void __launch_bounds__(128) k_conv3x3(const ConvArgs a)
+// MINB CTAs per SM: 4 leave a thread 120 registers, 5 (what the compiler chooses by itself) 96.  conv_mma takes
+// the larger number where it saves a wave of CTAs, and the registers where it does not.
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_conv3x3(const ConvArgs a)
 {
     __shared__ __align__(16) bf16 sx[CT_IH * CT_IW * PS];
     __shared__ __align__(16) bf16 sw[9 * CT_CO * PS];
@@ -984,7 +987,9 @@ cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
 cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s)
 {
     dim3 grid((a.W + CT_W - 1) / CT_W, (a.H + CT_H - 1) / CT_H, a.B * ((a.Co + CT_CO - 1) / CT_CO));
-    k_conv3x3<<<grid, 128, 0, s>>>(a);
+    const long long ctas = (long long)grid.x * grid.y * grid.z, n_sm = sm_count();
+    if ((ctas + 5 * n_sm - 1) / (5 * n_sm) < (ctas + 4 * n_sm - 1) / (4 * n_sm)) k_conv3x3<5><<<grid, 128, 0, s>>>(a);
+    else k_conv3x3<4><<<grid, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 

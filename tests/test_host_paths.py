@@ -288,3 +288,12 @@ def test_tile_shape_by_size_and_rings(fake, nx, ny, scalar, rings, grid):
     assert fake.L.lb_step(h, 1) == LB_OK
     assert [(int(c[2]), int(c[3])) for c in fake.launches("k_fused")] == [grid]
     fake.L.lb_destroy(h)
+
+
+@pytest.mark.parametrize("B,H,W,Ci,Co,minb", [(1, 32, 32, 1024, 256, 4), (2, 64, 64, 512, 512, 4), (1, 1024, 1024, 16, 16, 5),
+                                              (16, 64, 64, 128, 128, 4), (1, 2048, 2048, 16, 32, 5)])
+def test_mma_convolution_takes_registers_or_occupancy_by_its_waves(conv, B, H, W, Ci, Co, minb):
+    conv.L.lb_conv_kernel(0)
+    assert conv.L.lb_conv3x3(X, Ci, 0, WT, None, GX, None, Co, 0, B, H, W, Ci, Co, 1, None) == LB_OK
+    conv.L.lb_conv_kernel(1)
+    assert ["k_conv3x3ILi%dE" % minb in c[1] for c in conv.launches("k_conv3x3")] == [True]
