@@ -44,7 +44,8 @@ constexpr int PS = 24;                          // shared row of 16 channels + 8
 
 // MINB CTAs per SM: 4 leave a thread 120 registers, 5 (what the compiler chooses by itself) 96.  conv_mma takes
 // the larger number where it saves a wave of CTAs, and the registers where it does not.
-template <int MINB>
+// ODD: a BF16 output at an odd pixel stride or address, stored value by value.
+template <int MINB, bool ODD>
 __global__ void __launch_bounds__(128, MINB) k_conv3x3(const ConvArgs a)
 {
     __shared__ __align__(16) bf16 sx[CT_IH * CT_IW * PS];
@@ -133,7 +134,13 @@ __global__ void __launch_bounds__(128, MINB) k_conv3x3(const ConvArgs a)
                     a.yf[o] = v0;
                     a.yf[o + 1] = v1;
                 } else {
-                    *reinterpret_cast<__nv_bfloat162*>(a.y + o) = __floats2bfloat162_rn(v0, v1);
+                    const __nv_bfloat162 r = __floats2bfloat162_rn(v0, v1);
+                    if (!ODD) {
+                        *reinterpret_cast<__nv_bfloat162*>(a.y + o) = r;
+                    } else {
+                        a.y[o] = r.x;
+                        a.y[o + 1] = r.y;
+                    }
                 }
             }
         }
@@ -988,8 +995,9 @@ cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s)
 {
     dim3 grid((a.W + CT_W - 1) / CT_W, (a.H + CT_H - 1) / CT_H, a.B * ((a.Co + CT_CO - 1) / CT_CO));
     const long long ctas = (long long)grid.x * grid.y * grid.z, n_sm = sm_count();
-    if ((ctas + 5 * n_sm - 1) / (5 * n_sm) < (ctas + 4 * n_sm - 1) / (4 * n_sm)) k_conv3x3<5><<<grid, 128, 0, s>>>(a);
-    else k_conv3x3<4><<<grid, 128, 0, s>>>(a);
+    if (!a.yf && (a.ldy % 2 != 0 || ((uintptr_t)(a.y + a.yoff) & 3) != 0)) k_conv3x3<4, true><<<grid, 128, 0, s>>>(a);
+    else if ((ctas + 5 * n_sm - 1) / (5 * n_sm) < (ctas + 4 * n_sm - 1) / (4 * n_sm)) k_conv3x3<5, false><<<grid, 128, 0, s>>>(a);
+    else k_conv3x3<4, false><<<grid, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 

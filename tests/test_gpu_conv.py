@@ -123,3 +123,25 @@ def test_network_output_at_any_address(shift):
     assert torch.equal(got, ref)
     assert (buf[:shift] == 9).all() and (buf[shift + size:] == 9).all()
     n.close()
+
+
+@pytest.mark.parametrize("ldy,shift", [(25, 0), (25, 1), (24, 1), (27, 2), (24, 0)])
+def test_outputs_at_odd_strides_and_addresses(ldy, shift):
+    # both kernels store a BF16 output at any pixel stride and element address, and nothing beside it
+    torch, lb = _gpu()
+    B, H, W, Ci, Co = 2, 9, 21, 16, 24
+    x = torch.randn(B, H, W, Ci, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(9, Co, Ci, device="cuda") / 12).to(torch.bfloat16)
+    ref = _conv64(torch, x.double(), w.double())
+    try:
+        for kernel in (1, 0):
+            lb.conv_kernel(kernel)
+            buf = torch.full((B * H * W * ldy + shift + 8,), 7.0, dtype=torch.bfloat16, device="cuda")
+            lb.conv3x3(x, w, None, out_f32=False, ldy=ldy, y=buf[shift:])
+            torch.cuda.synchronize()
+            y = buf[shift:shift + B * H * W * ldy].reshape(B, H, W, ldy)
+            # as in test_forward_edges_vs_fp64
+            assert torch.all((y[..., :Co].double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5 * ref.abs().max())
+            assert (y[..., Co:] == 7).all() and (buf[:shift] == 7).all() and (buf[-8:] == 7).all()
+    finally:
+        lb.conv_kernel(1)

@@ -297,3 +297,11 @@ def test_mma_convolution_takes_registers_or_occupancy_by_its_waves(conv, B, H, W
     assert conv.L.lb_conv3x3(X, Ci, 0, WT, None, GX, None, Co, 0, B, H, W, Ci, Co, 1, None) == LB_OK
     conv.L.lb_conv_kernel(1)
     assert ["k_conv3x3ILi%dE" % minb in c[1] for c in conv.launches("k_conv3x3")] == [True]
+
+
+@pytest.mark.parametrize("ldy,shift,odd", [(16, 0, False), (16, 2, True), (17, 0, True), (18, 4, False), (17, 2, True)])
+def test_mma_convolution_stores_pairs_at_even_addresses_only(conv, ldy, shift, odd):
+    conv.L.lb_conv_kernel(0)
+    assert conv.L.lb_conv3x3(X, 16, 0, WT, None, GX + shift, None, ldy, 0, 1, 9, 9, 16, 16, 1, None) == LB_OK
+    conv.L.lb_conv_kernel(1)
+    assert [c[1].split("k_conv3x3IL")[1].split("EE")[0].endswith("b1") for c in conv.launches("k_conv3x3")] == [odd]
