@@ -3,6 +3,7 @@
 // output channels as N and K = 9 Ci, weight gradients with the input channels as M, the output channels
 // as N and the pixels as K.
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include "lb_conv.h"
@@ -900,10 +901,15 @@ __global__ void k_conv_pack(const __grid_constant__ PackArgs p)
     }
 }
 
+// SMs of the current device
 int sm_count()
 {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    static std::atomic<int> known[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 152;
+    if (dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 152;
+    if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -947,7 +953,7 @@ cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
     if (a.Ci % 16 != 0 || !a.wp || !conv_tc_fits(a.B, a.H, a.W)) return cudaErrorInvalidValue;
     const cudaError_t e = conv_err_init();
     if (e != cudaSuccess) return e;
-    static const int n_sm = sm_count();
+    const int n_sm = sm_count();
     ConvGeo g = {};
     g.cpk = (a.Co + 15) / 16 * 16;
     const long long flat_n = (long long)a.B * (a.H + 1) * (a.W + 1);
@@ -1005,7 +1011,7 @@ cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s)
 // many as wanted).  Returns S.
 static int wgrad_geo(int B, int H, int W, int Ci, int Co, long long room, WgradGeo& g)
 {
-    static const int n_sm = sm_count();
+    const int n_sm = sm_count();
     const int nb_o = (Co + WG_NMAX - 1) / WG_NMAX, nb_i = (Ci + 127) / 128;
     g.cob = ((Co + nb_o - 1) / nb_o + 15) / 16 * 16;
     g.cib = ((Ci / 8 + nb_i - 1) / nb_i) * 8;

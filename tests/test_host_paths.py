@@ -305,3 +305,13 @@ def test_mma_convolution_stores_pairs_at_even_addresses_only(conv, ldy, shift, o
     assert conv.L.lb_conv3x3(X, 16, 0, WT, None, GX + shift, None, ldy, 0, 1, 9, 9, 16, 16, 1, None) == LB_OK
     conv.L.lb_conv_kernel(1)
     assert [c[1].split("k_conv3x3IL")[1].split("EE")[0].endswith("b1") for c in conv.launches("k_conv3x3")] == [odd]
+
+
+def test_work_is_split_over_the_sms_of_the_current_device(conv):
+    # device 0 of the stand-in has 152 SMs, device 1 has 76
+    def grid(dev):
+        conv.L.fake_device(dev)
+        conv.clear()
+        assert conv.L.lb_conv3x3_wgrad(X, GZ, GW, GB, 4, 256, 256, 32, 32, None) == LB_OK
+        return conv.launches("k_wgrad_tc")[0][2]
+    assert [grid(d) for d in (0, 1, 0)] == ["152", "76", "152"]
