@@ -948,31 +948,51 @@ cudaError_t conv_pack(const PackArgs& p, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// How a call's positions and channels are split over CTAs.
+struct ConvSplit {
+    bool flat;
+    int mt, cop, n_cot;      // MMA tiles and channels per CTA, CTAs of the channels
+    long long tiles;         // CTAs of the positions
+    long long ctas() const { return tiles * n_cot; }
+};
+
+static ConvSplit conv_split(int B, int H, int W, int Co)
+{
+    const int n_sm = sm_count(), cpk = (Co + 15) / 16 * 16;
+    const long long flat_n = (long long)B * (H + 1) * (W + 1);
+    ConvSplit c;
+    c.flat = W <= 128 && flat_n < (1LL << 30);
+    auto tiles = [&](int mt) -> long long {
+        if (c.flat) return (flat_n + 128 * mt - 1) / (128 * mt);
+        return (long long)((W + 29) / 30) * ((H + 4 * mt - 1) / (4 * mt)) * B;
+    };
+    // channels per CTA: all up to 128, in equal parts beyond; MMA tiles per CTA: as many as leave one and
+    // a half CTAs per SM, fit half the tensor memory and (tiles form, 4 rows each) hold rows of the image
+    // (1 x 100000, 16 -> 16 channels: 79 us with four of them, 60 with one); then, where the CTAs would leave
+    // SMs empty, the channels are split further (each part stages the input again)
+    c.n_cot = (cpk + 127) / 128;
+    c.cop = ((cpk + c.n_cot - 1) / c.n_cot + 15) / 16 * 16;
+    c.mt = 4;
+    while (c.mt > 1 && (c.mt * c.cop > 256 || 2 * tiles(c.mt) * c.n_cot < 3 * n_sm || (!c.flat && H <= 2 * c.mt))) c.mt /= 2;
+    while (c.cop > 16 && 4 * tiles(c.mt) * ((cpk + c.cop - 1) / c.cop) < 3 * n_sm) c.cop = (c.cop / 2 + 15) / 16 * 16;
+    c.n_cot = (cpk + c.cop - 1) / c.cop;
+    c.tiles = tiles(c.mt);
+    return c;
+}
+
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
 {
     if (a.Ci % 16 != 0 || !a.wp || !conv_tc_fits(a.B, a.H, a.W)) return cudaErrorInvalidValue;
     const cudaError_t e = conv_err_init();
     if (e != cudaSuccess) return e;
-    const int n_sm = sm_count();
+    const ConvSplit c = conv_split(a.B, a.H, a.W, a.Co);
+    const int mt = c.mt, n_cot = c.n_cot;
     ConvGeo g = {};
     g.cpk = (a.Co + 15) / 16 * 16;
-    const long long flat_n = (long long)a.B * (a.H + 1) * (a.W + 1);
-    g.flat = a.W <= 128 && flat_n < (1LL << 30) ? 1 : 0;
+    g.cop = c.cop;
+    g.flat = c.flat ? 1 : 0;
     g.pitch = g.flat ? a.W + 1 : 32;
     g.tx = (a.W + 29) / 30;
-    auto tiles = [&](int mt) -> long long {
-        if (g.flat) return (flat_n + 128 * mt - 1) / (128 * mt);
-        return (long long)g.tx * ((a.H + 4 * mt - 1) / (4 * mt)) * a.B;
-    };
-    // channels per CTA: all up to 128, in equal parts beyond; MMA tiles per CTA: as many as leave one and
-    // a half CTAs per SM and fit half the tensor memory; then, where the CTAs would leave SMs empty, the
-    // channels are split further (each part stages the input again)
-    int n_cot = (g.cpk + 127) / 128;
-    g.cop = ((g.cpk + n_cot - 1) / n_cot + 15) / 16 * 16;
-    int mt = 4;
-    while (mt > 1 && (mt * g.cop > 256 || 2 * tiles(mt) * n_cot < 3 * n_sm)) mt /= 2;
-    while (g.cop > 16 && 4 * tiles(mt) * ((g.cpk + g.cop - 1) / g.cop) < 3 * n_sm) g.cop = (g.cop / 2 + 15) / 16 * 16;
-    n_cot = (g.cpk + g.cop - 1) / g.cop;
     g.ty = (a.H + 4 * mt - 1) / (4 * mt);
     // positions: a multiple of 4 that is not one of 8, which spreads the k-halves over the banks
     g.npix = g.flat ? 128 * mt + 2 * g.pitch + 2 : (4 * mt + 2) * 32 + 8;
@@ -984,11 +1004,11 @@ cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
     // stages: all chunks where one CTA has an SM to itself, else what lets two share it; the widest
     // stage of which two fit
     const int cbytes = g.npix * 32 + 288 * g.cop, nchunk = a.Ci / 16;
-    const int room = (tiles(mt) * n_cot <= n_sm ? 220 : 110) * 1024 - TC_HEAD - g.npix * 4;
+    const int room = (c.ctas() <= sm_count() ? 220 : 110) * 1024 - TC_HEAD - g.npix * 4;
     for (g.cw = 4, g.lgh = 3; g.cw > 1; g.cw /= 2, --g.lgh)
         if (nchunk % g.cw == 0 && std::min(2, nchunk / g.cw) * g.cw * cbytes <= room) break;
     g.slots = std::max(1, std::min(std::min(nchunk / g.cw, TC_SLOTS), room / (g.cw * cbytes)));
-    const long long m_tiles = tiles(mt);
+    const long long m_tiles = c.tiles;
     if (m_tiles > 0x7fffffffLL || n_cot > 65535) return cudaErrorInvalidConfiguration;
     switch (mt) {
     case 4: return launch_tc<4>(a, g, (unsigned)m_tiles, n_cot, s, pdl);

@@ -315,3 +315,9 @@ def test_work_is_split_over_the_sms_of_the_current_device(conv):
         assert conv.L.lb_conv3x3_wgrad(X, GZ, GW, GB, 4, 256, 256, 32, 32, None) == LB_OK
         return conv.launches("k_wgrad_tc")[0][2]
     assert [grid(d) for d in (0, 1, 0)] == ["152", "76", "152"]
+
+
+@pytest.mark.parametrize("H,W,mt", [(1, 100000, 1), (4, 100000, 1), (8, 100000, 2), (9, 100000, 4), (1024, 1024, 4)])
+def test_tiles_of_a_convolution_are_no_taller_than_the_image(conv, H, W, mt):
+    assert conv.L.lb_conv3x3(X, 16, 0, WT, None, GX, None, 16, 0, 1, H, W, 16, 16, 1, None) == LB_OK
+    assert ["k_conv_tcILi%dE" % mt in c[1] for c in conv.launches("k_conv_tc")] == [True]
