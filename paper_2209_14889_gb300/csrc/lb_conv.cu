@@ -342,7 +342,8 @@ __device__ __forceinline__ int in_pixel(const ConvArgs& a, const ConvGeo& g, int
     return (b * a.H + y) * a.W + x;
 }
 
-template <int MT>
+// DIRECT: the weights come as they lie in memory (a.w), by the copying warps
+template <int MT, bool DIRECT>
 __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ ConvArgs a, const __grid_constant__ ConvGeo g,
                                                         int* err)
 {
@@ -386,6 +387,19 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
             const int s = k % slots;
             if (k >= slots) ok = mbar_wait(&S.empty[s], (unsigned)((k / slots - 1) & 1));
             if (!ok) break;
+            if (DIRECT) {
+                // the weights as they lie in memory: a row (tap, output channel) of the stage's channels is
+                // one run of 16-byte units
+                const int units = min(g.cop, a.Co - co0) << g.lgh;
+                for (int v = tid; v < units; v += TC_COPY) {
+                    const int hw = v & ((1 << g.lgh) - 1), co = v >> g.lgh;
+                    const bf16* src = a.w + (long long)(co0 + co) * a.Ci + 16 * g.cw * k + 8 * hw;
+                    const unsigned d = stage0 + (unsigned)(s * sbytes + xbytes + (((hw >> 1) * 18 + (hw & 1)) * g.cop + co) * 16);
+#pragma unroll
+                    for (int t = 0; t < 9; ++t)
+                        cp_async16(d + (unsigned)(t * 2 * g.cop * 16), src + (long long)t * a.Co * a.Ci, 16);
+                }
+            }
             const unsigned dst = stage0 + (unsigned)(s * sbytes + h * g.npix * 16);
             const bf16* base = a.x + a.xoff + 16 * g.cw * k + 8 * h;
 #pragma unroll 4
@@ -400,7 +414,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
         // ---- weights: 18 bulk copies (tap, k-half) of the CTA's channels per chunk
         const unsigned nb = (unsigned)min(g.cop, g.cpk - co0) * 16u;
         int issued = 0;
-        for (int k = 0; k < nstage && ok; ++k) {
+        for (int k = 0; !DIRECT && k < nstage && ok; ++k) {
             const int s = k % slots;
             if (k >= slots) ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], (unsigned)((k / slots - 1) & 1)));
             if (!ok) break;
@@ -422,7 +436,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
         for (int k = 0; k < nstage && ok; ++k) {
             const int s = k % slots;
             const unsigned par = (unsigned)((k / slots) & 1);
-            ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], par) && mbar_wait(&S.wfull[s], par));
+            ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[s], par) && (DIRECT || mbar_wait(&S.wfull[s], par)));
             if (!ok) break;
             // the input was written through the generic proxy, the tensor core reads through the
             // asynchronous one
@@ -923,19 +937,19 @@ cudaError_t conv_err_init()
     return e;
 }
 
-template <int MT>
+template <int MT, bool DIRECT>
 cudaError_t launch_tc(const ConvArgs& a, const ConvGeo& g, unsigned m_tiles, int n_cot, cudaStream_t s, bool pdl)
 {
     static unsigned long long attr = 0;      // per device
     if (!done_on_device(attr)) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_tc<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(k_conv_tc<MT, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) {
             attr = 0;
             return e;
         }
     }
     const size_t smem = TC_HEAD + (size_t)g.npix * 4 + (size_t)g.slots * g.cw * (g.npix * 32 + 288 * g.cop);
-    return launch_pdl(k_conv_tc<MT>, dim3(m_tiles, n_cot), TC_THREADS, smem, s, pdl, a, g, g_conv_err);
+    return launch_pdl(k_conv_tc<MT, DIRECT>, dim3(m_tiles, n_cot), TC_THREADS, smem, s, pdl, a, g, g_conv_err);
 }
 
 }  // namespace
@@ -980,9 +994,16 @@ static ConvSplit conv_split(int B, int H, int W, int Co)
     return c;
 }
 
+bool conv_direct(int B, int H, int W, int Ci, int Co)
+{
+    const ConvSplit c = conv_split(B, H, W, Co);
+    const int n_sm = sm_count();
+    return 2 * c.ctas() <= 3 * n_sm || (Ci * (long long)c.cop <= 1024 && (c.ctas() <= 3 * n_sm || c.mt == 1));
+}
+
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
 {
-    if (a.Ci % 16 != 0 || !a.wp || !conv_tc_fits(a.B, a.H, a.W)) return cudaErrorInvalidValue;
+    if (a.Ci % 16 != 0 || (!a.wp && !a.w) || !conv_tc_fits(a.B, a.H, a.W)) return cudaErrorInvalidValue;
     const cudaError_t e = conv_err_init();
     if (e != cudaSuccess) return e;
     const ConvSplit c = conv_split(a.B, a.H, a.W, a.Co);
@@ -1008,12 +1029,15 @@ cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl)
     for (g.cw = 4, g.lgh = 3; g.cw > 1; g.cw /= 2, --g.lgh)
         if (nchunk % g.cw == 0 && std::min(2, nchunk / g.cw) * g.cw * cbytes <= room) break;
     g.slots = std::max(1, std::min(std::min(nchunk / g.cw, TC_SLOTS), room / (g.cw * cbytes)));
-    const long long m_tiles = c.tiles;
-    if (m_tiles > 0x7fffffffLL || n_cot > 65535) return cudaErrorInvalidConfiguration;
-    switch (mt) {
-    case 4: return launch_tc<4>(a, g, (unsigned)m_tiles, n_cot, s, pdl);
-    case 2: return launch_tc<2>(a, g, (unsigned)m_tiles, n_cot, s, pdl);
-    default: return launch_tc<1>(a, g, (unsigned)m_tiles, n_cot, s, pdl);
+    if (c.tiles > 0x7fffffffLL || n_cot > 65535) return cudaErrorInvalidConfiguration;
+    const unsigned m = (unsigned)c.tiles;
+    switch (2 * mt + (a.wp ? 0 : 1)) {
+    case 9: return launch_tc<4, true>(a, g, m, n_cot, s, pdl);
+    case 8: return launch_tc<4, false>(a, g, m, n_cot, s, pdl);
+    case 5: return launch_tc<2, true>(a, g, m, n_cot, s, pdl);
+    case 4: return launch_tc<2, false>(a, g, m, n_cot, s, pdl);
+    case 3: return launch_tc<1, true>(a, g, m, n_cot, s, pdl);
+    default: return launch_tc<1, false>(a, g, m, n_cot, s, pdl);
     }
 }
 

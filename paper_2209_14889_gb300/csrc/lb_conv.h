@@ -15,8 +15,8 @@ struct ConvArgs {
     const bf16* x;          // input, pixel stride ldx, channels at xoff .. xoff + Ci
     long long ldx;
     int xoff;
-    const bf16* w;          // [9][Co][Ci] (read by the mma.sync kernel)
-    const bf16* wp;         // the same weights packed (conv_pack_elems), read by the tcgen05 kernel
+    const bf16* w;          // [9][Co][Ci] (read by the mma.sync kernel, and by the tcgen05 one without wp)
+    const bf16* wp;         // the same weights packed (conv_pack_elems), read by the tcgen05 kernel, or null
     const float* bias;      // [Co] or nullptr
     bf16* y;                // BF16 output (pixel stride ldy, channel offset yoff), or
     float* yf;              // FP32 output
@@ -60,7 +60,15 @@ inline bool conv_tc_fits(int B, int H, int W) { return (long long)B * H * W < (1
 
 // The tcgen05 convolution of a (Ci % 16 == 0, conv_tc_fits).  pdl: the launch may start while the kernel
 // before it in the stream finishes (that kernel must not be the one that wrote the weights).
+// The weights are read packed (a.wp) or, where a.wp is null, as they lie in memory (a.w).
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl);
+// Whether a single call does better with the weights as they lie in memory: packing them costs a launch and
+// its scratch (7 us of a call, and 30 at 1024 -> 1024 channels), but bulk copies bring a CTA's packed weights
+// in sooner than 16-byte copies of rows that each CTA makes anew.  Few CTAs, or few weights (us, packed and
+// not: 8^2, 16 -> 16 channels 34, 26; 16^2, 1024 -> 1024 106, 72; 32^2, 1024 -> 256 78, 51; 75 x 100, 64 -> 96
+// 36, 32; 9 x 3000, 32 -> 32 34, 32; beyond, 8 x 128^2, 32 -> 64 42, 44; 256^2, 128 -> 128 51, 57; 2 x 64^2,
+// 512 -> 512 81, 123).
+bool conv_direct(int B, int H, int W, int Ci, int Co);
 // The mma.sync convolution (ym, up and yf2 are not supported).
 cudaError_t conv_mma(const ConvArgs& a, cudaStream_t s);
 

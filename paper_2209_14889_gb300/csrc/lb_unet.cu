@@ -764,6 +764,7 @@ int lb_conv3x3(const void* x, int64_t ldx, int32_t xoff, const void* w, const fl
     a.y = static_cast<bf16*>(y); a.yf = yf; a.ldy = ldy; a.yoff = yoff;
     a.B = B; a.H = H; a.W = W; a.Ci = Ci; a.Co = Co; a.act = act ? 1 : 0;
     if (g_conv_kernel == 0 || !conv_tc_fits(B, H, W)) return conv_code(conv_mma(a, s));
+    if (conv_direct(B, H, W, Ci, Co)) return conv_code(conv_tc(a, s, false));
     void* wp = nullptr;
     cudaError_t e = scratch(&wp, sizeof(bf16) * (size_t)conv_pack_elems(Ci, Co), s);
     if (e != cudaSuccess) return conv_code(e);

@@ -321,3 +321,18 @@ def test_work_is_split_over_the_sms_of_the_current_device(conv):
 def test_tiles_of_a_convolution_are_no_taller_than_the_image(conv, H, W, mt):
     assert conv.L.lb_conv3x3(X, 16, 0, WT, None, GX, None, 16, 0, 1, H, W, 16, 16, 1, None) == LB_OK
     assert ["k_conv_tcILi%dE" % mt in c[1] for c in conv.launches("k_conv_tc")] == [True]
+
+
+@pytest.mark.parametrize("B,H,W,Ci,Co,direct", [(1, 8, 8, 16, 16, True), (1, 75, 100, 64, 96, True), (1, 32, 32, 1024, 256, True),
+                                                (1, 9, 3000, 32, 32, True), (2, 64, 64, 512, 512, False),
+                                                (1, 1024, 1024, 16, 16, False), (4, 256, 256, 32, 32, False)])
+def test_small_forward_layer_is_one_launch_without_scratch(conv, B, H, W, Ci, Co, direct):
+    live = conv.L.fake_live()
+    args = arguments(conv, "k_conv_tc", ConvArgs)
+    conv.L.lb_conv3x3(X, 16, 0, WT, None, GX, None, 16, 0, 1, 8, 8, 16, 16, 1, None)       # the error flag's allocation
+    conv.clear()
+    del args[:]
+    assert conv.L.lb_conv3x3(X, Ci, 0, WT, None, GX, None, Co, 0, B, H, W, Ci, Co, 1, None) == LB_OK
+    assert args[0].w == WT and bool(args[0].wp) == (not direct)
+    assert len(conv.calls("launch")) == (1 if direct else 2)
+    assert [c for c in conv.calls() if "alloc" in c[0].lower()] == [] if direct else conv.L.fake_live() <= live + 1
