@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
         // ---- weights: 18 bulk copies (tap, k-half) of the CTA's channels per chunk
         const unsigned nb = (unsigned)min(g.cop, g.cpk - co0) * 16u;
         int issued = 0;
+        if (!DIRECT && a.w_late) pdl_wait();
         for (int k = 0; !DIRECT && k < nstage && ok; ++k) {
             const int s = k % slots;
             if (k >= slots) ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], (unsigned)((k / slots - 1) & 1)));
@@ -890,6 +891,7 @@ __global__ void __launch_bounds__(256) k_sum_parts(const float4* part, int S, in
 // its data-gradient form (chunk over o, tap, half, c)
 __global__ void k_conv_pack(const __grid_constant__ PackArgs p)
 {
+    pdl_trigger();               // a convolution of w_late reads nothing of this before it has waited
     const PackLayer L = p.L[blockIdx.y];
     const int cof = (L.Co + 15) / 16 * 16, cid = (L.Ci + 15) / 16 * 16;
     const int nf = L.fwd ? L.Ci / 16 * 18 * cof : 0, nd = L.dgrad ? L.Co / 16 * 18 * cid : 0;
@@ -958,7 +960,15 @@ int* conv_err_flag() { return g_conv_err; }
 
 cudaError_t conv_pack(const PackArgs& p, cudaStream_t s)
 {
-    k_conv_pack<<<dim3(48, p.n), 256, 0, s>>>(p);
+    // a unit per thread for a single layer; the network's layers together fill the GPU with 48 CTAs each
+    long long blocks = 48;
+    if (p.n == 1) {
+        const PackLayer& L = p.L[0];
+        const long long u = (L.fwd ? conv_pack_elems(L.Ci, L.Co) / 8 : 0) + (L.dgrad ? conv_pack_elems(L.Co, L.Ci) / 8 : 0) +
+                            (L.wt ? 9LL * L.Ci * L.Co : 0);
+        blocks = std::max(1LL, std::min((u + 255) / 256, 8LL * sm_count()));
+    }
+    k_conv_pack<<<dim3((unsigned)blocks, p.n), 256, 0, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -34,6 +34,7 @@ struct ConvArgs {
     bf16* up;
     long long ldu;
     float* yf2;             // optional, with an FP32 output: a second dense copy (pixel stride ldy)
+    int w_late;             // 1: the kernel before this one in the stream writes wp (conv_pack)
 };
 
 // BF16 elements of the packed weights of a layer: [Ci / 16][9][2][Co rounded up to 16][8]
@@ -59,7 +60,7 @@ cudaError_t conv_pack(const PackArgs& p, cudaStream_t s);
 inline bool conv_tc_fits(int B, int H, int W) { return (long long)B * H * W < (1LL << 31); }
 
 // The tcgen05 convolution of a (Ci % 16 == 0, conv_tc_fits).  pdl: the launch may start while the kernel
-// before it in the stream finishes (that kernel must not be the one that wrote the weights).
+// before it in the stream finishes (with w_late that kernel may be the one that writes the weights).
 // The weights are read packed (a.wp) or, where a.wp is null, as they lie in memory (a.w).
 cudaError_t conv_tc(const ConvArgs& a, cudaStream_t s, bool pdl);
 // Whether a single call does better with the weights as they lie in memory: packing them costs a launch and

@@ -740,8 +740,8 @@ cudaError_t scratch(void** p, size_t bytes, cudaStream_t s)
 // anywhere and a fault of its kernels is its own return code.
 cudaError_t finish(void* p, cudaError_t e, cudaStream_t s)
 {
-    const cudaError_t f = cudaFreeAsync(p, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    const cudaError_t f = cudaFreeAsync(p, s);
     return e != cudaSuccess ? e : f;
 }
 
@@ -772,8 +772,9 @@ int lb_conv3x3(const void* x, int64_t ldx, int32_t xoff, const void* w, const fl
     p.n = 1;
     p.L[0] = PackLayer{a.w, Ci, Co, static_cast<bf16*>(wp), nullptr, nullptr};
     a.wp = static_cast<bf16*>(wp);
+    a.w_late = 1;
     e = conv_pack(p, s);
-    if (e == cudaSuccess) e = conv_tc(a, s, false);
+    if (e == cudaSuccess) e = conv_tc(a, s, true);
     const cudaError_t f = cudaFreeAsync(wp, s);
     return conv_code(e != cudaSuccess ? e : f);
 }
@@ -794,10 +795,11 @@ int lb_conv3x3_dgrad(const void* gz, const void* w, void* gx, int32_t B, int32_t
     ConvArgs a = {};
     a.x = static_cast<const bf16*>(gz); a.ldx = Co;
     (tc ? a.wp : a.w) = static_cast<bf16*>(wt);
+    a.w_late = 1;
     a.y = static_cast<bf16*>(gx); a.ldy = Ci;
     a.B = B; a.H = H; a.W = W; a.Ci = Co; a.Co = Ci;
     e = conv_pack(p, s);
-    if (e == cudaSuccess) e = tc ? conv_tc(a, s, false) : conv_mma(a, s);
+    if (e == cudaSuccess) e = tc ? conv_tc(a, s, true) : conv_mma(a, s);
     return conv_code(finish(wt, e, s));
 }
 

@@ -29,7 +29,7 @@ def fake(built):
 class ConvArgs(ctypes.Structure):            # csrc/lb_conv.h
     _fields_ = [("x", P), ("ldx", I64), ("xoff", I32), ("w", P), ("wp", P), ("bias", P), ("y", P), ("yf", P),
                 ("ldy", I64), ("yoff", I32), ("B", I32), ("H", I32), ("W", I32), ("Ci", I32), ("Co", I32), ("act", I32),
-                ("ym", P), ("ldm", I64), ("moff", I32), ("up", P), ("ldu", I64), ("yf2", P)]
+                ("ym", P), ("ldm", I64), ("moff", I32), ("up", P), ("ldu", I64), ("yf2", P), ("w_late", I32)]
 
 
 class PackLayer(ctypes.Structure):
@@ -336,3 +336,12 @@ def test_small_forward_layer_is_one_launch_without_scratch(conv, B, H, W, Ci, Co
     assert args[0].w == WT and bool(args[0].wp) == (not direct)
     assert len(conv.calls("launch")) == (1 if direct else 2)
     assert [c for c in conv.calls() if "alloc" in c[0].lower()] == [] if direct else conv.L.fake_live() <= live + 1
+
+
+@pytest.mark.parametrize("Ci,Co,blocks", [(16, 16, 2), (64, 96, 27), (1024, 1024, 1216)])
+def test_convolution_starts_beside_the_packing_and_waits_for_it(conv, Ci, Co, blocks):
+    # a unit of 16 bytes per thread; the convolution's launch overlaps the packing (w_late: its weights wait)
+    args = arguments(conv, "k_conv_tc", ConvArgs)
+    assert conv.L.lb_conv3x3_dgrad(GZ, WT, GX, 1, 16, 16, Ci, Co, None) == LB_OK
+    assert args[0].w_late == 1 and [c[-1] for c in conv.launches("k_conv_tc")] == ["1"]
+    assert [int(c[2]) for c in conv.launches("k_conv_pack")] == [blocks]
