@@ -457,6 +457,9 @@ int lb_conv3x3_dgrad(const void* gz, const void* w, void* gx, int32_t B, int32_t
                      void* stream);
 int lb_conv3x3_wgrad(const void* x, const void* gz, float* gw, float* gb, int32_t B, int32_t H, int32_t W, int32_t Ci,
                      int32_t Co, void* stream);
+/* The single-layer calls keep at most 64 MB of scratch per device between them; this gives back what no call
+ * is using (any thread, any time; later calls take it anew). */
+int lb_conv_release(void);
 
 /*
  * The learned stepper (no counterpart in the paper: a surrogate of 16 steps of its method, used

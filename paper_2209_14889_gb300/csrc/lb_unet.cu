@@ -709,29 +709,31 @@ namespace {
 
 // Stream-ordered scratch of the single-layer calls, from a pool of its own per device that keeps at
 // most 64 MB between calls (the default pool would hand its memory back, and map it again, at every
-// synchronisation).
+// synchronisation) until lb_conv_release.
+constexpr int MAX_DEVICES = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[MAX_DEVICES] = {};
+
 cudaError_t scratch(void** p, size_t bytes, cudaStream_t s)
 {
-    static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaMallocAsync(p, bytes, s);
+    if (dev < 0 || dev >= MAX_DEVICES) return cudaMallocAsync(p, bytes, s);
     cudaMemPool_t pool;
     {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!pools[dev]) {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (!g_pools[dev]) {
             cudaMemPoolProps props = {};
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = dev;
-            e = cudaMemPoolCreate(&pools[dev], &props);
+            e = cudaMemPoolCreate(&g_pools[dev], &props);
             if (e != cudaSuccess) return e;
             uint64_t keep = 64ull << 20;
-            cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+            cudaMemPoolSetAttribute(g_pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
         }
-        pool = pools[dev];
+        pool = g_pools[dev];
     }
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
@@ -815,6 +817,18 @@ int lb_conv3x3_wgrad(const void* x, const void* gz, float* gw, float* gb, int32_
     e = conv_wgrad(s, static_cast<const bf16*>(x), Ci, 0, static_cast<const bf16*>(gz), B, H, W, Ci, Co,
                    static_cast<float*>(part), room, gw, gb, false);
     return conv_code(finish(part, e, s));
+}
+
+int lb_conv_release(void)
+{
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    cudaError_t e = cudaSuccess;
+    for (cudaMemPool_t p : g_pools)
+        if (p) {
+            const cudaError_t f = cudaMemPoolTrimTo(p, 0);
+            if (e == cudaSuccess) e = f;
+        }
+    return conv_code(e);
 }
 
 }  // extern "C"

@@ -152,6 +152,7 @@ def lib():
             "lb_learned_destroy": (None, [_L]),
             "lb_conv_kernel": (ctypes.c_int, [i32]),
             "lb_conv_status": (ctypes.c_int, []),
+            "lb_conv_release": (ctypes.c_int, []),
             "lb_conv3x3": (ctypes.c_int, [vp, i64, i32, vp, vp, vp, vp, i64, i32, i32, i32, i32, i32, i32,
                                           i32, vp]),
             "lb_conv3x3_dgrad": (ctypes.c_int, [vp, vp, vp, i32, i32, i32, i32, i32, vp]),
@@ -634,3 +635,8 @@ def conv_kernel(kernel: int):
 
 def conv_status():
     _check(None, lib().lb_conv_status())
+
+
+def conv_release():
+    """Give back the scratch memory that the single-layer calls keep between them."""
+    _check(None, lib().lb_conv_release())

@@ -222,8 +222,11 @@ cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStrea
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return release("cudaFreeAsync", p); }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) { return make("cudaMemPoolCreate", p); }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
-cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t keep) { note("cudaMemPoolTrimTo %p %zu", (void*)p, keep); return cudaSuccess; }
-cudaError_t cudaMemPoolDestroy(cudaMemPool_t p) { note("cudaMemPoolDestroy %p", (void*)p); return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t keep)
+{
+    note("cudaMemPoolTrimTo %p %zu", (void*)p, keep);
+    return err("cudaMemPoolTrimTo");
+}
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind k) { return copy("cudaMemcpy", d, s, n, k, nullptr); }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t st)
 {

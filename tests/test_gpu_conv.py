@@ -145,3 +145,20 @@ def test_outputs_at_odd_strides_and_addresses(ldy, shift):
             assert (y[..., Co:] == 7).all() and (buf[:shift] == 7).all() and (buf[-8:] == 7).all()
     finally:
         lb.conv_kernel(1)
+
+
+def test_scratch_is_given_back():
+    torch, lb = _gpu()
+    x = torch.randn(1, 128, 128, 128, device="cuda").to(torch.bfloat16)
+    gz = torch.randn(1, 128, 128, 96, device="cuda").to(torch.bfloat16)
+    gw, gb = lb.conv3x3_wgrad(x, gz)                # partial sums of 9 x 128 x 96 for some tens of CTAs
+    torch.cuda.synchronize()
+    lb.conv_release()
+    free0 = torch.cuda.mem_get_info()[0]
+    again = lb.conv3x3_wgrad(x, gz)
+    torch.cuda.synchronize()
+    kept = free0 - torch.cuda.mem_get_info()[0]
+    lb.conv_release()
+    assert 0 < kept <= 64 << 20
+    assert torch.cuda.mem_get_info()[0] >= free0
+    assert torch.equal(again[0], gw) and torch.equal(again[1], gb)

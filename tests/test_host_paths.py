@@ -345,3 +345,17 @@ def test_convolution_starts_beside_the_packing_and_waits_for_it(conv, Ci, Co, bl
     assert conv.L.lb_conv3x3_dgrad(GZ, WT, GX, 1, 16, 16, Ci, Co, None) == LB_OK
     assert args[0].w_late == 1 and [c[-1] for c in conv.launches("k_conv_tc")] == ["1"]
     assert [int(c[2]) for c in conv.launches("k_conv_pack")] == [blocks]
+
+
+def test_scratch_of_the_single_layer_calls_is_given_back_on_request(conv):
+    pools = set()
+    for dev in (0, 1):
+        conv.L.fake_device(dev)
+        assert conv.L.lb_conv3x3_wgrad(X, GZ, GW, GB, 1, 9, 40, 32, 16, None) == LB_OK
+        pools |= {c[1] for c in conv.calls("cudaMemPoolCreate")}
+    conv.clear()
+    assert conv.L.lb_conv_release() == LB_OK
+    trims = conv.calls("cudaMemPoolTrimTo")
+    assert len(trims) == 2 and all(c[2] == "0" for c in trims) and pools <= {c[1] for c in trims}
+    conv.fail("cudaMemPoolTrimTo", 1, 700)
+    assert conv.L.lb_conv_release() == LB_ECUDA
