@@ -652,7 +652,7 @@ int lb_readout(lb_handle* h, int32_t field, void* dst, size_t bytes, int32_t dst
     } else if (field <= LB_FIELD_UY) {
         FusedArgs fa = fused_args(h);
         fa.moments_out = out;
-        fa.moments_only = 1 + field - LB_FIELD_DRHO;
+        fa.moments_only = 1 + field - LB_FIELD_UX;
         CK(h, launch_fused(fa, MODE_MOMENTS, h->stream));
     } else {
         CK(h, plane_to_f32(h, h->cur, field <= LB_FIELD_PY ? PL_SXX + field - LB_FIELD_SXX : field - LB_FIELD_POP0, out));

@@ -5,11 +5,11 @@
 // instances' lattice tiles (k_batch_tiles, the tile kernel's occupancy of three CTAs per SM),
 // then their diffusion passes beside their rings' node steps -- in stream order, so no kernel waits
 // on another inside a launch.  A group holds instances of one tile shape, those with diffusion
-// sub-steps apart from those without, which make two groups: instances are independent, so every group has a stream of its
-// own and its short launches run beside the lattice launches of the others (20 lattices of 128^2 to
-// 512^2, 30 steps: 6109 -> 5500 us).  Alternatively (lb_batch_set_persistent) one persistent cooperative
-// kernel per group runs the whole chunk, each step having three phases separated by a grid
-// barrier:
+// sub-steps apart from those without, which make two groups: instances are independent, so where there
+// are several groups each has a stream of its own and its short launches run beside the lattice launches
+// of the others (20 lattices of 128^2 to 512^2, 30 steps: 6109 -> 5500 us).
+// Alternatively (lb_batch_set_persistent) one persistent cooperative kernel per group runs the whole
+// chunk, each step having three phases separated by a grid barrier:
 //   lattice  the fused step of every tile of every instance (tile shape per instance, chosen by
 //            the autotuner among 32x16, 32x8, 64x8, 16x16), the tile code of lb_tile.cuh;
 //   sigma    diffusion passes of the instances whose D_p exceeds the Heun bound;
@@ -200,7 +200,8 @@ __global__ void __launch_bounds__(BT, 3) k_batch_tiles(const BatchArgs B, int s)
     extern __shared__ __align__(16) float sm[];
     const int par = (*B.cur + s) & 1;
     const int item = blockIdx.x;
-    // one load where a search among the prefix sums is log2 n dependent ones at the start of every CTA (a sweep of 20 lattices, 30 steps: 5482 -> 5344 us)
+    // one load where a search among the prefix sums is log2 n dependent ones at the start of every CTA
+    // (a sweep of 20 lattices, 30 steps: 5482 -> 5344 us)
     const int i = __ldg(B.tile_inst + item);
     const BatchInst& I = B.inst[i];
     const int local = item - __ldg(B.tile_begin + i);

@@ -265,7 +265,8 @@ constexpr int TC_THREADS = TC_COPY + 64;         // and the MMA warp and the wei
 constexpr int TC_SLOTS = 16;                     // most stages
 constexpr int TC_HEAD = 1024;                    // shared bytes of the barriers and the bias
 
-// division of 0 <= n < 2^31 by a constant d >= 1: n / d = (n m) >> (32 + s) with 2^s >= d
+// division of 0 <= n < 2^31 by a constant d >= 1 by a multiplication and a shift (Granlund and Montgomery,
+// Division by invariant integers using multiplication, 1994): n / d = ((n m >> 32) + n) >> s with 2^s >= d
 struct FastDiv {
     unsigned m, s, d;
     FastDiv() = default;

@@ -15,7 +15,8 @@ namespace {
 
 // One sub-step, started by programmatic dependent launch behind the lattice kernel or the sub-step
 // before it (on a lattice of one wave of tiles a launch that waits for the end of the former one costs
-// more than the sub-step: 333 x 190, three sub-steps, 42.2 -> 30.3 us per step).  early: the kernel behind this one waits for it before it reads anything.
+// more than the sub-step: 333 x 190, three sub-steps, 42.2 -> 30.3 us per step).  early: the kernel behind
+// this one waits for it before it reads anything.
 __global__ void __launch_bounds__(DNT) k_diffuse(const float* src, float* dst, long long NP, int nx, int ny, float D, int early)
 {
     extern __shared__ __align__(16) float sm[];

@@ -78,7 +78,8 @@ struct NodeArgs {
     int n_ctas;                  // CTAs of a node launch: one per ring, at least one
     const double2* X;            // FP64 master node positions, wrapped into [0, n) (read)
     double2* X_out;              // the advanced positions (written; a different buffer than X when
-                                 // advancing: other CTAs read their halo nodes from X meanwhile)
+                                 // advancing: every tile that meets a ring loads nodes of X ahead of its
+                                 // arrival, while the last one to arrive may be writing)
     int2* node_cell;
     float2* node_frac;
     float2* node_force;
@@ -121,7 +122,7 @@ struct FusedArgs {
     Ctl* ctl;
     int every;                   // readout period
     float* moments_out;          // MOMENTS mode: drho, ux, uy planes, or
-    int moments_only;            // ... with 1 + k the k-th of them alone (0: all three)
+    int moments_only;            // ... with 1 or 2, u_x or u_y alone (0: all three)
     float* forces_out;           // MOMENTS mode, optional: Fx, Fy planes (total lattice force)
     // STEP mode with node_tail = 1: the node step of the same time step runs in the kernel's
     // tail.  Every tile whose staged region meets a ring's work box counts itself in

@@ -35,11 +35,12 @@ constexpr int TILE_X = 32, TILE_Y = 16;   // tile of the single-lattice kernel
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
 constexpr int al4(int x) { return (x + 3) & ~3; }   // 16-byte alignment in floats
 
-// Geometry and shared-memory layout (in floats) of a TX x TY output tile.
 // The early arrival of a small tile at its ring (tile_step, node_tail): what the node step needs of
 // the ring, the tiles that meet it, and whether this one was the last of them.
-enum { AR_BOX = 0, AR_BOX_OFF = 4, AR_COUNT = 6, AR_RING, AR_NODES, AR_OFF, AR_CAP_W, AR_CAP_H, AR_TRAP, AR_LAST, AR_N = 16 };
+enum { AR_BOX = 0, AR_BOX_OFF = 4, AR_COUNT = 6, AR_RING, AR_NODES, AR_OFF, AR_CAP_W, AR_CAP_H, AR_TRAP, AR_LAST,
+       AR_N = 16 };
 
+// Geometry and shared-memory layout (in floats) of a TX x TY output tile.
 template <int TX, int TY>
 struct TileGeo {
     static constexpr int R4W = TX + 8, R4H = TY + 8, R4 = R4W * R4H;
@@ -248,8 +249,8 @@ __device__ __forceinline__ void stage(const FusedArgs& a, const TileMem<TX, TY>&
 
 // ---- IB: gather f_IB on the halo-2 region from the nodes of every ring near the tile ----
 // A node at cell c with fraction f reaches the cells c - 1 .. c + 2 per axis with the weights
-// phi(f + 1), phi(f), phi(f - 1), phi(f - 2).  Each cell sums the nodes in ring and index order, so the result does not depend on the
-// tile.  A ring is taken 256 nodes at a time, one per thread; the chunk's nodes are listed per row
+// phi(f + 1), phi(f), phi(f - 1), phi(f - 2).  Each cell sums the nodes in ring and index order, so the
+// result does not depend on the tile.  A ring is taken 256 nodes at a time, one per thread; the chunk's nodes are listed per row
 // and per column of the region as bit masks, and a cell visits only the nodes in both of its lists
 // (a handful: testing every node of the ring at every cell and evaluating the kernel there made the
 // gather 16 000 of the 28 000 cycles of a tile that holds a ring of 157 nodes).
@@ -466,7 +467,7 @@ __device__ __forceinline__ void moments_out(const FusedArgs& a, const TileMem<TX
         const int j = (ly + 2) * G::R2W + lx + 2;
         const long long g = (long long)gy * a.nx + gx;
         if (IL && a.moments_only) {
-            a.moments_out[g] = a.moments_only == 1 ? m.sM[2 * G::R2 + j] : m.sM[2 * j + a.moments_only - 2];
+            a.moments_out[g] = m.sM[2 * j + a.moments_only - 1];
         } else if (IL) {
             const float2 u = reinterpret_cast<const float2*>(m.sM)[j];
             a.moments_out[g] = m.sM[2 * G::R2 + j];
