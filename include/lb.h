@@ -353,8 +353,8 @@ void lb_destroy(lb_handle* h);
  * equal; the readout sums of the lattice may differ in the last bits with the tile shape).
  *
  * lb_batch_create: handles[0..n-1] (n >= 1) must be distinct, have their fields and bodies set
- *   (lb_init_fields, lb_set_body), use the FP32 state and one model (all tensorial or all scalar), share one stream and be at the same
- *   buffer parity (an equal step count mod 2).  The batch keeps the pointers: the handles must
+ *   (lb_init_fields, lb_set_body), use the FP32 state and one model (all tensorial or all scalar),
+ *   share one stream and be at the same buffer parity (an equal step count mod 2).  The batch keeps the pointers: the handles must
  *   outlive it and must not be stepped with lb_step while it exists.  Readouts (lb_readout,
  *   lb_series, ...) on the handles stay valid and are ordered after the batch's steps.
  *   Returns LB_ESTATE for a handle not ready, LB_EINVAL for a mismatch.
@@ -364,7 +364,8 @@ void lb_destroy(lb_handle* h);
  * lb_batch_set_shape: tile shape of instance inst (-1: all): 0 = 32x16, 1 = 32x8, 2 = 64x8,
  *   3 = 16x16 cells, 4 = the warp-strip kernel (LB_KERNEL_STRIP's step; periodic instances with
  *   nx >= 64 even and ny >= 32, phase launches only, else LB_EINVAL).  lb_batch_shape returns
- *   it (-1 for a bad index).
+ *   it (-1 for a bad index).  When this call, lb_batch_set_persistent or lb_batch_autotune fails with
+ *   LB_ENOMEM or LB_ECUDA, lb_batch_step may return LB_ESTATE until one of them succeeds.
  * lb_batch_autotune: time `steps` steps with each shape that applies, first for the whole batch
  *   (one shape for all untuned sizes), then per distinct lattice size from the best of those,
  *   and keep the fastest; the states are saved and restored, so the simulation does not advance.  cache_path
