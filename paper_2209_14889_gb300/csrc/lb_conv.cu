@@ -504,23 +504,25 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
 #pragma unroll
                         for (int e = 0; e < 16; ++e) f[e] = fmaxf(f[e], SLOPE * f[e]);      // LeakyReLU, 0 < SLOPE < 1
                     }
-                    const bool whole = co0 + j + 16 <= a.Co;
+                    // stores of a whole sector where the address allows, in eights (the last block of a
+                    // channel count that is no multiple of 16 has one), else value by value
+                    const int n8 = min(2, (a.Co - co0 - j) / 8);
                     if (a.yf) {
-                        if (whole && (((uintptr_t)(a.yf + o) | (a.yf2 ? (uintptr_t)(a.yf2 + o) : 0)) & 31) == 0) {
-                            const unsigned(*w)[8] = reinterpret_cast<const unsigned(*)[8]>(f);
-                            st32(a.yf + o, w[0]);
-                            st32(a.yf + o + 8, w[1]);
-                            if (a.yf2) {
-                                st32(a.yf2 + o, w[0]);
-                                st32(a.yf2 + o + 8, w[1]);
-                            }
-                        } else {
+                        const unsigned(*w)[8] = reinterpret_cast<const unsigned(*)[8]>(f);
+                        const bool sect = (((uintptr_t)(a.yf + o) | (a.yf2 ? (uintptr_t)(a.yf2 + o) : 0)) & 31) == 0;
 #pragma unroll
-                            for (int e = 0; e < 16; ++e)
-                                if (co0 + j + e < a.Co) {
+                        for (int q8 = 0; q8 < 2; ++q8) {
+                            if (q8 >= n8) break;
+                            if (sect) {
+                                st32(a.yf + o + 8 * q8, w[q8]);
+                                if (a.yf2) st32(a.yf2 + o + 8 * q8, w[q8]);
+                            } else {
+#pragma unroll
+                                for (int e = 8 * q8; e < 8 * q8 + 8; ++e) {
                                     a.yf[o + e] = f[e];
                                     if (a.yf2) a.yf2[o + e] = f[e];
                                 }
+                            }
                         }
                         continue;
                     }
@@ -538,12 +540,16 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
                         }
                     }
                     const unsigned(&w)[8] = *reinterpret_cast<const unsigned(*)[8]>(r);
-                    if (whole && ((uintptr_t)(a.y + o) & 31) == 0) {
+                    if (n8 == 2 && ((uintptr_t)(a.y + o) & 31) == 0) {
                         st32(a.y + o, w);
+                    } else if (((uintptr_t)(a.y + o) & 15) == 0) {
+                        const uint4* v8 = reinterpret_cast<const uint4*>(r);
+                        if (n8 > 0) reinterpret_cast<uint4*>(a.y + o)[0] = v8[0];
+                        if (n8 > 1) reinterpret_cast<uint4*>(a.y + o)[1] = v8[1];
                     } else {
 #pragma unroll
                         for (int e = 0; e < 16; ++e)
-                            if (co0 + j + e < a.Co) a.y[o + e] = e & 1 ? r[e >> 1].y : r[e >> 1].x;
+                            if (e < 8 * n8) a.y[o + e] = e & 1 ? r[e >> 1].y : r[e >> 1].x;
                     }
                     if (a.up) {                     // the network's own buffers: whole blocks, aligned
 #pragma unroll
