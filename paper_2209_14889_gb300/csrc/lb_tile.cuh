@@ -450,6 +450,9 @@ __device__ __forceinline__ void box_write(const FusedArgs& a, unsigned mask, lon
 // fixed-order reduction of the tile's double-float readout sums into its partial slot
 __device__ __forceinline__ void readout_reduce(const FusedArgs& a, const DF* acc, double* sRed, int tile_index)
 {
+    // a warp with lanes outside a ragged lattice comes here in two halves, and the reduction and the tail behind
+    // it ran once for each (250 x 256 without rings, 16x16 tiles, a readout every step: 19.4 us, 13.9 so)
+    __syncwarp();
     store_partial(a.partials, tile_index, acc, reinterpret_cast<float*>(sRed));
 }
 
