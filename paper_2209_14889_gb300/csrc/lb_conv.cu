@@ -505,7 +505,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
                         for (int e = 0; e < 16; ++e) f[e] = fmaxf(f[e], SLOPE * f[e]);      // LeakyReLU, 0 < SLOPE < 1
                     }
                     // stores of a whole sector where the address allows, in eights (the last block of a
-                    // channel count that is no multiple of 16 has one), else value by value
+                    // channel count that is no multiple of 16 has one, and every second pixel starts
+                    // between sectors), else value by value: 3 x 441 x 395, 32 -> 88 channels 268 us value
+                    // by value, 99 in eights
                     const int n8 = min(2, (a.Co - co0 - j) / 8);
                     if (a.yf) {
                         const unsigned(*w)[8] = reinterpret_cast<const unsigned(*)[8]>(f);
